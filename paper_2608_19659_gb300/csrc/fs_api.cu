@@ -168,7 +168,7 @@ struct fs_model {
   // page-locked staging: the last bounds upload (its copy may still be in
   // flight until up_done), and a synchronous call's outputs and status word
   HostBuf h_up, h_out;
-  cudaEvent_t up_done = nullptr;
+  cudaEvent_t up_done = nullptr, round_done = nullptr;  // (created on first use)
   bool up_pending = false;
   bool staged = false;  // the staging holds bounds the device copy does not have yet
   int th_bound = -1;    // threshold_bound of the current bounds (-1: not computed yet)
@@ -367,7 +367,7 @@ int ensure_items(fs_model* m, int n, int O) {
 }
 
 // The scoring sequence on stream s; cand_dev holds n_cand cell ids.
-int run_score(fs_model* m, const Set& set, const fs_samples* smp, const int32_t* cand_dev, double* gap,
+int run_score(fs_model* m, Set set, const fs_samples* smp, const int32_t* cand_dev, double* gap,
               double* score, float* gamma_t, int32_t* best, void* dump, cudaStream_t s,
               uint32_t* status_copy = nullptr) {
   const int n = smp->n_cand;
@@ -390,9 +390,9 @@ int run_score(fs_model* m, const Set& set, const fs_samples* smp, const int32_t*
   }
   const bool phases = timed && m->timing == 2;
   if (phases) FS_CUDA(cudaEventRecord(ev[0], s), "record timing event");
-  FS_CUDA(launch_solve(set, 2, nullptr, nullptr, nullptr, true, m->lc, s, true), "launch solve");
-  if (phases) FS_CUDA(cudaEventRecord(ev[1], s), "record timing event");
   if (m->th_bound < 0) m->th_bound = threshold_bound(m);
+  FS_CUDA(launch_thresh(set, m->lc.floors, m->th_bound, s), "launch thresholds");
+  if (phases) FS_CUDA(cudaEventRecord(ev[1], s), "record timing event");
   FS_CUDA(launch_prep(set, it, pl, (float*)m->tables.p, (uint64_t*)m->sums.p, true, m->sm_count, m->lc, s,
                       m->th_bound),
           "launch prep");
@@ -507,7 +507,8 @@ int fs_load_model(const fs_bounds* b, const float* slo, const float* demand, int
   const size_t o_theta = take(8 * (size_t)d.theta_cap), o_nth = take(8);
   const size_t o_rowc = take(8 * (size_t)d.K4), o_rowb = take(8 * (size_t)d.K4);
   const size_t o_base = take(2 * sizeof(fs_allocation)), o_status = take(4), o_work = take(32);
-  const size_t o_rtab = take(8 * (size_t)kRowTabMax);
+  const int rt_cap = (int)std::min<long long>((long long)d.K4 * d.theta_cap, kRowTabModel);
+  const size_t o_rtab = take(4 * (size_t)rt_cap), o_tpart = take(8 * (size_t)kThreshBlocks);
   rc = m->fixed.ensure(off, "model state");
   if (rc) {
     delete m;
@@ -530,7 +531,9 @@ int fs_load_model(const fs_bounds* b, const float* slo, const float* demand, int
   s.status = (uint32_t*)(base + o_status);
   s.work = (unsigned long long*)(base + o_work);
   s.skip = nullptr;
-  s.rtab = (int*)(base + o_rtab);
+  s.rtab = (uint16_t*)(base + o_rtab);
+  s.rt_cap = rt_cap;
+  s.tpart = (float*)(base + o_tpart);
 
   m->h_lam.assign(demand, demand + K);
   m->h_slo.assign(slo, slo + K);
@@ -673,7 +676,7 @@ int fs_solve(fs_model* m, const float* cap, const float* tail, fs_allocation* ou
   cudaStream_t s = m->stream;
   FS_CUDA(cudaMemcpyAsync(d_cap, cap, 4 * (size_t)cells, cudaMemcpyHostToDevice, s), "upload cap");
   FS_CUDA(cudaMemcpyAsync(d_tail, tail, 4 * (size_t)cells, cudaMemcpyHostToDevice, s), "upload tail");
-  FS_CUDA(launch_solve(m->set, 1, d_cap, d_tail, d_out, false, m->lc, s), "launch solve");
+  FS_CUDA(launch_solve(m->set, 1, d_cap, d_tail, d_out, m->lc, s), "launch solve");
   if ((rc = solve_lex_pass(m, m->set, 1, d_cap, d_tail, d_out, s))) return rc;
   FS_CUDA(cudaMemcpyAsync(out, d_out, sizeof(fs_allocation), cudaMemcpyDeviceToHost, s), "read allocation");
   return read_status(m, s);
@@ -688,7 +691,7 @@ int fs_solve_batch(fs_model* m, int32_t n, const float* cap_dev, const float* ta
   if (!cap_dev || !tail_dev || !out_dev) return fail(FS_EINVAL, "NULL device pointer");
   int rc = flush_bounds(m, (cudaStream_t)cuda_stream);
   if (rc) return rc;
-  FS_CUDA(launch_solve(m->set, n, cap_dev, tail_dev, out_dev, false, m->lc, (cudaStream_t)cuda_stream),
+  FS_CUDA(launch_solve(m->set, n, cap_dev, tail_dev, out_dev, m->lc, (cudaStream_t)cuda_stream),
           "launch solve");
   return solve_lex_pass(m, m->set, n, cap_dev, tail_dev, out_dev, (cudaStream_t)cuda_stream);
 }
@@ -699,7 +702,7 @@ int fs_solve_bounds(fs_model* m, fs_allocation* minus, fs_allocation* plus, floa
   cudaStream_t s = m->stream;
   int rc0 = flush_bounds(m, s);
   if (rc0) return rc0;
-  FS_CUDA(launch_solve(m->set, 2, nullptr, nullptr, nullptr, true, m->lc, s), "launch solve");
+  FS_CUDA(launch_solve(m->set, 2, nullptr, nullptr, nullptr, m->lc, s), "launch solve");
   if ((rc0 = solve_lex_pass(m, m->set, 2, nullptr, nullptr, nullptr, s))) return rc0;
   fs_allocation h[2];
   FS_CUDA(cudaMemcpyAsync(h, m->set.base, sizeof h, cudaMemcpyDeviceToHost, s), "read allocations");
@@ -812,17 +815,21 @@ int fs_score_goodput(fs_model* m, const fs_samples* smp, double* gap_out, double
     return fail(FS_EINVAL, "the goodput stage needs Q / O <= 2048 under the monotone prior, 4096 otherwise");
   const int saved = m->objective;
   m->objective = FS_OBJECTIVE_LEXICOGRAPHIC;  // the base solves to tier 4 (their goodput)
-  FS_CUDA(launch_solve(m->set, 2, nullptr, nullptr, nullptr, true, m->lc, s), "launch solve");
+  FS_CUDA(launch_solve(m->set, 2, nullptr, nullptr, nullptr, m->lc, s), "launch solve");
   rc = solve_lex_pass(m, m->set, 2, nullptr, nullptr, nullptr, s);
   m->objective = saved;
   if (rc) return rc;
   uint64_t* sums = static_cast<uint64_t*>(m->sums.p);
-  FS_CUDA(launch_prep(m->set, it, pl, static_cast<float*>(m->tables.p), sums, false, m->sm_count, m->lc, s),
+  if (m->th_bound < 0) m->th_bound = threshold_bound(m);
+  Set set = m->set;
+  FS_CUDA(launch_thresh(set, m->lc.floors, m->th_bound, s), "launch thresholds");
+  FS_CUDA(launch_prep(set, it, pl, static_cast<float*>(m->tables.p), sums, false, m->sm_count, m->lc, s,
+                      m->th_bound),
           "launch prep");
-  FS_CUDA(launch_score_goodput(m->set, it, pl, static_cast<const float*>(m->tables.p), sums, m->lc.floors,
+  FS_CUDA(launch_score_goodput(set, it, pl, static_cast<const float*>(m->tables.p), sums, m->lc.floors,
                                m->sm_count, s),
           "launch goodput scorer");
-  FS_CUDA(launch_finalize_goodput(m->set, it, pl, sums, lam_sum, d_gap, d_score, d_gamma, d_best, d_st, s),
+  FS_CUDA(launch_finalize_goodput(set, it, pl, sums, lam_sum, d_gap, d_score, d_gamma, d_best, d_st, s),
           "launch goodput reduction");
   if (sum_eo && n)
     FS_CUDA(cudaMemcpyAsync(sum_eo, sums, 8 * (size_t)n * smp->O, cudaMemcpyDeviceToHost, s), "read sums");
@@ -882,7 +889,8 @@ int fs_replay(fs_model* m, const fs_replay_spec* sp, int32_t* rounds, int32_t* s
   const size_t o_trace = take(4 * (size_t)P * (sp->max_rounds + 1));
   const size_t o_final = take((size_t)P * sizeof(fs_allocation)), o_active = take(4 * (size_t)P), o_nact = take(4);
   const size_t o_ip = take(4 * (size_t)P * cells), o_ic = take(4 * (size_t)P * cells);
-  const size_t o_rtab = take(8 * (size_t)P * kRowTabMax);
+  const int rt_cap = std::min(d.K4 * d.theta_cap, kRowTabMax);
+  const size_t o_rtab = take(4 * (size_t)P * rt_cap);
   const size_t o_prior = take(16 * (size_t)cells);
   Buf& all = m->replay;
   if ((rc = all.ensure(off, "replay state"))) return rc;
@@ -896,7 +904,10 @@ int fs_replay(fs_model* m, const fs_replay_spec* sp, int32_t* rounds, int32_t* s
   set.rowC = (float*)(base + o_rowc);
   set.rowB = (int*)(base + o_rowb);
   set.base = (fs_allocation*)(base + o_base);
-  set.rtab = (int*)(base + o_rtab);
+  set.rtab = (uint16_t*)(base + o_rtab);
+  set.rt_cap = rt_cap;
+  set.tpart = nullptr;
+  set.n_tpart = 0;  // t* comes from the base allocations
   ReplayState rs{};
   rs.truth = (const float*)(base + o_truth);
   rs.perm = (const int*)(base + o_perm);
@@ -916,6 +927,8 @@ int fs_replay(fs_model* m, const fs_replay_spec* sp, int32_t* rounds, int32_t* s
   set.skip = rs.state;
 
   cudaStream_t s = m->stream;
+  if ((rc = m->h_out.ensure(64, "host staging"))) return rc;
+  if (!m->round_done) FS_CUDA(cudaEventCreateWithFlags(&m->round_done, cudaEventDisableTiming), "create round event");
   auto run = [&]() -> int {
     FS_CUDA(cudaMemsetAsync(all.p, 0, off, s), "clear replay state");
     // the prior once; the init kernel gives every stream its copy
@@ -934,14 +947,19 @@ int fs_replay(fs_model* m, const fs_replay_spec* sp, int32_t* rounds, int32_t* s
     const int rc_sync = read_status(m, s);  // truth buffer must outlive the copy
     if (rc_sync) return rc_sync;
     for (int r = 0; r <= sp->max_rounds; ++r) {
-      FS_CUDA(launch_solve(set, 2 * P, nullptr, nullptr, nullptr, true, m->lc, s), "launch solve");
+      FS_CUDA(launch_solve(set, 2 * P, nullptr, nullptr, nullptr, m->lc, s), "launch solve");
       FS_CUDA(cudaMemsetAsync(rs.n_active, 0, 4, s), "clear active");
       const int per = cells - sp->r0 - r;  // candidates of each running stream this round
       // the certificate, and the running streams' candidate lists (scored reveals)
       FS_CUDA(launch_replay_certify(set, rs, r, sp->policy == 0 ? per : 0, s), "launch certify");
-      int n_active = 0;
-      FS_CUDA(cudaMemcpyAsync(&n_active, rs.n_active, 4, cudaMemcpyDeviceToHost, s), "read active");
-      FS_CUDA(cudaStreamSynchronize(s), "round sync");
+      // the thresholds of the streams that go on are queued behind the read of
+      // their count, so that they run while the host learns it
+      FS_CUDA(cudaMemcpyAsync(m->h_out.p, rs.n_active, 4, cudaMemcpyDeviceToHost, s), "read active");
+      FS_CUDA(cudaEventRecord(m->round_done, s), "record round event");
+      if (sp->policy == 0) FS_CUDA(launch_thresh(set, m->lc.floors, 0, s), "launch thresholds");
+      FS_CUDA(cudaEventSynchronize(m->round_done), "round sync");
+      int n_active;
+      std::memcpy(&n_active, m->h_out.p, 4);
       if (n_active == 0) break;
       if (per <= 0) break;
       if (sp->policy == 1) {
@@ -1085,6 +1103,7 @@ void fs_free_model(fs_model* m) {
   m->replay.release();
   for (cudaEvent_t e : m->ev) cudaEventDestroy(e);
   if (m->up_done) cudaEventDestroy(m->up_done);
+  if (m->round_done) cudaEventDestroy(m->round_done);
   m->h_up.release();
   m->h_out.release();
   delete m;

@@ -74,6 +74,16 @@ __device__ __forceinline__ double fixed_mean(unsigned long long v, long long n, 
   return __longlong_as_double((long long)(((unsigned long long)bexp << 52) | (m & ((1ull << 52) - 1ull))));
 }
 
+// t* of base realisation sigma of problem p: the maximum of k_thresh's parts in
+// a scoring call, else the base allocation's. Every lane of the warp gets it.
+__device__ __forceinline__ float base_tstar(const Set& set, int p, int sigma) {
+  if (!set.n_tpart) return __ldg(&set.base[2 * p + sigma].t_star);
+  uint32_t v = 0u;
+  for (int q = threadIdx.x & 31; q < set.n_tpart; q += 32)
+    v = max(v, __float_as_uint(__ldg(set.tpart + (size_t)sigma * set.n_tpart + q)));
+  return __uint_as_float(__reduce_max_sync(0xffffffffu, v));
+}
+
 // Items [beg, end) of problem p, whose first item is pos0 (candidate positions,
 // for the order of equal scores, count from there).
 __device__ inline Best finalize_problem(const Set& set, const Items& it, const Plan& pl, const uint64_t* sums,
@@ -84,7 +94,7 @@ __device__ inline Best finalize_problem(const Set& set, const Items& it, const P
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nwarp = blockDim.x >> 5;
   // inputs are read-only here (written by earlier kernels): every load goes
   // through the read-only path and is issued before any store
-  const float gt = __fsub_rn(__ldg(&set.base[2 * p + 1].t_star), __ldg(&set.base[2 * p].t_star));
+  const float gt = __fsub_rn(base_tstar(set, p, 1), base_tstar(set, p, 0));
   const long long gfix = (long long)fixed40(gt);
   const long long n = (long long)pl.O * pl.S;
   const int log2n = (n & (n - 1)) == 0 ? 63 - __clzll(n) : -1;

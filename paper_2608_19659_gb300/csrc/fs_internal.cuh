@@ -10,6 +10,8 @@
 //   rowC     [P][2][K*4]   f32   best SLO-feasible capacity per (class, TP)
 //   rowB     [P][2][K*4]   i32   its bin (-1: none)
 //   base     [P][2]        fs_allocation
+//   rtab     [P][2][rt_cap] u16  row tables (k_thresh), word (row rho, threshold k) at k K4 + rho
+//   tpart    [2][n_tpart]  f32   scoring calls: each k_thresh block's largest feasible threshold
 //   work     [4]           u64   chunk counter of the Monte-Carlo kernel, the reduction's ticket,
 //                                 table entries evaluated and scenarios that tested their tail
 //                                 gate (both accumulate across calls; the host zeroes them)
@@ -31,15 +33,23 @@ namespace fs {
 
 constexpr int kT = 4;                 // TP degrees {1, 2, 4, 8}
 constexpr int kCostInf = 0x3FFFFFFF;  // "no option covers the threshold"
-constexpr int kSolveThreads = 256;
-constexpr int kSolveThreadsWide = 512;  // a scoring solve of a model with more than 256 cells
+constexpr int kSolveWideMax = 608;    // most realisations solved by a block each (else a warp each)
+constexpr int kThreshThreads = 256;
+constexpr int kThreshBlocks = 64;     // most blocks of k_thresh per realisation
 constexpr int kPrepThreads = 256;
 constexpr int kScoreThreads = 256;
 constexpr int kTableHeader = 20;      // floats before the three table arrays (16-byte multiple)
 constexpr int kSmemTableCap = 256;    // table entries staged in shared memory per realisation (pow2)
-// Row table of a scoring solve: one word per (row, threshold) pair, built when
-// K4 x |Theta| is at most this (else the per-candidate preparation searches).
-constexpr int kRowTabMax = 8192;
+// Row table of a realisation: one word per (row, threshold) pair, kept when K4
+// x |Theta| is at most the set's rt_cap (else the per-candidate preparation
+// searches): a model's own table holds every pair up to kRowTabModel words
+// (2 MB a realisation), the allocation-free path's and a replay stream's
+// kRowTabMax. A word: bits 0-14 the replicas the row may use once the other
+// classes cover the threshold (at most floor(G / tau) <= 32767), bit 15 set if
+// another row of its class covers it.
+constexpr int kRowTabMax = 16384;
+constexpr uint32_t kRowOther = 0x8000u;
+constexpr int kRowTabModel = 1 << 20;
 
 // Table header words (floats unless noted).
 enum : int {
@@ -104,8 +114,10 @@ struct Set {
                              // evaluated and scenarios that tested their tail gate in the Monte-Carlo
                              // kernel (summed over calls, zeroed by the host)
   const int* skip;      // [P] or nullptr: base solves skip problems with skip[p] >= 0
-  int* rtab;            // [P][2][kRowTabMax] or nullptr: row tables of the scoring solves,
-                        // word (row rho, threshold k) at k K4 + rho
+  uint16_t* rtab;       // [P][2][rt_cap]: row tables (k_thresh), word (row rho, threshold k) at k K4 + rho
+  int rt_cap;           // words per row table
+  int n_tpart;          // scoring calls: k_thresh blocks per realisation (0: t* comes from base)
+  float* tpart;         // [2][n_tpart] each block's largest feasible threshold (t* is their maximum)
   int prior;            // interval refit after a measurement: 0 the measured cell only,
                         // 1 also its row's other bins (capacity and tail nondecreasing in load)
 };
@@ -244,47 +256,39 @@ __device__ __forceinline__ bool row_in_range(float c, float lam) {
   return (c == 0.0f || (c >= 0x1p-60f && c <= 0x1p44f)) && in_markstein_range(lam);
 }
 
-// Smallest n in [1, M] with fulfil(n, c) >= t, or 0 if none (fulfil is
-// nondecreasing in n under round-to-nearest). The real-valued answer is
-// t lambda / c; the rounded fulfilment differs from n c / lambda by at most
-// two roundings (relative 2^-22), so for n <= 32767 the answer is within one
-// of ceil(t lambda / c) even with an approximate division. Five candidates
-// around that estimate are tested at once; a plain bisection is kept for the
-// case the bracket does not hold.
-// Replica counts are handled as floats (integers up to 32767 are exact there),
-// so that no integer/float conversion sits on the dependent chain; M is the
-// replica cap as a float.
-template <bool FAST>
-__device__ __forceinline__ int min_replicas_impl(float t, float c, float lam, float rlam, float M) {
-  auto f = [&](float n) { return FAST ? fulfil_fast(n, c, lam, rlam) : fulfil(n, c, lam); };
-  const float fM = f(M);
-  const float y = ceilf(__fdividef(__fmul_rn(t, lam), c));  // estimate only
-  if (!(fM >= t)) return 0;  // also covers c == 0
-  const float n = fminf(fmaxf(y, 1.0f), M);
-  const float a = fmaxf(1.0f, n - 2.0f), b = fminf(M, n + 2.0f);
-  const bool left = a == 1.0f || f(a - 1.0f) < t;
-  const bool right = f(b) >= t;
-  if (left && right) {
-    float r = b;
-#pragma unroll
-    for (int k = 3; k >= 0; --k) {
-      const float v = a + (float)k;
-      if (v < b && f(v) >= t) r = v;
-    }
-    return (int)r;
-  }
+// Smallest n in [1, M] with fulfil(n, c) >= t, or 0 if none, for t > 0 (fulfil
+// is nondecreasing in n under round-to-nearest). The real-valued answer is
+// t lambda / c; the rounded fulfilment differs from n c / lambda by at most two
+// roundings (relative 2^-22), so for n <= 32767 the answer is within one of
+// ceil(t lambda / c) even with an approximate division. Replica counts are
+// handled as floats (integers up to 32767 are exact there), so that no
+// integer/float conversion sits on the dependent chain; M is the replica cap as
+// a float.
+
+// Rows outside Markstein's range, where the estimate may be anything: a
+// bisection. Out of line: such rows are rare, and the kernels that call
+// min_replicas in a latency-bound chain fetch less code without it.
+static __device__ __noinline__ int min_replicas_ieee(float t, float c, float lam, float M) {
+  if (!(fulfil(M, c, lam) >= t)) return 0;  // also covers c == 0
   int lo = 1, hi = (int)M;
   while (lo < hi) {
     const int mid = (lo + hi) >> 1;
-    if (f((float)mid) >= t) hi = mid; else lo = mid + 1;
+    if (fulfil((float)mid, c, lam) >= t) hi = mid; else lo = mid + 1;
   }
   return lo;
 }
 
+// In range, the answer is reached from the estimate by steps of one: two
+// fulfilments when the estimate is right (the bracket of seven tested at once
+// that stood here before took 2.5 times the instructions).
 __device__ __forceinline__ int min_replicas(float t, float c, float lam, float rlam, float M) {
   if (!(M >= 1.0f)) return 0;
-  return row_in_range(c, lam) ? min_replicas_impl<true>(t, c, lam, rlam, M)
-                              : min_replicas_impl<false>(t, c, lam, rlam, M);
+  if (!row_in_range(c, lam)) return min_replicas_ieee(t, c, lam, M);
+  const float y = ceilf(__fdividef(__fmul_rn(t, lam), c));  // estimate only (c == 0: infinite)
+  float n = fminf(fmaxf(y, 1.0f), M);
+  while (n > 1.0f && fulfil_fast(n - 1.0f, c, lam, rlam) >= t) n -= 1.0f;
+  while (n <= M && fulfil_fast(n, c, lam, rlam) < t) n += 1.0f;
+  return n <= M ? (int)n : 0;
 }
 
 // Philox4x32-10 (Salmon, Moraes, Dror, Shaw, SC'11): ten rounds of the 4x32
@@ -467,7 +471,7 @@ cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t s
 constexpr int kScoreVariants = 4;
 struct LaunchCache {
   int floors = 0;  // some class has a floor > 0: launch the kernel instances with floors
-  size_t solve_smem[2] = {0, 0}, prep_smem[4] = {0, 0, 0, 0};
+  size_t prep_smem[4] = {0, 0, 0, 0};
   size_t score_smem[kScoreVariants][4] = {};
   // resident blocks per SM of 256, 128 and 64 threads
   int score_blocks_per_sm[kScoreVariants][4][3] = {};
@@ -477,24 +481,24 @@ cudaError_t launch_qtable(float* qn, int Q, cudaStream_t s);
 // Base or explicit realisations: realisation r of `n` reads cap/tail either
 // from the problem set's bounds (explicit == nullptr: r = 2 p + sigma) or from
 // cap_x / tail_x [n][cells].
-// tstar_only: the allocations' per-class choice is not needed (the scoring
-// call reads only t* and the thresholds); total_gpus is then -1 unless the
-// model has floors.
 cudaError_t launch_solve(const Set& set, int n, const float* cap_x, const float* tail_x,
-                         fs_allocation* out, bool write_theta, LaunchCache& lc, cudaStream_t s,
-                         bool tstar_only = false);
+                         fs_allocation* out, LaunchCache& lc, cudaStream_t s);
+// Sorted thresholds, rows and row tables of both realisations of every
+// problem of the set. th_bound > 0: a bound on either realisation's threshold
+// count (theta_cap otherwise). With set.tpart (one problem) the launch's block
+// count is left in set.n_tpart, and the parts hold t*.
+cudaError_t launch_thresh(Set& set, int floors, int th_bound, cudaStream_t s);
 // early: the candidate ids and bounds were complete before the preceding
 // kernel started, so the bounds-only work may run before the PDL wait.
 // Blocks of 256 threads, or of 64 when the launch holds more than two waves
 // of 256-thread blocks (sm_count SMs): each block is mostly a chain of
 // dependent latencies, so more of them in flight per SM finish sooner.
-// th_cap > 0: a bound on both base solves' threshold counts small enough that
-// the solves build row tables (4K th_cap <= kRowTabMax); shared memory then
-// holds th_cap thresholds instead of theta_cap, so that more blocks fit an SM
-// (a count above it is reported as ST_TABLE, never read past).
+// th_bound > 0: a bound on both realisations' threshold counts. Where it (or
+// theta_cap) guarantees row tables, no shared memory is set aside for the
+// search without one (a count above it is reported as ST_TABLE).
 cudaError_t launch_prep(const Set& set, const Items& it, const Plan& pl, float* tables,
                         uint64_t* sums, bool early, int sm_count, LaunchCache& lc, cudaStream_t s,
-                        int th_cap = 0);
+                        int th_bound = 0);
 cudaError_t launch_score(const Set& set, const Items& it, const Plan& pl, const float* tables,
                          uint64_t* sums, void* dump, int dump_stride, int sm_count, LaunchCache& lc,
                          cudaStream_t s);

@@ -26,10 +26,10 @@
 //
 // k_prep builds, per (candidate, realisation), the part of that table a
 // scenario can reach: Theta entries with kappa in (Cexcl, max(Cexcl, cap_hi_e)].
-// m(t) and "P(t) <= A(t)" depend only on (r, t): a scoring solve tabulates
-// them per realisation (the row table, k_solve), and k_prep then finds the
-// range's ends as counts of feasible thresholds and each kappa by one thread;
-// without a table it searches, evaluating the rows per probe.
+// m(t) and "P(t) <= A(t)" depend only on (r, t): k_thresh tabulates them per
+// realisation (the row table), and k_prep then finds the range's ends as counts
+// of feasible thresholds and each kappa by one thread; without a table it
+// searches, evaluating the rows per probe.
 // It also maps each outcome's quantile stratum into the candidate's capacity
 // interval and records where the stratum's tail values stop passing the SLO
 // (the map is monotone, so the gate of Eq. 5 is a position test).
@@ -159,10 +159,9 @@ __device__ __forceinline__ float tstar_of(float C, const float* kap, const float
 // critical (the model has floors).
 template <bool FL, bool RF>
 __global__ void __launch_bounds__(kPrepThreads) k_prep(Set set, Items it, Plan pl, float* rec,
-                                                       uint64_t* sums, int early, int th_cap) {
+                                                       uint64_t* sums, int early, int sure) {
   extern __shared__ __align__(16) unsigned char smraw[];
-  float* sC = reinterpret_cast<float*>(smraw);  // [256]
-  float* sTh = sC + 256;                          // [th_cap]
+  float* sTh = reinterpret_cast<float*>(smraw);  // [theta_cap], unless a table beyond a thread each is sure
   __shared__ float s_cx, s_cmax, s_pc, s_po, s_lf, s_hf;
   __shared__ int s_bx, s_row;
   __shared__ float sLam[FS_MAX_CLASSES], sRl[FS_MAX_CLASSES];  // demand and RN(1/demand)
@@ -347,63 +346,80 @@ __global__ void __launch_bounds__(kPrepThreads) k_prep(Set set, Items it, Plan p
       }
     }
   }
-  if (early) pdl_wait();  // thresholds and rows come from k_solve
+  if (early) pdl_wait();  // thresholds and rows come from k_thresh
 
   const size_t ps = (size_t)p * 2 + sigma;
   const float* th_g = set.theta + ps * d.theta_cap;
-  // this candidate's row of the base solve's row table (word k at k K4), when
-  // the solve built one; with at most one threshold per thread and a table
-  // that holds every threshold the model allows, each thread loads its
-  // threshold and word together with the count (one memory round trip; the
-  // entries past the count are never used)
-  const int* rt_g = set.rtab ? set.rtab + ps * kRowTabMax + rr : nullptr;
-  const bool ahead = d.theta_cap <= (int)blockDim.x && d.K4 * d.theta_cap <= kRowTabMax;
+  // this candidate's row of the realisation's row table (word k at k K4). With
+  // at most one threshold per thread and a table that holds every threshold the
+  // model allows (`ahead`), each thread loads its threshold and word together
+  // with the count (one memory round trip; the entries past the count are never
+  // used); a longer table is read where it is, a search's probes only; without a
+  // table the thresholds are staged for the search.
+  const uint16_t* rt_g = set.rtab + ps * set.rt_cap + rr;
+  const bool ahead = d.theta_cap <= (int)blockDim.x && d.K4 * d.theta_cap <= set.rt_cap;
   float th_a = 0.0f;
-  int rt_a = 0;
+  uint16_t rt_a = 0;
   if (ahead && tid < d.theta_cap) {
     th_a = th_g[tid];
-    if (rt_g) rt_a = rt_g[(size_t)tid * d.K4];
+    rt_a = rt_g[(size_t)tid * d.K4];
   }
-  // a count above the launch's bound (reported below; the call then fails) is
-  // cut to it, so that no index passes the shared arrays
-  const int total_raw = set.ntheta[ps];
-  const int total = min(total_raw, th_cap);
-  const bool rtab = rt_g != nullptr && d.K4 * total <= kRowTabMax;
-  int* sRt = reinterpret_cast<int*>(sTh + th_cap);  // [min(th_cap, kRowTabMax / 4)]
-  for (int rho = tid; rho < d.K4; rho += blockDim.x) sC[rho] = set.rowC[ps * d.K4 + rho];
+  const int total = set.ntheta[ps];
+  const bool rtab = d.K4 * total <= set.rt_cap;
+  if (sure && !rtab) {  // the host's bound on the count was wrong: the call fails
+    if (tid == 0) atomicOr(set.status, ST_TABLE);
+    return;
+  }
+  const float* th = th_g;  // the thresholds, and with a table the row's words (stride rts)
+  const uint16_t* rt = rt_g;
+  int rts = d.K4;
+  float* sC = sTh + d.theta_cap;  // [K4] (without a table)
   if (ahead) {
+    uint16_t* sRt = reinterpret_cast<uint16_t*>(sTh + d.theta_cap);  // [theta_cap]
     if (tid < total) {
       sTh[tid] = th_a;
-      if (rtab) sRt[tid] = rt_a;  // (the words' shared array exists only with a table)
+      sRt[tid] = rt_a;
     }
-  } else {
-    for (int k = tid; k < total; k += blockDim.x) {
-      sTh[k] = th_g[k];
-      if (rtab) sRt[k] = rt_g[(size_t)k * d.K4];
-    }
+    th = sTh;
+    rt = sRt;
+    rts = 1;
+  } else if (!rtab) {
+    for (int rho = tid; rho < d.K4; rho += blockDim.x) sC[rho] = set.rowC[ps * d.K4 + rho];
+    for (int k = tid; k < total; k += blockDim.x) sTh[k] = th_g[k];
+    th = sTh;
   }
   __syncthreads();
-  if (total_raw > th_cap && tid == 0) atomicOr(set.status, ST_TABLE);
   const float cx = s_cx, cmax = s_cmax;
   const int msent = d.K == 1 ? rep_cap(d, jr) : 0;  // above every threshold only a lone class can go on
 
   // b0: last index feasible at Cexcl; b1: last index feasible at max(Cexcl, cap_hi).
   // Feasibility is nonincreasing along the sorted thresholds, so with the row
-  // table each is the count of feasible indices less one (one barrier per 256
-  // indices); without it, a joint search.
+  // table each is the count of feasible indices less one: block-wide counts over
+  // the indices, after one over evenly spaced indices where there are more of
+  // them than threads; without it, a joint search.
   int b0, b1;
   if (rtab) {
-    int n0 = 0, n1 = 0;
-    for (int k0 = 0; k0 < total; k0 += blockDim.x) {
-      const int k = k0 + tid;
-      bool f0 = false, f1 = false;
-      if (k < total) {
-        const int e = sRt[k], m = e & 0xFFFF;
-        const bool other = (e >> 16) & 1;
-        const float te = FL ? fmaxf(sTh[k], dle) : sTh[k];
-        f0 = other || (m >= 1 && fulfil_r((float)m, cx, lam, rl) >= te);
-        f1 = other || (m >= 1 && fulfil_r((float)m, cmax, lam, rl) >= te);
-      }
+    auto feas = [&](int k, float C) {
+      const uint32_t e = rt[(size_t)k * rts], m = e & (kRowOther - 1u);
+      const float te = FL ? fmaxf(th[k], dle) : th[k];
+      return (e & kRowOther) || (m >= 1 && fulfil_r((float)m, C, lam, rl) >= te);
+    };
+    const int T = (int)blockDim.x;
+    int lo0 = 0, hi0 = total, lo1 = 0, hi1 = total;  // [lo, hi): indices not settled yet, all below lo feasible
+    if (total > T) {
+      auto at = [&](int q) { return (int)(((long long)(q + 1) * total) / (T + 1)); };
+      const int k = at(tid);
+      const int c0 = __syncthreads_count(feas(k, cx)), c1 = __syncthreads_count(feas(k, cmax));
+      if (c0) lo0 = at(c0 - 1) + 1;
+      if (c0 < T) hi0 = at(c0);
+      if (c1) lo1 = at(c1 - 1) + 1;
+      if (c1 < T) hi1 = at(c1);
+    }
+    int n0 = lo0, n1 = lo1;
+    const int span = max(hi0 - lo0, hi1 - lo1);
+    for (int k0 = tid; k0 < span + tid; k0 += T) {
+      const int ka = lo0 + k0, kb = lo1 + k0;
+      const bool f0 = ka < hi0 && feas(ka, cx), f1 = kb < hi1 && feas(kb, cmax);
       n0 += __syncthreads_count(f0);
       n1 += __syncthreads_count(f1);
     }
@@ -467,12 +483,12 @@ __global__ void __launch_bounds__(kPrepThreads) k_prep(Set set, Items it, Plan p
     const uint32_t bx = __float_as_uint(cx) & 0x7fffffffu, bmax = __float_as_uint(cmax) & 0x7fffffffu;
     for (int u = tid; u <= Lt; u += blockDim.x) {
       const int k = b0 + 1 + u;
-      const int m = k < total ? (sRt[k] & 0xFFFF) : msent;
+      const int m = k < total ? (int)(rt[(size_t)k * rts] & (kRowOther - 1u)) : msent;
       if (u < Lt) {
-        const float th = sTh[k], t = FL ? fmaxf(th, dle) : th;
+        const float tk = th[k], t = FL ? fmaxf(tk, dle) : tk;
         const float c0 = __fdividef(__fmul_rn(t, lam), (float)m);  // an estimate: the walk is exact
         kap[u] = __uint_as_float(kappa_walk((float)m, t, lam, rl, bx, bmax, __float_as_uint(c0)));
-        thx[u + 1] = th;
+        thx[u + 1] = tk;
       }
       if (m >= 1) s_row = 1;
       mnx[u] = (float)m;
@@ -493,7 +509,7 @@ __global__ void __launch_bounds__(kPrepThreads) k_prep(Set set, Items it, Plan p
         // the values). First the 32 patterns around the real solution t lambda / m,
         // one per lane; if the answer is not among them, a 32-ary search over the
         // whole interval.
-        const float th = sTh[k], t = FL ? fmaxf(th, dle) : th;
+        const float tk = sTh[k], t = FL ? fmaxf(tk, dle) : tk;
         // Cexcl = -0 as +0 (the same smallest capacity), as in the table branch
         const uint32_t bx = __float_as_uint(cx) & 0x7fffffffu, bmax = __float_as_uint(cmax) & 0x7fffffffu;
         const float c0 = __fdividef(__fmul_rn(t, lam), (float)m);  // an estimate: the window is checked exactly
@@ -519,7 +535,7 @@ __global__ void __launch_bounds__(kPrepThreads) k_prep(Set set, Items it, Plan p
         }
         if (lane == 0) {
           kap[u] = __uint_as_float(hi);
-          thx[u + 1] = th;
+          thx[u + 1] = tk;
         }
       }
       if (lane == 0) {
@@ -535,7 +551,7 @@ __global__ void __launch_bounds__(kPrepThreads) k_prep(Set set, Items it, Plan p
       mnx[u] = 0.0f;
     }
   }
-  if (tid == 0) thx[0] = b0 >= 0 ? sTh[b0] : 0.0f;
+  if (tid == 0) thx[0] = b0 >= 0 ? th[b0] : 0.0f;
   __syncthreads();
   if (tid == 0) {
     // every row-term quotient x / lambda of a scenario has x = m C' with
@@ -544,7 +560,7 @@ __global__ void __launch_bounds__(kPrepThreads) k_prep(Set set, Items it, Plan p
     // (under the prior every C' lies in [cx, cmax])
     const bool fast = in_markstein_range(lam) && cmax <= 0x1p44f &&
                       (cx >= 0x1p-60f || (!RF && cx == 0.0f && (lo_c >= 0x1p-60f || hi_c == 0.0f)));
-    tab[H_TH_BASE] = b0 >= 0 ? sTh[b0] : 0.0f;
+    tab[H_TH_BASE] = b0 >= 0 ? th[b0] : 0.0f;
     // t* at row capacity Cexcl (no kappa entry is at or below it): the value of
     // every scenario of this candidate whose tail gate is closed
     tab[H_TCL] = tstar_of<2, FL>(cx, kap, thx, mnx, Lt ? P >> 1 : 0, lam, rl, dle);
@@ -1163,9 +1179,12 @@ __global__ void __launch_bounds__(kScoreThreads, 4) k_score(Set set, Items it, P
   }
 }
 
+// (both reductions let the next call's first kernel be placed while they run:
+// it waits for their completion before it reads or writes anything)
 __global__ void k_finalize(Set set, Items it, Plan pl, const uint64_t* sums, double* gap, double* score,
                            float* gamma_t, int32_t* best, uint32_t* status_copy) {
   pdl_wait();
+  pdl_trigger();
   const int p = blockIdx.x;
   const int beg = it.off ? it.off[p] : 0;
   const int end = it.off ? it.off[p + 1] : it.n;
@@ -1182,6 +1201,7 @@ __global__ void k_finalize(Set set, Items it, Plan pl, const uint64_t* sums, dou
 __global__ void k_finalize_split(Set set, Items it, Plan pl, const uint64_t* sums, double* gap, double* score,
                                  float* gamma_t, int32_t* best, uint32_t* status_copy, uint64_t* part) {
   pdl_wait();
+  pdl_trigger();
   const int nb = (int)gridDim.x, per = (it.n + nb - 1) / nb;
   const int beg = min(it.n, (int)blockIdx.x * per), end = min(it.n, beg + per);
   const Best b = finalize_problem(set, it, pl, sums, 0, beg, end, gap, score,
@@ -1209,18 +1229,18 @@ __global__ void k_finalize_split(Set set, Items it, Plan pl, const uint64_t* sum
   }
 }
 
-// rowC, the thresholds and, with a row table, the candidate row's words
-static size_t prep_smem_bytes(const Set& set, int th_cap) {
-  return (size_t)(256 + th_cap + (set.rtab ? std::min(th_cap, kRowTabMax / 4) : 0)) * 4;
-}
-
 cudaError_t launch_prep(const Set& set, const Items& it, const Plan& pl, float* tables, uint64_t* sums,
-                        bool early, int sm_count, LaunchCache& lc, cudaStream_t s, int th_cap) {
+                        bool early, int sm_count, LaunchCache& lc, cudaStream_t s, int th_bound) {
   if (it.n <= 0) return cudaSuccess;
   const Dims& d = set.d;
-  const int cap = th_cap > 0 && th_cap < d.theta_cap && set.rtab && d.K4 * th_cap <= kRowTabMax ? th_cap
-                                                                                                   : d.theta_cap;
-  const size_t smem = prep_smem_bytes(set, cap);
+  const int bound = th_bound > 0 ? std::min(th_bound, d.theta_cap) : d.theta_cap;
+  const bool sure = (long long)d.K4 * bound <= set.rt_cap;  // both realisations have row tables
+  // (five 256-thread blocks fit an SM by registers; 64-thread blocks need at
+  // least 64 threads for the classes' demands, K <= 64)
+  const int tb = (long long)it.n * 2 > 2LL * 5 * sm_count ? 64 : kPrepThreads;
+  const bool ahead = d.theta_cap <= tb && d.K4 * d.theta_cap <= set.rt_cap;
+  // thresholds with the row's words or (a search) the rows; nothing for a table read in place
+  const size_t smem = ahead ? 6 * (size_t)d.theta_cap : sure ? 16 : 4 * (size_t)(d.theta_cap + d.K4);
   const int fl = lc.floors ? 1 : 0, mode = fl + (set.prior == 1 ? 2 : 0);
   auto kern = mode == 0 ? k_prep<false, false> : mode == 1 ? k_prep<true, false>
             : mode == 2 ? k_prep<false, true> : k_prep<true, true>;
@@ -1229,10 +1249,7 @@ cudaError_t launch_prep(const Set& set, const Items& it, const Plan& pl, float* 
     if (e != cudaSuccess) return e;
     lc.prep_smem[mode] = smem;
   }
-  // (five 256-thread blocks fit an SM by registers; 64-thread blocks need at
-  // least 64 threads for the classes' demands, K <= 64)
-  const int tb = (long long)it.n * 2 > 2LL * 5 * sm_count ? 64 : kPrepThreads;
-  return launch_pdl(kern, dim3(it.n * 2), dim3(tb), smem, s, set, it, pl, tables, sums, early ? 1 : 0, cap);
+  return launch_pdl(kern, dim3(it.n * 2), dim3(tb), smem, s, set, it, pl, tables, sums, early ? 1 : 0, sure ? 1 : 0);
 }
 
 static int score_lcap(const Dims& d) { return d.lcap < kSmemTableCap ? d.lcap : kSmemTableCap; }

@@ -1,36 +1,38 @@
 // Allocation solver (Section 3, Eqs. 1-5; tier 2 of the objective) and the
 // quantile table, for sm_103a.
 //
-// One CTA solves one realisation (a capacity and a tail value per cell):
+// One warp (or, for a few realisations, one block of eight) solves one
+// realisation (a capacity and a tail value per cell):
 //   1. rows: for every (class i, TP index j) the best SLO-feasible bin
-//      (largest capacity, then lowest bin; Eq. 5 gates l <= L_i) -> C_ij.
-//      All cells are read once, coalesced; a 32-bit shared-memory atomicMax
-//      of the feasible cells' capacity bits per row, then an atomicMin of the
-//      bins that hold that capacity (a 64-bit atomicMax of (capacity, -bin)
-//      is no native operation: under contention it measured 15x slower);
-//   2. thresholds: the positive fulfilments f(n, C_ij), n = 1..floor(G/tau_j)
-//      (cut at the first n with f = 1), written to shared memory and
-//      bitonic-sorted;
-//   3. t*: the largest threshold t whose cheapest per-class covers fit in G.
-//      A scoring solve tabulates every row's cover of every threshold (the
-//      row table the per-candidate preparation reads) and counts; otherwise a
-//      search, each probe one group of lanes (a row per lane, shuffles for the
-//      per-class minimum over the four TP lanes and the sum), the groups of the
-//      CTA probing evenly spaced points per round;
-//   4. choice at t*: per class the cheapest cover, ties to the lower TP.
+//      (largest capacity, then lowest bin; Eq. 5 gates l <= L_i) -> C_ij;
+//   2. t*: the largest threshold t whose cheapest per-class covers fit in G,
+//      the thresholds being the rows' positive fulfilments f(n, C_ij), n =
+//      1..floor(G/tau_j). The covers of t change only just above a threshold,
+//      so t fits exactly when the smallest threshold at or above it does, and
+//      t* is found without a list of thresholds: a search over the bit
+//      patterns of t, each probe one group of lanes (a row per lane, shuffles
+//      for the per-class minimum over the four TP lanes and the sum). The
+//      probes also count the thresholds below them, so the search ends when
+//      one threshold is left between the last t that fits and the first that
+//      does not: t* is the smallest threshold at or above the former;
+//   3. choice at t*: per class the cheapest cover, ties to the lower TP.
 // For a fixed (TP, n) a larger capacity never lowers f, so the best bin of
-// each row is the option the tie rule (larger capacity, then lower bin)
-// picks; and t* is the largest threshold t of the rows' values at which the
-// total fits, as cost(t) is constant between consecutive thresholds.
-// Critical floors (tier 1 of the objective): a row of a critical class i
-// starts at its first fulfilment >= delta_i (lower ones are not options), and
-// class i covers max(t, delta_i) at threshold t. Step 4 also prices every
-// critical class's cheapest cover of its floor: the floors are met when those
-// fit in G together; with t* = 0 and the floors met, that cover is the
-// class's allocation.
+// each row is the option the tie rule (larger capacity, then lower bin) picks.
+// Critical floors (tier 1 of the objective): options of a critical class i
+// below delta_i are none, so it covers max(t, delta_i) at threshold t. Step 3
+// also prices every critical class's cheapest cover of its floor: the floors
+// are met when those fit in G together; with t* = 0 and the floors met, that
+// cover is the class's allocation.
+// What bounds it: the dependent chain of about a dozen probes (latency for a
+// few realisations, issue slots for a batch). Before, a 256-thread block per
+// realisation listed and sorted the thresholds first; measured: see
+// launch_solve.
 #include <cuda_runtime.h>
 
+#include <cstddef>
+
 #include "fs_internal.cuh"
+#include "fs_rows.cuh"
 
 namespace fs {
 
@@ -49,25 +51,31 @@ __global__ void k_qtable(float* qn, int Q) {
   qn[k] = x;
 }
 
-// Total GPUs of the cheapest per-class covers of threshold t (class i covers
-// max(t, delta_i)), or kCostInf if some class has no cover, evaluated by an
-// aligned group of gsz lanes (a power of two in [4, 32]); lane gl takes rows
-// gl, gl + gsz, ... (rho = 4 i + j).
-// After the per-class minimum (two xor-shuffles) all four lanes of a class
-// hold its cost; xor-sums over the offsets 4 .. gsz/2 then add one lane per
-// class, so every lane of the group ends with the total (uncovered classes
-// counted above bit 24: a cost is at most G <= 32767, 64 classes < 2^21).
+// One realisation's state shared by its lanes (NW > 1, or more than 32 rows).
+struct SolveSmem {
+  float C[256], lam[FS_MAX_CLASSES], rl[FS_MAX_CLASSES], dl[FS_MAX_CLASSES];
+  int bin[256];
+  int4 end[16];  // per warp, alternate rounds: the search's ends and their sums
+  fs_allocation out;
+};
+
+constexpr uint32_t kAboveOne = 0x3F800001u;  // the float pattern after 1
+
+// Covers of threshold t by one aligned group of gsz lanes, lane gl taking rows
+// gl, gl + gsz, ...: the classes' cheapest covers summed (an uncovered class
+// counted as 2^24: a cost is at most G <= 32767, 64 of them stay below 2^21)
+// and `below`, the rows' first covering counts summed (M + 1 for a row that
+// does not cover t), which differ between two thresholds by the number of
+// option fulfilments in between. Every lane of the group gets both.
 template <bool FL>
-__device__ __forceinline__ int group_total_cost(float t, const float* sC, const float* sLam, const float* sRl,
-                                                const float* sDl, const Dims& d, int gl, int gsz) {
-  int packed = 0;
+__device__ __forceinline__ int group_cover(float t, const SolveSmem& sm, const Dims& d, int gl, int gsz, int* below) {
+  int packed = 0, u = 0;
   for (int base = 0; base < d.K4; base += gsz) {
-    const int rho = base + gl;
+    const int rho = base + gl, j = rho & 3, i = rho >> 2;
     int cost = kCostInf;
     if (rho < d.K4) {
-      const int j = rho & 3;
-      const float tc = FL ? fmaxf(t, sDl[rho >> 2]) : t;
-      const int n = min_replicas(tc, sC[rho], sLam[rho >> 2], sRl[rho >> 2], rep_capf(d, j));
+      const int n = min_replicas(FL ? fmaxf(t, sm.dl[i]) : t, sm.C[rho], sm.lam[i], sm.rl[i], rep_capf(d, j));
+      u += n ? n : rep_cap(d, j) + 1;
       if (n) cost = n << j;
     }
     cost = min(cost, __shfl_xor_sync(0xffffffffu, cost, 1));
@@ -76,37 +84,72 @@ __device__ __forceinline__ int group_total_cost(float t, const float* sC, const 
     for (int off = 4; off < gsz; off <<= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
     packed += v;
   }
-  return (packed >> 24) ? kCostInf : packed;
+  for (int off = 1; off < gsz; off <<= 1) u += __shfl_xor_sync(0xffffffffu, u, off);
+  *below = u;
+  return packed;
 }
 
-// FL: some class is critical (the model has floors); the instance without floors does
-// none of the floor work.
-template <bool FL>
-__global__ void __launch_bounds__(kSolveThreadsWide) k_solve(Set set, int n_real, const float* cap_x,
-                                                         const float* tail_x, fs_allocation* out_x,
-                                                         int mode) {
-  const bool write_theta = (mode & 1) != 0;
-  // the per-class choice at t* (step 4); a scoring call needs only t* and the
-  // thresholds, and without floors skips it
-  const bool choice = FL || (mode & 2) == 0;
-  extern __shared__ __align__(16) unsigned char smraw[];
+// Estimates of t* (patterns in [1, that of 1], aim_lo <= aim_hi) that start the
+// search; they only place the first probes. With replica counts real numbers,
+// class i takes t min_j tau_j lambda_i / C_ij GPUs, so t* is at most G over the
+// sum of those (aim_hi, with a margin for rounding); rounding the counts up adds
+// at most the chosen TP degrees (aim_lo). One warp; every lane gets both.
+__device__ __forceinline__ void search_aims(const SolveSmem& sm, const Dims& d, int lane, uint32_t& aim_lo,
+                                            uint32_t& aim_hi) {
+  float rate = 0.0f, extra = 0.0f;
+  for (int base = 0; base < d.K4; base += 32) {
+    const int rho = base + lane;
+    const float inf = __int_as_float(0x7f800000);
+    float c = inf;
+    if (rho < d.K4 && sm.C[rho] > 0.0f) c = __fdividef(sm.lam[rho >> 2] * (float)(1 << (rho & 3)), sm.C[rho]);
+    float m = fminf(c, __shfl_xor_sync(0xffffffffu, c, 1));
+    m = fminf(m, __shfl_xor_sync(0xffffffffu, m, 2));
+    const uint32_t who = (__ballot_sync(0xffffffffu, c == m) >> (lane & 28)) & 15u;  // the class's cheapest degrees
+    if ((lane & 3) == 0 && rho < d.K4) {
+      rate += m;
+      extra += (float)(1 << (__ffs(who | 8u) - 1));
+    }
+  }
+  for (int o = 16; o; o >>= 1) {
+    rate += __shfl_xor_sync(0xffffffffu, rate, o);
+    extra += __shfl_xor_sync(0xffffffffu, extra, o);
+  }
+  const float G = (float)d.G;
+  const float top = fminf(1.0f, __fdividef(G, rate) * 1.0001f);  // (0 when some class has no option)
+  const float bottom = top * fmaxf(0.25f, 1.0f - __fdividef(extra, G));
+  aim_hi = min(max(__float_as_uint(top), 1u), 0x3F800000u);
+  aim_lo = min(max(__float_as_uint(bottom), 1u), aim_hi);
+}
+
+// FL: some class is critical (the model has floors). NW warps per realisation:
+// 1 (four realisations a block) for batches, 8 for a few realisations, whose
+// latency counts: the rows and the probes are then spread over the warps.
+template <bool FL, int NW>
+__global__ void __launch_bounds__(NW == 1 ? 128 : 32 * NW) k_solve(Set set, int n_real, const float* cap_x,
+                                                                   const float* tail_x, fs_allocation* out_x) {
+  constexpr int kPerBlock = NW == 1 ? 4 : 1;  // realisations per block
+  __shared__ SolveSmem smem[kPerBlock];
   const Dims& d = set.d;  // kernel-parameter space: no local copy
-  const int r = blockIdx.x;
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int lane = threadIdx.x & 31, warp = NW == 1 ? 0 : (int)threadIdx.x >> 5;
+  const int slot = NW == 1 ? (int)threadIdx.x >> 5 : 0, ltid = warp * 32 + lane;
+  SolveSmem& sm = smem[slot];
+  const int r = (int)blockIdx.x * kPerBlock + slot;
   pdl_trigger();
   if (r >= n_real) return;
+  auto sync = [] {
+    if (NW == 1) __syncwarp();
+    else __syncthreads();
+  };
 
   const float* cap;
   const float* tail;
-  int p = 0, sigma = 0;
   fs_allocation* out;
   if (cap_x) {
     cap = cap_x + (size_t)r * d.cells;
     tail = tail_x + (size_t)r * d.cells;
     out = out_x + r;
   } else {
-    p = r >> 1;
-    sigma = r & 1;
+    const int p = r >> 1, sigma = r & 1;
     if (set.skip && set.skip[p] >= 0) return;
     const float* bp = set.bounds + (size_t)p * 4 * d.cells;
     cap = bp + (size_t)(sigma ? CAP_HI : CAP_LO) * d.cells;
@@ -114,409 +157,146 @@ __global__ void __launch_bounds__(kSolveThreadsWide) k_solve(Set set, int n_real
     out = set.base + r;
   }
 
-  uint32_t* sRowCap = reinterpret_cast<uint32_t*>(smraw);  // [256] best feasible capacity bits per row
-  uint32_t* sRowBin = sRowCap + 256;                       // [256] lowest bin holding it (~0u: none)
-  float* sC = reinterpret_cast<float*>(sRowBin + 256);    // [256]
-  int* sB = reinterpret_cast<int*>(sC + 256);             // [256]
-  int* sN0 = sB + 256;                                    // [256]
-  int* sOff = sN0 + 256;                                  // [260]
-  int* sProbe = sOff + 260;                               // [32]
-  int* sMisc = sProbe + 32;                               // [8]
-  float* sTheta = reinterpret_cast<float*>(sMisc + 8);    // [pow2 >= theta_cap]
+  // 1. rows
+  for (int i = ltid; i < d.K; i += 32 * NW) {
+    const float lam = set.lam[i];
+    sm.lam[i] = lam;
+    sm.rl[i] = __frcp_rn(lam);
+    if (FL) sm.dl[i] = set.slo[d.K + i];
+  }
+  best_rows<NW>(d, cap, tail, set.slo, warp, lane, sm.C, sm.bin);
+  sync();
 
-  // 1. rows: the best SLO-feasible bin of each row (largest capacity, then
-  // lowest bin). The inputs of the first pass (demands, and each thread's
-  // first kPre cells, every cell of a model with at most kPre x 256) are all
-  // loaded before anything waits on one of them: one memory round trip. Both
-  // passes read those cells from registers; any further cells from memory.
-  __shared__ float sLam[FS_MAX_CLASSES], sRl[FS_MAX_CLASSES];  // demand and RN(1/demand)
-  __shared__ float sDl[FS_MAX_CLASSES];                          // floor delta_i (0: not critical)
-  constexpr int kPre = 4;
-  const float lam_v = tid < d.K ? set.lam[tid] : 1.0f;
-  const float dl_v = FL && tid < d.K ? set.slo[d.K + tid] : 0.0f;
-  float tailp[kPre], capp[kPre], slop[kPre];
-#pragma unroll
-  for (int k = 0; k < kPre; ++k) {
-    const int c = tid + k * (int)blockDim.x;
-    const bool in = c < d.cells;
-    tailp[k] = in ? tail[c] : 0.0f;
-    capp[k] = in ? cap[c] : 0.0f;
-    slop[k] = in ? set.slo[(c / d.B) >> 2] : 0.0f;
-  }
-  for (int rho = tid; rho < d.K4; rho += blockDim.x) {
-    sRowCap[rho] = 0u;
-    sRowBin[rho] = ~0u;
-  }
-  if (tid < 8) sMisc[tid] = 0;
-  if (tid < d.K) {
-    sLam[tid] = lam_v;
-    sRl[tid] = __frcp_rn(lam_v);
-    if (FL) sDl[tid] = dl_v;
-  }
-  __syncthreads();
-  // feasible cells: their capacity's bits (-0 -> +0: nonnegative floats order
-  // like their bit patterns), first the row maximum, then the lowest bin
-  // holding it
-  bool okp[kPre];
-  uint32_t cbp[kPre];
-  int rhop[kPre];
-#pragma unroll
-  for (int k = 0; k < kPre; ++k) {
-    const int c = tid + k * (int)blockDim.x;
-    rhop[k] = c < d.cells ? c / d.B : 0;
-    okp[k] = c < d.cells && tailp[k] <= slop[k];
-    cbp[k] = __float_as_uint(__fadd_rn(capp[k], 0.0f));
-    if (okp[k]) atomicMax(&sRowCap[rhop[k]], cbp[k]);
-  }
-  const int c_rest = tid + kPre * (int)blockDim.x;
-  for (int c = c_rest; c < d.cells; c += blockDim.x) {
-    const int rho = c / d.B;
-    if (tail[c] <= set.slo[rho >> 2]) atomicMax(&sRowCap[rho], __float_as_uint(__fadd_rn(cap[c], 0.0f)));
-  }
-  __syncthreads();
-#pragma unroll
-  for (int k = 0; k < kPre; ++k) {
-    const int c = tid + k * (int)blockDim.x;
-    if (okp[k] && cbp[k] == sRowCap[rhop[k]]) atomicMin(&sRowBin[rhop[k]], (uint32_t)(c - rhop[k] * d.B));
-  }
-  for (int c = c_rest; c < d.cells; c += blockDim.x) {
-    const int rho = c / d.B;
-    const uint32_t cb = __float_as_uint(__fadd_rn(cap[c], 0.0f));
-    if (tail[c] <= set.slo[rho >> 2] && cb == sRowCap[rho]) atomicMin(&sRowBin[rho], (uint32_t)(c - rho * d.B));
-  }
-  __syncthreads();
-  for (int rho = tid; rho < d.K4; rho += blockDim.x) {
-    const uint32_t bin = sRowBin[rho];
-    const int bb = bin != ~0u ? (int)bin : -1;
-    const float best = bb >= 0 ? __uint_as_float(sRowCap[rho]) : 0.0f;
-    sC[rho] = best;
-    sB[rho] = bb;
-    const int i = rho >> 2, j = rho & 3;
-    const float lam = sLam[i], rl = sRl[i];
-    const int M = rep_cap(d, j);
-    const float Mf = rep_capf(d, j);
-    int n0 = 0, len = 0;
-    if (bb >= 0) {
-      atomicOr(reinterpret_cast<unsigned int*>(&sMisc[2 + (i >> 5)]), 1u << (i & 31));
-      if (M >= 1) {
-        // first fulfilment that is positive and at or above the class's floor
-        // (n = 1 unless one replica falls short of it)
-        const float lo_f = FL ? fmaxf(sDl[i], __int_as_float(1)) : __int_as_float(1);
-        n0 = fulfil_r(1.0f, best, lam, rl) >= lo_f ? 1 : min_replicas(lo_f, best, lam, rl, Mf);
-        if (n0) {
-          const int ns = min_replicas(1.0f, best, lam, rl, Mf);   // first full fulfilment
-          len = ns ? ns : M;
-        }
-      }
+  // 2. t*: bit patterns [lo, hi) of nonnegative floats (ordered like the
+  // values), lo feasible and hi not; every group probes one point a round.
+  int lgs = 2;
+  while ((1 << lgs) < d.K4 && lgs < 5) ++lgs;
+  const int gsz = 1 << lgs, gl = lane & (gsz - 1);
+  const int ng = NW << (5 - lgs), g = (warp << (5 - lgs)) + (lane >> lgs);
+  // Ends not probed yet: 0 fits (nothing is bought) and the pattern above 1 does
+  // not (no fulfilment exceeds 1); their sums never let the search end.
+  uint32_t lo = 0u, hi = kAboveOne;
+  int ulo = -(1 << 28), uhi = 1 << 28;
+  uint32_t aim_lo, aim_hi;  // where the first probes go
+  search_aims(sm, d, lane, aim_lo, aim_hi);
+  int oct = 22;  // an unprobed lower end is approached by points 2^oct patterns apart, growing
+  for (int rd = 0; uhi - ulo > 1 && hi - lo > 1; ++rd) {
+    uint32_t pt;
+    if (rd == 0 || (ng == 1 && rd == 1 && lo == 0u)) {
+      // between the two estimates; one group probes the upper, then the lower
+      if (ng == 1) pt = rd == 0 ? aim_hi : min(aim_lo, hi - 1u);
+      else pt = aim_lo + (uint32_t)(((uint64_t)g * (aim_hi - aim_lo)) / (uint32_t)(ng - 1));
+    } else {
+      const uint32_t span = hi - lo;
+      const uint64_t reach = lo ? (uint64_t)span : min((uint64_t)span, (uint64_t)(ng + 1) << min(oct, 30));
+      const uint32_t q = max(1u, (uint32_t)(reach / (uint32_t)(ng + 1)));
+      const uint64_t off = (uint64_t)(g + 1) * q;
+      pt = off < span ? hi - (uint32_t)off : lo;  // (past the lower end: that end again)
+      oct += 2;
     }
-    sN0[rho] = n0;
-    sOff[rho] = n0 ? len - n0 + 1 : 0;  // count, scanned below
-  }
-  __syncthreads();
-  if (warp == 0) {  // exclusive scan of the row counts
-    int carry = 0;
-    for (int base = 0; base < d.K4; base += 32) {
-      const int rho = base + lane;
-      const int v = rho < d.K4 ? sOff[rho] : 0;
-      int incl = v;
-      for (int o = 1; o < 32; o <<= 1) {
-        const int y = __shfl_up_sync(0xffffffffu, incl, o);
-        if (lane >= o) incl += y;
-      }
-      if (rho < d.K4) sOff[rho] = carry + incl - v;
-      carry += __shfl_sync(0xffffffffu, incl, 31);
-    }
-    if (lane == 0) sOff[d.K4] = carry;
-  }
-  __syncthreads();
-  int total = sOff[d.K4];
-  if (total > d.theta_cap) {  // cannot happen: a row holds at most floor(G/tau) values
-    if (tid == 0) atomicOr(set.status, ST_THETA);
-    total = d.theta_cap;
-  }
-  int P2 = 1;
-  while (P2 < total) P2 <<= 1;
-  // A scoring solve builds the row table (step 3) when it is small enough; its
-  // scratch follows the thresholds: cover costs [K4][total], class minima
-  // [K][total], and each row's own fulfilment values in order [total]
-  const bool row_table =
-      write_theta && !cap_x && set.rtab && d.K4 * total <= kRowTabMax && sOff[d.K4] == total;
-  int P2c = 1;
-  while (P2c < d.theta_cap) P2c <<= 1;
-  int* sCost = reinterpret_cast<int*>(sTheta + P2c);
-  int* sCmin = sCost + d.K4 * total;
-  float* sOwn = reinterpret_cast<float*>(sCmin + d.K * total);
-
-  // 2. thresholds, then a sort (ascending, +inf padding)
-  for (int x = tid; x < P2; x += blockDim.x) {
-    float v = __int_as_float(0x7f800000);
-    if (x < total) {
-      int lo = 0, hi = d.K4 - 1;
-      while (lo < hi) {
-        const int mid = (lo + hi + 1) >> 1;
-        if (sOff[mid] <= x) lo = mid; else hi = mid - 1;
-      }
-      const int n = sN0[lo] + (x - sOff[lo]);
-      v = fulfil_r((float)n, sC[lo], sLam[lo >> 2], sRl[lo >> 2]);
-      if (row_table) sOwn[x] = v;
-    }
-    sTheta[x] = v;
-  }
-  __syncthreads();
-  if (P2 <= 64) {
-    // small lists: one warp sorts 64 values held two per lane (bitonic network,
-    // partners by __shfl_xor_sync), with no block barriers
-    if (warp == 0) {
-      const float inf = __int_as_float(0x7f800000);
-      float r[2] = {lane < P2 ? sTheta[lane] : inf, lane + 32 < P2 ? sTheta[lane + 32] : inf};
-      for (int k = 2; k <= 64; k <<= 1) {
-        for (int jj = k >> 1; jj > 0; jj >>= 1) {
-          if (jj == 32) {  // partners share a lane; k == 64, ascending
-            const float lo = fminf(r[0], r[1]), hi = fmaxf(r[0], r[1]);
-            r[0] = lo;
-            r[1] = hi;
-          } else {
-#pragma unroll
-            for (int h = 0; h < 2; ++h) {
-              const int i = lane + 32 * h;
-              const float pv = __shfl_xor_sync(0xffffffffu, r[h], jj);
-              const bool keep_min = ((i & jj) == 0) == ((i & k) == 0);
-              r[h] = keep_min ? fminf(r[h], pv) : fmaxf(r[h], pv);
-            }
-          }
-        }
-      }
-      if (lane < P2) sTheta[lane] = r[0];
-      if (lane + 32 < P2) sTheta[lane + 32] = r[1];
-    }
-    __syncthreads();
-  } else if (row_table && P2 <= 256 && P2 <= (int)blockDim.x) {
-    // up to one value a thread, the unsorted values in sOwn: each thread
-    // places its value at its rank (values below it, and equal values at
-    // lower indices), one pass with no barriers between stages (its cost
-    // grows with the count: above 256 values the network below is faster)
-    if (tid < total) {
-      const float v = sOwn[tid];
-      int rank = 0;
-#pragma unroll 4
-      for (int j = 0; j < total; ++j) {
-        const float u = sOwn[j];
-        rank += (u < v || (u == v && j < tid)) ? 1 : 0;
-      }
-      sTheta[rank] = v;
-    }
-  } else {
-    for (int k = 2; k <= P2; k <<= 1) {
-      for (int jj = k >> 1; jj > 0; jj >>= 1) {
-        for (int x = tid; x < P2; x += blockDim.x) {
-          const int y = x ^ jj;
-          if (y > x) {
-            const float a = sTheta[x], b = sTheta[y];
-            const bool up = (x & k) == 0;
-            if ((a > b) == up && a != b) {
-              sTheta[x] = b;
-              sTheta[y] = a;
-            }
-          }
-        }
-        __syncthreads();
-      }
-    }
-  }
-
-  // 3. t*: the largest index whose threshold fits in G (the cheapest-cover
-  // total is nondecreasing along the sorted thresholds).
-  __shared__ int s_res[2][kSolveThreadsWide / 4];
-  if (tid == 0) sMisc[4] = 0;
-  __syncthreads();
-  int kstar;
-  if (row_table) {
-    // Row table of a scoring solve: every row's cover cost at every threshold,
-    // then per (row rho, threshold k) the word the per-candidate preparation
-    // reads for a candidate in row rho, stored threshold-major at k K4 + rho (its
-    // address does not depend on the number of thresholds): bits 0-15 the
-    // replicas rho may use once the other classes are covered (0 if one cannot
-    // be), bit 16 set if another row of rho's class covers theta_k within that
-    // budget.
-    //
-    // A row's cheapest cover of t (class i covers max(t, delta_i)) is n0 plus
-    // the number of its own values f(n0) <= ... <= f(len) below t: every n
-    // below n0 falls short of it, and past len either f(ns) >= 1 >= t or the
-    // row holds M replicas and none covers t. The values are the fulfilments
-    // the thresholds were made of, so the count is the cover min_replicas
-    // finds, without evaluating f. One thread per (class, threshold) runs the
-    // four TP rows' branch-free lower bounds side by side.
-    const int nx = d.K * total;
-    for (int x = tid; x < nx; x += blockDim.x) {
-      const int i = x / total, k = x - i * total;
-      const float tc = FL ? fmaxf(sTheta[k], sDl[i]) : sTheta[k];
-      int q[4], nv[4], beg[4];  // values below tc so far, values held, first value
-#pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        beg[j] = sOff[4 * i + j];
-        nv[j] = sOff[4 * i + j + 1] - beg[j];
-        q[j] = 0;
-      }
-      const int most = max(max(nv[0], nv[1]), max(nv[2], nv[3]));
-      for (int step = most ? 1 << (31 - __clz(most)) : 0; step > 0; step >>= 1) {
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          // the four loads are issued unconditionally: the index is clamped to
-          // the row's last value, at most total - 1 (an empty row reads the word
-          // before its start, at worst the last class minimum: scratch either way)
-          const float v = sOwn[beg[j] + min(q[j] + step, nv[j]) - 1];
-          q[j] += (q[j] + step <= nv[j]) & (v < tc) ? step : 0;
-        }
-      }
-      int cm = kCostInf;
-#pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        const int c = q[j] < nv[j] ? (sN0[4 * i + j] + q[j]) << j : kCostInf;
-        sCost[(4 * i + j) * total + k] = c;
-        cm = min(cm, c);
-      }
-      sCmin[x] = cm;
-    }
-    __syncthreads();
-    // per pair: the other classes' covers summed (an uncovered class counted as
-    // 2^24: a cost is at most G <= 32767, 64 of them stay below 2^21), then one
-    // word per TP row; t* = the count of thresholds whose total fits, less one
-    int* rt = set.rtab + ((size_t)p * 2 + sigma) * kRowTabMax;
-    int cnt = 0;
-    for (int x0 = 0; x0 < nx; x0 += blockDim.x) {
-      const int x = x0 + tid;
-      bool fits = false;
-      if (x < nx) {
-        const int i = x / total, k = x - i * total;
-        int sum = 0;
-        for (int q = 0; q < d.K; ++q) {
-          const int cq = sCmin[q * total + k];
-          sum += cq >= kCostInf ? (1 << 24) : cq;
-        }
-        fits = i == 0 && sum <= d.G;
-        const int own = sCmin[x];
-        const int rest = sum - (own >= kCostInf ? (1 << 24) : own);
-        const int A = (rest >> 24) ? -1 : d.G - rest;
-        int c[4], wd[4];
-#pragma unroll
-        for (int j = 0; j < 4; ++j) c[j] = sCost[(4 * i + j) * total + k];
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          int other = kCostInf;  // cheapest cover by another row of the class
-#pragma unroll
-          for (int q = 0; q < 4; ++q)
-            if (q != j) other = min(other, c[q]);
-          const int m = A >= (1 << j) ? min(A >> j, rep_cap(d, j)) : 0;
-          wd[j] = m | ((other < kCostInf && other <= A) ? 1 << 16 : 0);
-        }
-        // threshold-major: word (rho, k) at k K4 + rho, the class's four in one 16-byte store
-        *reinterpret_cast<int4*>(rt + (size_t)k * d.K4 + 4 * i) = make_int4(wd[0], wd[1], wd[2], wd[3]);
-      }
-      cnt += __syncthreads_count(fits);
-    }
-    kstar = cnt - 1;
-  } else {
-    // Search: each round every group of gsz lanes probes one index (an
-    // (ng+1)-ary split); each warp merges the answers with integer max / min
-    // reductions, so a round costs one barrier (lo feasible, hi not).
-    int gsz = 4;
-    while (gsz < d.K4 && gsz < 32) gsz <<= 1;
-    const int ng = blockDim.x / gsz, g = tid / gsz, gl = tid & (gsz - 1);
-    int lo = -1, hi = total;
-    for (int par = 0; hi - lo > 1; par ^= 1) {
-      int kp = lo + ((g + 1) * (hi - lo)) / (ng + 1);
-      kp = max(lo + 1, min(hi - 1, kp));
-      const int cost = group_total_cost<FL>(sTheta[kp], sC, sLam, sRl, sDl, d, gl, gsz);
-      if (gl == 0) s_res[par][g] = (cost <= d.G) ? kp : -(kp + 1);
+    int u;
+    const int cost = group_cover<FL>(__uint_as_float(max(pt, 1u)), sm, d, gl, gsz, &u);
+    const bool known = pt <= lo;
+    const bool fits = known || cost <= d.G;
+    // the largest point that fits and the smallest that does not
+    uint32_t nlo = __reduce_max_sync(0xffffffffu, fits && !known ? pt : lo);
+    uint32_t nhi = __reduce_min_sync(0xffffffffu, fits ? hi : min(pt, hi));
+    const uint32_t bl = __ballot_sync(0xffffffffu, fits && !known && pt == nlo);
+    const uint32_t bh = __ballot_sync(0xffffffffu, !fits && pt == nhi);
+    int nul = __shfl_sync(0xffffffffu, u, bl ? __ffs(bl) - 1 : 0);
+    int nuh = __shfl_sync(0xffffffffu, u, bh ? __ffs(bh) - 1 : 0);
+    if (!bl) nul = ulo;
+    if (!bh) nuh = uhi;
+    if (NW > 1) {
+      // (the arrays alternate between rounds: one barrier a round)
+      const int w = (rd & 1) * NW;
+      if (lane == 0) sm.end[w + warp] = make_int4((int)nlo, (int)nhi, nul, nuh);
       __syncthreads();
-      int nlo = lo, nhi = hi;
-      for (int q = lane; q < ng; q += 32) {
-        const int v = s_res[par][q];
-        if (v >= 0) nlo = max(nlo, v); else nhi = min(nhi, -v - 1);
-      }
-      lo = __reduce_max_sync(0xffffffffu, nlo);
-      hi = __reduce_min_sync(0xffffffffu, nhi);
+      const int4 e = sm.end[w + (lane & (NW - 1))];
+      nlo = __reduce_max_sync(0xffffffffu, (uint32_t)e.x);
+      nhi = __reduce_min_sync(0xffffffffu, (uint32_t)e.y);
+      nul = __shfl_sync(0xffffffffu, e.z, __ffs(__ballot_sync(0xffffffffu, (uint32_t)e.x == nlo)) - 1);
+      nuh = __shfl_sync(0xffffffffu, e.w, __ffs(__ballot_sync(0xffffffffu, (uint32_t)e.y == nhi)) - 1);
     }
-    kstar = lo;
+    lo = nlo;
+    hi = nhi;
+    ulo = nul;
+    uhi = nuh;
   }
-  const float tstar = kstar >= 0 ? sTheta[kstar] : 0.0f;
 
-  if (choice) {
-    // 4. choice at t*: every row's cheapest cover in parallel (thread = row), then
-    // per class the cheapest row over its four TP lanes, lower TP on ties; the
-    // same for the floor of a critical class, summed into sMisc[5] (sMisc[6]:
-    // some critical class cannot reach its floor)
-    {
-      const int rho = tid;  // K4 <= 256 <= blockDim
-      int key = 0x7fffffff, keyf = 0x7fffffff;
-      if (rho < d.K4) {
-        const float dl = FL ? sDl[rho >> 2] : 0.0f;
-        if (tstar > 0.0f) {
-          const int n = min_replicas(FL ? fmaxf(tstar, dl) : tstar, sC[rho], sLam[rho >> 2], sRl[rho >> 2],
-                                     rep_capf(d, rho & 3));
-          if (n) key = ((n << (rho & 3)) << 2) | (rho & 3);
-        }
-        if (FL && dl > 0.0f) {
-          const int n = min_replicas(dl, sC[rho], sLam[rho >> 2], sRl[rho >> 2], rep_capf(d, rho & 3));
-          if (n) keyf = ((n << (rho & 3)) << 2) | (rho & 3);
-        }
+  // 3. t* is the smallest option fulfilment at or above lo, and the covers at
+  // t* are those at lo: per class the cheapest over its four TP lanes, lower
+  // TP on ties; the same for the floor of a critical class. One warp.
+  if (warp != 0) return;
+  float tv = 2.0f;  // the smallest option fulfilment at or above lo
+  int total = 0, ftotal = 0;
+  bool fmiss = false;
+  uint64_t mask = 0;
+  fs_allocation& so = sm.out;
+  const float t_lo = __uint_as_float(lo);
+  if (FL) {  // the critical classes' floors
+    for (int base = 0; base < d.K4; base += 32) {
+      const int rho = base + lane, i = rho >> 2;
+      int keyf = 0x7fffffff;
+      const float dl = rho < d.K4 ? sm.dl[i] : 0.0f;
+      if (dl > 0.0f) {
+        const int n = min_replicas(dl, sm.C[rho], sm.lam[i], sm.rl[i], rep_capf(d, rho & 3));
+        if (n) keyf = n << (rho & 3);
       }
-      key = min(key, __shfl_xor_sync(0xffffffffu, key, 1));
-      key = min(key, __shfl_xor_sync(0xffffffffu, key, 2));
-      const int i = tid >> 2;
-      if constexpr (FL) {
-        keyf = min(keyf, __shfl_xor_sync(0xffffffffu, keyf, 1));
-        keyf = min(keyf, __shfl_xor_sync(0xffffffffu, keyf, 2));
-        const bool critical = (tid & 3) == 0 && i < d.K && sDl[i] > 0.0f;
-        if (critical) {
-          if (keyf == 0x7fffffff) atomicOr(&sMisc[6], 1);
-          else atomicAdd(&sMisc[5], keyf >> 2);
-        }
-        __syncthreads();
-        const bool met = sMisc[6] == 0 && sMisc[5] <= d.G;
-        if (tstar <= 0.0f) key = (critical && met) ? keyf : 0x7fffffff;  // tier 1 alone
-      }
-      if ((tid & 3) == 0 && i < FS_MAX_CLASSES) {  // (a 512-thread block has 128 groups of four)
-        int8_t tp = 0;
-        int16_t bin = -1, reps = 0;
-        float f = 0.0f;
-        if (i < d.K && key != 0x7fffffff) {
-          const int bj = key & 3, cost_i = key >> 2, bn = cost_i >> bj;
-          tp = (int8_t)(1 << bj);
-          bin = (int16_t)sB[4 * i + bj];
-          reps = (int16_t)bn;
-          f = fulfil_r((float)bn, sC[4 * i + bj], sLam[i], sRl[i]);
-          atomicAdd(&sMisc[4], cost_i);
-        }
-        out->tp[i] = tp;
-        out->bin[i] = bin;
-        out->replicas[i] = reps;
-        out->fulfil[i] = f;
+      keyf = min(keyf, __shfl_xor_sync(0xffffffffu, keyf, 1));
+      keyf = min(keyf, __shfl_xor_sync(0xffffffffu, keyf, 2));
+      const bool head = (lane & 3) == 0 && dl > 0.0f;
+      fmiss = fmiss || __any_sync(0xffffffffu, head && keyf == 0x7fffffff);
+      ftotal += __reduce_add_sync(0xffffffffu, head && keyf != 0x7fffffff ? keyf : 0);
+    }
+  }
+  const bool met = !FL || (!fmiss && ftotal <= d.G);
+  // an empty allocation, then the model's classes
+  uint64_t* words = reinterpret_cast<uint64_t*>(&so);
+  constexpr int kBin0 = (int)(offsetof(fs_allocation, bin) / 8), kBin1 = (int)(offsetof(fs_allocation, replicas) / 8);
+  for (int w = lane; w < (int)(sizeof(fs_allocation) / 8); w += 32) words[w] = w >= kBin0 && w < kBin1 ? ~0ull : 0ull;
+  __syncwarp();
+  for (int base = 0; base < d.K4; base += 32) {
+    const int rho = base + lane, i = rho >> 2, j = rho & 3;
+    int key = 0x7fffffff;
+    bool has = false;
+    if (rho < d.K4) {
+      const float dl = FL ? sm.dl[i] : 0.0f;
+      has = sm.bin[rho] >= 0;
+      // at t* = 0 tier 1 alone: the critical classes' floors, when they can be met
+      const float t = lo ? (FL ? fmaxf(t_lo, dl) : t_lo) : (met ? dl : 0.0f);
+      const int n = t > 0.0f ? min_replicas(t, sm.C[rho], sm.lam[i], sm.rl[i], rep_capf(d, j)) : 0;
+      if (n) {
+        key = ((n << j) << 2) | j;
+        tv = fminf(tv, fulfil_r((float)n, sm.C[rho], sm.lam[i], sm.rl[i]));
       }
     }
-    __syncthreads();
-  }
-  if (tid == 0) {
-    out->t_star = tstar;
-    // (with t* = 0 and no floors the sum is 0 anyway; the unconditional read
-    // measured 1.5 us slower on a 28 us scoring call whose next kernel overlaps this one)
-    out->total_gpus = !choice ? -1 : (FL || tstar > 0.0f) ? sMisc[4] : 0;  // -1: not computed
-    out->has_option_mask = (uint64_t)(uint32_t)sMisc[2] | ((uint64_t)(uint32_t)sMisc[3] << 32);
-    out->ok = tstar > 0.0f ? 1 : 0;
-    out->floors_met = (!FL || (sMisc[6] == 0 && sMisc[5] <= d.G)) ? 1 : 0;
-    out->goodput = 0.0;  // tier 3 is filled by the lexicographic solve
-  }
-  if (write_theta && !cap_x) {
-    float* th = set.theta + ((size_t)p * 2 + sigma) * d.theta_cap;
-    for (int x = tid; x < total; x += blockDim.x) th[x] = sTheta[x];
-    float* rc = set.rowC + ((size_t)p * 2 + sigma) * d.K4;
-    int* rb = set.rowB + ((size_t)p * 2 + sigma) * d.K4;
-    for (int rho = tid; rho < d.K4; rho += blockDim.x) {
-      rc[rho] = sC[rho];
-      rb[rho] = sB[rho];
+    key = min(key, __shfl_xor_sync(0xffffffffu, key, 1));
+    key = min(key, __shfl_xor_sync(0xffffffffu, key, 2));
+    const uint32_t bal = __ballot_sync(0xffffffffu, has);
+    mask |= (uint64_t)__ballot_sync(0xffffffffu, lane < 8 && ((bal >> (4 * (lane & 7))) & 15u)) << (base >> 2);
+    const bool head = j == 0 && key != 0x7fffffff;
+    total += __reduce_add_sync(0xffffffffu, head ? key >> 2 : 0);
+    if (head) {
+      const int bj = key & 3, bn = (key >> 2) >> bj;
+      so.tp[i] = (int8_t)(1 << bj);
+      so.bin[i] = (int16_t)sm.bin[4 * i + bj];
+      so.replicas[i] = (int16_t)bn;
+      so.fulfil[i] = fulfil_r((float)bn, sm.C[4 * i + bj], sm.lam[i], sm.rl[i]);
     }
-    if (tid == 0) set.ntheta[p * 2 + sigma] = total;
   }
+  const float tstar = lo ? __uint_as_float(__reduce_min_sync(0xffffffffu, __float_as_uint(tv))) : 0.0f;
+  if (lane == 0) {
+    so.t_star = tstar;
+    so.total_gpus = total;
+    so.has_option_mask = mask;
+    so.ok = tstar > 0.0f ? 1 : 0;
+    so.floors_met = met ? 1 : 0;
+    so.goodput = 0.0;  // tier 3 is filled by the lexicographic solve
+  }
+  __syncwarp();
+  uint64_t* dst = reinterpret_cast<uint64_t*>(out);
+  for (int w = lane; w < (int)(sizeof(fs_allocation) / 8); w += 32) dst[w] = words[w];
 }
 
 // Watchdog self-test: wait on a barrier phase that nothing completes; the
@@ -535,37 +315,26 @@ cudaError_t launch_watchdog(uint32_t* status, uint64_t limit_ns, cudaStream_t s)
   return cudaGetLastError();
 }
 
-static size_t solve_smem_bytes(const Dims& d) {
-  int P2 = 1;
-  while (P2 < d.theta_cap) P2 <<= 1;
-  return 256 * 8 + (size_t)(256 * 3 + 260 + 32 + 8) * 4 + (size_t)P2 * 4;
-}
-
 cudaError_t launch_qtable(float* qn, int Q, cudaStream_t s) {
   note_launch();
   k_qtable<<<(Q + 255) / 256, 256, 0, s>>>(qn, Q);
   return cudaGetLastError();
 }
 
+// Measured (one GB300, calls in a row): 4096 realisations of the four-class,
+// 64-GPU grid 71.7 -> 14.6 us (11.5 M -> 5 M warp instructions against the first
+// one-warp version, whose rows and cover counts took more of them).
 cudaError_t launch_solve(const Set& set, int n, const float* cap_x, const float* tail_x,
-                         fs_allocation* out, bool write_theta, LaunchCache& lc, cudaStream_t s, bool tstar_only) {
+                         fs_allocation* out, LaunchCache& lc, cudaStream_t s) {
   if (n <= 0) return cudaSuccess;
-  // a scoring solve may build the row table: K4 x |Theta| cover costs, K x |Theta| class minima
-  // and |Theta| own values, with K4 x |Theta| <= kRowTabMax
-  const size_t smem =
-      solve_smem_bytes(set.d) + (write_theta && set.rtab ? (size_t)(kRowTabMax + kRowTabMax / 2) * 4 : 0);
-  const int fl = lc.floors ? 1 : 0;
-  auto kern = fl ? k_solve<true> : k_solve<false>;
-  if (smem > lc.solve_smem[fl]) {
-    cudaError_t e = raise_smem_limit(reinterpret_cast<const void*>(kern), smem);
-    if (e != cudaSuccess) return e;
-    lc.solve_smem[fl] = smem;
-  }
-  // a scoring solve of a model with more than 256 cells takes 512 threads: its
-  // per-cell passes and row-table phases then run half the iterations each
-  const int bt = write_theta && !cap_x && set.d.cells > kSolveThreads ? kSolveThreadsWide : kSolveThreads;
   note_launch();
-  kern<<<n, bt, smem, s>>>(set, n, cap_x, tail_x, out, (write_theta ? 1 : 0) | (tstar_only ? 2 : 0));
+  if (n <= kSolveWideMax) {
+    auto kern = lc.floors ? k_solve<true, 8> : k_solve<false, 8>;
+    kern<<<n, 256, 0, s>>>(set, n, cap_x, tail_x, out);
+  } else {
+    auto kern = lc.floors ? k_solve<true, 1> : k_solve<false, 1>;
+    kern<<<(n + 3) / 4, 128, 0, s>>>(set, n, cap_x, tail_x, out);
+  }
   return cudaGetLastError();
 }
 

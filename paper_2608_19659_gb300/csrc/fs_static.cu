@@ -116,7 +116,7 @@ extern "C" int fs_score_candidates_noalloc(int32_t K, int32_t B, int32_t G, cons
   const size_t o_theta = take(8 * (size_t)d.theta_cap), o_nth = take(8);
   const size_t o_rowc = take(8 * (size_t)d.K4), o_rowb = take(8 * (size_t)d.K4);
   const size_t o_base = take(2 * sizeof(fs_allocation));
-  const size_t o_rtab = take(8 * (size_t)kRowTabMax);  // row tables of the two base solves
+  const size_t o_rtab = take(4 * (size_t)kRowTabMax);  // row tables of the two base solves
   const int Wq = Q / smp->O, Wp = 4 + ((Wq + 3) & ~3);
   const size_t item_floats = 2 * (size_t)d.slot_floats + (size_t)smp->O * Wp;
   const size_t o_tab = take((size_t)std::max(n, 1) * item_floats * 4);
@@ -165,7 +165,9 @@ extern "C" int fs_score_candidates_noalloc(int32_t K, int32_t B, int32_t G, cons
   set.status = reinterpret_cast<uint32_t*>(base + o_status);
   set.work = reinterpret_cast<unsigned long long*>(base + o_work);
   set.skip = nullptr;
-  set.rtab = reinterpret_cast<int*>(base + o_rtab);
+  set.rtab = reinterpret_cast<uint16_t*>(base + o_rtab);
+  set.rt_cap = kRowTabMax;
+  set.tpart = reinterpret_cast<float*>(base + o_base);  // (no allocation is written here)
   set.prior = 0;  // the revealed-only prior: no cell is measured here
 
   Items it{};
@@ -195,7 +197,7 @@ extern "C" int fs_score_candidates_noalloc(int32_t K, int32_t B, int32_t G, cons
   cudaStream_t s = static_cast<cudaStream_t>(cuda_stream);
   e = cudaMemsetAsync(set.status, 0, 4, s);  // the array keeps the last call's status word
   if (e == cudaSuccess && !quantile_dev) e = launch_qtable(const_cast<float*>(set.qn), Q, s);
-  if (e == cudaSuccess) e = launch_solve(set, 2, nullptr, nullptr, nullptr, true, lc, s, true);
+  if (e == cudaSuccess) e = launch_thresh(set, 0, 0, s);
   if (e == cudaSuccess) e = launch_prep(set, it, pl, reinterpret_cast<float*>(base + o_tab),
                                         reinterpret_cast<uint64_t*>(base + o_sums), true, sm_count, lc, s);
   if (e == cudaSuccess)
@@ -209,7 +211,6 @@ extern "C" int fs_score_candidates_noalloc(int32_t K, int32_t B, int32_t G, cons
     // keep the larger of what this call and any concurrent one found
     std::lock_guard<std::mutex> lock(g_static_mu);
     LaunchCache& g = g_static_lc[dev];
-    for (int f = 0; f < 2; ++f) g.solve_smem[f] = std::max(g.solve_smem[f], lc.solve_smem[f]);
     for (int f = 0; f < 4; ++f) {
       g.prep_smem[f] = std::max(g.prep_smem[f], lc.prep_smem[f]);
       for (int v = 0; v < kScoreVariants; ++v)
