@@ -408,23 +408,27 @@ int run_score(fs_model* m, Set set, const fs_samples* smp, const int32_t* cand_d
   return FS_OK;
 }
 
+double demand_sum(const fs_model* m) {
+  double t = 0.0;
+  for (float v : m->h_lam) t += (double)v;
+  return t;
+}
+
 // Tiers 3-4 (fs_lex.cu) of n realisations whose tier-2 allocations are in out
 // (or the base), when the model's objective asks for them.
 int solve_lex_pass(fs_model* m, const Set& set, int n, const float* cap_x, const float* tail_x, fs_allocation* out,
                    cudaStream_t s) {
   if (m->objective != FS_OBJECTIVE_LEXICOGRAPHIC || n <= 0) return FS_OK;
-  const size_t per_real = lex_scratch_cells(m->d) * kLexCellBytes;
-  const int per_launch = (int)std::max<size_t>(1, std::min<size_t>((size_t)n, (64u << 20) / per_real));
-  int rc = m->lex.ensure(per_real * per_launch, "lexicographic scratch");
-  if (rc) return rc;
-  FS_CUDA(launch_solve_lex(set, n, cap_x, tail_x, out, m->lex.p, per_launch, s), "launch lexicographic solve");
+  const bool pack = demand_sum(m) <= 67108864.0;
+  int per_launch = n;
+  if (lex_needs_scratch(m->d, n, pack)) {
+    const size_t per_real = lex_scratch_cells(m->d) * kLexCellBytes;
+    per_launch = (int)std::max<size_t>(1, std::min<size_t>((size_t)n, (64u << 20) / per_real));
+    int rc = m->lex.ensure(per_real * per_launch, "lexicographic scratch");
+    if (rc) return rc;
+  }
+  FS_CUDA(launch_solve_lex(set, n, cap_x, tail_x, out, m->lex.p, per_launch, pack, s), "launch lexicographic solve");
   return FS_OK;
-}
-
-double demand_sum(const fs_model* m) {
-  double t = 0.0;
-  for (float v : m->h_lam) t += (double)v;
-  return t;
 }
 
 }  // namespace

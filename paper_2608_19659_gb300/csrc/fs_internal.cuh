@@ -521,8 +521,11 @@ constexpr size_t kLexCellBytes = 16;  // one cell of the programme over classes 
 size_t lex_scratch_cells(const Dims& d);  // (K + 1)(G + 1) cells per realisation
 // Realisations [0, n) (as launch_solve reads them; their tier-2 allocations in
 // out / the base), per_launch of them at a time through scratch.
+// pack: sum lambda <= 2^26 (goodput and GPUs fit one word). scratch: needed
+// when lex_needs_scratch says so (the cells do not fit shared memory).
+bool lex_needs_scratch(const Dims& d, int n, bool pack);
 cudaError_t launch_solve_lex(const Set& set, int n, const float* cap_x, const float* tail_x, fs_allocation* out,
-                             void* scratch, int per_launch, cudaStream_t s);
+                             void* scratch, int per_launch, bool pack, cudaStream_t s);
 // Threads per block of the goodput scorer (a multiple of 32, at most 256) and
 // its dynamic shared memory, or 0 when one warp's share does not fit.
 constexpr size_t kGoodputSmemMax = 220 * 1024;  // of the 227 KB a block may opt into, less its static arrays

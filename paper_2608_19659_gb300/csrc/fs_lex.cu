@@ -21,9 +21,10 @@
 // GPUs, S_K = 0, S_i(g) = max over class i's options (cost <= g) of their
 // goodput plus S_{i+1}(g - cost).
 //
-// k_solve_lex: one CTA per realisation; the table S in global scratch,
-//   threads over g, one class per step; thread 0 then walks the classes
-//   forward taking the preferred option that keeps the optimum.
+// k_solve_lex: one warp (a block of 16 for a few) per realisation, threads over
+//   g, one class per step, over the GPUs that the classes' cheapest options
+//   leave; then a walk over the classes, lanes over a class's options, taking
+//   the preferred option that keeps the optimum.
 // k_score_goodput: the goodput stage of the Monte-Carlo score. Within a
 //   segment (candidate e, outcome o) a scenario's goodput gap
 //   |GP(A+') - GP(A-')| depends on its draw only through (c_y position,
@@ -37,6 +38,7 @@
 
 #include "fs_finalize.cuh"
 #include "fs_internal.cuh"
+#include "fs_rows.cuh"
 #include "fs_sample.cuh"
 
 namespace fs {
@@ -61,12 +63,134 @@ __device__ __forceinline__ bool lex_better(long long gpa, int gpusa, long long g
 
 // --------------------------------------------------------------------------- tiers 3-4
 
-__global__ void __launch_bounds__(256) k_solve_lex(Set set, int n_real, const float* cap_x, const float* tail_x,
-                                                   fs_allocation* out_x, LexCell* scratch, int r0) {
+// A programme value: goodput first, then fewest GPUs. Packed into one 64-bit
+// word (goodput 2^16 less GPUs: both parts add, and more goodput or the same
+// with fewer GPUs is the larger word) while goodput stays below 2^46, which the
+// host knows from sum lambda <= 2^26; the two-word form otherwise.
+template <bool PACK>
+struct Lex;
+template <>
+struct Lex<true> {
+  using T = long long;
+  static __device__ __forceinline__ T make(long long gp, int gpus) { return (gp << 16) - gpus; }
+  static __device__ __forceinline__ T add(T a, T b) { return a + b; }
+  static __device__ __forceinline__ bool better(T a, T b) { return a > b; }
+  static __device__ __forceinline__ bool same(T a, T b) { return a == b; }
+  static __device__ __forceinline__ long long gp(T a) { return (a + 0xFFFF) >> 16; }
+  static __device__ __forceinline__ T worst() { return -0x7FFFFFFFFFFFFFFFLL - 1; }
+  static __device__ __forceinline__ T shfl_xor(T a, int o) { return __shfl_xor_sync(0xffffffffu, a, o); }
+};
+template <>
+struct Lex<false> {
+  using T = LexCell;
+  static __device__ __forceinline__ T make(long long gp, int gpus) { return LexCell{gp, gpus}; }
+  static __device__ __forceinline__ T add(T a, T b) { return LexCell{a.gp + b.gp, a.gpus + b.gpus}; }
+  static __device__ __forceinline__ bool better(T a, T b) { return lex_better(a.gp, a.gpus, b.gp, b.gpus); }
+  static __device__ __forceinline__ bool same(T a, T b) { return a.gp == b.gp && a.gpus == b.gpus; }
+  static __device__ __forceinline__ long long gp(T a) { return a.gp; }
+  static __device__ __forceinline__ T worst() { return LexCell{-1, 0x7fffffff}; }
+  static __device__ __forceinline__ T shfl_xor(T a, int o) {
+    return LexCell{__shfl_xor_sync(0xffffffffu, a.gp, o), __shfl_xor_sync(0xffffffffu, a.gpus, o)};
+  }
+};
+
+// First n in [1, M] with fl(n c) >= lambda (the whole demand served: further
+// replicas add GPUs and no goodput), else M + 1; fl(n c) is nondecreasing in n.
+// In range the answer is within one of ceil(lambda / c) and is reached from an
+// estimate by steps of one, as in min_replicas; else by bisection.
+__device__ __forceinline__ int first_full(float c, float lam, int M) {
+  if (row_in_range(c, lam) && c > 0.0f) {
+    const float Mf = (float)M;
+    float n = fminf(fmaxf(ceilf(__fdividef(lam, c)), 1.0f), Mf);
+    while (n > 1.0f && !(__fmul_rn(n - 1.0f, c) < lam)) n -= 1.0f;
+    while (n <= Mf && __fmul_rn(n, c) < lam) n += 1.0f;
+    return (int)n;
+  }
+  int a = 1, b = M + 1;
+  while (a < b) {
+    const int mid = (a + b) >> 1;
+    if (!(__fmul_rn((float)mid, c) < lam)) b = mid;
+    else a = mid + 1;
+  }
+  return a;
+}
+
+// Class i's options on row (i, tau = 2^j) at capacity C are the replica
+// counts n in [1, M = G / tau] whose fulfilment reaches T (all of them when
+// T = 0), up to the first that serves the whole demand. Both ends are monotone
+// in n, so the options are one range [lo, hi]. lo = 0: none.
+__device__ __forceinline__ void row_range(float C, bool ok, int M, float T, float lam, float rl, int& lo, int& hi) {
+  lo = hi = 0;
+  if (!ok || M < 1) return;
+  lo = T > 0.0f ? min_replicas(T, C, lam, rl, (float)M) : 1;
+  if (lo) hi = min(M, max(lo, first_full(C, lam, M)));
+}
+
+__device__ __forceinline__ float class_threshold(float t, float dl) { return t > 0.0f ? fmaxf(t, dl) : dl; }
+
+// Dynamic shared memory of k_solve_lex per realisation: the rows (best
+// capacity, its bin, its option range), the classes (cheapest option), one
+// class's option values (opt of them; more are evaluated where they are used)
+// and the programme's cells, when they fit (cells of them; else in scratch).
+struct LexSmem {
+  size_t rows, cls, opt, cells, total;
+  int n_opt, n_cells;
+};
+
+__host__ __device__ inline LexSmem lex_smem(int K, int G, bool pack, int most_opt, size_t most_cell_bytes) {
+  LexSmem m{};
+  const size_t cell = pack ? 8 : sizeof(LexCell);
+  auto up = [](size_t x) { return (x + 15) & ~(size_t)15; };
+  m.n_opt = G + (G >> 1) + (G >> 2) + (G >> 3);
+  if (m.n_opt > most_opt) m.n_opt = most_opt;
+  const size_t all = (size_t)(K + 1) * (G + 1);
+  m.n_cells = all * cell <= most_cell_bytes ? (int)all : 0;
+  m.rows = 0;
+  m.cls = up(m.rows + 16 * (size_t)(4 * K));
+  m.opt = up(m.cls + 8 * (size_t)K);
+  m.cells = up(m.opt + cell * (size_t)m.n_opt);
+  m.total = up(m.cells + cell * (size_t)m.n_cells);
+  return m;
+}
+
+constexpr int kLexWideWarps = 16;       // warps of a realisation when there are few
+constexpr int kLexOptWarp = 512;        // option values kept per class (one warp, kLexWideWarps)
+constexpr int kLexOptWide = 2048;
+constexpr size_t kLexCellsWarp = 12 * 1024;   // bytes of programme cells in shared memory
+constexpr size_t kLexCellsWide = 128 * 1024;
+
+// NW warps per realisation: 1 (four realisations a block) for batches, 16 for
+// a few realisations, whose latency counts.
+//
+// The programme runs over the GPUs left beyond what must be kept: class i's
+// cheapest option costs m_i (0 when it may stay empty), so of G only slack = G -
+// sum m_i can be spent freely, and S_i is needed (and reachable) for h = 0..slack
+// GPUs above the cheapest options of classes i..K-1. An option of cost c takes e
+// = c - m_i of them. Where t* is tight the slack is a few GPUs and a class's
+// options with e <= slack are few; the table over all of [0, G] that stood here
+// before, with a division per option and cell, took 66 us on 1000 realisations of
+// the four-class, 64-GPU grid and 180 us on two of the eight-class, 256-GPU one
+// (its last step, the walk forward, one thread's); measured now: see
+// launch_solve_lex.
+template <bool PACK, int NW>
+__global__ void __launch_bounds__(NW == 1 ? 128 : 32 * NW) k_solve_lex(Set set, int n_real, const float* cap_x,
+                                                                       const float* tail_x, fs_allocation* out_x,
+                                                                       unsigned char* scratch, int r0, LexSmem lay) {
+  using L = Lex<PACK>;
+  using V = typename L::T;
+  constexpr int kPerBlock = NW == 1 ? 4 : 1, kThreads = 32 * NW;
+  extern __shared__ __align__(16) unsigned char smraw[];
+  __shared__ int s_slack[kPerBlock];
+  __shared__ V s_top[NW];
   const Dims& d = set.d;
-  const int r = r0 + blockIdx.x;
-  const int tid = threadIdx.x;
+  const int lane = threadIdx.x & 31, warp = NW == 1 ? 0 : (int)threadIdx.x >> 5;
+  const int slot = NW == 1 ? (int)threadIdx.x >> 5 : 0, tid = warp * 32 + lane;
+  const int rel = (int)blockIdx.x * kPerBlock + slot, r = r0 + rel;
   if (r >= n_real) return;
+  auto sync = [] {
+    if (NW == 1) __syncwarp();
+    else __syncthreads();
+  };
   const float* cap;
   const float* tail;
   fs_allocation* out;
@@ -81,107 +205,188 @@ __global__ void __launch_bounds__(256) k_solve_lex(Set set, int n_real, const fl
     tail = bp + (size_t)(sigma ? TAIL_LO : TAIL_HI) * d.cells;
     out = set.base + r;
   }
-  LexCell* S = scratch + (size_t)blockIdx.x * (size_t)(d.K + 1) * (d.G + 1);
-  __shared__ float sC[256];
-  __shared__ int sB[256];
-  __shared__ float sT[FS_MAX_CLASSES];
-  __shared__ int sEmpty[FS_MAX_CLASSES];
   const float tstar = out->t_star;
-  const int met = out->floors_met;
-  // rows: best SLO-feasible bin (largest capacity, then lowest bin)
-  for (int rho = tid; rho < d.K4; rho += blockDim.x) {
-    const int i = rho >> 2;
-    const float L = set.slo[i];
-    float best = 0.0f;
-    int bb = -1;
-    for (int b = 0; b < d.B; ++b) {
-      const size_t c = (size_t)rho * d.B + b;
-      if (tail[c] <= L) {
-        const float v = __fadd_rn(cap[c], 0.0f);  // -0 as +0
-        if (bb < 0 || v > best) {
-          best = v;
-          bb = b;
-        }
-      }
-    }
-    sC[rho] = best;
-    sB[rho] = bb;
-  }
-  for (int i = tid; i < d.K; i += blockDim.x) {
-    const float dl = set.slo[d.K + i];  // floors follow the SLOs (0: not critical)
-    sT[i] = tstar > 0.0f ? fmaxf(tstar, dl) : dl;
-    sEmpty[i] = !(tstar > 0.0f) && !(dl > 0.0f);
-  }
-  if (!met) {  // tier 1 cannot hold: nothing is allocated (k_solve wrote the empty allocation)
+  if (!out->floors_met) {  // tier 1 cannot hold: nothing is allocated (k_solve wrote the empty allocation)
     if (tid == 0) out->goodput = 0.0;
     return;
   }
-  for (int g = tid; g <= d.G; g += blockDim.x) S[(size_t)d.K * (d.G + 1) + g] = LexCell{0, 0};
-  __syncthreads();
-  for (int i = d.K - 1; i >= 0; --i) {
-    const LexCell* nxt = S + (size_t)(i + 1) * (d.G + 1);
-    LexCell* cur = S + (size_t)i * (d.G + 1);
-    const float lam = set.lam[i], T = sT[i];
-    for (int g = tid; g <= d.G; g += blockDim.x) {
-      LexCell best{-1, 0};
-      if (sEmpty[i] && nxt[g].gp >= 0) best = nxt[g];
+  unsigned char* mem = smraw + (size_t)slot * lay.total;
+  float* sC = reinterpret_cast<float*>(mem + lay.rows);
+  int* sB = reinterpret_cast<int*>(sC + d.K4);
+  int* sLo = sB + d.K4;
+  int* sHi = sLo + d.K4;
+  int* sMin = reinterpret_cast<int*>(mem + lay.cls);     // cheapest option's GPUs
+  int* sEmpty = sMin + d.K;                               // 1: the class may stay empty
+  V* sOpt = reinterpret_cast<V*>(mem + lay.opt);
+  V* S = lay.n_cells ? reinterpret_cast<V*>(mem + lay.cells)
+                     : reinterpret_cast<V*>(scratch) + (size_t)rel * (size_t)(d.K + 1) * (d.G + 1);
+  best_rows<NW>(d, cap, tail, set.slo, warp, lane, sC, sB);
+  sync();
+  for (int rho = tid; rho < d.K4; rho += kThreads) {
+    const int i = rho >> 2;
+    const float lam = set.lam[i], T = class_threshold(tstar, set.slo[d.K + i]);
+    int lo, hi;
+    row_range(sC[rho], sB[rho] >= 0, rep_cap(d, rho & 3), T, lam, __frcp_rn(lam), lo, hi);
+    sLo[rho] = lo;
+    sHi[rho] = hi;
+  }
+  sync();
+  if (warp == 0) {
+    int sum = 0;
+    for (int i = lane; i < d.K; i += 32) {
+      const bool empty = !(tstar > 0.0f) && !(set.slo[d.K + i] > 0.0f);
+      int m = empty ? 0 : kCostInf;
+      for (int j = 0; j < kT && !empty; ++j)
+        if (sLo[4 * i + j]) m = min(m, sLo[4 * i + j] << j);
+      sMin[i] = m;
+      sEmpty[i] = empty;
+      sum += min(m, 1 << 24);
+    }
+    sum = __reduce_add_sync(0xffffffffu, sum);
+    if (lane == 0) s_slack[slot] = d.G - sum;
+  }
+  sync();
+  const int slack = s_slack[slot], H = slack + 1;
+  if (slack < 0) {  // cannot happen: t* and the floors were found feasible
+    if (tid == 0) {
+      atomicOr(set.status, ST_THETA);
+      out->goodput = 0.0;
+    }
+    return;
+  }
+  // class i's options with e <= slack in the order of preference (no replicas,
+  // lower TP, fewer replicas): x = 0.. over `empty`, then row j's lo..top
+  struct Opts {
+    int empty, e1, e2, e3, total, lo[kT], m;
+  };
+  auto options = [&](int i) {
+    Opts o;
+    o.empty = sEmpty[i];
+    o.m = sMin[i];
+    int cnt[kT];
+#pragma unroll
+    for (int j = 0; j < kT; ++j) {
+      o.lo[j] = sLo[4 * i + j];
+      cnt[j] = o.lo[j] ? max(0, min(sHi[4 * i + j], (slack + o.m) >> j) - o.lo[j] + 1) : 0;
+    }
+    o.e1 = o.empty + cnt[0];
+    o.e2 = o.e1 + cnt[1];
+    o.e3 = o.e2 + cnt[2];
+    o.total = o.e3 + cnt[3];
+    return o;
+  };
+  auto pick = [&](const Opts& o, int x, int& j, int& n) {
+    if (x < o.empty) { j = 0; n = 0; }
+    else if (x < o.e1) { j = 0; n = o.lo[0] + (x - o.empty); }
+    else if (x < o.e2) { j = 1; n = o.lo[1] + (x - o.e1); }
+    else if (x < o.e3) { j = 2; n = o.lo[2] + (x - o.e2); }
+    else { j = 3; n = o.lo[3] + (x - o.e3); }
+  };
+  auto value = [&](int i, int j, int n) {
+    return L::make(n ? goodput_fx((float)n, sC[4 * i + j], set.lam[i]) : 0, n << j);
+  };
+  for (int h = tid; h < H; h += kThreads) S[(size_t)d.K * H + h] = L::make(0, 0);
+  sync();
+  for (int i = d.K - 1; i >= 1; --i) {
+    const V* nxt = S + (size_t)(i + 1) * H;
+    V* cur = S + (size_t)i * H;
+    const Opts o = options(i);
+    const int kept = min(o.total, lay.n_opt);
+    for (int x = tid; x < kept; x += kThreads) {
+      int j, n;
+      pick(o, x, j, n);
+      sOpt[x] = value(i, j, n);
+    }
+    sync();
+    for (int h = tid; h < H; h += kThreads) {
+      V best = L::worst();
+      if (o.empty) best = nxt[h];
+      int x = o.empty;
+#pragma unroll
       for (int j = 0; j < kT; ++j) {
-        if (sB[4 * i + j] < 0) continue;
-        const float C = sC[4 * i + j];
-        const int M = rep_cap(d, j);
-        for (int n = 1; n <= M && (n << j) <= g; ++n) {
-          const float nf = (float)n;
-          if (T > 0.0f && !(fulfil(nf, C, lam) >= T)) continue;
-          const LexCell pv = nxt[g - (n << j)];
-          if (pv.gp >= 0) {
-            const long long v = goodput_fx(nf, C, lam) + pv.gp;
-            const int u = (n << j) + pv.gpus;
-            if (best.gp < 0 || lex_better(v, u, best.gp, best.gpus)) best = LexCell{v, u};
-          }
-          if (!(__fmul_rn(nf, C) < lam)) break;  // the whole demand served: more replicas add nothing
+        const int end = j == 0 ? o.e1 : j == 1 ? o.e2 : j == 2 ? o.e3 : o.total;
+        int e = (o.lo[j] << j) - o.m;
+        for (; x < end && e <= h; ++x, e += 1 << j) {
+          const V v = L::add(x < kept ? sOpt[x] : value(i, j, (e + o.m) >> j), nxt[h - e]);
+          if (L::better(v, best)) best = v;
         }
+        x = end;
       }
-      cur[g] = best;
+      cur[h] = best;
     }
-    __syncthreads();
+    sync();
   }
-  if (tid != 0) return;
-  // forward: class by class the preferred option that keeps the optimum
-  int left = d.G, total = 0;
-  const long long gp_all = S[d.G].gp;
+  // the first class: its best over all threads
+  V top = L::worst();
+  {
+    const Opts o = options(0);
+    for (int x = tid; x < o.total; x += kThreads) {
+      int j, n;
+      pick(o, x, j, n);
+      const int e = (n << j) - o.m;
+      if (e <= slack) {
+        const V v = L::add(value(0, j, n), S[(size_t)H + slack - e]);
+        if (L::better(v, top)) top = v;
+      }
+    }
+    for (int off = 16; off; off >>= 1) {
+      const V v = L::shfl_xor(top, off);
+      if (L::better(v, top)) top = v;
+    }
+    if (NW > 1) {
+      if (lane == 0) s_top[warp] = top;
+      __syncthreads();
+      if (warp != 0) return;
+      top = s_top[lane & (NW - 1)];
+      for (int off = 16; off; off >>= 1) {
+        const V v = L::shfl_xor(top, off);
+        if (L::better(v, top)) top = v;
+      }
+    }
+  }
+  // forward: class by class the first option, in the order of preference, that
+  // keeps the optimum (lanes over the options). One warp.
+  int left = slack, total = 0;
+  V target = top;
   for (int i = 0; i < d.K; ++i) {
-    const LexCell target = S[(size_t)i * (d.G + 1) + left];
-    const LexCell* nxt = S + (size_t)(i + 1) * (d.G + 1);
-    const float lam = set.lam[i], T = sT[i];
-    int cj = -1, cn = 0;
-    if (!(sEmpty[i] && nxt[left].gp == target.gp && nxt[left].gpus == target.gpus)) {
-      for (int j = 0; j < kT && cj < 0; ++j) {
-        if (sB[4 * i + j] < 0) continue;
-        const float C = sC[4 * i + j];
-        const int M = rep_cap(d, j);
-        for (int n = 1; n <= M && (n << j) <= left; ++n) {
-          const float nf = (float)n;
-          if (T > 0.0f && !(fulfil(nf, C, lam) >= T)) continue;
-          const LexCell pv = nxt[left - (n << j)];
-          if (pv.gp >= 0 && goodput_fx(nf, C, lam) + pv.gp == target.gp && (n << j) + pv.gpus == target.gpus) {
-            cj = j;
-            cn = n;
-            break;
-          }
-        }
+    const V* nxt = S + (size_t)(i + 1) * H;
+    const Opts o = options(i);
+    int j = 0, n = 0, e = 0;
+    bool found = false;
+    for (int x0 = 0; x0 < o.total && !found; x0 += 32) {
+      const int x = x0 + lane;
+      bool hit = false;
+      if (x < o.total) {
+        pick(o, x, j, n);
+        e = (n << j) - o.m;
+        hit = e <= left && L::same(L::add(value(i, j, n), nxt[left - e]), target);
+      }
+      const uint32_t bal = __ballot_sync(0xffffffffu, hit);
+      if (bal) {
+        const int src = __ffs(bal) - 1;
+        j = __shfl_sync(0xffffffffu, j, src);
+        n = __shfl_sync(0xffffffffu, n, src);
+        e = __shfl_sync(0xffffffffu, e, src);
+        found = true;
       }
     }
-    out->tp[i] = (int8_t)(cj >= 0 ? 1 << cj : 0);
-    out->bin[i] = (int16_t)(cj >= 0 ? sB[4 * i + cj] : -1);
-    out->replicas[i] = (int16_t)cn;
-    out->fulfil[i] = cj >= 0 ? fulfil((float)cn, sC[4 * i + cj], lam) : 0.0f;
-    if (cj >= 0) {
-      left -= cn << cj;
-      total += cn << cj;
+    if (lane == 0) {
+      const bool some = found && n > 0;
+      out->tp[i] = (int8_t)(some ? 1 << j : 0);
+      out->bin[i] = (int16_t)(some ? sB[4 * i + j] : -1);
+      out->replicas[i] = (int16_t)(some ? n : 0);
+      out->fulfil[i] = some ? fulfil((float)n, sC[4 * i + j], set.lam[i]) : 0.0f;
+    }
+    if (found) {
+      total += n << j;
+      left -= e;
+      target = nxt[left];
     }
   }
-  out->total_gpus = total;
-  out->goodput = (double)gp_all * 0x1p-20;
+  if (lane == 0) {
+    out->total_gpus = total;
+    out->goodput = (double)L::gp(top) * 0x1p-20;
+  }
 }
 
 // --------------------------------------------------------------------------- goodput stage
@@ -204,26 +409,6 @@ struct RowOpt {
   float a, b;
 };
 
-// Class i's options on row (i, tau = 2^j) at capacity C are the replica
-// counts n in [1, M = G / tau] whose fulfilment reaches T (all of them when
-// T = 0), up to the first that serves the whole demand (fl(n C) >= lambda:
-// more replicas add GPUs and no goodput). Both ends are monotone in n, so the
-// options are one range [lo, hi]: the smallest feasible count by
-// min_replicas, the first saturating count by bisection. lo = 0: none.
-__device__ __forceinline__ void row_range(float C, bool ok, int M, float T, float lam, float rl, int& lo, int& hi) {
-  lo = hi = 0;
-  if (!ok || M < 1) return;
-  lo = T > 0.0f ? min_replicas(T, C, lam, rl, (float)M) : 1;
-  if (lo == 0) return;
-  int a = 1, b = M + 1;  // the first n in [1, M] with fl(n C) >= lambda, else M + 1
-  while (a < b) {
-    const int mid = (a + b) >> 1;
-    if (!(__fmul_rn((float)mid, C) < lam)) b = mid;
-    else a = mid + 1;
-  }
-  hi = min(M, max(lo, a));
-}
-
 // The row's range and the interval of thresholds that gives the same lo (and
 // so the same hi): fulfil(lo - 1) < T <= fulfil(lo) for lo >= 1 (no lower end
 // at lo = 1), T > fulfil(M) for lo = 0 (fulfil is nondecreasing in n).
@@ -239,8 +424,6 @@ __device__ __forceinline__ RowOpt row_opt(float C, bool ok, int M, float T, floa
   }
   return r;
 }
-
-__device__ __forceinline__ float class_threshold(float t, float dl) { return t > 0.0f ? fmaxf(t, dl) : dl; }
 
 // The best tier-3 goodput of every class but `skip` within g GPUs, for g in
 // [0, G], at tiers 1-2 value t (-1: the floors of those classes cannot be
@@ -580,16 +763,39 @@ __global__ void k_finalize_goodput(Set set, Items it, Plan pl, const uint64_t* s
 
 size_t lex_scratch_cells(const Dims& d) { return (size_t)(d.K + 1) * (d.G + 1); }
 
-cudaError_t launch_solve_lex(const Set& set, int n, const float* cap_x, const float* tail_x, fs_allocation* out,
-                             void* scratch, int per_launch, cudaStream_t s) {
+// Whether the programme of n realisations needs scratch in global memory.
+static LexSmem lex_layout(const Dims& d, int n, bool pack) {
+  return n <= kSolveWideMax ? lex_smem(d.K, d.G, pack, kLexOptWide, kLexCellsWide)
+                            : lex_smem(d.K, d.G, pack, kLexOptWarp, kLexCellsWarp);
+}
+
+bool lex_needs_scratch(const Dims& d, int n, bool pack) { return lex_layout(d, n, pack).n_cells == 0; }
+
+template <bool PACK, int NW>
+static cudaError_t launch_lex(const Set& set, int n, const float* cap_x, const float* tail_x, fs_allocation* out,
+                              void* scratch, int per_launch, const LexSmem& lay, cudaStream_t s) {
+  constexpr int kPerBlock = NW == 1 ? 4 : 1;
+  auto kern = k_solve_lex<PACK, NW>;
+  const size_t smem = kPerBlock * lay.total;
+  cudaError_t e = raise_smem_limit(reinterpret_cast<const void*>(kern), smem);
+  if (e != cudaSuccess) return e;
   for (int r0 = 0; r0 < n; r0 += per_launch) {
     const int m = n - r0 < per_launch ? n - r0 : per_launch;
     note_launch();
-    k_solve_lex<<<m, 256, 0, s>>>(set, n, cap_x, tail_x, out, static_cast<LexCell*>(scratch), r0);
-    cudaError_t e = cudaGetLastError();
+    kern<<<(m + kPerBlock - 1) / kPerBlock, NW == 1 ? 128 : 32 * NW, smem, s>>>(
+        set, r0 + m, cap_x, tail_x, out, static_cast<unsigned char*>(scratch), r0, lay);
+    e = cudaGetLastError();
     if (e != cudaSuccess) return e;
   }
   return cudaSuccess;
+}
+
+cudaError_t launch_solve_lex(const Set& set, int n, const float* cap_x, const float* tail_x, fs_allocation* out,
+                             void* scratch, int per_launch, bool pack, cudaStream_t s) {
+  const LexSmem lay = lex_layout(set.d, n, pack);
+  auto go = n <= kSolveWideMax ? (pack ? launch_lex<true, kLexWideWarps> : launch_lex<false, kLexWideWarps>)
+                               : (pack ? launch_lex<true, 1> : launch_lex<false, 1>);
+  return go(set, n, cap_x, tail_x, out, scratch, per_launch, lay, s);
 }
 
 int goodput_threads(const Dims& d, const Plan& pl, bool rf, size_t* smem) {
