@@ -158,7 +158,7 @@ struct fs_model {
   Buf fixed;      // lam, slo + floors, qn, bounds, revealed, theta, ntheta, rowC, rowB, base, status
   Set set{};
   // per-call scratch
-  Buf cand, tables, sums, outs, real, lex;
+  Buf cand, tables, sums, outs, real, lex, gp;
   Buf replay;     // fs_replay's state of every stream (grown on demand, kept)
   int objective = FS_OBJECTIVE_MAXMIN;  // FS_OBJECTIVE_LEXICOGRAPHIC: fs_solve* and the certificate to tier 4
   // host mirrors
@@ -815,25 +815,26 @@ int fs_score_goodput(fs_model* m, const fs_samples* smp, double* gap_out, double
   it.n = n;
   it.cell = reinterpret_cast<const int32_t*>(hd + out_bytes);
   const Plan pl = make_plan(m, smp, n);
-  if (goodput_threads(m->d, pl, m->set.prior == 1, nullptr) == 0)
+  if (pl.W > (m->set.prior == 1 ? 2048 : 4096))  // a segment's table of positions lives in shared memory
     return fail(FS_EINVAL, "the goodput stage needs Q / O <= 2048 under the monotone prior, 4096 otherwise");
-  const int saved = m->objective;
-  m->objective = FS_OBJECTIVE_LEXICOGRAPHIC;  // the base solves to tier 4 (their goodput)
-  FS_CUDA(launch_solve(m->set, 2, nullptr, nullptr, nullptr, m->lc, s), "launch solve");
-  rc = solve_lex_pass(m, m->set, 2, nullptr, nullptr, nullptr, s);
-  m->objective = saved;
-  if (rc) return rc;
-  uint64_t* sums = static_cast<uint64_t*>(m->sums.p);
   if (m->th_bound < 0) m->th_bound = threshold_bound(m);
+  // the rows wanted and the base goodputs, then the pool of rows
+  const size_t rows = goodput_pool_rows(m->d, m->th_bound, kGoodputPoolMax);
+  const size_t head = 4 * (size_t)kGoodputSpanInts + 256;
+  if ((rc = m->gp.ensure(head + rows * goodput_row_bytes(m->d), "goodput tables"))) return rc;
+  int* span = static_cast<int*>(m->gp.p);
+  long long* base = reinterpret_cast<long long*>(span + kGoodputSpanInts);
+  uint64_t* sums = static_cast<uint64_t*>(m->sums.p);
   Set set = m->set;
+  set.gp_span = span;
   FS_CUDA(launch_thresh(set, m->lc.floors, m->th_bound, s), "launch thresholds");
-  FS_CUDA(launch_prep(set, it, pl, static_cast<float*>(m->tables.p), sums, false, m->sm_count, m->lc, s,
-                      m->th_bound),
+  FS_CUDA(launch_prep(set, it, pl, static_cast<float*>(m->tables.p), sums, true, m->sm_count, m->lc, s, m->th_bound),
           "launch prep");
-  FS_CUDA(launch_score_goodput(set, it, pl, static_cast<const float*>(m->tables.p), sums, m->lc.floors,
-                               m->sm_count, s),
+  FS_CUDA(launch_score_goodput(set, it, pl, static_cast<const float*>(m->tables.p), sums, span, base,
+                               static_cast<char*>(m->gp.p) + head, rows, m->lc.floors, m->th_bound, m->sm_count, s),
           "launch goodput scorer");
-  FS_CUDA(launch_finalize_goodput(set, it, pl, sums, lam_sum, d_gap, d_score, d_gamma, d_best, d_st, s),
+  FS_CUDA(launch_finalize_goodput(set, it, pl, sums, base, lam_sum, d_gap, d_score, d_gamma, d_best, d_st,
+                                  sums + nn * smp->O, s),
           "launch goodput reduction");
   if (sum_eo && n)
     FS_CUDA(cudaMemcpyAsync(sum_eo, sums, 8 * (size_t)n * smp->O, cudaMemcpyDeviceToHost, s), "read sums");
@@ -1104,6 +1105,7 @@ void fs_free_model(fs_model* m) {
   m->outs.release();
   m->real.release();
   m->lex.release();
+  m->gp.release();
   m->replay.release();
   for (cudaEvent_t e : m->ev) cudaEventDestroy(e);
   if (m->up_done) cudaEventDestroy(m->up_done);

@@ -53,7 +53,7 @@ constexpr int kRowTabModel = 1 << 20;
 
 // Table header words (floats unless noted).
 enum : int {
-  H_TH_BASE = 0,  // threshold below the first table entry (0 if none)
+  H_B0 = 0,       // index of the threshold below the first table entry (int, -1 if none)
   H_TCL = 1,      // t* of this realisation at row capacity Cexcl: every scenario whose tail gate is closed
   H_L = 2,        // entries (int)
   H_LPAD = 3,     // entries padded to 4 (int)
@@ -118,6 +118,8 @@ struct Set {
   int rt_cap;           // words per row table
   int n_tpart;          // scoring calls: k_thresh blocks per realisation (0: t* comes from base)
   float* tpart;         // [2][n_tpart] each block's largest feasible threshold (t* is their maximum)
+  int* gp_span;         // goodput stage (else nullptr): [2][2][K] rows of the other classes' tables that
+                        // the candidates can reach, least then most; k_thresh empties it, k_prep fills it
   int prior;            // interval refit after a measurement: 0 the measured cell only,
                         // 1 also its row's other bins (capacity and tail nondecreasing in load)
 };
@@ -526,15 +528,20 @@ size_t lex_scratch_cells(const Dims& d);  // (K + 1)(G + 1) cells per realisatio
 bool lex_needs_scratch(const Dims& d, int n, bool pack);
 cudaError_t launch_solve_lex(const Set& set, int n, const float* cap_x, const float* tail_x, fs_allocation* out,
                              void* scratch, int per_launch, bool pack, cudaStream_t s);
-// Threads per block of the goodput scorer (a multiple of 32, at most 256) and
-// its dynamic shared memory, or 0 when one warp's share does not fit.
-constexpr size_t kGoodputSmemMax = 220 * 1024;  // of the 227 KB a block may opt into, less its static arrays
-int goodput_threads(const Dims& d, const Plan& pl, bool rf, size_t* smem);
+// The goodput stage's tables of the other classes' best goodput: rows of
+// goodput_row_bytes each, goodput_pool_rows of them (every row the call can
+// want, or as many whole classes' as most_bytes holds, at least one's: the
+// scorer then takes the classes in several passes).
+constexpr size_t kGoodputPoolMax = 512u << 20;
+size_t goodput_pool_rows(const Dims& d, int th_bound, size_t most_bytes);
+size_t goodput_row_bytes(const Dims& d);
+constexpr int kGoodputSpanInts = 4 * FS_MAX_CLASSES;  // wanted rows per (realisation, class): least, most
 cudaError_t launch_score_goodput(const Set& set, const Items& it, const Plan& pl, const float* tables,
-                                 uint64_t* sums, int floors, int sm_count, cudaStream_t s);
+                                 uint64_t* sums, int* span, long long* base, void* pool, size_t pool_rows,
+                                 int floors, int th_bound, int sm_count, cudaStream_t s);
 cudaError_t launch_finalize_goodput(const Set& set, const Items& it, const Plan& pl, const uint64_t* sums,
-                                    double lam_sum, double* gap, double* score, double* gamma, int32_t* best,
-                                    uint32_t* status_copy, cudaStream_t s);
+                                    const long long* base, double lam_sum, double* gap, double* score, double* gamma,
+                                    int32_t* best, uint32_t* status_copy, uint64_t* part, cudaStream_t s);
 
 // replay
 struct ReplayState {

@@ -25,16 +25,18 @@
 //   g, one class per step, over the GPUs that the classes' cheapest options
 //   leave; then a walk over the classes, lanes over a class's options, taking
 //   the preferred option that keeps the optimum.
-// k_score_goodput: the goodput stage of the Monte-Carlo score. Within a
+// k_other, k_score_goodput: the goodput stage of the Monte-Carlo score. Within a
 //   segment (candidate e, outcome o) a scenario's goodput gap
 //   |GP(A+') - GP(A-')| depends on its draw only through (c_y position,
-//   tail gate), as its t* does: the block tabulates those values (a warp per
-//   entry: each realisation's row capacity and t* as the scorer computes
-//   them, then the programme over the classes with row r patched, lanes over
-//   g), then draws every scenario's position and sums the entries.
+//   tail gate), as its t* does: the block tabulates those values, a thread per
+//   entry, on top of tables of the other classes' best goodput that k_other
+//   makes once per call, then draws every scenario's position and sums the
+//   entries.
 // k_finalize_goodput: E[Gamma_gp,t+1 | e] = sum 2^-20 / (O S) / sum lambda,
 //   the score Gamma_gp,t - E and the argmax (same order as the max-min stage).
 #include <cuda_runtime.h>
+
+#include <algorithm>
 
 #include "fs_finalize.cuh"
 #include "fs_internal.cuh"
@@ -409,338 +411,406 @@ struct RowOpt {
   float a, b;
 };
 
-// The row's range and the interval of thresholds that gives the same lo (and
-// so the same hi): fulfil(lo - 1) < T <= fulfil(lo) for lo >= 1 (no lower end
-// at lo = 1), T > fulfil(M) for lo = 0 (fulfil is nondecreasing in n).
-__device__ __forceinline__ RowOpt row_opt(float C, bool ok, int M, float T, float lam, float rl) {
-  RowOpt r{C, 0, 0, -INFINITY, INFINITY};
-  row_range(C, ok, M, T, lam, rl, r.lo, r.hi);
-  if (!ok || M < 1) return r;
-  if (r.lo == 0) {
-    r.a = fulfil((float)M, C, lam);
-  } else {
-    r.b = fulfil((float)r.lo, C, lam);
-    if (r.lo > 1) r.a = fulfil((float)(r.lo - 1), C, lam);
-  }
-  return r;
-}
-
-// The best tier-3 goodput of every class but `skip` within g GPUs, for g in
-// [0, G], at tiers 1-2 value t (-1: the floors of those classes cannot be
-// met within g), by one warp: the programme over the classes (no replicas,
-// when class i may stay empty: T_i = 0 and no floor; else one range of
-// replica counts on each of its rows) with lanes over g. Also leaves in opt
-// every row's range at t (those of `skip` for warp_best_with; row `fixed`,
-// whose capacity varies, with no interval). dpa, dpb: the warp's two arrays
-// of G + 1 cells. Returns the array that holds the result.
-template <bool FL>
-__device__ const long long* warp_other(const Dims& d, const float* sCs, const int* sOk, const float* sLam,
-                                       const float* sRl, const float* sDl, int skip, int fixed, float t,
-                                       RowOpt* opt, long long* dpa, long long* dpb) {
-  const int lane = threadIdx.x & 31;
-  __syncwarp();  // the previous result and ranges are no longer read
-  for (int rho = lane; rho < d.K4; rho += 32) {
-    const int i = rho >> 2;
-    RowOpt r = row_opt(sCs[rho], sOk[rho] != 0, d.G >> (rho & 3), class_threshold(t, FL ? sDl[i] : 0.0f),
-                       sLam[i], sRl[i]);
-    if (rho == fixed) r.a = -INFINITY, r.b = INFINITY;
-    opt[rho] = r;
-  }
-  for (int g = lane; g <= d.G; g += 32) dpa[g] = 0;
-  __syncwarp();
-  long long* cur = dpa;  // S_{i+1}
-  long long* nxt = dpb;
-  for (int i = d.K - 1; i >= 0; --i) {
-    if (i == skip) continue;
-    const float dl = FL ? sDl[i] : 0.0f;
-    const bool may_empty = !(t > 0.0f) && !(dl > 0.0f);
-    const float lam = sLam[i];
-    for (int g = lane; g <= d.G; g += 32) {
-      long long best = may_empty ? cur[g] : -1;
-#pragma unroll
-      for (int j = 0; j < kT; ++j) {
-        const RowOpt ro = opt[4 * i + j];
-        const int top = min(ro.hi, g >> j);
-        for (int n = ro.lo; n <= top && n > 0; ++n) {
-          const long long pv = cur[g - (n << j)];
-          if (pv >= 0) {
-            const long long v = goodput_fx20((float)n, ro.C, lam) + pv;
-            best = v > best ? v : best;
-          }
-        }
-      }
-      nxt[g] = best;
-    }
-    __syncwarp();
-    long long* x = cur;
-    cur = nxt;
-    nxt = x;
-  }
-  return cur;
-}
-
-// Whether the ranges in opt (left by warp_other at a value t0 with
-// (t0 > 0) = pos) hold at t as well: then so do the programme's result and
-// class i_r's other rows. One warp.
-template <bool FL>
-__device__ bool warp_ranges_hold(const Dims& d, const float* sDl, const RowOpt* opt, float t, bool pos) {
-  const int lane = threadIdx.x & 31;
-  bool ok = (t > 0.0f) == pos;
-  for (int rho = lane; rho < d.K4; rho += 32) {
-    const float T = class_threshold(t, FL ? sDl[rho >> 2] : 0.0f);
-    ok = ok && opt[rho].a < T && T <= opt[rho].b;
-  }
-  return __all_sync(0xffffffffu, ok);
-}
-
-// Tier-3 goodput of one realisation with row rr at capacity Cr (its range
-// [lor, hir] at t), at tiers 1-2 value t, given other = warp_other(..., skip
-// = class of rr, t): the best over class i_r's choices (nothing, when it may
-// stay empty; else n replicas on one of its rows) of its goodput plus the
-// others' best within the GPUs left; -1 when the floors cannot be met. Lanes
-// over the choices, one warp.
-template <bool FL>
-__device__ long long warp_best_with(const Dims& d, const float* sLam, const float* sDl, const RowOpt* opt, int rr,
-                                    float Cr, int lor, int hir, float t, const long long* other) {
-  const int lane = threadIdx.x & 31, ir = rr >> 2, jr = rr & 3;
-  const float lam = sLam[ir];
-  const float dl = FL ? sDl[ir] : 0.0f;
-  int cnt[kT], lo[kT];
-  float C[kT];
-#pragma unroll
-  for (int j = 0; j < kT; ++j) {
-    const RowOpt ro = opt[4 * ir + j];
-    lo[j] = j == jr ? lor : ro.lo;
-    const int hi = j == jr ? hir : ro.hi;
-    C[j] = j == jr ? Cr : ro.C;
-    cnt[j] = lo[j] > 0 ? hi - lo[j] + 1 : 0;
-  }
-  long long best = (!(t > 0.0f) && !(dl > 0.0f)) ? other[d.G] : -1;
-  const int e1 = cnt[0], e2 = e1 + cnt[1], e3 = e2 + cnt[2], total = e3 + cnt[3];
-  for (int x = lane; x < total; x += 32) {
-    int j, n;
-    float Cj;
-    if (x < e1) { j = 0; n = lo[0] + x; Cj = C[0]; }
-    else if (x < e2) { j = 1; n = lo[1] + (x - e1); Cj = C[1]; }
-    else if (x < e3) { j = 2; n = lo[2] + (x - e2); Cj = C[2]; }
-    else { j = 3; n = lo[3] + (x - e3); Cj = C[3]; }
-    const long long pv = other[d.G - (n << j)];
-    if (pv >= 0) {
-      const long long v = goodput_fx20((float)n, Cj, lam) + pv;
-      best = v > best ? v : best;
-    }
-  }
-  for (int off = 16; off; off >>= 1) {
-    const long long o = __shfl_xor_sync(0xffffffffu, best, off);
-    best = o > best ? o : best;
-  }
-  return best;
-}
-
-// t* of realisation sigma at row capacity C, from the candidate's table in
-// global memory (the IEEE row term: every input).
-template <bool FL>
-__device__ __forceinline__ float tstar_global(const float* h, float C) {
-  const int Lp = __float_as_int(h[H_LPAD]);
-  const float* kap = h + kTableHeader;
-  const float* thx = kap + Lp;
-  const float* mnx = thx + Lp;
-  int pos = 0;
-  for (int step = __float_as_int(h[H_STEP0]); step > 0; step >>= 1) pos += kap[pos + step - 1] <= C ? step : 0;
-  const float thb = thx[pos];
-  const float m = mnx[pos];
-  const float tr = m >= 1.0f ? fulfil(m, C, h[H_LAM]) : 0.0f;
-  if (FL) return (tr > thb && tr >= h[H_DLT]) ? tr : thb;
-  return tr > thb ? tr : thb;
-}
-
-// Shared memory of k_score_goodput: per table entry its gap (8 bytes), both
-// realisations' row capacities (8) and values (16: t*, then the goodput),
-// one flag byte; per warp its K4 row ranges and two programme arrays.
-struct GoodputSmem {
-  size_t gtab, cap, val, flag, warps, per_warp, total;
+// Value tables of one goodput call. A realisation's goodput depends on a
+// scenario only through its patched row capacity C' (t* is a function of C').
+// It splits at the candidate's class i_r: the best of class i_r's choices plus
+// `other`, the best goodput of the other classes within the GPUs left, which
+// depends on t* only through the replica ranges it leaves the other classes'
+// rows. Those change only just above a threshold of the realisation, so `other`
+// is the same for every t* in (theta_{k-1}, theta_k]: one table per
+// (realisation, class, k), shared by every candidate of the class and every
+// outcome. Row kk of a (realisation, class): 0 holds t* = 0, k + 1 holds t* in
+// (theta_{k-1}, theta_k], total + 1 holds t* above every threshold. The
+// preparation records the rows its candidates can reach (span), k_other fills
+// them.
+struct GoodputTables {
+  int* span;            // [2 (least, most)][2][K] rows wanted per (realisation, class); least > most: none
+  long long* base;      // [2] the base realisations' goodput, 2^-20 req/s
+  long long* rows;      // pool of rows of `stride` words
+  int stride;           // G + 1 values by GPUs, then kT: the best without each row of the class
+  int pool;             // rows the pool holds
+  int c0, c1;           // classes of this pass (the pool may not hold every class's rows at once)
 };
 
-__host__ __device__ inline GoodputSmem goodput_smem(int K4, int G, int gt_len, int nwarp) {
-  GoodputSmem m{};
+// First row of (sigma, class i) in the pool: the rows wanted by the pass's
+// classes in order (a few dozen additions; every caller finds the same).
+__device__ __forceinline__ int span_rows(const GoodputTables& g, int K, int sc) {
+  const int lo = g.span[sc], hi = g.span[2 * K + sc];
+  const int i = sc < K ? sc : sc - K;
+  return i >= g.c0 && i < g.c1 && hi >= lo ? hi - lo + 1 : 0;
+}
+
+// Inclusive scan over the lanes (rows of the (realisation, class) pairs lane,
+// lane + 32, .. < 2K handled by the caller).
+__device__ __forceinline__ int warp_scan(int v, int lane) {
+  for (int o = 1; o < 32; o <<= 1) {
+    const int y = __shfl_up_sync(0xffffffffu, v, o);
+    if (lane >= o) v += y;
+  }
+  return v;
+}
+
+// Tasks of k_other: one warp per (realisation, class, row), and two more for
+// the base realisations' goodput (t* itself, every class).
+//
+// A programme over the other classes within g GPUs, lanes over g, over the GPUs
+// that their cheapest options leave (h = g - need; below need nothing reaches):
+// options cost e = cost - cheapest of them. Then the best of class i's own rows
+// at their base capacities on top, for candidates on another of its rows.
+// What bounds it: issue slots of the inner step (two shared loads, an add and a
+// maximum), about 5 k warp instructions a row at eight classes and 256 GPUs.
+constexpr int kOtherWarps = 4;
+
+struct OtherSmem {
+  size_t rows, lohi, mins, opt, dp, per_warp, total;
+  int n_opt;
+};
+
+__host__ __device__ inline OtherSmem other_smem(int K, int G) {
+  OtherSmem m{};
   auto up = [](size_t x) { return (x + 15) & ~(size_t)15; };
-  m.gtab = 0;
-  m.cap = up(m.gtab + 8 * (size_t)gt_len);
-  m.val = up(m.cap + 8 * (size_t)gt_len);
-  m.flag = up(m.val + 16 * (size_t)gt_len);
-  m.warps = up(m.flag + (size_t)gt_len);
-  m.per_warp = up(sizeof(RowOpt) * (size_t)K4) + 16 * ((size_t)G + 1);
-  m.total = m.warps + (size_t)nwarp * m.per_warp;
+  m.n_opt = G + (G >> 1) + (G >> 2) + (G >> 3);
+  m.rows = 0;                                    // per block: base capacities [2][4K], feasible [2][4K]
+  const size_t shared = up(16 * (size_t)(4 * K));
+  m.lohi = 0;                                    // per warp: option ranges [4K] x 2
+  m.mins = up(8 * (size_t)(4 * K));              // [K]
+  m.opt = up(m.mins + 4 * (size_t)K);            // one class's option values
+  m.dp = up(m.opt + 8 * (size_t)m.n_opt);        // two arrays of G + 1
+  m.per_warp = up(m.dp + 16 * ((size_t)G + 1));
+  m.total = shared + kOtherWarps * m.per_warp;
+  m.rows = shared;
   return m;
 }
 
-// One block per segment (candidate e, outcome o) at a time. Entries: [0, W)
-// open gate at position k; [W, 2W) closed gate at position k - W (under the
-// prior), or W alone (closed, one value). A realisation's goodput depends on
-// an entry only through its patched row capacity C' (t* is a function of
-// C'), and consecutive entries often share C' (every position whose c_y lies
-// at or below Cexcl, or is clamped by the refit): a run of equal C' takes one
-// evaluation. The evaluation splits the programme at class i_r: the other
-// classes' best within g GPUs depends on the entry only through the replica
-// ranges that t* leaves their rows, which change at few values of t* in a
-// segment, so a warp reruns that part only where a range changes and
-// otherwise only combines it with class i_r's choices. Then the same draws
-// and sums as the table path.
-// MINB: resident blocks per SM the registers are capped for (2, or 4 for
-// launches of many segments, whose throughput gains more from the occupancy
-// than each block loses).
-template <bool FL, bool RF, int MINB>
-__global__ void __launch_bounds__(256, MINB) k_score_goodput(Set set, Items it, Plan pl, const float* rec,
-                                                          uint64_t* sums) {
+template <bool FL>
+__global__ void __launch_bounds__(32 * kOtherWarps) k_other(Set set, GoodputTables gt, OtherSmem lay) {
   extern __shared__ __align__(16) unsigned char smraw[];
   const Dims& d = set.d;
-  const int W = pl.W, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nwarp = blockDim.x >> 5;
-  const int gt_len = RF ? 2 * W : W + 1;
-  const GoodputSmem lay = goodput_smem(d.K4, d.G, gt_len, nwarp);
-  uint64_t* gtab = reinterpret_cast<uint64_t*>(smraw + lay.gtab);
-  float* cap = reinterpret_cast<float*>(smraw + lay.cap);          // [2][gt_len]
-  long long* val = reinterpret_cast<long long*>(smraw + lay.val);  // [2][gt_len]
-  uint8_t* flag = smraw + lay.flag;  // bit 0 / 1: a run starts here (realisation 0 / 1); bit 2: reachable
-  unsigned char* wbase = smraw + lay.warps + (size_t)warp * lay.per_warp;
-  RowOpt* opt = reinterpret_cast<RowOpt*>(wbase);
-  long long* dpa = reinterpret_cast<long long*>(wbase + ((sizeof(RowOpt) * (size_t)d.K4 + 15) & ~(size_t)15));
-  long long* dpb = dpa + (d.G + 1);
-  __shared__ float sC[2][256];
-  __shared__ int sOk[2][256];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   __shared__ float sLam[FS_MAX_CLASSES], sRl[FS_MAX_CLASSES], sDl[FS_MAX_CLASSES];
-  for (int x = tid; x < 2 * d.K4; x += blockDim.x) {
-    const int sg = x / d.K4, rho = x - sg * d.K4;
-    sC[sg][rho] = set.rowC[(size_t)sg * d.K4 + rho];
-    sOk[sg][rho] = set.rowB[(size_t)sg * d.K4 + rho] >= 0;
+  __shared__ int sBeg[2 * FS_MAX_CLASSES + 1];
+  float* sC = reinterpret_cast<float*>(smraw);   // [2][K4]
+  int* sOk = reinterpret_cast<int*>(sC + 2 * d.K4);
+  unsigned char* mem = smraw + lay.rows + (size_t)warp * lay.per_warp;
+  int* sLo = reinterpret_cast<int*>(mem + lay.lohi);
+  int* sHi = sLo + d.K4;
+  int* sMin = reinterpret_cast<int*>(mem + lay.mins);
+  long long* sOpt = reinterpret_cast<long long*>(mem + lay.opt);
+  long long* cur = reinterpret_cast<long long*>(mem + lay.dp);
+  long long* nxt = cur + (d.G + 1);
+  pdl_wait();
+  pdl_trigger();
+  for (int x = threadIdx.x; x < 2 * d.K4; x += blockDim.x) {
+    sC[x] = set.rowC[x];
+    sOk[x] = set.rowB[x] >= 0;
   }
-  for (int i = tid; i < d.K; i += blockDim.x) {
-    sLam[i] = set.lam[i];
-    sRl[i] = __frcp_rn(set.lam[i]);
+  for (int i = threadIdx.x; i < d.K; i += blockDim.x) {
+    const float lam = set.lam[i];
+    sLam[i] = lam;
+    sRl[i] = __frcp_rn(lam);
     sDl[i] = FL ? set.slo[d.K + i] : 0.0f;
   }
+  if (warp == 0) {  // first task of each (realisation, class)
+    int carry = 0;
+    for (int b = 0; b < 2 * d.K; b += 32) {
+      const int sc = b + lane;
+      const int incl = warp_scan(sc < 2 * d.K ? span_rows(gt, d.K, sc) : 0, lane);
+      if (sc < 2 * d.K) sBeg[sc + 1] = carry + incl;
+      carry += __shfl_sync(0xffffffffu, incl, 31);
+    }
+    if (lane == 0) sBeg[0] = 0;
+  }
   __syncthreads();
-  const PhiloxKeys keys{};  // (the plan's round keys serve a one-problem launch)
-  const long long n_seg = (long long)it.n * pl.O;
-  for (long long seg = blockIdx.x; seg < n_seg; seg += gridDim.x) {
-    const long long* other = nullptr;  // the warp's programme over the other classes, for this segment
-    bool other_pos = false;
-    int other_sg = 0;
-    const int item = (int)(seg / pl.O), o = (int)(seg - (long long)item * pl.O);
-    const float* r = rec + (size_t)item * pl.item_floats;
-    const float* h0 = r;
-    const float* h1 = r + d.slot_floats;
-    const float* win = r + 2 * (size_t)d.slot_floats + (size_t)o * pl.Wp;
-    const int cell = __float_as_int(h0[H_CELL]);
-    if (cell < 0 || cell >= d.cells) continue;  // flagged by the preparation (uniform over the block)
-    const int rr = cell / d.B;
-    const uint32_t kgs = (uint32_t)__float_as_int(win[0]) << pl.sh;
-    const uint32_t kgs16 = (uint32_t)min((unsigned long long)kgs << 16, 0xFFFFFFFFull);
-    const bool any_open = kgs != 0u, any_closed = kgs16 != 0xFFFFFFFFu;
-    const RowCap a0 = row_cap_of(h0), a1 = row_cap_of(h1);
-    auto reachable = [&](int k) { return k < W ? any_open : any_closed; };
-    // each entry's patched row capacity in both realisations
-    for (int k = tid; k < gt_len; k += blockDim.x) {
-      const bool g = k < W;
-      const float cy = g ? win[4 + k] : (RF ? win[4 + k - W] : 0.0f);
-      cap[k] = RF ? row_cap(a0, cy, g) : (g ? fmaxf(a0.pc, cy) : a0.pc);
-      cap[gt_len + k] = RF ? row_cap(a1, cy, g) : (g ? fmaxf(a1.pc, cy) : a1.pc);
-    }
-    __syncthreads();
-    // where runs of equal capacity start, and t* there
-    for (int k = tid; k < gt_len; k += blockDim.x) {
-      uint8_t f = 0;
-      if (reachable(k)) {
-        f = 4;
-        const bool first = k == 0 || !reachable(k - 1);
-        const float c0 = cap[k], c1 = cap[gt_len + k];
-        if (first || __float_as_uint(c0) != __float_as_uint(cap[k - 1])) {
-          f |= 1;
-          val[k] = (long long)__float_as_uint(tstar_global<FL>(h0, c0));
-        }
-        if (first || __float_as_uint(c1) != __float_as_uint(cap[gt_len + k - 1])) {
-          f |= 2;
-          val[gt_len + k] = (long long)__float_as_uint(tstar_global<FL>(h1, c1));
-        }
+  const int rows = sBeg[2 * d.K];
+  if (rows > gt.pool) {  // cannot happen: the host sized the pool for the most rows there can be
+    if (blockIdx.x == 0 && threadIdx.x == 0) atomicOr(set.status, ST_TABLE);
+    return;
+  }
+  const int n_base = gt.c0 == 0 ? 2 : 0;  // (the first pass)
+  for (int task = (int)blockIdx.x * kOtherWarps + warp; task < rows + n_base; task += (int)gridDim.x * kOtherWarps) {
+    const bool base = task >= rows;
+    int sigma, cls, kk = 0;
+    float t;
+    if (base) {
+      sigma = task - rows;
+      cls = 0;
+      t = base_tstar(set, 0, sigma);
+    } else {
+      int sc = 0, hi = 2 * d.K - 1;
+      while (sc < hi) {
+        const int mid = (sc + hi + 1) >> 1;
+        if (sBeg[mid] <= task) sc = mid; else hi = mid - 1;
       }
-      flag[k] = f;
+      sigma = sc >= d.K ? 1 : 0;
+      cls = sc - sigma * d.K;
+      kk = gt.span[sc] + task - sBeg[sc];
+      const int total = set.ntheta[sigma];
+      const float* th = set.theta + (size_t)sigma * d.theta_cap;
+      if (kk == 0) t = 0.0f;
+      else if (kk <= total) t = th[kk - 1];
+      else t = total ? __uint_as_float(__float_as_uint(th[total - 1]) + 1u) : __uint_as_float(1u);
     }
-    __syncthreads();
-    // the warps take chunks of 32 entries of one realisation in turn; a chunk's
-    // first reachable entry starts a run. Every run start's row-r range comes
-    // from its own lane; the others' programme is rerun only where a row's
-    // range changes with t*
-    {
-      const int ir = rr >> 2, jr = rr & 3;
-      const float lam_r = sLam[ir], rl_r = sRl[ir], dl_r = FL ? sDl[ir] : 0.0f;
-      const int n_chunk = (gt_len + 31) >> 5;
-      for (int task = warp; task < 2 * n_chunk; task += nwarp) {
-        const int sg = task & 1, kk = ((task >> 1) << 5) + lane;
-        const float* cs = cap + (size_t)sg * gt_len;
-        long long* v = val + (size_t)sg * gt_len;
-        const bool reach = kk < gt_len && (flag[kk] & 4);
-        const bool start = reach && ((flag[kk] >> sg) & 1);
-        const unsigned rb = __ballot_sync(0xffffffffu, reach);
-        const bool head = start || (rb && lane == __ffs(rb) - 1);
-        float c = 0.0f, t = 0.0f;
-        int lor = 0, hir = 0;
-        if (head) {  // t* stored where a run starts, else evaluated
-          c = cs[kk];
-          t = start ? __uint_as_float((uint32_t)v[kk]) : tstar_global<FL>(sg ? h1 : h0, c);
-          row_range(c, true, d.G >> jr, class_threshold(t, dl_r), lam_r, rl_r, lor, hir);
+    // option ranges of every row at t, and each class's cheapest option
+    const float* C = sC + sigma * d.K4;
+    __syncwarp();
+    for (int rho = lane; rho < d.K4; rho += 32) {
+      const int i = rho >> 2;
+      int lo, hi;
+      row_range(C[rho], sOk[sigma * d.K4 + rho] != 0, rep_cap(d, rho & 3), class_threshold(t, FL ? sDl[i] : 0.0f),
+                sLam[i], sRl[i], lo, hi);
+      sLo[rho] = lo;
+      sHi[rho] = hi;
+    }
+    __syncwarp();
+    int need = 0;
+    for (int b = 0; b < d.K; b += 32) {
+      const int i = b + lane;
+      int m = 0;
+      if (i < d.K) {
+        const bool empty = !(t > 0.0f) && !(FL && sDl[i] > 0.0f);
+        if (!empty) {
+          m = 1 << 24;  // (above every budget: 64 of them stay below 2^31)
+          for (int j = 0; j < kT; ++j)
+            if (sLo[4 * i + j]) m = min(m, sLo[4 * i + j] << j);
         }
-        unsigned heads = __ballot_sync(0xffffffffu, head);
-        long long mine = 0;
-        while (heads) {
-          const int p = __ffs(heads) - 1;
-          heads &= heads - 1;
-          const float tp = __shfl_sync(0xffffffffu, t, p), cp = __shfl_sync(0xffffffffu, c, p);
-          const int lop = __shfl_sync(0xffffffffu, lor, p), hip = __shfl_sync(0xffffffffu, hir, p);
-          if (other == nullptr || other_sg != sg || !warp_ranges_hold<FL>(d, sDl, opt, tp, other_pos)) {
-            other = warp_other<FL>(d, sC[sg], sOk[sg], sLam, sRl, sDl, ir, rr, tp, opt, dpa, dpb);
-            other_pos = tp > 0.0f;
-            other_sg = sg;
+        sMin[i] = m;
+      }
+      need += __reduce_add_sync(0xffffffffu, i < d.K && i != cls ? m : 0);
+    }
+    __syncwarp();
+    const int H = need <= d.G ? d.G - need + 1 : 0;  // GPUs above the cheapest options: 0..H-1
+    for (int h = lane; h < H; h += 32) cur[h] = 0;
+    __syncwarp();
+    if (H > 0)
+      for (int i = 0; i < d.K; ++i) {
+        if (i == cls) continue;
+        const int m = sMin[i];
+        const bool empty = !(t > 0.0f) && !(FL && sDl[i] > 0.0f);
+        int cnt[kT], beg[kT], all = 0;
+#pragma unroll
+        for (int j = 0; j < kT; ++j) {
+          const int lo = sLo[4 * i + j];
+          cnt[j] = lo ? max(0, min(sHi[4 * i + j], (H - 1 + m) >> j) - lo + 1) : 0;
+          beg[j] = all;
+          all += cnt[j];
+        }
+        for (int x = lane; x < all; x += 32) {
+          int j = 0;
+#pragma unroll
+          for (int q = 1; q < kT; ++q)
+            if (x >= beg[q]) j = q;
+          sOpt[x] = goodput_fx20((float)(sLo[4 * i + j] + x - beg[j]), C[4 * i + j], sLam[i]);
+        }
+        __syncwarp();
+        for (int h = lane; h < H; h += 32) {
+          long long best = empty ? cur[h] : -1;
+#pragma unroll
+          for (int j = 0; j < kT; ++j) {
+            int e = (sLo[4 * i + j] << j) - m;
+            for (int x = 0; x < cnt[j] && e <= h; ++x, e += 1 << j) {
+              const long long v = sOpt[beg[j] + x] + cur[h - e];
+              best = v > best ? v : best;
+            }
           }
-          long long gv = warp_best_with<FL>(d, sLam, sDl, opt, rr, cp, lop, hip, tp, other);
-          gv = gv < 0 ? 0 : gv;
-          if (lane >= p) mine = gv;
+          nxt[h] = best;
         }
-        if (reach) v[kk] = mine;
+        __syncwarp();
+        long long* x = cur;
+        cur = nxt;
+        nxt = x;
+      }
+    // other[g] = cur[g - need], -1 below; the class's own rows on top
+    long long row_best[kT];
+    const bool empty = !(t > 0.0f) && !(FL && sDl[cls] > 0.0f);
+#pragma unroll
+    for (int j = 0; j < kT; ++j) {
+      long long best = -1;
+      const int lo = sLo[4 * cls + j];
+      if (lo && H > 0) {
+        const int top = min(sHi[4 * cls + j], (H - 1) >> j);
+        for (int n = lo + lane; n <= top; n += 32) {
+          const long long v = goodput_fx20((float)n, C[4 * cls + j], sLam[cls]) + cur[H - 1 - (n << j)];
+          best = v > best ? v : best;
+        }
+      }
+      for (int o = 16; o; o >>= 1) {
+        const long long v = __shfl_xor_sync(0xffffffffu, best, o);
+        best = v > best ? v : best;
+      }
+      row_best[j] = best;
+    }
+    const long long none = empty && H > 0 ? cur[H - 1] : -1;  // no replicas for the class
+    if (base) {
+      long long best = none;
+#pragma unroll
+      for (int j = 0; j < kT; ++j) best = row_best[j] > best ? row_best[j] : best;
+      if (lane == 0) gt.base[sigma] = best < 0 ? 0 : best;
+    } else {
+      long long* row = gt.rows + (size_t)task * gt.stride;
+      for (int g = lane; g <= d.G; g += 32) row[g] = g >= need ? cur[g - need] : -1;
+      if (lane < kT) {
+        long long best = none;
+#pragma unroll
+        for (int j = 0; j < kT; ++j)
+          if (j != lane && row_best[j] > best) best = row_best[j];
+        row[d.G + 1 + lane] = best;
       }
     }
-    __syncthreads();
-    for (int k = tid; k < gt_len; k += blockDim.x) {
-      if (!(flag[k] & 4)) continue;
-      const long long g0 = val[k], g1 = val[gt_len + k];
-      const unsigned long long gap = (unsigned long long)(g1 > g0 ? g1 - g0 : g0 - g1);
-      gtab[k] = gap;
-    }
-    __syncthreads();
-    unsigned long long v = sample_gtab<true, RF>(pl, keys, o, cell, 0, pl.calls, smem_u32(gtab), kgs16);
-    for (int off = 16; off; off >>= 1) v += __shfl_down_sync(0xffffffffu, v, off);
-    if (lane == 0 && v) atomicAdd(reinterpret_cast<unsigned long long*>(&sums[(size_t)seg]), v);
-    __syncthreads();  // the tables are rebuilt for the next segment
   }
 }
 
-// E, score and argmax of the goodput stage for one problem (one CTA).
-__global__ void k_finalize_goodput(Set set, Items it, Plan pl, const uint64_t* sums, double lam_sum, double* gap,
-                                   double* score, double* gamma, int32_t* best, uint32_t* status_copy) {
+// What a scenario's goodput in one realisation needs besides C'.
+struct GoodputCtx {
+  const float* h;          // the candidate's table (header, kappa, theta, m) in global memory
+  const long long* rows;   // other rows of (realisation, class), indexed by kk
+  int stride, G, jr, M, lpad, step0, b0, fast;
+  float lam, rl, dl;
+};
+
+// Tier-3 goodput at row capacity C (2^-20 req/s; 0 when the floors cannot be
+// met): t* as the scorer finds it, then the best over row r's replica counts at
+// C on top of the others' best, or the class's best without row r.
+template <bool FL>
+__device__ __forceinline__ long long goodput_at(const GoodputCtx& c, float C) {
+  const float* kap = c.h + kTableHeader;
+  int pos = 0;
+  for (int step = c.step0; step > 0; step >>= 1) pos += kap[pos + step - 1] <= C ? step : 0;
+  const float thb = kap[c.lpad + pos], m = kap[2 * c.lpad + pos];
+  const float tr = m >= 1.0f ? (c.fast ? fulfil_fast(m, C, c.lam, c.rl) : fulfil(m, C, c.lam)) : 0.0f;
+  const bool own = FL ? tr > thb && tr >= c.dl : tr > thb;
+  const float t = own ? tr : thb;
+  const long long* row = c.rows + (size_t)(c.b0 + 1 + pos + (own ? 1 : 0)) * c.stride;
+  int lo, hi;
+  row_range(C, true, c.M, class_threshold(t, FL ? c.dl : 0.0f), c.lam, c.rl, lo, hi);
+  long long best = row[c.G + 1 + c.jr];
+  if (lo) {
+    const int top = min(hi, c.G >> c.jr);
+    for (int n = lo; n <= top; ++n) {
+      const long long pv = row[c.G - (n << c.jr)];
+      if (pv >= 0) {
+        const long long v = goodput_fx20((float)n, C, c.lam) + pv;
+        best = v > best ? v : best;
+      }
+    }
+  }
+  return best < 0 ? 0 : best;
+}
+
+template <bool FL>
+__device__ __forceinline__ GoodputCtx goodput_ctx(const Set& set, const GoodputTables& gt, const float* h, int sigma,
+                                                  int rr) {
+  const Dims& d = set.d;
+  GoodputCtx c;
+  const int i = rr >> 2;
+  c.h = h;
+  c.stride = gt.stride;
+  c.G = d.G;
+  c.jr = rr & 3;
+  c.M = rep_cap(d, c.jr);
+  c.lpad = __float_as_int(h[H_LPAD]);
+  c.step0 = __float_as_int(h[H_STEP0]);
+  c.b0 = __float_as_int(h[H_B0]);
+  c.fast = __float_as_int(h[H_FAST]);
+  c.lam = h[H_LAM];
+  c.rl = h[H_RLAM];
+  c.dl = FL ? h[H_DLT] : 0.0f;
+  const int sc = sigma * d.K + i;
+  int first = 0;  // the class's first row in the pool
+  for (int q = 0; q < sc; ++q) first += span_rows(gt, d.K, q);
+  c.rows = gt.rows + ((long long)first - gt.span[sc]) * gt.stride;
+  return c;
+}
+
+// One block per segment (candidate e, outcome o): entries [0, W) hold the gap
+// with an open gate at position k, W with a closed one (under the prior [W, 2W),
+// position k - W). A thread per entry; without the prior every entry at or
+// below a realisation's Cexcl takes that realisation's closed-gate goodput,
+// evaluated once. Then the same draws and sums as the table path.
+template <bool FL, bool RF>
+__global__ void __launch_bounds__(256) k_score_goodput(Set set, Items it, Plan pl, const float* rec, uint64_t* sums,
+                                                       GoodputTables gt) {
+  extern __shared__ __align__(16) unsigned char smraw[];
+  uint64_t* gtab = reinterpret_cast<uint64_t*>(smraw);
+  __shared__ long long s_closed[2];
+  __shared__ GoodputCtx s_ctx[2];
+  const Dims& d = set.d;
+  const int W = pl.W, tid = threadIdx.x, lane = tid & 31;
+  pdl_wait();
+  pdl_trigger();
+  const PhiloxKeys keys{};  // (the plan's round keys serve a one-problem launch)
+  const long long n_seg = (long long)it.n * pl.O;
+  for (long long seg = blockIdx.x; seg < n_seg; seg += gridDim.x) {
+    const int item = (int)(seg / pl.O), o = (int)(seg - (long long)item * pl.O);
+    const float* h0 = rec + (size_t)item * pl.item_floats;
+    const float* h1 = h0 + d.slot_floats;
+    const float* win = h0 + 2 * (size_t)d.slot_floats + (size_t)o * pl.Wp;
+    const int cell = __float_as_int(h0[H_CELL]);
+    if (cell < 0 || cell >= d.cells) continue;  // flagged by the preparation (uniform over the block)
+    const int rr = cell / d.B, ir = rr >> 2;
+    if (ir < gt.c0 || ir >= gt.c1) continue;    // another pass's class (uniform)
+    const uint32_t kgs = (uint32_t)__float_as_int(win[0]) << pl.sh;
+    const uint32_t kgs16 = (uint32_t)min((unsigned long long)kgs << 16, 0xFFFFFFFFull);
+    const bool any_open = kgs != 0u, any_closed = kgs16 != 0xFFFFFFFFu;
+    if ((tid & 31) == 0 && tid < 64 ) {
+      const int sg = tid >> 5;
+      const float* h = sg ? h1 : h0;
+      s_ctx[sg] = goodput_ctx<FL>(set, gt, h, sg, rr);
+      if (!RF) s_closed[sg] = goodput_at<FL>(s_ctx[sg], h[H_CX]);
+    }
+    __syncthreads();
+    const RowCap a0 = row_cap_of(h0), a1 = row_cap_of(h1);
+    const int k0 = any_open ? 0 : W, k1 = RF ? (any_closed ? 2 * W : W) : any_open ? W + 1 : W + 1;
+    for (int k = k0 + tid; k < k1; k += blockDim.x) {
+      const bool g = k < W;
+      long long g0, g1;
+      if (RF) {
+        const float cy = win[4 + (g ? k : k - W)];
+        g0 = goodput_at<FL>(s_ctx[0], row_cap(a0, cy, g));
+        g1 = goodput_at<FL>(s_ctx[1], row_cap(a1, cy, g));
+      } else {
+        const float cy = g ? win[4 + k] : 0.0f;
+        g0 = g && cy > a0.pc ? goodput_at<FL>(s_ctx[0], cy) : s_closed[0];
+        g1 = g && cy > a1.pc ? goodput_at<FL>(s_ctx[1], cy) : s_closed[1];
+      }
+      gtab[k] = (unsigned long long)(g1 > g0 ? g1 - g0 : g0 - g1);
+    }
+    __syncthreads();
+    unsigned long long v;
+    if (!any_open || !any_closed)  // the gate is the same at every position
+      v = sample_gtab<true, RF, false>(pl, keys, o, cell, 0, pl.calls, smem_u32(gtab) + (any_open ? 0u : 8u * (uint32_t)W),
+                                       0u, (!RF && !any_open) ? pl.uniform_stride : pl.entry_bytes);
+    else
+      v = sample_gtab<true, RF, true>(pl, keys, o, cell, 0, pl.calls, smem_u32(gtab), kgs16);
+    for (int off = 16; off; off >>= 1) v += __shfl_down_sync(0xffffffffu, v, off);
+    if (lane == 0 && v) atomicAdd(reinterpret_cast<unsigned long long*>(&sums[(size_t)seg]), v);
+    __syncthreads();  // the table is rebuilt for the next segment
+  }
+}
+
+// E, score and argmax of the goodput stage for one problem, its candidates
+// split over the blocks: each leaves its best in part[2 b ..], the last to take a
+// ticket (work[1], zeroed by the preparation) merges them.
+__global__ void k_finalize_goodput(Set set, Items it, Plan pl, const uint64_t* sums, const long long* base,
+                                   double lam_sum, double* gap, double* score, double* gamma, int32_t* best,
+                                   uint32_t* status_copy, uint64_t* part) {
   __shared__ Best sb[32];
-  // every earlier kernel of the call has completed: the status word travels
-  // with the outputs
-  if (threadIdx.x == 0 && status_copy) *status_copy = *set.status;
+  __shared__ int s_last;
+  pdl_wait();
+  pdl_trigger();
   const Dims& d = set.d;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nwarp = blockDim.x >> 5;
-  const long long gm = __double2ll_rn(__dmul_rn(set.base[0].goodput, 0x1p20));
-  const long long gpl = __double2ll_rn(__dmul_rn(set.base[1].goodput, 0x1p20));
+  const int nb = (int)gridDim.x, per = (it.n + nb - 1) / nb;
+  const int beg = min(it.n, (int)blockIdx.x * per), end = min(it.n, beg + per);
+  const long long gm = base[0], gpl = base[1];
   const long long gfix = gpl > gm ? gpl - gm : gm - gpl;
   const long long n = (long long)pl.O * pl.S;
   const double dn = __ll2double_rn(n);
   Best b = no_best();
-  for (int q = tid; q < it.n; q += blockDim.x) {
+  for (int q = beg + tid; q < end; q += blockDim.x) {
     const int cell = it.cell[q];
     long long tot = 0;
-    for (int o = 0; o < pl.O; ++o) tot += (long long)sums[(size_t)q * pl.O + o];
+#pragma unroll 8
+    for (int o = 0; o < pl.O; ++o) tot += (long long)__ldg(sums + (size_t)q * pl.O + o);
     const long long sc = gfix * n - tot;
     if (gap) gap[q] = __ddiv_rn(__ddiv_rn(__dmul_rn(__ll2double_rn(tot), 0x1p-20), dn), lam_sum);
     if (score) score[q] = __ddiv_rn(__ddiv_rn(__dmul_rn(__ll2double_rn(sc), 0x1p-20), dn), lam_sum);
@@ -750,12 +820,32 @@ __global__ void k_finalize_goodput(Set set, Items it, Plan pl, const uint64_t* s
   b = warp_best(b);
   if (lane == 0) sb[warp] = b;
   __syncthreads();
-  if (warp == 0) {
-    b = warp_best(lane < nwarp ? sb[lane] : no_best());
+  if (warp != 0) return;
+  b = warp_best(lane < nwarp ? sb[lane] : no_best());
+  if (nb > 1) {
     if (lane == 0) {
-      if (best) *best = b.valid() ? b.cell : -1;
-      if (gamma) *gamma = __ddiv_rn(__dmul_rn(__ll2double_rn(gfix), 0x1p-20), lam_sum);
+      part[2 * blockIdx.x] = (uint64_t)b.hi;
+      part[2 * blockIdx.x + 1] = ((uint64_t)b.lo << 32) | (uint32_t)b.cell;
+      __threadfence();
+      s_last = atomicAdd(&set.work[1], 1ull) == (unsigned long long)(nb - 1);
     }
+    __syncwarp();
+    if (!s_last) return;
+    __threadfence();
+    b = no_best();
+    for (int q = lane; q < nb; q += 32) {
+      const uint64_t w = __ldcg(part + 2 * q + 1);
+      const Best c{(long long)__ldcg(part + 2 * q), (uint32_t)(w >> 32), (int)(uint32_t)w};
+      if (better(c, b)) b = c;
+    }
+    b = warp_best(b);
+  }
+  if (lane == 0) {
+    if (best) *best = b.valid() ? b.cell : -1;
+    if (gamma) *gamma = __ddiv_rn(__dmul_rn(__ll2double_rn(gfix), 0x1p-20), lam_sum);
+    // every earlier kernel of the call has completed: the status word travels
+    // with the outputs
+    if (status_copy) *status_copy = *set.status;
   }
 }
 
@@ -798,52 +888,68 @@ cudaError_t launch_solve_lex(const Set& set, int n, const float* cap_x, const fl
   return go(set, n, cap_x, tail_x, out, scratch, per_launch, lay, s);
 }
 
-int goodput_threads(const Dims& d, const Plan& pl, bool rf, size_t* smem) {
-  const int gt_len = rf ? 2 * pl.W : pl.W + 1;
-  for (int nw = 8; nw >= 1; --nw) {
-    const GoodputSmem m = goodput_smem(d.K4, d.G, gt_len, nw);
-    if (m.total <= kGoodputSmemMax) {
-      if (smem) *smem = m.total;
-      return 32 * nw;
-    }
-  }
-  return 0;
+// Rows a (realisation, class) can want: t* = 0, every threshold, one above them.
+static long long goodput_rows_per_class(const Dims& d, int th_bound) {
+  const int bound = th_bound > 0 && th_bound < d.theta_cap ? th_bound : d.theta_cap;
+  return 2LL * (bound + 2);
 }
 
+size_t goodput_pool_rows(const Dims& d, int th_bound, size_t most_bytes) {
+  const long long per = goodput_rows_per_class(d, th_bound);
+  const long long row = 8LL * (d.G + 1 + kT);
+  long long classes = (long long)most_bytes / (per * row);
+  classes = classes < 1 ? 1 : classes > d.K ? d.K : classes;
+  return (size_t)(classes * per);
+}
+
+size_t goodput_row_bytes(const Dims& d) { return 8 * (size_t)(d.G + 1 + kT); }
+
 cudaError_t launch_score_goodput(const Set& set, const Items& it, const Plan& pl, const float* tables,
-                                 uint64_t* sums, int floors, int sm_count, cudaStream_t s) {
-  if (it.n <= 0) return cudaSuccess;
+                                 uint64_t* sums, int* span, long long* base, void* pool, size_t pool_rows,
+                                 int floors, int th_bound, int sm_count, cudaStream_t s) {
+  const Dims& d = set.d;
   const bool rf = set.prior == 1;
-  size_t smem = 0;
-  const int threads = goodput_threads(set.d, pl, rf, &smem);
-  if (threads == 0) return cudaErrorInvalidValue;  // refused by the host before this point
-  // many segments (beyond four waves of two blocks per SM): the instance with
-  // registers for four blocks per SM (measured 5.94 -> 3.44 ms on the
-  // eight-class workload, 0.375 -> 0.325 ms on the mid one at three times its
-  // demands; the paper-scale call, one wave, slower: 0.17 -> 0.19 ms)
-  const long long n_seg = (long long)it.n * pl.O;
-  const bool wide = n_seg > 4LL * 2 * sm_count;
-#define FS_GP(MB) \
-  (floors ? (rf ? k_score_goodput<true, true, MB> : k_score_goodput<true, false, MB>) \
-          : (rf ? k_score_goodput<false, true, MB> : k_score_goodput<false, false, MB>))
-  auto kern = wide ? FS_GP(4) : FS_GP(2);
-#undef FS_GP
-  cudaError_t e = raise_smem_limit(reinterpret_cast<const void*>(kern), smem);
+  GoodputTables gt{};
+  gt.span = span;
+  gt.base = base;
+  gt.rows = static_cast<long long*>(pool);
+  gt.stride = d.G + 1 + kT;
+  gt.pool = (int)pool_rows;
+  const long long per = goodput_rows_per_class(d, th_bound);
+  const int classes = (int)(gt.pool / per);  // classes a pass (all of them unless the pool is at its limit)
+  if (classes < 1) return cudaErrorInvalidValue;
+  const OtherSmem lay = other_smem(d.K, d.G);
+  auto other = floors ? k_other<true> : k_other<false>;
+  const size_t smem = 8 * (size_t)(rf ? 2 * pl.W : pl.W + 1);
+  auto kern = floors ? (rf ? k_score_goodput<true, true> : k_score_goodput<true, false>)
+                     : (rf ? k_score_goodput<false, true> : k_score_goodput<false, false>);
+  cudaError_t e = raise_smem_limit(reinterpret_cast<const void*>(other), lay.total);
+  if (e == cudaSuccess) e = raise_smem_limit(reinterpret_cast<const void*>(kern), smem);
   if (e != cudaSuccess) return e;
-  // one block per segment: segments differ widely in cost (where row r sets
-  // t*, its ranges change often), and the block scheduler evens them out
-  const long long grid = n_seg < 0x7fffffffLL ? n_seg : 0x7fffffffLL;
-  note_launch();
-  kern<<<(unsigned)grid, threads, smem, s>>>(set, it, pl, tables, sums);
-  return cudaGetLastError();
+  // one block per segment: segments differ in cost, and the block scheduler
+  // evens them out
+  const long long n_seg = (long long)it.n * pl.O;
+  const unsigned grid = (unsigned)(n_seg < 0x7fffffffLL ? n_seg : 0x7fffffffLL);
+  for (gt.c0 = 0; gt.c0 < d.K; gt.c0 = gt.c1) {
+    gt.c1 = gt.c0 + classes < d.K ? gt.c0 + classes : d.K;
+    // a warp per row wanted, as many blocks as run at once (the count is not
+    // known here; the rows are dealt to the warps)
+    const long long most = ((long long)(gt.c1 - gt.c0) * per + 2 + kOtherWarps - 1) / kOtherWarps;
+    const long long fit = 8LL * sm_count;
+    e = launch_pdl(other, dim3((unsigned)(most < fit ? most : fit)), dim3(32 * kOtherWarps), lay.total, s, set, gt, lay);
+    if (e != cudaSuccess) return e;
+    if (it.n > 0) e = launch_pdl(kern, dim3(grid), dim3(256), smem, s, set, it, pl, tables, sums, gt);
+    if (e != cudaSuccess) return e;
+  }
+  return cudaSuccess;
 }
 
 cudaError_t launch_finalize_goodput(const Set& set, const Items& it, const Plan& pl, const uint64_t* sums,
-                                    double lam_sum, double* gap, double* score, double* gamma, int32_t* best,
-                                    uint32_t* status_copy, cudaStream_t s) {
-  note_launch();
-  k_finalize_goodput<<<1, 256, 0, s>>>(set, it, pl, sums, lam_sum, gap, score, gamma, best, status_copy);
-  return cudaGetLastError();
+                                    const long long* base, double lam_sum, double* gap, double* score, double* gamma,
+                                    int32_t* best, uint32_t* status_copy, uint64_t* part, cudaStream_t s) {
+  const int nb = std::max(1, finalize_blocks(it));
+  return launch_pdl(k_finalize_goodput, dim3(nb), dim3(256), 0, s, set, it, pl, sums, base, lam_sum, gap, score, gamma,
+                    best, status_copy, part);
 }
 
 }  // namespace fs

@@ -560,7 +560,11 @@ __global__ void __launch_bounds__(kPrepThreads) k_prep(Set set, Items it, Plan p
     // (under the prior every C' lies in [cx, cmax])
     const bool fast = in_markstein_range(lam) && cmax <= 0x1p44f &&
                       (cx >= 0x1p-60f || (!RF && cx == 0.0f && (lo_c >= 0x1p-60f || hi_c == 0.0f)));
-    tab[H_TH_BASE] = b0 >= 0 ? th[b0] : 0.0f;
+    tab[H_B0] = __int_as_float(b0);
+    if (set.gp_span) {  // t* = theta_b0 (or 0) .. above theta_b1: rows b0 + 1 .. b1 + 2
+      atomicMin(&set.gp_span[sigma * d.K + ie], b0 + 1);
+      atomicMax(&set.gp_span[(2 + sigma) * d.K + ie], min(b1 + 2, total + 1));
+    }
     // t* at row capacity Cexcl (no kappa entry is at or below it): the value of
     // every scenario of this candidate whose tail gate is closed
     tab[H_TCL] = tstar_of<2, FL>(cx, kap, thx, mnx, Lt ? P >> 1 : 0, lam, rl, dle);

@@ -115,6 +115,10 @@ __global__ void __launch_bounds__(kThreshThreads) k_thresh(Set set) {
       set.rowB[ps * d.K4 + rho] = sB[rho];
     }
     if (tid == 0) set.ntheta[ps] = total;
+    if (set.gp_span && tid < d.K) {
+      set.gp_span[sigma * d.K + tid] = 0x7fffffff;
+      set.gp_span[(2 + sigma) * d.K + tid] = -1;
+    }
   }
 
   int lgs = 2;
