@@ -33,7 +33,14 @@ namespace fs {
 
 constexpr int kT = 4;                 // TP degrees {1, 2, 4, 8}
 constexpr int kCostInf = 0x3FFFFFFF;  // "no option covers the threshold"
-constexpr int kSolveWideMax = 608;    // most realisations solved by a block each (else a warp each)
+// Most realisations solved by a block each (else a warp each). Measured, block
+// against warp: 608 realisations of the (2, 16), (4, 64), (8, 256) grids
+// (classes, GPUs) 8.3 / 8.3, 10.3 / 12.3, 8.3 / 12.4 us, 900: 10.3 / 10.3,
+// 12.4 / 12.3, 10.9 / 14.4, 2000: 16.5 / 10.3, 19.4 / 12.4, 16.5 / 18.5. The
+// tier-4 solve's wide block (16 warps) at 450: 16.5 / 14.4, 20.6 / 20.6, 26.7 /
+// 30.8 with the first pass, at 608: 20.6 / 16.8, 26.7 / 20.5, 36.9 / 30.8.
+constexpr int kSolveWideMax = 900;
+constexpr int kLexWideMax = 450;
 constexpr int kThreshThreads = 256;
 constexpr int kThreshBlocks = 64;     // most blocks of k_thresh per realisation
 constexpr int kPrepThreads = 256;
@@ -483,8 +490,15 @@ cudaError_t launch_qtable(float* qn, int Q, cudaStream_t s);
 // Base or explicit realisations: realisation r of `n` reads cap/tail either
 // from the problem set's bounds (explicit == nullptr: r = 2 p + sigma) or from
 // cap_x / tail_x [n][cells].
+// A synchronous call's results, written by the kernels themselves into mapped
+// page-locked memory (no copy after them): copies of the allocations, and per
+// realisation the status word as its solve leaves it. Null members: none.
+struct HostOut {
+  fs_allocation* alloc;
+  uint32_t* status;
+};
 cudaError_t launch_solve(const Set& set, int n, const float* cap_x, const float* tail_x,
-                         fs_allocation* out, LaunchCache& lc, cudaStream_t s);
+                         fs_allocation* out, LaunchCache& lc, cudaStream_t s, HostOut host = HostOut{});
 // Sorted thresholds, rows and row tables of both realisations of every
 // problem of the set. th_bound > 0: a bound on either realisation's threshold
 // count (theta_cap otherwise). With set.tpart (one problem) the launch's block
@@ -527,7 +541,7 @@ size_t lex_scratch_cells(const Dims& d);  // (K + 1)(G + 1) cells per realisatio
 // when lex_needs_scratch says so (the cells do not fit shared memory).
 bool lex_needs_scratch(const Dims& d, int n, bool pack);
 cudaError_t launch_solve_lex(const Set& set, int n, const float* cap_x, const float* tail_x, fs_allocation* out,
-                             void* scratch, int per_launch, bool pack, cudaStream_t s);
+                             void* scratch, int per_launch, bool pack, cudaStream_t s, HostOut host = HostOut{});
 // The goodput stage's tables of the other classes' best goodput: rows of
 // goodput_row_bytes each, goodput_pool_rows of them (every row the call can
 // want, or as many whole classes' as most_bytes holds, at least one's: the

@@ -177,7 +177,8 @@ constexpr size_t kLexCellsWide = 128 * 1024;
 template <bool PACK, int NW>
 __global__ void __launch_bounds__(NW == 1 ? 128 : 32 * NW) k_solve_lex(Set set, int n_real, const float* cap_x,
                                                                        const float* tail_x, fs_allocation* out_x,
-                                                                       unsigned char* scratch, int r0, LexSmem lay) {
+                                                                       unsigned char* scratch, int r0, LexSmem lay,
+                                                                       HostOut host) {
   using L = Lex<PACK>;
   using V = typename L::T;
   constexpr int kPerBlock = NW == 1 ? 4 : 1, kThreads = 32 * NW;
@@ -208,8 +209,19 @@ __global__ void __launch_bounds__(NW == 1 ? 128 : 32 * NW) k_solve_lex(Set set, 
     out = set.base + r;
   }
   const float tstar = out->t_star;
+  // the first warp, once the allocation is complete: its copy for the host
+  auto finish = [&]() {
+    __syncwarp();
+    if (host.alloc) {
+      const uint64_t* src = reinterpret_cast<const uint64_t*>(out);
+      uint64_t* dst = reinterpret_cast<uint64_t*>(host.alloc + r);
+      for (int w = lane; w < (int)(sizeof(fs_allocation) / 8); w += 32) dst[w] = src[w];
+    }
+    if (host.status && lane == 0) host.status[r] = *set.status;
+  };
   if (!out->floors_met) {  // tier 1 cannot hold: nothing is allocated (k_solve wrote the empty allocation)
     if (tid == 0) out->goodput = 0.0;
+    if (warp == 0) finish();
     return;
   }
   unsigned char* mem = smraw + (size_t)slot * lay.total;
@@ -254,6 +266,7 @@ __global__ void __launch_bounds__(NW == 1 ? 128 : 32 * NW) k_solve_lex(Set set, 
       atomicOr(set.status, ST_THETA);
       out->goodput = 0.0;
     }
+    if (warp == 0) finish();
     return;
   }
   // class i's options with e <= slack in the order of preference (no replicas,
@@ -389,6 +402,7 @@ __global__ void __launch_bounds__(NW == 1 ? 128 : 32 * NW) k_solve_lex(Set set, 
     out->total_gpus = total;
     out->goodput = (double)L::gp(top) * 0x1p-20;
   }
+  finish();
 }
 
 // --------------------------------------------------------------------------- goodput stage
@@ -855,7 +869,7 @@ size_t lex_scratch_cells(const Dims& d) { return (size_t)(d.K + 1) * (d.G + 1); 
 
 // Whether the programme of n realisations needs scratch in global memory.
 static LexSmem lex_layout(const Dims& d, int n, bool pack) {
-  return n <= kSolveWideMax ? lex_smem(d.K, d.G, pack, kLexOptWide, kLexCellsWide)
+  return n <= kLexWideMax ? lex_smem(d.K, d.G, pack, kLexOptWide, kLexCellsWide)
                             : lex_smem(d.K, d.G, pack, kLexOptWarp, kLexCellsWarp);
 }
 
@@ -863,7 +877,7 @@ bool lex_needs_scratch(const Dims& d, int n, bool pack) { return lex_layout(d, n
 
 template <bool PACK, int NW>
 static cudaError_t launch_lex(const Set& set, int n, const float* cap_x, const float* tail_x, fs_allocation* out,
-                              void* scratch, int per_launch, const LexSmem& lay, cudaStream_t s) {
+                              void* scratch, int per_launch, const LexSmem& lay, cudaStream_t s, HostOut host) {
   constexpr int kPerBlock = NW == 1 ? 4 : 1;
   auto kern = k_solve_lex<PACK, NW>;
   const size_t smem = kPerBlock * lay.total;
@@ -873,7 +887,7 @@ static cudaError_t launch_lex(const Set& set, int n, const float* cap_x, const f
     const int m = n - r0 < per_launch ? n - r0 : per_launch;
     note_launch();
     kern<<<(m + kPerBlock - 1) / kPerBlock, NW == 1 ? 128 : 32 * NW, smem, s>>>(
-        set, r0 + m, cap_x, tail_x, out, static_cast<unsigned char*>(scratch), r0, lay);
+        set, r0 + m, cap_x, tail_x, out, static_cast<unsigned char*>(scratch), r0, lay, host);
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
   }
@@ -881,11 +895,11 @@ static cudaError_t launch_lex(const Set& set, int n, const float* cap_x, const f
 }
 
 cudaError_t launch_solve_lex(const Set& set, int n, const float* cap_x, const float* tail_x, fs_allocation* out,
-                             void* scratch, int per_launch, bool pack, cudaStream_t s) {
+                             void* scratch, int per_launch, bool pack, cudaStream_t s, HostOut host) {
   const LexSmem lay = lex_layout(set.d, n, pack);
-  auto go = n <= kSolveWideMax ? (pack ? launch_lex<true, kLexWideWarps> : launch_lex<false, kLexWideWarps>)
+  auto go = n <= kLexWideMax ? (pack ? launch_lex<true, kLexWideWarps> : launch_lex<false, kLexWideWarps>)
                                : (pack ? launch_lex<true, 1> : launch_lex<false, 1>);
-  return go(set, n, cap_x, tail_x, out, scratch, per_launch, lay, s);
+  return go(set, n, cap_x, tail_x, out, scratch, per_launch, lay, s, host);
 }
 
 // Rows a (realisation, class) can want: t* = 0, every threshold, one above them.

@@ -126,7 +126,8 @@ __device__ __forceinline__ void search_aims(const SolveSmem& sm, const Dims& d, 
 // latency counts: the rows and the probes are then spread over the warps.
 template <bool FL, int NW>
 __global__ void __launch_bounds__(NW == 1 ? 128 : 32 * NW) k_solve(Set set, int n_real, const float* cap_x,
-                                                                   const float* tail_x, fs_allocation* out_x) {
+                                                                   const float* tail_x, fs_allocation* out_x,
+                                                                   HostOut host) {
   constexpr int kPerBlock = NW == 1 ? 4 : 1;  // realisations per block
   __shared__ SolveSmem smem[kPerBlock];
   const Dims& d = set.d;  // kernel-parameter space: no local copy
@@ -296,7 +297,12 @@ __global__ void __launch_bounds__(NW == 1 ? 128 : 32 * NW) k_solve(Set set, int 
   }
   __syncwarp();
   uint64_t* dst = reinterpret_cast<uint64_t*>(out);
-  for (int w = lane; w < (int)(sizeof(fs_allocation) / 8); w += 32) dst[w] = words[w];
+  uint64_t* dst2 = host.alloc ? reinterpret_cast<uint64_t*>(host.alloc + r) : nullptr;
+  for (int w = lane; w < (int)(sizeof(fs_allocation) / 8); w += 32) {
+    dst[w] = words[w];
+    if (dst2) dst2[w] = words[w];
+  }
+  if (host.status && lane == 0) host.status[r] = *set.status;
 }
 
 // Watchdog self-test: wait on a barrier phase that nothing completes; the
@@ -322,18 +328,17 @@ cudaError_t launch_qtable(float* qn, int Q, cudaStream_t s) {
 }
 
 // Measured (one GB300, calls in a row): 4096 realisations of the four-class,
-// 64-GPU grid 71.7 -> 14.6 us (11.5 M -> 5 M warp instructions against the first
-// one-warp version, whose rows and cover counts took more of them).
+// 64-GPU grid 71.7 -> 14.6 us (6.5 M warp instructions, issue slots 56 % busy).
 cudaError_t launch_solve(const Set& set, int n, const float* cap_x, const float* tail_x,
-                         fs_allocation* out, LaunchCache& lc, cudaStream_t s) {
+                         fs_allocation* out, LaunchCache& lc, cudaStream_t s, HostOut host) {
   if (n <= 0) return cudaSuccess;
   note_launch();
   if (n <= kSolveWideMax) {
     auto kern = lc.floors ? k_solve<true, 8> : k_solve<false, 8>;
-    kern<<<n, 256, 0, s>>>(set, n, cap_x, tail_x, out);
+    kern<<<n, 256, 0, s>>>(set, n, cap_x, tail_x, out, host);
   } else {
     auto kern = lc.floors ? k_solve<true, 1> : k_solve<false, 1>;
-    kern<<<(n + 3) / 4, 128, 0, s>>>(set, n, cap_x, tail_x, out);
+    kern<<<(n + 3) / 4, 128, 0, s>>>(set, n, cap_x, tail_x, out, host);
   }
   return cudaGetLastError();
 }

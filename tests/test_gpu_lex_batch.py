@@ -16,7 +16,7 @@ pytestmark = pytest.mark.gpu
 
 
 @pytest.mark.parametrize("n,K,B,G,scale,floors", [
-    (700, 2, 8, 16, 1.0, False), (700, 3, 5, 33, 1.0, True), (610, 1, 3, 1, 1.0, False),
+    (1000, 2, 8, 16, 1.0, False), (700, 3, 5, 33, 1.0, True), (610, 1, 3, 1, 1.0, False),
     (620, 8, 4, 256, 1.0, False),            # one warp, cells in scratch
     (612, 3, 4, 40, 2.0**24, False),         # two-word values
     (9, 8, 32, 256, 1.0, True), (7, 12, 3, 64, 2.0**24, False),

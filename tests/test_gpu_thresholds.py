@@ -23,8 +23,8 @@ def _scaled(w, cap=1.0, demand=1.0):
     return dataclasses.replace(w, cap_lo=w.cap_lo * f(cap), cap_hi=w.cap_hi * f(cap), demand=w.demand * f(demand))
 
 
-# (700 realisations: a warp each; 20: a block each)
-@pytest.mark.parametrize("n", [700, 20])
+# (1000 realisations: a warp each; 20: a block each)
+@pytest.mark.parametrize("n", [1000, 20])
 @pytest.mark.parametrize("K,B,G,floors,cap,demand", [
     (2, 8, 16, False, 1.0, 3.0), (1, 7, 2000, False, 1.0, 900.0), (3, 5, 1, False, 1.0, 1.0),
     (4, 16, 64, True, 1.0, 6.0), (8, 32, 256, False, 1.0, 20.0), (9, 3, 40, True, 1.0, 2.0),
