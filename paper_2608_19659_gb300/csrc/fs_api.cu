@@ -376,7 +376,8 @@ int run_score(fs_model* m, Set set, const fs_samples* smp, const int32_t* cand_d
   it.p = nullptr;
   it.cell = cand_dev;
   it.off = nullptr;
-  const Plan pl = make_plan(m, smp, n);
+  Plan pl = make_plan(m, smp, n);
+  pl.few = !dump && few_path(pl, n) ? 1 : 0;
   const bool timed = m->timing && n > 0 && m->ev_used + 5 <= kMaxTimedEvents;
   cudaEvent_t* ev = nullptr;
   if (timed) {
@@ -1002,7 +1003,8 @@ int fs_replay(fs_model* m, const fs_replay_spec* sp, int32_t* rounds, int32_t* s
       it.cell = rs.item_cell;
       it.off = nullptr;
       fs_samples smp{sp->seed, 0, (uint32_t)r, n_items, sp->O, sp->S, 0, nullptr};
-      const Plan pl = make_plan(m, &smp, n_items);
+      Plan pl = make_plan(m, &smp, n_items);
+      pl.few = few_path(pl, n_items) ? 1 : 0;
       FS_CUDA(launch_prep(set, it, pl, (float*)m->tables.p, (uint64_t*)m->sums.p, false, m->sm_count, m->lc, s),
               "launch prep");
       FS_CUDA(launch_score(set, it, pl, (const float*)m->tables.p, (uint64_t*)m->sums.p, nullptr, 0, m->sm_count,

@@ -188,6 +188,7 @@ struct Plan {
   // A parameter like the others: every scenario still computes its position
   // and its entry's address, and the kernel is not specialised for that table
   uint32_t uniform_stride;
+  int few;              // 1: few samples per segment (few_path): no mapped windows, k_score_few
 };
 
 // Round keys of problem 0 for the plan (host).
@@ -515,6 +516,8 @@ cudaError_t launch_thresh(Set& set, int floors, int th_bound, cudaStream_t s);
 cudaError_t launch_prep(const Set& set, const Items& it, const Plan& pl, float* tables,
                         uint64_t* sums, bool early, int sm_count, LaunchCache& lc, cudaStream_t s,
                         int th_bound = 0);
+// Whether a launch takes k_score_few (the plan's `few`, set before launch_prep).
+bool few_path(const Plan& pl, int n_items);
 cudaError_t launch_score(const Set& set, const Items& it, const Plan& pl, const float* tables,
                          uint64_t* sums, void* dump, int dump_stride, int sm_count, LaunchCache& lc,
                          cudaStream_t s);

@@ -290,11 +290,12 @@ __global__ void __launch_bounds__(kPrepThreads) k_prep(Set set, Items it, Plan p
     }
   }
 
-  // Mapped strata. Window of outcome o: word 0 = the number of leading
+  // Mapped strata (unless the samples are few, whose scorer maps its draws).
+  // Window of outcome o: word 0 = the number of leading
   // positions whose tail value passes the SLO (the mapped tails are
   // nondecreasing in the position, so exactly one position ends the run of
   // passes), words 4.. = the W capacities.
-  {
+  if (!pl.few) {
     const int W = pl.W;
     const float d_c = __fsub_rn(hi_c, lo_c), d_l = __fsub_rn(hi_l, lo_l);
     const long long n_idx = (long long)((pl.O - sigma + 1) >> 1) * W;
@@ -1183,6 +1184,87 @@ __global__ void __launch_bounds__(kScoreThreads, 4) k_score(Set set, Items it, P
   }
 }
 
+// Few samples per segment: gsz lanes (a power of two, at most 32) per segment,
+// a call each at a time, everything read where it is (the candidates' tables
+// through L1, shared by the segments of a block): no staging, no windows (each
+// draw's capacity and tail are mapped from its quantiles and the tail compared
+// with the SLO, as the dump does), no chunks and no atomics: the group's sum is
+// the segment's. A call's four samples search each realisation's table side by
+// side. What bounds it: the dependent loads of those searches. A block per
+// segment (the plain path) left all but calls of its 256 threads idle: measured
+// on 1024 x 8 x 60 scenarios of the eight-class, 256-GPU grid: see few_path.
+constexpr int kFewThreads = 128;
+
+template <bool FL, bool RF>
+__global__ void __launch_bounds__(kFewThreads) k_score_few(Set set, Items it, Plan pl, const float* rec, uint64_t* sums,
+                                                           int lgs) {
+  pdl_wait();
+  pdl_trigger();
+  const Dims& d = set.d;
+  const int gsz = 1 << lgs;
+  const long long seg = ((long long)blockIdx.x * kFewThreads + threadIdx.x) >> lgs;
+  const int gl = threadIdx.x & (gsz - 1);
+  const bool live = seg < (long long)it.n * pl.O;
+  uint64_t sum = 0;
+  if (live) {
+    const int item = (int)(seg >> pl.logO), o = (int)seg & (pl.O - 1);
+    const float* h0 = rec + (size_t)item * pl.item_floats;
+    const float* h1 = h0 + d.slot_floats;
+    const int cell = __float_as_int(h0[H_CELL]);
+    if (cell >= 0 && cell < d.cells) {  // (a bad device-side id was flagged by k_prep)
+      const int p = __float_as_int(h0[H_P]);
+      const float* bp = set.bounds + (size_t)p * 4 * d.cells + cell;
+      const float lo_c = bp[0], hi_c = bp[(size_t)d.cells];
+      const float lo_l = h0[H_LO_L], hi_l = h0[H_HI_L], L = h0[H_SLO];
+      const float d_c = __fsub_rn(hi_c, lo_c), d_l = __fsub_rn(hi_l, lo_l);
+      const float lam = h0[H_LAM], rl = h0[H_RLAM], dl = FL ? h0[H_DLT] : 0.0f;
+      const uint32_t key1 = pl.key1 ^ (pl.stream_base + (uint32_t)p);
+      const float* q = set.qn + (size_t)o * pl.W;
+      const uint32_t w = (uint32_t)pl.w;
+      for (int call = gl; call < pl.calls; call += gsz) {
+        const uint4 x = philox4x32_10(make_uint4((uint32_t)call, (uint32_t)o, (uint32_t)cell, pl.round), pl.key0, key1);
+        const uint32_t word[4] = {x.x, x.y, x.z, x.w};
+        float cy[4], t0[4];
+        bool g[4];
+#pragma unroll
+        for (int h = 0; h < 4; ++h) {
+          cy[h] = map_into(lo_c, d_c, hi_c, __ldg(q + __funnelshift_lc(word[h], 0u, w)));
+          g[h] = map_into(lo_l, d_l, hi_l, __ldg(q + ((word[h] & 0xFFFFu) >> pl.sh))) <= L;
+        }
+#pragma unroll
+        for (int sg = 0; sg < 2; ++sg) {
+          const float* h = sg ? h1 : h0;
+          const int Lp = __float_as_int(h[H_LPAD]);
+          const float* kap = h + kTableHeader;
+          const bool fast = __float_as_int(h[H_FAST]) != 0;
+          const RowCap rc = row_cap_of(h);
+          float C[4];
+          int pos[4] = {0, 0, 0, 0};
+#pragma unroll
+          for (int k = 0; k < 4; ++k) C[k] = RF ? row_cap(rc, cy[k], g[k]) : fmaxf(rc.pc, g[k] ? cy[k] : 0.0f);
+          for (int step = __float_as_int(h[H_STEP0]); step > 0; step >>= 1) {
+#pragma unroll
+            for (int k = 0; k < 4; ++k) pos[k] += kap[pos[k] + step - 1] <= C[k] ? step : 0;
+          }
+#pragma unroll
+          for (int k = 0; k < 4; ++k) {
+            const float thb = kap[Lp + pos[k]], m = kap[2 * Lp + pos[k]];
+            float t = thb;
+            if (m >= 1.0f) {
+              const float tr = fast ? fulfil_fast(m, C[k], lam, rl) : fulfil(m, C[k], lam);
+              if (tr > thb && (!FL || tr >= dl)) t = tr;
+            }
+            if (sg == 0) t0[k] = t;
+            else if (4 * call + k < pl.S) sum += fixed40(__fsub_rn(t, t0[k]));
+          }
+        }
+      }
+    }
+  }
+  for (int off = gsz >> 1; off; off >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, off);
+  if (live && gl == 0) sums[seg] = sum;
+}
+
 // (both reductions let the next call's first kernel be placed while they run:
 // it waits for their completion before it reads or writes anything)
 __global__ void k_finalize(Set set, Items it, Plan pl, const uint64_t* sums, double* gap, double* score,
@@ -1256,19 +1338,44 @@ cudaError_t launch_prep(const Set& set, const Items& it, const Plan& pl, float* 
   return launch_pdl(kern, dim3(it.n * 2), dim3(tb), smem, s, set, it, pl, tables, sums, early ? 1 : 0, sure ? 1 : 0);
 }
 
+static bool table_path(const Plan& pl) {
+  const long long chunk_min = std::min<long long>(pl.S, 2LL * 4 * kScoreThreads);
+  return pl.W <= 4096 && 3LL * (pl.W + 1) <= 2 * chunk_min;
+}
+
+// Off the table path: one call a lane, or up to four where segments are many.
+// Measured against the plain path (us a call, few / plain; classes, GPUs,
+// candidates x outcomes): 32 calls 18.6 / 18.5 (2, 16, 64 x 1), 26.8 / 30.5 (8,
+// 256, 1024 x 1), 28.7 / 36.8 (8, 256, 1024 x 4); 64 calls 20.5 / 18.4, 22.5 /
+// 20.5 (4, 64, 256 x 1), 28.7 / 30.8, 30.8 / 36.8; 128 calls 22.7 / 18.5, 24.8 /
+// 20.5, 30.9 / 31.2, 35.0 / 37.6; 256 calls 45.1 / 41.5 at the largest. The
+// 1024 x 8 x 60 scenarios of the eight-class, 256-GPU grid 49.9 -> 30.0 us.
+bool few_path(const Plan& pl, int n_items) {
+  return !table_path(pl) && (pl.calls <= 32 || (pl.calls <= 128 && (long long)n_items * pl.O >= 2048));
+}
+
 static int score_lcap(const Dims& d) { return d.lcap < kSmemTableCap ? d.lcap : kSmemTableCap; }
 
 cudaError_t launch_score(const Set& set, const Items& it, const Plan& pl, const float* tables, uint64_t* sums,
                          void* dump, int dump_stride, int sm_count, LaunchCache& lc, cudaStream_t s) {
   if (it.n <= 0) return cudaSuccess;
+  if (pl.few) {
+    int lgs = 2;
+    while ((1 << lgs) < pl.calls && lgs < 5) ++lgs;
+    const bool rf = set.prior == 1;
+    auto kern = lc.floors ? (rf ? k_score_few<true, true> : k_score_few<true, false>)
+                          : (rf ? k_score_few<false, true> : k_score_few<false, false>);
+    const long long threads = ((long long)it.n * pl.O) << lgs;  // (n O <= 2^30)
+    return launch_pdl(kern, dim3((unsigned)((threads + kFewThreads - 1) / kFewThreads)), dim3(kFewThreads), 0, s, set, it,
+                      pl, tables, sums, lgs);
+  }
   ScoreGrid sg{};
   sg.lcap_s = score_lcap(set.d);
   sg.tcopy = kTableHeader + 3 * sg.lcap_s;
   // the table path when a segment's W + 1 entries cost well under a chunk's
   // samples (an entry costs about one scenario of the plain path, a scenario
   // about a third of one there); the smallest chunk holds 2 calls per thread
-  const long long chunk_min = std::min<long long>(pl.S, 2LL * 4 * kScoreThreads);
-  const bool table = !dump && pl.W <= 4096 && 3LL * (pl.W + 1) <= 2 * chunk_min;
+  const bool table = !dump && table_path(pl);
   const bool rf = set.prior == 1;
   const size_t stages = 16 + 2 * (size_t)(pl.Wp + 2 * sg.tcopy) * 4;
   const size_t gt_len = rf ? 2 * (size_t)pl.W : (size_t)pl.W + 1;

@@ -192,6 +192,7 @@ extern "C" int fs_score_candidates_noalloc(int32_t K, int32_t B, int32_t G, cons
   pl.Wp = Wp;
   pl.item_floats = (long long)item_floats;
   plan_round_keys(pl);
+  pl.few = few_path(pl, n) ? 1 : 0;
 
   // --- the scoring pipeline on the caller's stream, then wait and report
   cudaStream_t s = static_cast<cudaStream_t>(cuda_stream);
