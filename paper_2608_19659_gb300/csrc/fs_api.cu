@@ -843,10 +843,10 @@ int fs_score_goodput(fs_model* m, const fs_samples* smp, double* gap_out, double
   if (m->th_bound < 0) m->th_bound = threshold_bound(m);
   // the rows wanted and the base goodputs, then the pool of rows
   const size_t rows = goodput_pool_rows(m->d, m->th_bound, kGoodputPoolMax);
-  const size_t head = 4 * (size_t)kGoodputSpanInts + 256;
+  const size_t head = align_up(8 * (size_t)kGoodputSpanInts + 16 * (nn + 1), 256);
   if ((rc = m->gp.ensure(head + rows * goodput_row_bytes(m->d), "goodput tables"))) return rc;
   int* span = static_cast<int*>(m->gp.p);
-  long long* base = reinterpret_cast<long long*>(span + kGoodputSpanInts);
+  long long* base = reinterpret_cast<long long*>(span + 2 * kGoodputSpanInts);
   uint64_t* sums = static_cast<uint64_t*>(m->sums.p);
   Set set = m->set;
   set.gp_span = span;

@@ -439,7 +439,10 @@ struct RowOpt {
 // them.
 struct GoodputTables {
   int* span;            // [2 (least, most)][2][K] rows wanted per (realisation, class); least > most: none
+  int* first;           // [2][K] first row of each in the pool (k_other)
   long long* base;      // [2] the base realisations' goodput, 2^-20 req/s
+  long long* closed;    // [items][2] goodput at Cexcl: every scenario whose tail gate is closed
+                        // (nullptr: few segments, each evaluates it itself)
   long long* rows;      // pool of rows of `stride` words
   int stride;           // G + 1 values by GPUs, then kT: the best without each row of the class
   int pool;             // rows the pool holds
@@ -464,19 +467,21 @@ __device__ __forceinline__ int warp_scan(int v, int lane) {
   return v;
 }
 
-// Tasks of k_other: one warp per (realisation, class, row), and two more for
+// Tasks of k_other: one block per (realisation, class, row), and two more for
 // the base realisations' goodput (t* itself, every class).
 //
-// A programme over the other classes within g GPUs, lanes over g, over the GPUs
-// that their cheapest options leave (h = g - need; below need nothing reaches):
-// options cost e = cost - cheapest of them. Then the best of class i's own rows
-// at their base capacities on top, for candidates on another of its rows.
-// What bounds it: issue slots of the inner step (two shared loads, an add and a
-// maximum), about 5 k warp instructions a row at eight classes and 256 GPUs.
-constexpr int kOtherWarps = 4;
+// A programme over the other classes within g GPUs, over the GPUs that their
+// cheapest options leave (h = g - need; below need nothing reaches): options
+// cost e = cost - cheapest of them. Threads over (h, TP degree): four lanes take
+// a class's four rows for one h and merge by two shuffles. Then the best of class
+// i's own rows at their base capacities on top, for candidates on another of its
+// rows. What bounds it: the chain of K - 1 dependent steps of a task (some 800
+// tasks on the eight-class, 256-GPU grid). A warp per task, lanes over h, took 35
+// us there; measured now: see launch_score_goodput.
+constexpr int kOtherThreads = 128;
 
 struct OtherSmem {
-  size_t rows, lohi, mins, opt, dp, per_warp, total;
+  size_t lohi, mins, opt, dp, total;
   int n_opt;
 };
 
@@ -484,41 +489,38 @@ __host__ __device__ inline OtherSmem other_smem(int K, int G) {
   OtherSmem m{};
   auto up = [](size_t x) { return (x + 15) & ~(size_t)15; };
   m.n_opt = G + (G >> 1) + (G >> 2) + (G >> 3);
-  m.rows = 0;                                    // per block: base capacities [2][4K], feasible [2][4K]
-  const size_t shared = up(16 * (size_t)(4 * K));
-  m.lohi = 0;                                    // per warp: option ranges [4K] x 2
-  m.mins = up(8 * (size_t)(4 * K));              // [K]
+  m.lohi = up(16 * (size_t)(4 * K));             // base capacities [2][4K], feasible [2][4K]; option ranges [4K] x 2
+  m.mins = up(m.lohi + 8 * (size_t)(4 * K));     // [K]
   m.opt = up(m.mins + 4 * (size_t)K);            // one class's option values
   m.dp = up(m.opt + 8 * (size_t)m.n_opt);        // two arrays of G + 1
-  m.per_warp = up(m.dp + 16 * ((size_t)G + 1));
-  m.total = shared + kOtherWarps * m.per_warp;
-  m.rows = shared;
+  m.total = up(m.dp + 16 * ((size_t)G + 1));
   return m;
 }
 
 template <bool FL>
-__global__ void __launch_bounds__(32 * kOtherWarps) k_other(Set set, GoodputTables gt, OtherSmem lay) {
+__global__ void __launch_bounds__(kOtherThreads) k_other(Set set, GoodputTables gt, OtherSmem lay) {
   extern __shared__ __align__(16) unsigned char smraw[];
   const Dims& d = set.d;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   __shared__ float sLam[FS_MAX_CLASSES], sRl[FS_MAX_CLASSES], sDl[FS_MAX_CLASSES];
   __shared__ int sBeg[2 * FS_MAX_CLASSES + 1];
+  __shared__ long long sRow[kT];
+  __shared__ int s_need;
   float* sC = reinterpret_cast<float*>(smraw);   // [2][K4]
   int* sOk = reinterpret_cast<int*>(sC + 2 * d.K4);
-  unsigned char* mem = smraw + lay.rows + (size_t)warp * lay.per_warp;
-  int* sLo = reinterpret_cast<int*>(mem + lay.lohi);
+  int* sLo = reinterpret_cast<int*>(smraw + lay.lohi);
   int* sHi = sLo + d.K4;
-  int* sMin = reinterpret_cast<int*>(mem + lay.mins);
-  long long* sOpt = reinterpret_cast<long long*>(mem + lay.opt);
-  long long* cur = reinterpret_cast<long long*>(mem + lay.dp);
+  int* sMin = reinterpret_cast<int*>(smraw + lay.mins);
+  long long* sOpt = reinterpret_cast<long long*>(smraw + lay.opt);
+  long long* cur = reinterpret_cast<long long*>(smraw + lay.dp);
   long long* nxt = cur + (d.G + 1);
   pdl_wait();
   pdl_trigger();
-  for (int x = threadIdx.x; x < 2 * d.K4; x += blockDim.x) {
+  for (int x = tid; x < 2 * d.K4; x += kOtherThreads) {
     sC[x] = set.rowC[x];
     sOk[x] = set.rowB[x] >= 0;
   }
-  for (int i = threadIdx.x; i < d.K; i += blockDim.x) {
+  for (int i = tid; i < d.K; i += kOtherThreads) {
     const float lam = set.lam[i];
     sLam[i] = lam;
     sRl[i] = __frcp_rn(lam);
@@ -528,8 +530,12 @@ __global__ void __launch_bounds__(32 * kOtherWarps) k_other(Set set, GoodputTabl
     int carry = 0;
     for (int b = 0; b < 2 * d.K; b += 32) {
       const int sc = b + lane;
-      const int incl = warp_scan(sc < 2 * d.K ? span_rows(gt, d.K, sc) : 0, lane);
-      if (sc < 2 * d.K) sBeg[sc + 1] = carry + incl;
+      const int v = sc < 2 * d.K ? span_rows(gt, d.K, sc) : 0;
+      const int incl = warp_scan(v, lane);
+      if (sc < 2 * d.K) {
+        sBeg[sc + 1] = carry + incl;
+        if (blockIdx.x == 0) gt.first[sc] = carry + incl - v;
+      }
       carry += __shfl_sync(0xffffffffu, incl, 31);
     }
     if (lane == 0) sBeg[0] = 0;
@@ -537,11 +543,11 @@ __global__ void __launch_bounds__(32 * kOtherWarps) k_other(Set set, GoodputTabl
   __syncthreads();
   const int rows = sBeg[2 * d.K];
   if (rows > gt.pool) {  // cannot happen: the host sized the pool for the most rows there can be
-    if (blockIdx.x == 0 && threadIdx.x == 0) atomicOr(set.status, ST_TABLE);
+    if (blockIdx.x == 0 && tid == 0) atomicOr(set.status, ST_TABLE);
     return;
   }
   const int n_base = gt.c0 == 0 ? 2 : 0;  // (the first pass)
-  for (int task = (int)blockIdx.x * kOtherWarps + warp; task < rows + n_base; task += (int)gridDim.x * kOtherWarps) {
+  for (int task = (int)blockIdx.x; task < rows + n_base; task += (int)gridDim.x) {
     const bool base = task >= rows;
     int sigma, cls, kk = 0;
     float t;
@@ -566,8 +572,8 @@ __global__ void __launch_bounds__(32 * kOtherWarps) k_other(Set set, GoodputTabl
     }
     // option ranges of every row at t, and each class's cheapest option
     const float* C = sC + sigma * d.K4;
-    __syncwarp();
-    for (int rho = lane; rho < d.K4; rho += 32) {
+    auto empty_ok = [&](int i) { return !(t > 0.0f) && !(FL && sDl[i] > 0.0f); };
+    for (int rho = tid; rho < d.K4; rho += kOtherThreads) {
       const int i = rho >> 2;
       int lo, hi;
       row_range(C[rho], sOk[sigma * d.K4 + rho] != 0, rep_cap(d, rho & 3), class_threshold(t, FL ? sDl[i] : 0.0f),
@@ -575,75 +581,86 @@ __global__ void __launch_bounds__(32 * kOtherWarps) k_other(Set set, GoodputTabl
       sLo[rho] = lo;
       sHi[rho] = hi;
     }
-    __syncwarp();
-    int need = 0;
-    for (int b = 0; b < d.K; b += 32) {
-      const int i = b + lane;
-      int m = 0;
-      if (i < d.K) {
-        const bool empty = !(t > 0.0f) && !(FL && sDl[i] > 0.0f);
-        if (!empty) {
-          m = 1 << 24;  // (above every budget: 64 of them stay below 2^31)
-          for (int j = 0; j < kT; ++j)
-            if (sLo[4 * i + j]) m = min(m, sLo[4 * i + j] << j);
-        }
-        sMin[i] = m;
-      }
-      need += __reduce_add_sync(0xffffffffu, i < d.K && i != cls ? m : 0);
-    }
-    __syncwarp();
-    const int H = need <= d.G ? d.G - need + 1 : 0;  // GPUs above the cheapest options: 0..H-1
-    for (int h = lane; h < H; h += 32) cur[h] = 0;
-    __syncwarp();
-    if (H > 0)
-      for (int i = 0; i < d.K; ++i) {
-        if (i == cls) continue;
-        const int m = sMin[i];
-        const bool empty = !(t > 0.0f) && !(FL && sDl[i] > 0.0f);
-        int cnt[kT], beg[kT], all = 0;
-#pragma unroll
-        for (int j = 0; j < kT; ++j) {
-          const int lo = sLo[4 * i + j];
-          cnt[j] = lo ? max(0, min(sHi[4 * i + j], (H - 1 + m) >> j) - lo + 1) : 0;
-          beg[j] = all;
-          all += cnt[j];
-        }
-        for (int x = lane; x < all; x += 32) {
-          int j = 0;
-#pragma unroll
-          for (int q = 1; q < kT; ++q)
-            if (x >= beg[q]) j = q;
-          sOpt[x] = goodput_fx20((float)(sLo[4 * i + j] + x - beg[j]), C[4 * i + j], sLam[i]);
-        }
-        __syncwarp();
-        for (int h = lane; h < H; h += 32) {
-          long long best = empty ? cur[h] : -1;
-#pragma unroll
-          for (int j = 0; j < kT; ++j) {
-            int e = (sLo[4 * i + j] << j) - m;
-            for (int x = 0; x < cnt[j] && e <= h; ++x, e += 1 << j) {
-              const long long v = sOpt[beg[j] + x] + cur[h - e];
-              best = v > best ? v : best;
-            }
+    __syncthreads();
+    if (warp == 0) {
+      int need = 0;
+      for (int b = 0; b < d.K; b += 32) {
+        const int i = b + lane;
+        int m = 0;
+        if (i < d.K) {
+          if (!empty_ok(i)) {
+            m = 1 << 24;  // (above every budget: 64 of them stay below 2^31)
+            for (int j = 0; j < kT; ++j)
+              if (sLo[4 * i + j]) m = min(m, sLo[4 * i + j] << j);
           }
-          nxt[h] = best;
+          sMin[i] = m;
         }
-        __syncwarp();
-        long long* x = cur;
-        cur = nxt;
-        nxt = x;
+        need += __reduce_add_sync(0xffffffffu, i < d.K && i != cls ? m : 0);
       }
-    // other[g] = cur[g - need], -1 below; the class's own rows on top
-    long long row_best[kT];
-    const bool empty = !(t > 0.0f) && !(FL && sDl[cls] > 0.0f);
+      if (lane == 0) s_need = need;
+    }
+    __syncthreads();
+    const int need = s_need;
+    const int H = need <= d.G ? d.G - need + 1 : 0;  // GPUs above the cheapest options: 0..H-1
+    for (int h = tid; h < H; h += kOtherThreads) cur[h] = 0;
+    const int j = tid & 3;  // this thread's TP degree
+    for (int i = 0; H > 0 && i < d.K; ++i) {
+      if (i == cls) continue;
+      const int m = sMin[i];
+      int cnt[kT], beg[kT], all = 0;
 #pragma unroll
-    for (int j = 0; j < kT; ++j) {
+      for (int q = 0; q < kT; ++q) {
+        const int lo = sLo[4 * i + q];
+        cnt[q] = lo ? max(0, min(sHi[4 * i + q], (H - 1 + m) >> q) - lo + 1) : 0;
+        beg[q] = all;
+        all += cnt[q];
+      }
+      for (int x = tid; x < all; x += kOtherThreads) {
+        int q = 0;
+#pragma unroll
+        for (int y = 1; y < kT; ++y)
+          if (x >= beg[y]) q = y;
+        const int lo = sLo[4 * i + q], at = q == 0 ? 0 : q == 1 ? beg[1] : q == 2 ? beg[2] : beg[3];
+        sOpt[x] = goodput_fx20((float)(lo + x - at), C[4 * i + q], sLam[i]);
+      }
+      __syncthreads();
+      const int my_cnt = j == 0 ? cnt[0] : j == 1 ? cnt[1] : j == 2 ? cnt[2] : cnt[3];
+      const long long* opt = sOpt + (j == 0 ? 0 : j == 1 ? beg[1] : j == 2 ? beg[2] : beg[3]);
+      const int e0 = (sLo[4 * i + j] << j) - m;
+      const bool empty = empty_ok(i);
+      for (int h0 = 0; h0 < H; h0 += kOtherThreads / 4) {
+        const int h = h0 + (tid >> 2);
+        long long best = -1;
+        if (h < H) {
+          if (empty && j == 0) best = cur[h];
+          int e = e0;
+          for (int x = 0; x < my_cnt && e <= h; ++x, e += 1 << j) {
+            const long long v = opt[x] + cur[h - e];
+            best = v > best ? v : best;
+          }
+        }
+#pragma unroll
+        for (int o = 1; o <= 2; o <<= 1) {
+          const long long v = __shfl_xor_sync(0xffffffffu, best, o);
+          best = v > best ? v : best;
+        }
+        if (j == 0 && h < H) nxt[h] = best;
+      }
+      __syncthreads();
+      long long* x = cur;
+      cur = nxt;
+      nxt = x;
+    }
+    // (a lone class's programme is all zeros)
+    if (H > 0) __syncthreads();
+    // the class's own rows on top, a warp each: replicas over the lanes
+    {
       long long best = -1;
-      const int lo = sLo[4 * cls + j];
+      const int lo = sLo[4 * cls + warp];
       if (lo && H > 0) {
-        const int top = min(sHi[4 * cls + j], (H - 1) >> j);
+        const int top = min(sHi[4 * cls + warp], (H - 1) >> warp);
         for (int n = lo + lane; n <= top; n += 32) {
-          const long long v = goodput_fx20((float)n, C[4 * cls + j], sLam[cls]) + cur[H - 1 - (n << j)];
+          const long long v = goodput_fx20((float)n, C[4 * cls + warp], sLam[cls]) + cur[H - 1 - (n << warp)];
           best = v > best ? v : best;
         }
       }
@@ -651,25 +668,28 @@ __global__ void __launch_bounds__(32 * kOtherWarps) k_other(Set set, GoodputTabl
         const long long v = __shfl_xor_sync(0xffffffffu, best, o);
         best = v > best ? v : best;
       }
-      row_best[j] = best;
+      if (lane == 0) sRow[warp] = best;
     }
-    const long long none = empty && H > 0 ? cur[H - 1] : -1;  // no replicas for the class
+    __syncthreads();
+    const long long none = empty_ok(cls) && H > 0 ? cur[H - 1] : -1;  // no replicas for the class
     if (base) {
       long long best = none;
 #pragma unroll
-      for (int j = 0; j < kT; ++j) best = row_best[j] > best ? row_best[j] : best;
-      if (lane == 0) gt.base[sigma] = best < 0 ? 0 : best;
+      for (int q = 0; q < kT; ++q) best = sRow[q] > best ? sRow[q] : best;
+      if (tid == 0) gt.base[sigma] = best < 0 ? 0 : best;
     } else {
+      // other[g] = cur[g - need], -1 below
       long long* row = gt.rows + (size_t)task * gt.stride;
-      for (int g = lane; g <= d.G; g += 32) row[g] = g >= need ? cur[g - need] : -1;
-      if (lane < kT) {
+      for (int g = tid; g <= d.G; g += kOtherThreads) row[g] = g >= need ? cur[g - need] : -1;
+      if (tid < kT) {
         long long best = none;
 #pragma unroll
-        for (int j = 0; j < kT; ++j)
-          if (j != lane && row_best[j] > best) best = row_best[j];
-        row[d.G + 1 + lane] = best;
+        for (int q = 0; q < kT; ++q)
+          if (q != tid && sRow[q] > best) best = sRow[q];
+        row[d.G + 1 + tid] = best;
       }
     }
+    __syncthreads();  // the next task's ranges and programme
   }
 }
 
@@ -729,19 +749,36 @@ __device__ __forceinline__ GoodputCtx goodput_ctx(const Set& set, const GoodputT
   c.rl = h[H_RLAM];
   c.dl = FL ? h[H_DLT] : 0.0f;
   const int sc = sigma * d.K + i;
-  int first = 0;  // the class's first row in the pool
-  for (int q = 0; q < sc; ++q) first += span_rows(gt, d.K, q);
-  c.rows = gt.rows + ((long long)first - gt.span[sc]) * gt.stride;
+  c.rows = gt.rows + ((long long)gt.first[sc] - gt.span[sc]) * gt.stride;
   return c;
+}
+
+// Each candidate's goodput at Cexcl in both realisations, a thread each (without
+// the prior): what every entry at or below Cexcl and every closed gate takes.
+template <bool FL>
+__global__ void __launch_bounds__(128) k_goodput_closed(Set set, Items it, Plan pl, const float* rec, GoodputTables gt) {
+  pdl_wait();
+  pdl_trigger();
+  const Dims& d = set.d;
+  const long long x = (long long)blockIdx.x * 128 + threadIdx.x;
+  if (x >= 2LL * it.n) return;
+  const int item = (int)(x >> 1), sigma = (int)x & 1;
+  const float* h = rec + (size_t)item * pl.item_floats + (size_t)sigma * d.slot_floats;
+  const int cell = __float_as_int(h[H_CELL]);
+  if (cell < 0 || cell >= d.cells) return;  // flagged by the preparation
+  const int rr = cell / d.B, ir = rr >> 2;
+  if (ir < gt.c0 || ir >= gt.c1) return;    // another pass's class
+  const GoodputCtx c = goodput_ctx<FL>(set, gt, h, sigma, rr);
+  gt.closed[x] = goodput_at<FL>(c, h[H_CX]);
 }
 
 // One block per segment (candidate e, outcome o): entries [0, W) hold the gap
 // with an open gate at position k, W with a closed one (under the prior [W, 2W),
 // position k - W). A thread per entry; without the prior every entry at or
-// below a realisation's Cexcl takes that realisation's closed-gate goodput,
-// evaluated once. Then the same draws and sums as the table path.
+// below a realisation's Cexcl takes that realisation's closed-gate goodput. Then
+// the same draws and sums as the table path.
 template <bool FL, bool RF>
-__global__ void __launch_bounds__(256) k_score_goodput(Set set, Items it, Plan pl, const float* rec, uint64_t* sums,
+__global__ void __launch_bounds__(256, 4) k_score_goodput(Set set, Items it, Plan pl, const float* rec, uint64_t* sums,
                                                        GoodputTables gt) {
   extern __shared__ __align__(16) unsigned char smraw[];
   uint64_t* gtab = reinterpret_cast<uint64_t*>(smraw);
@@ -765,15 +802,16 @@ __global__ void __launch_bounds__(256) k_score_goodput(Set set, Items it, Plan p
     const uint32_t kgs = (uint32_t)__float_as_int(win[0]) << pl.sh;
     const uint32_t kgs16 = (uint32_t)min((unsigned long long)kgs << 16, 0xFFFFFFFFull);
     const bool any_open = kgs != 0u, any_closed = kgs16 != 0xFFFFFFFFu;
-    if ((tid & 31) == 0 && tid < 64 ) {
+    if (lane == 0 && tid < 64) {
       const int sg = tid >> 5;
       const float* h = sg ? h1 : h0;
       s_ctx[sg] = goodput_ctx<FL>(set, gt, h, sg, rr);
-      if (!RF) s_closed[sg] = goodput_at<FL>(s_ctx[sg], h[H_CX]);
+      if (!RF) s_closed[sg] = gt.closed ? gt.closed[2 * (long long)item + sg] : goodput_at<FL>(s_ctx[sg], h[H_CX]);
     }
     __syncthreads();
+    const long long c0 = s_closed[0], c1 = s_closed[1];
     const RowCap a0 = row_cap_of(h0), a1 = row_cap_of(h1);
-    const int k0 = any_open ? 0 : W, k1 = RF ? (any_closed ? 2 * W : W) : any_open ? W + 1 : W + 1;
+    const int k0 = any_open ? 0 : W, k1 = RF ? (any_closed ? 2 * W : W) : W + 1;
     for (int k = k0 + tid; k < k1; k += blockDim.x) {
       const bool g = k < W;
       long long g0, g1;
@@ -783,8 +821,8 @@ __global__ void __launch_bounds__(256) k_score_goodput(Set set, Items it, Plan p
         g1 = goodput_at<FL>(s_ctx[1], row_cap(a1, cy, g));
       } else {
         const float cy = g ? win[4 + k] : 0.0f;
-        g0 = g && cy > a0.pc ? goodput_at<FL>(s_ctx[0], cy) : s_closed[0];
-        g1 = g && cy > a1.pc ? goodput_at<FL>(s_ctx[1], cy) : s_closed[1];
+        g0 = g && cy > a0.pc ? goodput_at<FL>(s_ctx[0], cy) : c0;
+        g1 = g && cy > a1.pc ? goodput_at<FL>(s_ctx[1], cy) : c1;
       }
       gtab[k] = (unsigned long long)(g1 > g0 ? g1 - g0 : g0 - g1);
     }
@@ -925,6 +963,7 @@ cudaError_t launch_score_goodput(const Set& set, const Items& it, const Plan& pl
   const bool rf = set.prior == 1;
   GoodputTables gt{};
   gt.span = span;
+  gt.first = span + kGoodputSpanInts;
   gt.base = base;
   gt.rows = static_cast<long long*>(pool);
   gt.stride = d.G + 1 + kT;
@@ -934,6 +973,7 @@ cudaError_t launch_score_goodput(const Set& set, const Items& it, const Plan& pl
   if (classes < 1) return cudaErrorInvalidValue;
   const OtherSmem lay = other_smem(d.K, d.G);
   auto other = floors ? k_other<true> : k_other<false>;
+  auto closed = floors ? k_goodput_closed<true> : k_goodput_closed<false>;
   const size_t smem = 8 * (size_t)(rf ? 2 * pl.W : pl.W + 1);
   auto kern = floors ? (rf ? k_score_goodput<true, true> : k_score_goodput<true, false>)
                      : (rf ? k_score_goodput<false, true> : k_score_goodput<false, false>);
@@ -943,14 +983,23 @@ cudaError_t launch_score_goodput(const Set& set, const Items& it, const Plan& pl
   // one block per segment: segments differ in cost, and the block scheduler
   // evens them out
   const long long n_seg = (long long)it.n * pl.O;
+  // beyond a few waves of blocks the closed-gate goodputs are evaluated once per
+  // candidate rather than by each of its segments (294 us in all on the largest
+  // call with them and the block-wide k_other, 352 us before both; 1.2 us more of
+  // a launch on the paper-scale one, whose 512 segments are one wave)
+  gt.closed = !rf && n_seg > 8LL * sm_count ? base + 2 : nullptr;
   const unsigned grid = (unsigned)(n_seg < 0x7fffffffLL ? n_seg : 0x7fffffffLL);
+  // Measured (eight classes, 256 GPUs, about 800 rows; one GB300): k_other 35 us a
+  // warp per row, 21 us a block per row.
   for (gt.c0 = 0; gt.c0 < d.K; gt.c0 = gt.c1) {
     gt.c1 = gt.c0 + classes < d.K ? gt.c0 + classes : d.K;
-    // a warp per row wanted, as many blocks as run at once (the count is not
-    // known here; the rows are dealt to the warps)
-    const long long most = ((long long)(gt.c1 - gt.c0) * per + 2 + kOtherWarps - 1) / kOtherWarps;
+    // a block per row wanted, as many as run at once (the count is not known
+    // here; the rows are dealt to the blocks)
+    const long long most = (long long)(gt.c1 - gt.c0) * per + 2;
     const long long fit = 8LL * sm_count;
-    e = launch_pdl(other, dim3((unsigned)(most < fit ? most : fit)), dim3(32 * kOtherWarps), lay.total, s, set, gt, lay);
+    e = launch_pdl(other, dim3((unsigned)(most < fit ? most : fit)), dim3(kOtherThreads), lay.total, s, set, gt, lay);
+    if (e == cudaSuccess && gt.closed)
+      e = launch_pdl(closed, dim3((unsigned)((2LL * it.n + 127) / 128)), dim3(128), 0, s, set, it, pl, tables, gt);
     if (e != cudaSuccess) return e;
     if (it.n > 0) e = launch_pdl(kern, dim3(grid), dim3(256), smem, s, set, it, pl, tables, sums, gt);
     if (e != cudaSuccess) return e;
