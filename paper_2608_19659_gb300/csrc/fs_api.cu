@@ -186,6 +186,10 @@ size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 
 constexpr size_t kMaxTimedEvents = 5 * 4096;
 
+// Sums that a synchronous call's reduction writes into the mapped block itself
+// (more of them are copied after it: page-locked memory is kept by the model).
+constexpr size_t kMappedSums = 4u << 20;
+
 int check_cells(const float* a, int n, const char* name) {
   if (!a) return fail(FS_EINVAL, "%s is NULL", name);
   for (int i = 0; i < n; ++i)
@@ -368,7 +372,7 @@ int ensure_items(fs_model* m, int n, int O) {
 
 // The scoring sequence on stream s; cand_dev holds n_cand cell ids.
 int run_score(fs_model* m, Set set, const fs_samples* smp, const int32_t* cand_dev, double* gap,
-              double* score, float* gamma_t, int32_t* best, void* dump, cudaStream_t s,
+              double* score, float* gamma_t, int32_t* best, void* dump, uint64_t* sum_out, cudaStream_t s,
               uint32_t* status_copy = nullptr) {
   const int n = smp->n_cand;
   Items it{};
@@ -403,7 +407,7 @@ int run_score(fs_model* m, Set set, const fs_samples* smp, const int32_t* cand_d
           "launch score");
   if (timed) FS_CUDA(cudaEventRecord(ev[3], s), "record timing event");
   FS_CUDA(launch_finalize(set, it, pl, (const uint64_t*)m->sums.p, gap, score, gamma_t, best, status_copy,
-                          (uint64_t*)m->sums.p + (size_t)std::max(n, 1) * smp->O, s),
+                          (uint64_t*)m->sums.p + (size_t)std::max(n, 1) * smp->O, sum_out, s),
           "launch finalize");
   if (phases) FS_CUDA(cudaEventRecord(ev[4], s), "record timing event");
   return FS_OK;
@@ -644,7 +648,9 @@ int fs_score_candidates(fs_model* m, const fs_samples* smp, double* gap_out, dou
   // copy engine sits before the first kernel or after the last one.
   const size_t nn = (size_t)std::max(n, 1);
   const size_t out_bytes = align_up(16 * nn + 36, 16);
-  if ((rc = m->h_out.ensure(out_bytes + 4 * nn, "host staging"))) return rc;
+  const size_t sum_at = align_up(out_bytes + 4 * nn, 16), sum_bytes = sum_eo ? 8 * (size_t)n * smp->O : 0;
+  const bool sums_mapped = sum_bytes && sum_bytes <= kMappedSums;
+  if ((rc = m->h_out.ensure(sum_at + (sums_mapped ? sum_bytes : 0), "host staging"))) return rc;
   char* h = static_cast<char*>(m->h_out.p);
   char* hd = static_cast<char*>(m->h_out.dev);
   if (n > 0) std::memcpy(h + out_bytes, smp->cand, 4 * (size_t)n);
@@ -659,14 +665,15 @@ int fs_score_candidates(fs_model* m, const fs_samples* smp, double* gap_out, dou
   Set set = m->set;
   if (m->staged) set.bounds = static_cast<float*>(m->h_up.dev);
   rc = run_score(m, set, smp, reinterpret_cast<const int32_t*>(hd + out_bytes), d_gap, d_score, d_gt, d_best,
-                 dump_dev, s, d_st);
+                 dump_dev, sums_mapped ? reinterpret_cast<uint64_t*>(hd + sum_at) : nullptr, s, d_st);
   if (rc) return rc;
-  if (sum_eo && n)
-    FS_CUDA(cudaMemcpyAsync(sum_eo, m->sums.p, 8 * (size_t)n * smp->O, cudaMemcpyDeviceToHost, s), "read sums");
+  if (sum_bytes && !sums_mapped)
+    FS_CUDA(cudaMemcpyAsync(sum_eo, m->sums.p, sum_bytes, cudaMemcpyDeviceToHost, s), "read sums");
   FS_CUDA(cudaStreamSynchronize(s), "synchronize");
   uint32_t st;
   std::memcpy(&st, h + 16 * nn + 32, 4);
   if (st) return status_error(m, st);
+  if (sums_mapped) std::memcpy(sum_eo, h + sum_at, sum_bytes);
   if (gap_out && n) std::memcpy(gap_out, h, 8 * (size_t)n);
   if (score_out && n) std::memcpy(score_out, h + 8 * nn, 8 * (size_t)n);
   if (gamma_t) std::memcpy(gamma_t, h + 16 * nn, 4);
@@ -685,12 +692,8 @@ int fs_score_candidates_async(fs_model* m, const fs_samples* smp, double* gap_de
   if ((rc = ensure_items(m, n, smp->O))) return rc;
   cudaStream_t s = (cudaStream_t)cuda_stream;
   if ((rc = flush_bounds(m, s))) return rc;
-  rc = run_score(m, m->set, smp, smp->cand, gap_dev, score_dev, gamma_t_dev, best_dev, dump_dev, s);
-  if (rc) return rc;
-  if (sum_eo_dev && n)
-    FS_CUDA(cudaMemcpyAsync(sum_eo_dev, m->sums.p, 8 * (size_t)n * smp->O, cudaMemcpyDeviceToDevice, s),
-            "copy sums");
-  return FS_OK;
+  return run_score(m, m->set, smp, smp->cand, gap_dev, score_dev, gamma_t_dev, best_dev, dump_dev,
+                   reinterpret_cast<uint64_t*>(sum_eo_dev), s);
 }
 
 int fs_solve(fs_model* m, const float* cap, const float* tail, fs_allocation* out) {
@@ -825,7 +828,9 @@ int fs_score_goodput(fs_model* m, const fs_samples* smp, double* gap_out, double
   // candidate ids in and gap, score, gamma, best and the status word out
   const size_t nn = (size_t)std::max(n, 1);
   const size_t out_bytes = align_up(16 * nn + 16, 16);
-  if ((rc = m->h_out.ensure(out_bytes + 4 * nn, "host staging"))) return rc;
+  const size_t sum_at = align_up(out_bytes + 4 * nn, 16), sum_bytes = sum_eo ? 8 * (size_t)n * smp->O : 0;
+  const bool sums_mapped = sum_bytes && sum_bytes <= kMappedSums;
+  if ((rc = m->h_out.ensure(sum_at + (sums_mapped ? sum_bytes : 0), "host staging"))) return rc;
   char* h = static_cast<char*>(m->h_out.p);
   char* hd = static_cast<char*>(m->h_out.dev);
   if (n > 0) std::memcpy(h + out_bytes, smp->cand, 4 * (size_t)n);
@@ -857,14 +862,16 @@ int fs_score_goodput(fs_model* m, const fs_samples* smp, double* gap_out, double
                                static_cast<char*>(m->gp.p) + head, rows, m->lc.floors, m->th_bound, m->sm_count, s),
           "launch goodput scorer");
   FS_CUDA(launch_finalize_goodput(set, it, pl, sums, base, lam_sum, d_gap, d_score, d_gamma, d_best, d_st,
-                                  sums + nn * smp->O, s),
+                                  sums + nn * smp->O,
+                                  sums_mapped ? reinterpret_cast<uint64_t*>(hd + sum_at) : nullptr, s),
           "launch goodput reduction");
-  if (sum_eo && n)
-    FS_CUDA(cudaMemcpyAsync(sum_eo, sums, 8 * (size_t)n * smp->O, cudaMemcpyDeviceToHost, s), "read sums");
+  if (sum_bytes && !sums_mapped)
+    FS_CUDA(cudaMemcpyAsync(sum_eo, sums, sum_bytes, cudaMemcpyDeviceToHost, s), "read sums");
   FS_CUDA(cudaStreamSynchronize(s), "synchronize");
   uint32_t st;
   std::memcpy(&st, h + 16 * nn + 12, 4);
   if (st) return status_error(m, st);
+  if (sums_mapped) std::memcpy(sum_eo, h + sum_at, sum_bytes);
   if (gap_out && n) std::memcpy(gap_out, h, 8 * (size_t)n);
   if (score_out && n) std::memcpy(score_out, h + 8 * nn, 8 * (size_t)n);
   if (gamma_gp) std::memcpy(gamma_gp, h + 16 * nn, 8);

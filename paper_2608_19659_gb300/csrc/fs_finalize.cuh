@@ -84,6 +84,15 @@ __device__ __forceinline__ float base_tstar(const Set& set, int p, int sigma) {
   return __uint_as_float(__reduce_max_sync(0xffffffffu, v));
 }
 
+// The caller's copy of the sums of items [beg, end) (nullable), coalesced over the
+// block: the reduction reads them anyway, so no copy follows the call's last kernel.
+__device__ __forceinline__ void copy_sums(const Plan& pl, const uint64_t* sums, uint64_t* out, int beg, int end) {
+  if (!out) return;
+  const size_t b = (size_t)beg * pl.O, e = (size_t)end * pl.O;
+#pragma unroll 4
+  for (size_t x = b + threadIdx.x; x < e; x += blockDim.x) out[x] = __ldg(sums + x);
+}
+
 // Items [beg, end) of problem p, whose first item is pos0 (candidate positions,
 // for the order of equal scores, count from there).
 __device__ inline Best finalize_problem(const Set& set, const Items& it, const Plan& pl, const uint64_t* sums,

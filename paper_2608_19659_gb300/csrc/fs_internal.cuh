@@ -523,11 +523,12 @@ cudaError_t launch_score(const Set& set, const Items& it, const Plan& pl, const 
                          cudaStream_t s);
 // status_copy (nullable): the status word as it stands after the whole call.
 // part: 2 finalize_blocks(it) words of scratch (nullable when that is 0).
+// sum_out (nullable): the caller's copy of the sums.
 constexpr int kFinalizeMaxBlocks = 64;
 int finalize_blocks(const Items& it);
 cudaError_t launch_finalize(const Set& set, const Items& it, const Plan& pl, const uint64_t* sums,
                             double* gap, double* score, float* gamma_t, int32_t* best, uint32_t* status_copy,
-                            uint64_t* part, cudaStream_t s);
+                            uint64_t* part, uint64_t* sum_out, cudaStream_t s);
 cudaError_t launch_watchdog(uint32_t* status, uint64_t limit_ns, cudaStream_t s);
 // Measurement only: median time of `reps` launches of the table path's draws
 // alone (mode 0) or with its per-sample lookup (mode 1), W = 2^w, at least
@@ -558,7 +559,8 @@ cudaError_t launch_score_goodput(const Set& set, const Items& it, const Plan& pl
                                  int floors, int th_bound, int sm_count, cudaStream_t s);
 cudaError_t launch_finalize_goodput(const Set& set, const Items& it, const Plan& pl, const uint64_t* sums,
                                     const long long* base, double lam_sum, double* gap, double* score, double* gamma,
-                                    int32_t* best, uint32_t* status_copy, uint64_t* part, cudaStream_t s);
+                                    int32_t* best, uint32_t* status_copy, uint64_t* part, uint64_t* sum_out,
+                                    cudaStream_t s);
 
 // replay
 struct ReplayState {

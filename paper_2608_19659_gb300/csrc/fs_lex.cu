@@ -844,7 +844,7 @@ __global__ void __launch_bounds__(256, 4) k_score_goodput(Set set, Items it, Pla
 // ticket (work[1], zeroed by the preparation) merges them.
 __global__ void k_finalize_goodput(Set set, Items it, Plan pl, const uint64_t* sums, const long long* base,
                                    double lam_sum, double* gap, double* score, double* gamma, int32_t* best,
-                                   uint32_t* status_copy, uint64_t* part) {
+                                   uint32_t* status_copy, uint64_t* part, uint64_t* sum_out) {
   __shared__ Best sb[32];
   __shared__ int s_last;
   pdl_wait();
@@ -853,6 +853,7 @@ __global__ void k_finalize_goodput(Set set, Items it, Plan pl, const uint64_t* s
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nwarp = blockDim.x >> 5;
   const int nb = (int)gridDim.x, per = (it.n + nb - 1) / nb;
   const int beg = min(it.n, (int)blockIdx.x * per), end = min(it.n, beg + per);
+  copy_sums(pl, sums, sum_out, beg, end);
   const long long gm = base[0], gpl = base[1];
   const long long gfix = gpl > gm ? gpl - gm : gm - gpl;
   const long long n = (long long)pl.O * pl.S;
@@ -1009,10 +1010,11 @@ cudaError_t launch_score_goodput(const Set& set, const Items& it, const Plan& pl
 
 cudaError_t launch_finalize_goodput(const Set& set, const Items& it, const Plan& pl, const uint64_t* sums,
                                     const long long* base, double lam_sum, double* gap, double* score, double* gamma,
-                                    int32_t* best, uint32_t* status_copy, uint64_t* part, cudaStream_t s) {
+                                    int32_t* best, uint32_t* status_copy, uint64_t* part, uint64_t* sum_out,
+                                    cudaStream_t s) {
   const int nb = std::max(1, finalize_blocks(it));
   return launch_pdl(k_finalize_goodput, dim3(nb), dim3(256), 0, s, set, it, pl, sums, base, lam_sum, gap, score, gamma,
-                    best, status_copy, part);
+                    best, status_copy, part, sum_out);
 }
 
 }  // namespace fs

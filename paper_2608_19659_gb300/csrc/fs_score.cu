@@ -181,13 +181,18 @@ __global__ void __launch_bounds__(kPrepThreads) k_prep(Set set, Items it, Plan p
   }
   if (sigma == 0)
     for (int o = tid; o < pl.O; o += blockDim.x) sums[(size_t)item * pl.O + o] = 0ull;
-  if (cell < 0 || cell >= d.cells) {  // device-side candidate ids are checked here
+  // an item that cannot be scored: the status word says why, and the scorers
+  // leave a record without a cell alone
+  auto reject = [&](uint32_t why) {
     if (tid == 0) {
-      atomicOr(set.status, ST_CELL);
+      atomicOr(set.status, why);
       for (int k = 0; k < kTableHeader; ++k) tab[k] = 0.0f;
       tab[H_BX] = __int_as_float(-1);
       tab[H_CELL] = __int_as_float(-1);
     }
+  };
+  if (cell < 0 || cell >= d.cells) {  // device-side candidate ids are checked here
+    reject(ST_CELL);
     return;
   }
   const int rr = cell / d.B, be = cell - rr * d.B, ie = rr >> 2, jr = rr & 3;
@@ -368,7 +373,7 @@ __global__ void __launch_bounds__(kPrepThreads) k_prep(Set set, Items it, Plan p
   const int total = set.ntheta[ps];
   const bool rtab = d.K4 * total <= set.rt_cap;
   if (sure && !rtab) {  // the host's bound on the count was wrong: the call fails
-    if (tid == 0) atomicOr(set.status, ST_TABLE);
+    reject(ST_TABLE);
     return;
   }
   const float* th = th_g;  // the thresholds, and with a table the row's words (stride rts)
@@ -470,7 +475,7 @@ __global__ void __launch_bounds__(kPrepThreads) k_prep(Set set, Items it, Plan p
   while (P < Lt + 1) P <<= 1;
   const int Lpad = max(P, 4);
   if (Lpad > d.lcap) {  // cannot happen: Lt <= total <= theta_cap
-    if (tid == 0) atomicOr(set.status, ST_TABLE);
+    reject(ST_TABLE);
     return;
   }
   float* kap = tab + kTableHeader;
@@ -1268,12 +1273,13 @@ __global__ void __launch_bounds__(kFewThreads) k_score_few(Set set, Items it, Pl
 // (both reductions let the next call's first kernel be placed while they run:
 // it waits for their completion before it reads or writes anything)
 __global__ void k_finalize(Set set, Items it, Plan pl, const uint64_t* sums, double* gap, double* score,
-                           float* gamma_t, int32_t* best, uint32_t* status_copy) {
+                           float* gamma_t, int32_t* best, uint32_t* status_copy, uint64_t* sum_out) {
   pdl_wait();
   pdl_trigger();
   const int p = blockIdx.x;
   const int beg = it.off ? it.off[p] : 0;
   const int end = it.off ? it.off[p + 1] : it.n;
+  copy_sums(pl, sums, sum_out, beg, end);
   const Best b = finalize_problem(set, it, pl, sums, p, beg, end, gap, score, gamma_t ? gamma_t + p : nullptr, beg);
   if (threadIdx.x == 0 && best) best[p] = b.valid() ? b.cell : -1;
   // every kernel of the call has finished (stream order, and the wait above):
@@ -1285,11 +1291,13 @@ __global__ void k_finalize(Set set, Items it, Plan pl, const uint64_t* sums, dou
 // candidates' expectations and scores and its best entry into part[2 b ..],
 // and the last to finish (a ticket in work[1], zeroed by k_prep) reduces them.
 __global__ void k_finalize_split(Set set, Items it, Plan pl, const uint64_t* sums, double* gap, double* score,
-                                 float* gamma_t, int32_t* best, uint32_t* status_copy, uint64_t* part) {
+                                 float* gamma_t, int32_t* best, uint32_t* status_copy, uint64_t* part,
+                                 uint64_t* sum_out) {
   pdl_wait();
   pdl_trigger();
   const int nb = (int)gridDim.x, per = (it.n + nb - 1) / nb;
   const int beg = min(it.n, (int)blockIdx.x * per), end = min(it.n, beg + per);
+  copy_sums(pl, sums, sum_out, beg, end);
   const Best b = finalize_problem(set, it, pl, sums, 0, beg, end, gap, score,
                                   blockIdx.x == 0 ? gamma_t : nullptr, 0);
   __shared__ int s_last;
@@ -1473,13 +1481,13 @@ int finalize_blocks(const Items& it) {
 
 cudaError_t launch_finalize(const Set& set, const Items& it, const Plan& pl, const uint64_t* sums, double* gap,
                             double* score, float* gamma_t, int32_t* best, uint32_t* status_copy, uint64_t* part,
-                            cudaStream_t s) {
+                            uint64_t* sum_out, cudaStream_t s) {
   const int nb = finalize_blocks(it);
   if (nb > 0 && part)
     return launch_pdl(k_finalize_split, dim3(nb), dim3(256), 0, s, set, it, pl, sums, gap, score, gamma_t, best,
-                      status_copy, part);
+                      status_copy, part, sum_out);
   return launch_pdl(k_finalize, dim3(it.off ? set.P : 1), dim3(256), 0, s, set, it, pl, sums, gap, score, gamma_t,
-                    best, status_copy);
+                    best, status_copy, sum_out);
 }
 
 // ---------------------------------------------------------------- measurement floors (not part of the method)

@@ -206,7 +206,7 @@ extern "C" int fs_score_candidates_noalloc(int32_t K, int32_t B, int32_t G, cons
                      reinterpret_cast<uint64_t*>(base + o_sums), nullptr, 0, sm_count, lc, s);
   if (e == cudaSuccess)
     e = launch_finalize(set, it, pl, reinterpret_cast<const uint64_t*>(base + o_sums), gap_dev, score_dev,
-                        gamma_t_dev, best_dev, nullptr, reinterpret_cast<uint64_t*>(base + o_part), s);
+                        gamma_t_dev, best_dev, nullptr, reinterpret_cast<uint64_t*>(base + o_part), nullptr, s);
   {
     // launch shapes only grow (a kernel's shared-memory limit is only raised):
     // keep the larger of what this call and any concurrent one found
