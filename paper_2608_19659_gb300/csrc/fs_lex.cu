@@ -858,15 +858,31 @@ __global__ void k_finalize_goodput(Set set, Items it, Plan pl, const uint64_t* s
   const long long gfix = gpl > gm ? gpl - gm : gm - gpl;
   const long long n = (long long)pl.O * pl.S;
   const double dn = __ll2double_rn(n);
+  // x / n: a power of two's quotient is an exact scaling (no result is subnormal)
+  const bool p2 = (n & (n - 1)) == 0;
+  const double rn = p2 ? __longlong_as_double((1023LL - (63 - __clzll(n))) << 52) : 0.0;
+  auto mean = [&](long long v) {
+    const double x = __dmul_rn(__ll2double_rn(v), 0x1p-20);
+    return __ddiv_rn(p2 ? __dmul_rn(x, rn) : __ddiv_rn(x, dn), lam_sum);
+  };
   Best b = no_best();
-  for (int q = beg + tid; q < end; q += blockDim.x) {
-    const int cell = it.cell[q];
+  // lanes per candidate as in finalize_problem: four when split over blocks
+  const int lpc = nb > 1 ? 4 : 1, sub = tid & (lpc - 1), step = (int)blockDim.x / lpc;
+  for (int q0 = beg; q0 < end; q0 += step) {
+    const int q = q0 + tid / lpc;
+    const bool in = q < end;
     long long tot = 0;
+    int cell = 0;
+    if (in) {
+      cell = __ldg(it.cell + q);
 #pragma unroll 8
-    for (int o = 0; o < pl.O; ++o) tot += (long long)__ldg(sums + (size_t)q * pl.O + o);
+      for (int o = sub; o < pl.O; o += lpc) tot += (long long)__ldg(sums + (size_t)q * pl.O + o);
+    }
+    for (int o = 1; o < lpc; o <<= 1) tot += __shfl_xor_sync(0xffffffffu, tot, o);
+    if (!in) continue;
     const long long sc = gfix * n - tot;
-    if (gap) gap[q] = __ddiv_rn(__ddiv_rn(__dmul_rn(__ll2double_rn(tot), 0x1p-20), dn), lam_sum);
-    if (score) score[q] = __ddiv_rn(__ddiv_rn(__dmul_rn(__ll2double_rn(sc), 0x1p-20), dn), lam_sum);
+    if (sub == 0 && gap) gap[q] = mean(tot);
+    if (sub == lpc / 2 && score) score[q] = mean(sc);
     const Best c = make_best(sc, (cell / d.B) & 3, q, cell);
     if (better(c, b)) b = c;
   }

@@ -1298,8 +1298,8 @@ __global__ void k_finalize_split(Set set, Items it, Plan pl, const uint64_t* sum
   const int nb = (int)gridDim.x, per = (it.n + nb - 1) / nb;
   const int beg = min(it.n, (int)blockIdx.x * per), end = min(it.n, beg + per);
   copy_sums(pl, sums, sum_out, beg, end);
-  const Best b = finalize_problem(set, it, pl, sums, 0, beg, end, gap, score,
-                                  blockIdx.x == 0 ? gamma_t : nullptr, 0);
+  const Best b = finalize_problem<4>(set, it, pl, sums, 0, beg, end, gap, score,
+                                     blockIdx.x == 0 ? gamma_t : nullptr, 0);
   __shared__ int s_last;
   if (threadIdx.x == 0) {
     part[2 * blockIdx.x] = (uint64_t)b.hi;
@@ -1474,9 +1474,8 @@ cudaError_t launch_score(const Set& set, const Items& it, const Plan& pl, const 
 }
 
 int finalize_blocks(const Items& it) {
-  if (it.off) return 0;
-  const int nb = (it.n + 255) / 256;  // one candidate per thread
-  return nb < 2 ? 0 : (nb > kFinalizeMaxBlocks ? kFinalizeMaxBlocks : nb);
+  if (it.off || it.n <= 256) return 0;
+  return std::min(kFinalizeMaxBlocks, (it.n + 63) / 64);  // four lanes per candidate: one pass of a block
 }
 
 cudaError_t launch_finalize(const Set& set, const Items& it, const Plan& pl, const uint64_t* sums, double* gap,
