@@ -173,6 +173,8 @@ struct fs_model {
   bool staged = false;  // the staging holds bounds the device copy does not have yet
   int th_bound = -1;    // threshold_bound of the current bounds (-1: not computed yet)
   LaunchCache lc;
+  int t_half = 0;           // half of the t* parts the last scoring call used
+  bool rows_read = false;   // the last scoring call's scenarios read the rows (dump)
   // optional timing events: 5 per timed call (before solve, prep, score,
   // finalize, and after finalize); mode 1 records only the two around score
   int timing = 0;
@@ -373,7 +375,7 @@ int ensure_items(fs_model* m, int n, int O) {
 // The scoring sequence on stream s; cand_dev holds n_cand cell ids.
 int run_score(fs_model* m, Set set, const fs_samples* smp, const int32_t* cand_dev, double* gap,
               double* score, float* gamma_t, int32_t* best, void* dump, uint64_t* sum_out, cudaStream_t s,
-              uint32_t* status_copy = nullptr) {
+              uint32_t* status_copy = nullptr, bool late = false) {
   const int n = smp->n_cand;
   Items it{};
   it.n = n;
@@ -396,7 +398,10 @@ int run_score(fs_model* m, Set set, const fs_samples* smp, const int32_t* cand_d
   const bool phases = timed && m->timing == 2;
   if (phases) FS_CUDA(cudaEventRecord(ev[0], s), "record timing event");
   if (m->th_bound < 0) m->th_bound = threshold_bound(m);
-  FS_CUDA(launch_thresh(set, m->lc.floors, m->th_bound, s), "launch thresholds");
+  m->t_half ^= 1;
+  set.tpart += m->t_half * 2 * kThreshBlocks;
+  FS_CUDA(launch_thresh(set, m->lc.floors, m->th_bound, s, late && !m->rows_read), "launch thresholds");
+  m->rows_read = dump != nullptr;
   if (phases) FS_CUDA(cudaEventRecord(ev[1], s), "record timing event");
   FS_CUDA(launch_prep(set, it, pl, (float*)m->tables.p, (uint64_t*)m->sums.p, true, m->sm_count, m->lc, s,
                       m->th_bound),
@@ -543,7 +548,7 @@ int fs_load_model(const fs_bounds* b, const float* slo, const float* demand, int
   const size_t o_rowc = take(8 * (size_t)d.K4), o_rowb = take(8 * (size_t)d.K4);
   const size_t o_base = take(2 * sizeof(fs_allocation)), o_status = take(4), o_work = take(32);
   const int rt_cap = (int)std::min<long long>((long long)d.K4 * d.theta_cap, kRowTabModel);
-  const size_t o_rtab = take(4 * (size_t)rt_cap), o_tpart = take(8 * (size_t)kThreshBlocks);
+  const size_t o_rtab = take(4 * (size_t)rt_cap), o_tpart = take(16 * (size_t)kThreshBlocks);
   rc = m->fixed.ensure(off, "model state");
   if (rc) {
     delete m;
@@ -693,7 +698,7 @@ int fs_score_candidates_async(fs_model* m, const fs_samples* smp, double* gap_de
   cudaStream_t s = (cudaStream_t)cuda_stream;
   if ((rc = flush_bounds(m, s))) return rc;
   return run_score(m, m->set, smp, smp->cand, gap_dev, score_dev, gamma_t_dev, best_dev, dump_dev,
-                   reinterpret_cast<uint64_t*>(sum_eo_dev), s);
+                   reinterpret_cast<uint64_t*>(sum_eo_dev), s, nullptr, true);
 }
 
 int fs_solve(fs_model* m, const float* cap, const float* tail, fs_allocation* out) {

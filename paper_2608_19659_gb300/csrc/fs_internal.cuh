@@ -504,7 +504,7 @@ cudaError_t launch_solve(const Set& set, int n, const float* cap_x, const float*
 // problem of the set. th_bound > 0: a bound on either realisation's threshold
 // count (theta_cap otherwise). With set.tpart (one problem) the launch's block
 // count is left in set.n_tpart, and the parts hold t*.
-cudaError_t launch_thresh(Set& set, int floors, int th_bound, cudaStream_t s);
+cudaError_t launch_thresh(Set& set, int floors, int th_bound, cudaStream_t s, bool late = false);
 // early: the candidate ids and bounds were complete before the preceding
 // kernel started, so the bounds-only work may run before the PDL wait.
 // Blocks of 256 threads, or of 64 when the launch holds more than two waves

@@ -300,55 +300,52 @@ __global__ void __launch_bounds__(kPrepThreads) k_prep(Set set, Items it, Plan p
   // positions whose tail value passes the SLO (the mapped tails are
   // nondecreasing in the position, so exactly one position ends the run of
   // passes), words 4.. = the W capacities.
-  if (!pl.few) {
+  if (pl.few) {  // (word 1, 2 of the first window: the cell's capacity bounds, for its draws)
+    if (sigma == 0 && tid == 0) {
+      float* win0 = base_rec + 2 * (size_t)d.slot_floats;
+      win0[1] = lo_c;
+      win0[2] = hi_c;
+    }
+  } else {
     const int W = pl.W;
     const float d_c = __fsub_rn(hi_c, lo_c), d_l = __fsub_rn(hi_l, lo_l);
-    const long long n_idx = (long long)((pl.O - sigma + 1) >> 1) * W;
+    const int n_out = (pl.O - sigma + 1) >> 1;  // this block's outcomes
+    const int n_idx = n_out << pl.w;            // (at most Q <= 2^24 positions)
     float* wins = base_rec + 2 * (size_t)d.slot_floats;
+    // gate positions, an outcome per thread: every position where even the upper
+    // tail passes, none where not even the lower one does, else by bisection
+    for (int x = tid; x < n_out; x += blockDim.x) {
+      const int o = sigma + 2 * x;
+      int pass = hi_l <= L ? W : 0;
+      if (hi_l > L && lo_l <= L) {
+        const float* q = set.qn + (size_t)o * W;
+        for (int step = W; step > 0; step >>= 1)
+          if (pass + step <= W && map_into(lo_l, d_l, hi_l, __ldg(q + pass + step - 1)) <= L) pass += step;
+      }
+      wins[(size_t)o * pl.Wp] = __int_as_float(pass);
+    }
     if (W >= 4 && (reinterpret_cast<uintptr_t>(set.qn) & 15u) == 0) {
       // four consecutive positions per thread: one 16-byte load and store
-      // (windows start on 16-byte boundaries), plus the next position's value
-      const long long n4 = n_idx >> 2;
-#pragma unroll 2
-      for (long long g4 = tid; g4 < n4; g4 += blockDim.x) {
-        const long long idx = g4 << 2;
-        const int k = (int)(idx & (W - 1));
-        const int o = sigma + 2 * (int)(idx >> pl.w);
-        const float* q = set.qn + (size_t)o * W;
-        float* win = wins + (size_t)o * pl.Wp;
-        const float4 v = __ldg(reinterpret_cast<const float4*>(q + k));
-        const float vn = k + 4 < W ? __ldg(q + k + 4) : 0.0f;
+      // (windows start on 16-byte boundaries)
+      const int n4 = n_idx >> 2;
+#pragma unroll 4
+      for (int g4 = tid; g4 < n4; g4 += blockDim.x) {
+        const int k = (g4 << 2) & (W - 1), o = sigma + 2 * (g4 >> (pl.w - 2));
+        const float4 v = __ldg(reinterpret_cast<const float4*>(set.qn + (size_t)o * W + k));
         float4 cm;
         cm.x = map_into(lo_c, d_c, hi_c, v.x);
         cm.y = map_into(lo_c, d_c, hi_c, v.y);
         cm.z = map_into(lo_c, d_c, hi_c, v.z);
         cm.w = map_into(lo_c, d_c, hi_c, v.w);
-        *reinterpret_cast<float4*>(win + 4 + k) = cm;
-        const bool p0 = map_into(lo_l, d_l, hi_l, v.x) <= L, p1 = map_into(lo_l, d_l, hi_l, v.y) <= L;
-        const bool p2 = map_into(lo_l, d_l, hi_l, v.z) <= L, p3 = map_into(lo_l, d_l, hi_l, v.w) <= L;
-        const bool p4 = k + 4 < W && map_into(lo_l, d_l, hi_l, vn) <= L;
-        if (k == 0 && !p0) win[0] = __int_as_float(0);
-        if (p0 && !p1) win[0] = __int_as_float(k + 1);
-        if (p1 && !p2) win[0] = __int_as_float(k + 2);
-        if (p2 && !p3) win[0] = __int_as_float(k + 3);
-        if (p3 && !p4) win[0] = __int_as_float(k + 4);
+        *reinterpret_cast<float4*>(wins + (size_t)o * pl.Wp + 4 + k) = cm;
       }
     } else {
       // read-only loads, so that the unrolled iterations' loads are issued
       // together rather than each behind the previous iteration's stores
 #pragma unroll 4
-      for (long long idx = tid; idx < n_idx; idx += blockDim.x) {
-        const int k = (int)(idx & (W - 1));
-        const int o = sigma + 2 * (int)(idx >> pl.w);
-        const float* q = set.qn + (size_t)o * W;
-        float* win = wins + (size_t)o * pl.Wp;
-        const float qv = __ldg(q + k);
-        const float qnext = k + 1 < W ? __ldg(q + k + 1) : 0.0f;
-        win[4 + k] = map_into(lo_c, d_c, hi_c, qv);
-        const bool pass = map_into(lo_l, d_l, hi_l, qv) <= L;
-        const bool pass_next = k + 1 < W && map_into(lo_l, d_l, hi_l, qnext) <= L;
-        if (k == 0 && !pass) win[0] = __int_as_float(0);
-        if (pass && !pass_next) win[0] = __int_as_float(k + 1);
+      for (int idx = tid; idx < n_idx; idx += blockDim.x) {
+        const int k = idx & (W - 1), o = sigma + 2 * (idx >> pl.w);
+        wins[(size_t)o * pl.Wp + 4 + k] = map_into(lo_c, d_c, hi_c, __ldg(set.qn + (size_t)o * W + k));
       }
     }
   }
@@ -1218,8 +1215,8 @@ __global__ void __launch_bounds__(kFewThreads) k_score_few(Set set, Items it, Pl
     const int cell = __float_as_int(h0[H_CELL]);
     if (cell >= 0 && cell < d.cells) {  // (a bad device-side id was flagged by k_prep)
       const int p = __float_as_int(h0[H_P]);
-      const float* bp = set.bounds + (size_t)p * 4 * d.cells + cell;
-      const float lo_c = bp[0], hi_c = bp[(size_t)d.cells];
+      const float* win0 = h0 + 2 * (size_t)d.slot_floats;
+      const float lo_c = win0[1], hi_c = win0[2];
       const float lo_l = h0[H_LO_L], hi_l = h0[H_HI_L], L = h0[H_SLO];
       const float d_c = __fsub_rn(hi_c, lo_c), d_l = __fsub_rn(hi_l, lo_l);
       const float lam = h0[H_LAM], rl = h0[H_RLAM], dl = FL ? h0[H_DLT] : 0.0f;
@@ -1270,12 +1267,12 @@ __global__ void __launch_bounds__(kFewThreads) k_score_few(Set set, Items it, Pl
   if (live && gl == 0) sums[seg] = sum;
 }
 
-// (both reductions let the next call's first kernel be placed while they run:
-// it waits for their completion before it reads or writes anything)
+// (both reductions let the next call's first kernel start at once: see
+// launch_thresh for what it may do before they have finished)
 __global__ void k_finalize(Set set, Items it, Plan pl, const uint64_t* sums, double* gap, double* score,
                            float* gamma_t, int32_t* best, uint32_t* status_copy, uint64_t* sum_out) {
-  pdl_wait();
   pdl_trigger();
+  pdl_wait();
   const int p = blockIdx.x;
   const int beg = it.off ? it.off[p] : 0;
   const int end = it.off ? it.off[p + 1] : it.n;
@@ -1293,8 +1290,8 @@ __global__ void k_finalize(Set set, Items it, Plan pl, const uint64_t* sums, dou
 __global__ void k_finalize_split(Set set, Items it, Plan pl, const uint64_t* sums, double* gap, double* score,
                                  float* gamma_t, int32_t* best, uint32_t* status_copy, uint64_t* part,
                                  uint64_t* sum_out) {
-  pdl_wait();
   pdl_trigger();
+  pdl_wait();
   const int nb = (int)gridDim.x, per = (it.n + nb - 1) / nb;
   const int beg = min(it.n, (int)blockIdx.x * per), end = min(it.n, beg + per);
   copy_sums(pl, sums, sum_out, beg, end);
@@ -1446,7 +1443,7 @@ cudaError_t launch_score(const Set& set, const Items& it, const Plan& pl, const 
         const long long nch_u = (pl.calls + tb * u - 1) / (tb * u);
         const long long rounds = (n_seg * nch_u + res_b - 1) / res_b;
         const long long cost = rounds * lc.score_blocks_per_sm[v][mode][b] * tb * (180 + build + 72 * u);
-        if (best < 0 || cost < best) {
+        if (best < 0 || cost < best || (cost == best && tb < bt)) {  // (equal: the smaller block, measured faster)
           best = cost;
           U = u;
           bt = tb;

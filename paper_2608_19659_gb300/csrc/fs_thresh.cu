@@ -36,7 +36,7 @@ namespace fs {
 
 // FL: some class is critical (the model has floors).
 template <bool FL>
-__global__ void __launch_bounds__(kThreshThreads) k_thresh(Set set) {
+__global__ void __launch_bounds__(kThreshThreads) k_thresh(Set set, int late) {
   const Dims& d = set.d;  // kernel-parameter space: no local copy
   const int r = blockIdx.y, p = r >> 1, sigma = r & 1;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -46,10 +46,15 @@ __global__ void __launch_bounds__(kThreshThreads) k_thresh(Set set) {
   __shared__ float sLam[FS_MAX_CLASSES], sRl[FS_MAX_CLASSES], sDl[FS_MAX_CLASSES];
   __shared__ int sCover[kWarps][256];  // covers of one threshold (more than 32 rows)
   __shared__ uint32_t s_best;
-  // the previous kernels of the stream wrote what is read here, and may read
-  // what is written here (the last call's tables)
-  pdl_wait();
-  pdl_trigger();
+  // `late`: what is read here was complete before this kernel could start, and
+  // nothing that may still run reads what is written here (launch_thresh), so the
+  // wait for the previous kernel comes after the work: the last call's scenarios
+  // and this call's thresholds overlap. Only then may the preparation start, whose
+  // records those scenarios still read.
+  if (!late) {
+    pdl_wait();
+    pdl_trigger();
+  }
   if (set.skip && set.skip[p] >= 0) return;
   const float* bp = set.bounds + (size_t)p * 4 * d.cells;
   const float* cap = bp + (size_t)(sigma ? CAP_HI : CAP_LO) * d.cells;
@@ -186,13 +191,25 @@ __global__ void __launch_bounds__(kThreshThreads) k_thresh(Set set) {
     __syncthreads();
     if (tid == 0) set.tpart[sigma * gridDim.x + blockIdx.x] = __uint_as_float(s_best);
   }
+  if (late) {
+    pdl_wait();
+    pdl_trigger();
+  }
 }
 
 // Measured (one GB300, calls in a row): the eight-class, 256-GPU grid (about 1300
 // thresholds a realisation, 55 blocks each) 19.2 -> 7.3 us, and with its tables
 // the preparation of 1024 candidates 60.6 -> 14 us: 1024 x 16 x 16384 scenarios
 // 270 -> 206 us, 1024 x 8 x 60 116 -> 51 us; four classes, 64 GPUs 51 -> 45 us.
-cudaError_t launch_thresh(Set& set, int floors, int th_bound, cudaStream_t s) {
+//
+// late: for a scoring call on the model's own device bounds. They are only
+// written by copies (a full barrier in the stream). The thresholds, rows and
+// tables were last read by the previous call's preparation, which had finished
+// before its Monte-Carlo kernel let the reduction, and that let this kernel,
+// start; only a dump's scenarios and the goodput stage read rows later (not
+// late after the former; the latter is synchronous). The parts of t*, which the
+// previous reduction may still read, alternate between two halves.
+cudaError_t launch_thresh(Set& set, int floors, int th_bound, cudaStream_t s, bool late) {
   const Dims& d = set.d;
   const int bound = th_bound > 0 ? std::min(th_bound, d.theta_cap) : d.theta_cap;
   int gsz = 4;
@@ -202,7 +219,8 @@ cudaError_t launch_thresh(Set& set, int floors, int th_bound, cudaStream_t s) {
   const int per_block = 2 * (kThreshThreads / gsz);
   const int nb = set.P > 1 ? 1 : std::max(1, std::min(kThreshBlocks, (bound + per_block - 1) / per_block));
   set.n_tpart = set.tpart ? nb : 0;
-  return launch_pdl(floors ? k_thresh<true> : k_thresh<false>, dim3(nb, 2 * set.P), dim3(kThreshThreads), 0, s, set);
+  return launch_pdl(floors ? k_thresh<true> : k_thresh<false>, dim3(nb, 2 * set.P), dim3(kThreshThreads), 0, s, set,
+                    late ? 1 : 0);
 }
 
 }  // namespace fs

@@ -1,0 +1,77 @@
+"""Asynchronous scoring calls queued without a wait between them: a call's
+thresholds may be made while the previous call's scenarios still run, so calls
+with other bounds, other candidate lists (none among them), few and many
+samples, and dumps, whose scenarios read the rows, are queued in a mixed order
+on the model's stream, and every call's outputs must be those of the same call
+made alone."""
+
+import dataclasses
+
+import numpy as np
+import pytest
+
+from conftest import load_model
+from paper_2608_19659_gb300 import workloads
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("side_stream", [False, True])
+@pytest.mark.parametrize("K,B,G", [(2, 8, 16), (8, 6, 200)])
+def test_calls_in_a_row(fsb, cuda, oracle_lib, K, B, G, side_stream):
+    torch = cuda
+    rng = np.random.default_rng(K + G)
+    ws = [workloads.random_small(np.random.default_rng(s), K, B, G, p_infeasible=0.1) for s in (1, 2)]
+    lam = (ws[0].demand * np.float32(G / (4.0 * K))).astype(np.float32)
+    ws = [dataclasses.replace(w, demand=lam, slo=ws[0].slo) for w in ws]
+    st = torch.cuda.Stream() if side_stream else None
+    w = ws[0]
+    plans = [(rng.permutation(w.cells)[:n].astype(np.int32), O, S, dump)
+             for n, O, S, dump in ((16, 4, 2000, 0), (1, 8, 64, 0), (0, 4, 10, 0), (w.cells, 8, 1500, 0), (3, 4, 40, 1),
+                                   (40, 2, 4096, 0))]
+
+    def alone(m, plan, which):
+        cand, O, S, _ = plan
+        x = ws[which]
+        fsb.fs_update_bounds(m, x.cap_lo, x.cap_hi, x.tail_lo, x.tail_hi)
+        return fsb.fs_score_candidates(m, cand, O, S, 9)
+
+    with load_model(fsb, w) as m:
+        ref = {(k, b): alone(m, p, b) for k, p in enumerate(plans) for b in (0, 1)}
+        stride = fsb.fs_dump_stride(m)
+    m = fsb.fs_load_model(w.cap_lo, w.cap_hi, w.tail_lo, w.tail_hi, w.slo, w.demand, G, K, B, stream=st)
+    dev = [torch.from_numpy(p[0]).cuda() for p in plans]
+    torch.cuda.synchronize()
+    calls = []
+    with m:
+        at = 0
+        for _ in range(40):
+            k = int(rng.integers(len(plans)))
+            cand, O, S, dump = plans[k]
+            if rng.random() < 0.3:
+                at ^= 1
+                x = ws[at]
+                fsb.fs_update_bounds(m, x.cap_lo, x.cap_hi, x.tail_lo, x.tail_hi)
+            n = len(cand)
+            out = [torch.zeros(max(n, 1), dtype=torch.float64, device="cuda"), torch.zeros(1, device="cuda"),
+                   torch.zeros(1, dtype=torch.int32, device="cuda"),
+                   torch.zeros((max(n, 1), O), dtype=torch.int64, device="cuda")]
+            d = torch.zeros(n * O * S * stride, dtype=torch.uint8, device="cuda") if dump else None
+            calls.append((k, at, out, d))
+        torch.cuda.synchronize()  # the buffers are zeroed; the calls below queue back to back
+        at = 0
+        for k, b, out, d in calls:
+            if b != at:
+                at = b
+                x = ws[at]
+                fsb.fs_update_bounds(m, x.cap_lo, x.cap_hi, x.tail_lo, x.tail_hi)
+            cand, O, S, _ = plans[k]
+            fsb.fs_score_candidates_async(m, dev[k], O, S, 9, score_dev=out[0], gamma_t_dev=out[1], best_dev=out[2],
+                                          sum_eo_dev=out[3], dump_dev=d, stream=st)
+        fsb.fs_check(m)
+        torch.cuda.synchronize()
+    for k, b, out, _ in calls:
+        r, n = ref[(k, b)], len(plans[k][0])
+        assert float(out[1][0]) == r.gamma_t and int(out[2][0]) == r.best, (k, b)
+        assert np.array_equal(out[3].cpu().numpy()[:n], r.sum_eo), (k, b)
+        assert np.array_equal(out[0].cpu().numpy()[:n], r.score), (k, b)
