@@ -988,13 +988,13 @@ int fs_replay(fs_model* m, const fs_replay_spec* sp, int32_t* rounds, int32_t* s
     if (rc_sync) return rc_sync;
     for (int r = 0; r <= sp->max_rounds; ++r) {
       FS_CUDA(launch_solve(set, 2 * P, nullptr, nullptr, nullptr, m->lc, s), "launch solve");
-      FS_CUDA(cudaMemsetAsync(rs.n_active, 0, 4, s), "clear active");
       const int per = cells - sp->r0 - r;  // candidates of each running stream this round
       // the certificate, and the running streams' candidate lists (scored reveals)
-      FS_CUDA(launch_replay_certify(set, rs, r, sp->policy == 0 ? per : 0, s), "launch certify");
-      // the thresholds of the streams that go on are queued behind the read of
-      // their count, so that they run while the host learns it
-      FS_CUDA(cudaMemcpyAsync(m->h_out.p, rs.n_active, 4, cudaMemcpyDeviceToHost, s), "read active");
+      FS_CUDA(launch_replay_certify(set, rs, r, sp->policy == 0 ? per : 0, static_cast<int*>(m->h_out.dev), s),
+              "launch certify");
+      // the thresholds of the streams that go on are queued behind the event that
+      // their count (in mapped memory) waits for, so that they run while the host
+      // learns it
       FS_CUDA(cudaEventRecord(m->round_done, s), "record round event");
       if (sp->policy == 0) FS_CUDA(launch_thresh(set, m->lc.floors, 0, s), "launch thresholds");
       FS_CUDA(cudaEventSynchronize(m->round_done), "round sync");

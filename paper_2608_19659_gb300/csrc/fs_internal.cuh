@@ -585,7 +585,9 @@ cudaError_t launch_replay_init(const Set& set, const ReplayState& rs, const floa
                                cudaStream_t s);
 // Certificate of every running stream; with per > 0 also each running
 // stream's list of per candidates (items [slot][per]).
-cudaError_t launch_replay_certify(const Set& set, const ReplayState& rs, int round, int per, cudaStream_t s);
+// host_active (mapped): the number of streams that go on.
+cudaError_t launch_replay_certify(const Set& set, const ReplayState& rs, int round, int per, int* host_active,
+                                  cudaStream_t s);
 cudaError_t launch_replay_next(const Set& set, const ReplayState& rs, int n_active, cudaStream_t s);
 cudaError_t launch_replay_reveal(const Set& set, const ReplayState& rs, const Items& it,
                                  const Plan& pl, const uint64_t* sums, int n_active, cudaStream_t s);

@@ -189,6 +189,8 @@ __global__ void __launch_bounds__(NW == 1 ? 128 : 32 * NW) k_solve_lex(Set set, 
   const int lane = threadIdx.x & 31, warp = NW == 1 ? 0 : (int)threadIdx.x >> 5;
   const int slot = NW == 1 ? (int)threadIdx.x >> 5 : 0, tid = warp * 32 + lane;
   const int rel = (int)blockIdx.x * kPerBlock + slot, r = r0 + rel;
+  pdl_wait();
+  pdl_trigger();
   if (r >= n_real) return;
   auto sync = [] {
     if (NW == 1) __syncwarp();
@@ -940,10 +942,8 @@ static cudaError_t launch_lex(const Set& set, int n, const float* cap_x, const f
   if (e != cudaSuccess) return e;
   for (int r0 = 0; r0 < n; r0 += per_launch) {
     const int m = n - r0 < per_launch ? n - r0 : per_launch;
-    note_launch();
-    kern<<<(m + kPerBlock - 1) / kPerBlock, NW == 1 ? 128 : 32 * NW, smem, s>>>(
-        set, r0 + m, cap_x, tail_x, out, static_cast<unsigned char*>(scratch), r0, lay, host);
-    e = cudaGetLastError();
+    e = launch_pdl(kern, dim3((m + kPerBlock - 1) / kPerBlock), dim3(NW == 1 ? 128 : 32 * NW), smem, s, set, r0 + m,
+                   cap_x, tail_x, out, static_cast<unsigned char*>(scratch), r0, lay, host);
     if (e != cudaSuccess) return e;
   }
   return cudaSuccess;

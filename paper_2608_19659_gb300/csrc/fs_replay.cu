@@ -38,6 +38,7 @@ __global__ void k_replay_init(Set set, ReplayState rs, const float* prior, int r
   for (int q = threadIdx.x; q < cells; q += blockDim.x) rs.reveal_order[(size_t)p * cells + q] = -1;
   __syncthreads();
   if (threadIdx.x != 0) return;
+  if (p == 0) set.work[1] = 0ull;  // the certificate's ticket
   rs.n_revealed[p] = 0;
   rs.gpu_seconds[p] = 0.0;
   rs.rounds[p] = 0;
@@ -49,7 +50,7 @@ __global__ void k_replay_init(Set set, ReplayState rs, const float* prior, int r
 // that go on, and (per > 0) writes each one's candidate list: its unrevealed
 // cells in reveal order, 32 cells of the order at a time, each lane's place in
 // the list from a ballot of the unrevealed ones before it.
-__global__ void k_replay_certify(Set set, ReplayState rs, int round, int per) {
+__device__ __forceinline__ void certify_stream(const Set& set, const ReplayState& rs, int round, int per) {
   const int p = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5), lane = threadIdx.x & 31;
   if (p >= set.P || rs.state[p] >= 0) return;  // (the warp's lanes agree)
   const Dims& d = set.d;
@@ -104,9 +105,29 @@ __global__ void k_replay_certify(Set set, ReplayState rs, int round, int per) {
   if (lane == 0 && q < per) atomicOr(set.status, ST_TABLE);
 }
 
+// The last block to finish (a ticket) leaves the count of running streams for the
+// host and clears the device's for the next round.
+__global__ void k_replay_certify(Set set, ReplayState rs, int round, int per, int* host_active) {
+  pdl_wait();
+  pdl_trigger();
+  certify_stream(set, rs, round, per);
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    __threadfence();
+    const unsigned long long t = atomicAdd(&set.work[1], 1ull);
+    if (t == (unsigned long long)gridDim.x - 1) {
+      __threadfence();
+      *host_active = atomicExch(rs.n_active, 0);
+      set.work[1] = 0ull;
+    }
+  }
+}
+
 // Fixed-order policy: running stream slot a reveals its next unrevealed cell
 // in reveal order (the candidate list's first entry).
 __global__ void k_replay_next(Set set, ReplayState rs, int n_active) {
+  pdl_wait();
+  pdl_trigger();
   const int a = blockIdx.x * blockDim.x + threadIdx.x;
   if (a >= n_active) return;
   const int p = rs.active[a];
@@ -122,6 +143,8 @@ __global__ void k_replay_next(Set set, ReplayState rs, int n_active) {
 }
 
 __global__ void k_replay_reveal(Set set, ReplayState rs, Items it, Plan pl, const uint64_t* sums, int per) {
+  pdl_wait();
+  pdl_trigger();
   const int a = blockIdx.x;
   const int p = rs.active[a];
   const Best b = finalize_problem(set, it, pl, sums, p, a * per, (a + 1) * per, nullptr, nullptr, nullptr, a * per);
@@ -135,23 +158,18 @@ cudaError_t launch_replay_init(const Set& set, const ReplayState& rs, const floa
   return cudaGetLastError();
 }
 
-cudaError_t launch_replay_certify(const Set& set, const ReplayState& rs, int round, int per, cudaStream_t s) {
-  note_launch();
-  k_replay_certify<<<(set.P + 3) / 4, 128, 0, s>>>(set, rs, round, per);
-  return cudaGetLastError();
+cudaError_t launch_replay_certify(const Set& set, const ReplayState& rs, int round, int per, int* host_active,
+                                  cudaStream_t s) {
+  return launch_pdl(k_replay_certify, dim3((set.P + 3) / 4), dim3(128), 0, s, set, rs, round, per, host_active);
 }
 
 cudaError_t launch_replay_next(const Set& set, const ReplayState& rs, int n_active, cudaStream_t s) {
-  note_launch();
-  k_replay_next<<<(n_active + 127) / 128, 128, 0, s>>>(set, rs, n_active);
-  return cudaGetLastError();
+  return launch_pdl(k_replay_next, dim3((n_active + 127) / 128), dim3(128), 0, s, set, rs, n_active);
 }
 
 cudaError_t launch_replay_reveal(const Set& set, const ReplayState& rs, const Items& it, const Plan& pl,
                                  const uint64_t* sums, int n_active, cudaStream_t s) {
-  note_launch();
-  k_replay_reveal<<<n_active, 256, 0, s>>>(set, rs, it, pl, sums, it.n / n_active);
-  return cudaGetLastError();
+  return launch_pdl(k_replay_reveal, dim3(n_active), dim3(256), 0, s, set, rs, it, pl, sums, it.n / n_active);
 }
 
 }  // namespace fs

@@ -135,6 +135,7 @@ __global__ void __launch_bounds__(NW == 1 ? 128 : 32 * NW) k_solve(Set set, int 
   const int slot = NW == 1 ? (int)threadIdx.x >> 5 : 0, ltid = warp * 32 + lane;
   SolveSmem& sm = smem[slot];
   const int r = (int)blockIdx.x * kPerBlock + slot;
+  pdl_wait();
   pdl_trigger();
   if (r >= n_real) return;
   auto sync = [] {
@@ -332,15 +333,11 @@ cudaError_t launch_qtable(float* qn, int Q, cudaStream_t s) {
 cudaError_t launch_solve(const Set& set, int n, const float* cap_x, const float* tail_x,
                          fs_allocation* out, LaunchCache& lc, cudaStream_t s, HostOut host) {
   if (n <= 0) return cudaSuccess;
-  note_launch();
-  if (n <= kSolveWideMax) {
-    auto kern = lc.floors ? k_solve<true, 8> : k_solve<false, 8>;
-    kern<<<n, 256, 0, s>>>(set, n, cap_x, tail_x, out, host);
-  } else {
-    auto kern = lc.floors ? k_solve<true, 1> : k_solve<false, 1>;
-    kern<<<(n + 3) / 4, 128, 0, s>>>(set, n, cap_x, tail_x, out, host);
-  }
-  return cudaGetLastError();
+  if (n <= kSolveWideMax)
+    return launch_pdl(lc.floors ? k_solve<true, 8> : k_solve<false, 8>, dim3(n), dim3(256), 0, s, set, n, cap_x, tail_x,
+                      out, host);
+  return launch_pdl(lc.floors ? k_solve<true, 1> : k_solve<false, 1>, dim3((n + 3) / 4), dim3(128), 0, s, set, n, cap_x,
+                    tail_x, out, host);
 }
 
 }  // namespace fs
