@@ -291,14 +291,19 @@ static __device__ __noinline__ int min_replicas_ieee(float t, float c, float lam
 // In range, the answer is reached from the estimate by steps of one: two
 // fulfilments when the estimate is right (the bracket of seven tested at once
 // that stood here before took 2.5 times the instructions).
-__device__ __forceinline__ int min_replicas(float t, float c, float lam, float rlam, float M) {
-  if (!(M >= 1.0f)) return 0;
-  if (!row_in_range(c, lam)) return min_replicas_ieee(t, c, lam, M);
+// (row_in_range(c, lam) and M >= 1)
+__device__ __forceinline__ int min_replicas_fast(float t, float c, float lam, float rlam, float M) {
   const float y = ceilf(__fdividef(__fmul_rn(t, lam), c));  // estimate only (c == 0: infinite)
   float n = fminf(fmaxf(y, 1.0f), M);
   while (n > 1.0f && fulfil_fast(n - 1.0f, c, lam, rlam) >= t) n -= 1.0f;
   while (n <= M && fulfil_fast(n, c, lam, rlam) < t) n += 1.0f;
   return n <= M ? (int)n : 0;
+}
+
+__device__ __forceinline__ int min_replicas(float t, float c, float lam, float rlam, float M) {
+  if (!(M >= 1.0f)) return 0;
+  if (!row_in_range(c, lam)) return min_replicas_ieee(t, c, lam, M);
+  return min_replicas_fast(t, c, lam, rlam, M);
 }
 
 // Philox4x32-10 (Salmon, Moraes, Dror, Shaw, SC'11): ten rounds of the 4x32

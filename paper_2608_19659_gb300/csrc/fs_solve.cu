@@ -89,6 +89,41 @@ __device__ __forceinline__ int group_cover(float t, const SolveSmem& sm, const D
   return packed;
 }
 
+// A lane's row when every row has a lane of its own (at most 32 rows).
+struct OneRow {
+  float C, lam, rl, dl, M;
+  int j;
+  bool in, fast;  // a row; in Markstein's range
+};
+
+// min_replicas on it (the range test made once).
+__device__ __forceinline__ int row_cover(const OneRow& r, float t) {
+  if (!(r.M >= 1.0f)) return 0;
+  if (!r.fast) return min_replicas_ieee(t, r.C, r.lam, r.M);
+  return min_replicas_fast(t, r.C, r.lam, r.rl, r.M);
+}
+
+template <bool FL>
+__device__ __forceinline__ int one_cover(float t, const OneRow& r, int gsz, int* below) {
+  int cost = kCostInf, u = 0;
+  if (r.in) {
+    const int n = row_cover(r, FL ? fmaxf(t, r.dl) : t);
+    u = n ? n : (int)r.M + 1;
+    if (n) cost = n << r.j;
+  }
+  cost = min(cost, __shfl_xor_sync(0xffffffffu, cost, 1));
+  cost = min(cost, __shfl_xor_sync(0xffffffffu, cost, 2));
+  u += __shfl_xor_sync(0xffffffffu, u, 1);
+  u += __shfl_xor_sync(0xffffffffu, u, 2);
+  int v = r.in ? (cost >= kCostInf ? (1 << 24) : cost) : 0;
+  for (int off = 4; off < gsz; off <<= 1) {
+    v += __shfl_xor_sync(0xffffffffu, v, off);
+    u += __shfl_xor_sync(0xffffffffu, u, off);
+  }
+  *below = u;
+  return v;
+}
+
 // Estimates of t* (patterns in [1, that of 1], aim_lo <= aim_hi) that start the
 // search; they only place the first probes. With replica counts real numbers,
 // class i takes t min_j tau_j lambda_i / C_ij GPUs, so t* is at most G over the
@@ -181,6 +216,16 @@ __global__ void __launch_bounds__(NW == 1 ? 128 : 32 * NW) k_solve(Set set, int 
   int ulo = -(1 << 28), uhi = 1 << 28;
   uint32_t aim_lo, aim_hi;  // where the first probes go
   search_aims(sm, d, lane, aim_lo, aim_hi);
+  const bool one = d.K4 <= gsz;  // (the same for every lane)
+  OneRow mine;
+  mine.in = gl < d.K4;
+  mine.j = gl & 3;
+  mine.C = mine.in ? sm.C[gl] : 0.0f;
+  mine.lam = mine.in ? sm.lam[gl >> 2] : 1.0f;
+  mine.rl = mine.in ? sm.rl[gl >> 2] : 1.0f;
+  mine.dl = FL && mine.in ? sm.dl[gl >> 2] : 0.0f;
+  mine.M = rep_capf(d, mine.j);
+  mine.fast = row_in_range(mine.C, mine.lam);
   int oct = 22;  // an unprobed lower end is approached by points 2^oct patterns apart, growing
   for (int rd = 0; uhi - ulo > 1 && hi - lo > 1; ++rd) {
     uint32_t pt;
@@ -197,7 +242,8 @@ __global__ void __launch_bounds__(NW == 1 ? 128 : 32 * NW) k_solve(Set set, int 
       oct += 2;
     }
     int u;
-    const int cost = group_cover<FL>(__uint_as_float(max(pt, 1u)), sm, d, gl, gsz, &u);
+    const float tp = __uint_as_float(max(pt, 1u));
+    const int cost = one ? one_cover<FL>(tp, mine, gsz, &u) : group_cover<FL>(tp, sm, d, gl, gsz, &u);
     const bool known = pt <= lo;
     const bool fits = known || cost <= d.G;
     // the largest point that fits and the smallest that does not
