@@ -158,7 +158,8 @@ struct fs_model {
   Buf fixed;      // lam, slo + floors, qn, bounds, revealed, theta, ntheta, rowC, rowB, base, status
   Set set{};
   // per-call scratch
-  Buf cand, tables, sums, outs, real, lex, gp;
+  Buf real, lex, gp;
+  Buf tables, sums;  // records and sums, two halves each: asynchronous calls alternate (launch_thresh)
   Buf replay;     // fs_replay's state of every stream (grown on demand, kept)
   int objective = FS_OBJECTIVE_MAXMIN;  // FS_OBJECTIVE_LEXICOGRAPHIC: fs_solve* and the certificate to tier 4
   // host mirrors
@@ -173,7 +174,7 @@ struct fs_model {
   bool staged = false;  // the staging holds bounds the device copy does not have yet
   int th_bound = -1;    // threshold_bound of the current bounds (-1: not computed yet)
   LaunchCache lc;
-  int t_half = 0;           // half of the t* parts the last scoring call used
+  int half = 0;             // the set of what alternates that the last scoring call used
   bool rows_read = false;   // the last scoring call's scenarios read the rows (dump)
   // optional timing events: 5 per timed call (before solve, prep, score,
   // finalize, and after finalize); mode 1 records only the two around score
@@ -340,7 +341,7 @@ int check_samples(const fs_model* m, const fs_samples* s, bool host_cand) {
   return FS_OK;
 }
 
-Plan make_plan(const fs_model* m, const fs_samples* s, int n_items) {
+Plan make_plan(const Dims& d, const fs_samples* s) {
   Plan pl{};
   pl.key0 = (uint32_t)s->seed;
   pl.key1 = (uint32_t)(s->seed >> 32);
@@ -348,28 +349,46 @@ Plan make_plan(const fs_model* m, const fs_samples* s, int n_items) {
   pl.round = s->round;
   pl.O = s->O;
   pl.S = s->S;
-  pl.W = m->d.Q / s->O;
+  pl.W = d.Q / s->O;
   pl.w = log2i(pl.W);
   pl.sh = 16 - pl.w;
   pl.logO = log2i(s->O);
   pl.calls = (s->S + 3) / 4;
   pl.Wp = 4 + ((pl.W + 3) & ~3);
-  pl.item_floats = 2LL * m->d.slot_floats + (long long)s->O * pl.Wp;
+  pl.item_floats = 2LL * d.slot_floats + (long long)s->O * pl.Wp;
   plan_round_keys(pl);
-  (void)n_items;
   return pl;
 }
 
-int ensure_items(fs_model* m, int n, int O) {
+// Dims of a call whose realisations have at most th_bound thresholds: its
+// records' tables need no more entries.
+Dims call_dims(const fs_model* m, int th_bound) {
+  Dims d = m->d;
+  if (th_bound > 0 && th_bound < d.theta_cap) {
+    d.lcap = 4;
+    while (d.lcap < th_bound + 1) d.lcap <<= 1;
+    d.slot_floats = kTableHeader + 3 * d.lcap;
+  }
+  return d;
+}
+
+// Halves of the records and sums (their place depends on the buffers' size alone,
+// so that calls of different sizes never share a byte; a buffer that grows is
+// freed, which waits for the calls in flight).
+float* tables_half(const fs_model* m, int half) {
+  return reinterpret_cast<float*>(static_cast<char*>(m->tables.p) + half * (m->tables.bytes / 2));
+}
+uint64_t* sums_half(const fs_model* m, int half) {
+  return reinterpret_cast<uint64_t*>(static_cast<char*>(m->sums.p) + half * (m->sums.bytes / 2));
+}
+
+int ensure_items(fs_model* m, const Dims& d, int n, int O) {
   int rc;
-  if ((rc = m->cand.ensure((size_t)std::max(n, 1) * 4, "candidate list"))) return rc;
-  const int W = m->d.Q / O, Wp = 4 + ((W + 3) & ~3);
-  const size_t item_floats = 2 * (size_t)m->d.slot_floats + (size_t)O * Wp;
-  if ((rc = m->tables.ensure((size_t)std::max(n, 1) * item_floats * 4, "candidate records"))) return rc;
+  const int W = d.Q / O, Wp = 4 + ((W + 3) & ~3);
+  const size_t item_floats = 2 * (size_t)d.slot_floats + (size_t)O * Wp;
+  if ((rc = m->tables.ensure(2 * align_up((size_t)std::max(n, 1) * item_floats * 4, 256), "candidate records"))) return rc;
   // sums, then the split reduction's scratch (2 words per block)
-  if ((rc = m->sums.ensure((size_t)std::max(n, 1) * O * 8 + 16 * (size_t)kFinalizeMaxBlocks, "sums"))) return rc;
-  if ((rc = m->outs.ensure((size_t)std::max(n, 1) * 16 + 64, "outputs"))) return rc;
-  return FS_OK;
+  return m->sums.ensure(2 * align_up((size_t)std::max(n, 1) * O * 8 + 16 * (size_t)kFinalizeMaxBlocks, 256), "sums");
 }
 
 // The scoring sequence on stream s; cand_dev holds n_cand cell ids.
@@ -382,7 +401,20 @@ int run_score(fs_model* m, Set set, const fs_samples* smp, const int32_t* cand_d
   it.p = nullptr;
   it.cell = cand_dev;
   it.off = nullptr;
-  Plan pl = make_plan(m, smp, n);
+  // this call's set of what alternates: the other one in an asynchronous call,
+  // which may start before the last call has finished, the same in a synchronous
+  // one, which waits for it
+  if (m->th_bound < 0) m->th_bound = threshold_bound(m);
+  set.d = call_dims(m, m->th_bound);
+  if (late) m->half ^= 1;
+  const int half = m->half;
+  int rc = ensure_items(m, set.d, n, smp->O);
+  if (rc) return rc;
+  float* tables = tables_half(m, half);
+  uint64_t* sums = sums_half(m, half);
+  set.tpart += half * 2 * kThreshBlocks;
+  set.work += 4 * half;
+  Plan pl = make_plan(set.d, smp);
   pl.few = !dump && few_path(pl, n) ? 1 : 0;
   const bool timed = m->timing && n > 0 && m->ev_used + 5 <= kMaxTimedEvents;
   cudaEvent_t* ev = nullptr;
@@ -397,22 +429,15 @@ int run_score(fs_model* m, Set set, const fs_samples* smp, const int32_t* cand_d
   }
   const bool phases = timed && m->timing == 2;
   if (phases) FS_CUDA(cudaEventRecord(ev[0], s), "record timing event");
-  if (m->th_bound < 0) m->th_bound = threshold_bound(m);
-  m->t_half ^= 1;
-  set.tpart += m->t_half * 2 * kThreshBlocks;
-  FS_CUDA(launch_thresh(set, m->lc.floors, m->th_bound, s, late && !m->rows_read), "launch thresholds");
+  FS_CUDA(launch_thresh(set, m->lc.floors, m->th_bound, s, late && n > 0 && !m->rows_read), "launch thresholds");
   m->rows_read = dump != nullptr;
   if (phases) FS_CUDA(cudaEventRecord(ev[1], s), "record timing event");
-  FS_CUDA(launch_prep(set, it, pl, (float*)m->tables.p, (uint64_t*)m->sums.p, true, m->sm_count, m->lc, s,
-                      m->th_bound),
-          "launch prep");
+  FS_CUDA(launch_prep(set, it, pl, tables, sums, late ? 2 : 1, m->sm_count, m->lc, s, m->th_bound), "launch prep");
   if (timed) FS_CUDA(cudaEventRecord(ev[2], s), "record timing event");
-  FS_CUDA(launch_score(set, it, pl, (const float*)m->tables.p, (uint64_t*)m->sums.p, dump,
-                       fs_dump_stride(m), m->sm_count, m->lc, s),
-          "launch score");
+  FS_CUDA(launch_score(set, it, pl, tables, sums, dump, fs_dump_stride(m), m->sm_count, m->lc, s), "launch score");
   if (timed) FS_CUDA(cudaEventRecord(ev[3], s), "record timing event");
-  FS_CUDA(launch_finalize(set, it, pl, (const uint64_t*)m->sums.p, gap, score, gamma_t, best, status_copy,
-                          (uint64_t*)m->sums.p + (size_t)std::max(n, 1) * smp->O, sum_out, s),
+  FS_CUDA(launch_finalize(set, it, pl, sums, gap, score, gamma_t, best, status_copy,
+                          sums + (size_t)std::max(n, 1) * smp->O, sum_out, s),
           "launch finalize");
   if (phases) FS_CUDA(cudaEventRecord(ev[4], s), "record timing event");
   return FS_OK;
@@ -546,7 +571,7 @@ int fs_load_model(const fs_bounds* b, const float* slo, const float* demand, int
   const size_t o_bounds = take(16 * (size_t)cells), o_rev = take(cells);
   const size_t o_theta = take(8 * (size_t)d.theta_cap), o_nth = take(8);
   const size_t o_rowc = take(8 * (size_t)d.K4), o_rowb = take(8 * (size_t)d.K4);
-  const size_t o_base = take(2 * sizeof(fs_allocation)), o_status = take(4), o_work = take(32);
+  const size_t o_base = take(2 * sizeof(fs_allocation)), o_status = take(4), o_work = take(64);
   const int rt_cap = (int)std::min<long long>((long long)d.K4 * d.theta_cap, kRowTabModel);
   const size_t o_rtab = take(4 * (size_t)rt_cap), o_tpart = take(16 * (size_t)kThreshBlocks);
   rc = m->fixed.ensure(off, "model state");
@@ -646,7 +671,6 @@ int fs_score_candidates(fs_model* m, const fs_samples* smp, double* gap_out, dou
   int rc = check_samples(m, smp, true);
   if (rc) return rc;
   const int n = smp->n_cand;
-  if ((rc = ensure_items(m, n, smp->O))) return rc;
   // One mapped page-locked block carries the call's host data both ways: the
   // kernels read the candidate ids from it and write gap, score, gamma_t, best
   // and the status word into it (k_finalize copies the status word), so no
@@ -673,7 +697,7 @@ int fs_score_candidates(fs_model* m, const fs_samples* smp, double* gap_out, dou
                  dump_dev, sums_mapped ? reinterpret_cast<uint64_t*>(hd + sum_at) : nullptr, s, d_st);
   if (rc) return rc;
   if (sum_bytes && !sums_mapped)
-    FS_CUDA(cudaMemcpyAsync(sum_eo, m->sums.p, sum_bytes, cudaMemcpyDeviceToHost, s), "read sums");
+    FS_CUDA(cudaMemcpyAsync(sum_eo, sums_half(m, m->half), sum_bytes, cudaMemcpyDeviceToHost, s), "read sums");
   FS_CUDA(cudaStreamSynchronize(s), "synchronize");
   uint32_t st;
   std::memcpy(&st, h + 16 * nn + 32, 4);
@@ -693,8 +717,6 @@ int fs_score_candidates_async(fs_model* m, const fs_samples* smp, double* gap_de
   if (!m) return fail(FS_EINVAL, "model is NULL");
   int rc = check_samples(m, smp, false);
   if (rc) return rc;
-  const int n = smp->n_cand;
-  if ((rc = ensure_items(m, n, smp->O))) return rc;
   cudaStream_t s = (cudaStream_t)cuda_stream;
   if ((rc = flush_bounds(m, s))) return rc;
   return run_score(m, m->set, smp, smp->cand, gap_dev, score_dev, gamma_t_dev, best_dev, dump_dev,
@@ -826,7 +848,10 @@ int fs_score_goodput(fs_model* m, const fs_samples* smp, double* gap_out, double
   if (m->d.G > 1024) return fail(FS_EINVAL, "the goodput stage needs G <= 1024");
   if (lex_scratch_cells(m->d) * kLexCellBytes > (64u << 20)) return fail(FS_EINVAL, "(K + 1)(G + 1) too large");
   const int n = smp->n_cand;
-  if ((rc = ensure_items(m, n, smp->O))) return rc;
+  if (m->th_bound < 0) m->th_bound = threshold_bound(m);
+  Set set = m->set;
+  set.d = call_dims(m, m->th_bound);
+  if ((rc = ensure_items(m, set.d, n, smp->O))) return rc;
   cudaStream_t s = m->stream;
   if ((rc = flush_bounds(m, s))) return rc;
   // as in fs_score_candidates, one mapped page-locked block carries the
@@ -847,23 +872,22 @@ int fs_score_goodput(fs_model* m, const fs_samples* smp, double* gap_out, double
   Items it{};
   it.n = n;
   it.cell = reinterpret_cast<const int32_t*>(hd + out_bytes);
-  const Plan pl = make_plan(m, smp, n);
+  const Plan pl = make_plan(set.d, smp);
   if (pl.W > (m->set.prior == 1 ? 2048 : 4096))  // a segment's table of positions lives in shared memory
     return fail(FS_EINVAL, "the goodput stage needs Q / O <= 2048 under the monotone prior, 4096 otherwise");
-  if (m->th_bound < 0) m->th_bound = threshold_bound(m);
   // the rows wanted and the base goodputs, then the pool of rows
   const size_t rows = goodput_pool_rows(m->d, m->th_bound, kGoodputPoolMax);
   const size_t head = align_up(8 * (size_t)kGoodputSpanInts + 16 * (nn + 1), 256);
   if ((rc = m->gp.ensure(head + rows * goodput_row_bytes(m->d), "goodput tables"))) return rc;
   int* span = static_cast<int*>(m->gp.p);
   long long* base = reinterpret_cast<long long*>(span + 2 * kGoodputSpanInts);
-  uint64_t* sums = static_cast<uint64_t*>(m->sums.p);
-  Set set = m->set;
+  uint64_t* sums = sums_half(m, 0);
+  float* tables = tables_half(m, 0);
   set.gp_span = span;
   FS_CUDA(launch_thresh(set, m->lc.floors, m->th_bound, s), "launch thresholds");
-  FS_CUDA(launch_prep(set, it, pl, static_cast<float*>(m->tables.p), sums, true, m->sm_count, m->lc, s, m->th_bound),
+  FS_CUDA(launch_prep(set, it, pl, tables, sums, 1, m->sm_count, m->lc, s, m->th_bound),
           "launch prep");
-  FS_CUDA(launch_score_goodput(set, it, pl, static_cast<const float*>(m->tables.p), sums, span, base,
+  FS_CUDA(launch_score_goodput(set, it, pl, tables, sums, span, base,
                                static_cast<char*>(m->gp.p) + head, rows, m->lc.floors, m->th_bound, m->sm_count, s),
           "launch goodput scorer");
   FS_CUDA(launch_finalize_goodput(set, it, pl, sums, base, lam_sum, d_gap, d_score, d_gamma, d_best, d_st,
@@ -1007,7 +1031,7 @@ int fs_replay(fs_model* m, const fs_replay_spec* sp, int32_t* rounds, int32_t* s
         continue;
       }
       const int n_items = n_active * per;
-      int rc2 = ensure_items(m, n_items, sp->O);
+      int rc2 = ensure_items(m, m->d, n_items, sp->O);
       if (rc2) return rc2;
       Items it{};
       it.n = n_items;
@@ -1015,14 +1039,14 @@ int fs_replay(fs_model* m, const fs_replay_spec* sp, int32_t* rounds, int32_t* s
       it.cell = rs.item_cell;
       it.off = nullptr;
       fs_samples smp{sp->seed, 0, (uint32_t)r, n_items, sp->O, sp->S, 0, nullptr};
-      Plan pl = make_plan(m, &smp, n_items);
+      Plan pl = make_plan(m->d, &smp);
       pl.few = few_path(pl, n_items) ? 1 : 0;
-      FS_CUDA(launch_prep(set, it, pl, (float*)m->tables.p, (uint64_t*)m->sums.p, false, m->sm_count, m->lc, s),
+      FS_CUDA(launch_prep(set, it, pl, tables_half(m, 0), sums_half(m, 0), 0, m->sm_count, m->lc, s),
               "launch prep");
-      FS_CUDA(launch_score(set, it, pl, (const float*)m->tables.p, (uint64_t*)m->sums.p, nullptr, 0, m->sm_count,
+      FS_CUDA(launch_score(set, it, pl, tables_half(m, 0), sums_half(m, 0), nullptr, 0, m->sm_count,
                            m->lc, s),
               "launch score");
-      FS_CUDA(launch_replay_reveal(set, rs, it, pl, (const uint64_t*)m->sums.p, n_active, s), "launch reveal");
+      FS_CUDA(launch_replay_reveal(set, rs, it, pl, sums_half(m, 0), n_active, s), "launch reveal");
     }
     if (rounds) FS_CUDA(cudaMemcpyAsync(rounds, rs.rounds, 4 * (size_t)P, cudaMemcpyDeviceToHost, s), "read rounds");
     if (state) FS_CUDA(cudaMemcpyAsync(state, rs.state, 4 * (size_t)P, cudaMemcpyDeviceToHost, s), "read state");
@@ -1054,6 +1078,7 @@ int fs_check(fs_model* m, void* cuda_stream) {
 // The work counts (work[2..3]) of the model, zeroed in stream order.
 static int zero_entry_count(fs_model* m) {
   FS_CUDA(cudaMemsetAsync(m->set.work + 2, 0, 16, m->stream), "zero the entry count");
+  FS_CUDA(cudaMemsetAsync(m->set.work + 6, 0, 16, m->stream), "zero the entry count");
   FS_CUDA(cudaStreamSynchronize(m->stream), "zero the entry count");
   return FS_OK;
 }
@@ -1070,7 +1095,9 @@ int fs_timing_read(fs_model* m, double* kernel_ms, int32_t* launches, double* ph
   if (!m) return fail(FS_EINVAL, "model is NULL");
   if (work_counts) {
     FS_CUDA(cudaDeviceSynchronize(), "wait for the scoring calls");
-    FS_CUDA(cudaMemcpy(work_counts, m->set.work + 2, 16, cudaMemcpyDeviceToHost), "read the work counts");
+    uint64_t w[8];
+    FS_CUDA(cudaMemcpy(w, m->set.work, sizeof w, cudaMemcpyDeviceToHost), "read the work counts");
+    for (int q = 0; q < 2; ++q) work_counts[q] = w[2 + q] + w[6 + q];
     int rc = zero_entry_count(m);
     if (rc) return rc;
   }
@@ -1135,10 +1162,8 @@ void fs_free_model(fs_model* m) {
   if (m->stream) cudaStreamSynchronize(m->stream);
   else cudaDeviceSynchronize();
   m->fixed.release();
-  m->cand.release();
   m->tables.release();
   m->sums.release();
-  m->outs.release();
   m->real.release();
   m->lex.release();
   m->gp.release();

@@ -12,7 +12,7 @@
 //   base     [P][2]        fs_allocation
 //   rtab     [P][2][rt_cap] u16  row tables (k_thresh), word (row rho, threshold k) at k K4 + rho
 //   tpart    [2][n_tpart]  f32   scoring calls: each k_thresh block's largest feasible threshold
-//   work     [4]           u64   chunk counter of the Monte-Carlo kernel, the reduction's ticket,
+//   work     [4]           u64   (two sets, alternate calls) chunk counter of the Monte-Carlo kernel, the reduction's ticket,
 //                                 table entries evaluated and scenarios that tested their tail
 //                                 gate (both accumulate across calls; the host zeroes them)
 // Per scoring call (items = (problem, candidate cell) pairs), one record of
@@ -510,8 +510,10 @@ cudaError_t launch_solve(const Set& set, int n, const float* cap_x, const float*
 // count (theta_cap otherwise). With set.tpart (one problem) the launch's block
 // count is left in set.n_tpart, and the parts hold t*.
 cudaError_t launch_thresh(Set& set, int floors, int th_bound, cudaStream_t s, bool late = false);
-// early: the candidate ids and bounds were complete before the preceding
-// kernel started, so the bounds-only work may run before the PDL wait.
+// early: 0 nothing before the wait for the preceding kernel; 1 the candidate ids
+// and bounds were complete before that kernel let this one start, so the
+// bounds-only work runs before the wait; 2 the bounds were, the ids are read again
+// after it (k_thresh's late form).
 // Blocks of 256 threads, or of 64 when the launch holds more than two waves
 // of 256-thread blocks (sm_count SMs): each block is mostly a chain of
 // dependent latencies, so more of them in flight per SM finish sooner.
@@ -519,7 +521,7 @@ cudaError_t launch_thresh(Set& set, int floors, int th_bound, cudaStream_t s, bo
 // theta_cap) guarantees row tables, no shared memory is set aside for the
 // search without one (a count above it is reported as ST_TABLE).
 cudaError_t launch_prep(const Set& set, const Items& it, const Plan& pl, float* tables,
-                        uint64_t* sums, bool early, int sm_count, LaunchCache& lc, cudaStream_t s,
+                        uint64_t* sums, int early, int sm_count, LaunchCache& lc, cudaStream_t s,
                         int th_bound = 0);
 // Whether a launch takes k_score_few (the plan's `few`, set before launch_prep).
 bool few_path(const Plan& pl, int n_items);

@@ -172,7 +172,7 @@ __global__ void __launch_bounds__(kPrepThreads) k_prep(Set set, Items it, Plan p
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nwarp = blockDim.x >> 5;
   if (!early) pdl_wait();
   const int p = it.p ? it.p[item] : 0;
-  const int cell = it.cell[item];
+  int cell = it.cell[item];
   float* base_rec = rec + (size_t)item * pl.item_floats;
   float* tab = base_rec + (size_t)sigma * d.slot_floats;
   if (blockIdx.x == 0 && tid == 0) {
@@ -191,13 +191,29 @@ __global__ void __launch_bounds__(kPrepThreads) k_prep(Set set, Items it, Plan p
       tab[H_CELL] = __int_as_float(-1);
     }
   };
+  int rr = 0, ie = 0, jr = 0;
+  float lam = 1.0f, L = 0.0f, rl = 1.0f, dle = 0.0f, lo_c, hi_c, lo_l, hi_l;
+  // The part that reads only the bounds: once, or again when the candidate list
+  // turns out to have changed (read before the wait, it may have belonged to a
+  // kernel of the caller's that lets its dependents start before it has finished).
+  for (bool waited = !early;; waited = true) {
   if (cell < 0 || cell >= d.cells) {  // device-side candidate ids are checked here
+    if (!waited) pdl_wait();
+    if (!waited && early == 2) {
+      cell = __ldcg(it.cell + item);
+      if (cell >= 0 && cell < d.cells) continue;
+    }
     reject(ST_CELL);
     return;
   }
-  const int rr = cell / d.B, be = cell - rr * d.B, ie = rr >> 2, jr = rr & 3;
-  const float lam = set.lam[ie], L = set.slo[ie], rl = __frcp_rn(lam);
-  const float dle = FL ? set.slo[d.K + ie] : 0.0f;
+  rr = cell / d.B;
+  ie = rr >> 2;
+  jr = rr & 3;
+  const int be = cell - rr * d.B;
+  lam = set.lam[ie];
+  L = set.slo[ie];
+  rl = __frcp_rn(lam);
+  dle = FL ? set.slo[d.K + ie] : 0.0f;
   if (tid < d.K) {
     sLam[tid] = set.lam[tid];
     sRl[tid] = __frcp_rn(set.lam[tid]);
@@ -206,8 +222,10 @@ __global__ void __launch_bounds__(kPrepThreads) k_prep(Set set, Items it, Plan p
   const float* bp = set.bounds + (size_t)p * 4 * d.cells;
   const float* capS = bp + (size_t)(sigma ? CAP_HI : CAP_LO) * d.cells;
   const float* tailS = bp + (size_t)(sigma ? TAIL_LO : TAIL_HI) * d.cells;
-  const float lo_c = bp[(size_t)CAP_LO * d.cells + cell], hi_c = bp[(size_t)CAP_HI * d.cells + cell];
-  const float lo_l = bp[(size_t)TAIL_LO * d.cells + cell], hi_l = bp[(size_t)TAIL_HI * d.cells + cell];
+  lo_c = bp[(size_t)CAP_LO * d.cells + cell];
+  hi_c = bp[(size_t)CAP_HI * d.cells + cell];
+  lo_l = bp[(size_t)TAIL_LO * d.cells + cell];
+  hi_l = bp[(size_t)TAIL_HI * d.cells + cell];
 
   // best SLO-feasible capacity of row r without bin b_e (ties: lower bin)
   if (RF) {
@@ -349,7 +367,14 @@ __global__ void __launch_bounds__(kPrepThreads) k_prep(Set set, Items it, Plan p
       }
     }
   }
-  if (early) pdl_wait();  // thresholds and rows come from k_thresh
+  if (waited) break;
+  pdl_wait();  // thresholds and rows come from k_thresh
+  if (early != 2) break;
+  const int again = __ldcg(it.cell + item);
+  if (again == cell) break;
+  cell = again;  // (the same for the whole block)
+  __syncthreads();
+  }
 
   const size_t ps = (size_t)p * 2 + sigma;
   const float* th_g = set.theta + ps * d.theta_cap;
@@ -1321,7 +1346,7 @@ __global__ void k_finalize_split(Set set, Items it, Plan pl, const uint64_t* sum
 }
 
 cudaError_t launch_prep(const Set& set, const Items& it, const Plan& pl, float* tables, uint64_t* sums,
-                        bool early, int sm_count, LaunchCache& lc, cudaStream_t s, int th_bound) {
+                        int early, int sm_count, LaunchCache& lc, cudaStream_t s, int th_bound) {
   if (it.n <= 0) return cudaSuccess;
   const Dims& d = set.d;
   const int bound = th_bound > 0 ? std::min(th_bound, d.theta_cap) : d.theta_cap;
@@ -1340,7 +1365,7 @@ cudaError_t launch_prep(const Set& set, const Items& it, const Plan& pl, float* 
     if (e != cudaSuccess) return e;
     lc.prep_smem[mode] = smem;
   }
-  return launch_pdl(kern, dim3(it.n * 2), dim3(tb), smem, s, set, it, pl, tables, sums, early ? 1 : 0, sure ? 1 : 0);
+  return launch_pdl(kern, dim3(it.n * 2), dim3(tb), smem, s, set, it, pl, tables, sums, early, sure ? 1 : 0);
 }
 
 static bool table_path(const Plan& pl) {

@@ -49,12 +49,9 @@ __global__ void __launch_bounds__(kThreshThreads) k_thresh(Set set, int late) {
   // `late`: what is read here was complete before this kernel could start, and
   // nothing that may still run reads what is written here (launch_thresh), so the
   // wait for the previous kernel comes after the work: the last call's scenarios
-  // and this call's thresholds overlap. Only then may the preparation start, whose
-  // records those scenarios still read.
-  if (!late) {
-    pdl_wait();
-    pdl_trigger();
-  }
+  // overlap this call's thresholds and the part of the preparation before its wait.
+  if (!late) pdl_wait();
+  pdl_trigger();
   if (set.skip && set.skip[p] >= 0) return;
   const float* bp = set.bounds + (size_t)p * 4 * d.cells;
   const float* cap = bp + (size_t)(sigma ? CAP_HI : CAP_LO) * d.cells;
@@ -191,10 +188,7 @@ __global__ void __launch_bounds__(kThreshThreads) k_thresh(Set set, int late) {
     __syncthreads();
     if (tid == 0) set.tpart[sigma * gridDim.x + blockIdx.x] = __uint_as_float(s_best);
   }
-  if (late) {
-    pdl_wait();
-    pdl_trigger();
-  }
+  if (late) pdl_wait();
 }
 
 // Measured (one GB300, calls in a row): the eight-class, 256-GPU grid (about 1300
@@ -202,13 +196,20 @@ __global__ void __launch_bounds__(kThreshThreads) k_thresh(Set set, int late) {
 // the preparation of 1024 candidates 60.6 -> 14 us: 1024 x 16 x 16384 scenarios
 // 270 -> 206 us, 1024 x 8 x 60 116 -> 51 us; four classes, 64 GPUs 51 -> 45 us.
 //
-// late: for a scoring call on the model's own device bounds. They are only
-// written by copies (a full barrier in the stream). The thresholds, rows and
-// tables were last read by the previous call's preparation, which had finished
-// before its Monte-Carlo kernel let the reduction, and that let this kernel,
-// start; only a dump's scenarios and the goodput stage read rows later (not
-// late after the former; the latter is synchronous). The parts of t*, which the
-// previous reduction may still read, alternate between two halves.
+// late: for a scoring call n on the model's own device bounds, of at least one
+// candidate, after another on its stream. What may still run when it starts is
+// call n - 1's scenarios and reduction: that reduction let this kernel start, and
+// was itself let start by the scenarios, after call n - 1's preparation and so
+// (each waits for its predecessor) its thresholds had finished, which had waited
+// for call n - 2's reduction. So
+//   - the bounds are only written by copies (a full barrier in the stream);
+//   - thresholds, rows and tables have no reader left: the preparation of call n -
+//     1 was the last (a dump's scenarios read rows: not late after one; the goodput
+//     stage and the replay are synchronous);
+//   - the parts of t*, the records, the sums and the counters, which call n - 1
+//     still uses, alternate between two sets, call n - 2's being free.
+// A call without candidates has no preparation and scenarios to hand that on: it
+// waits first.
 cudaError_t launch_thresh(Set& set, int floors, int th_bound, cudaStream_t s, bool late) {
   const Dims& d = set.d;
   const int bound = th_bound > 0 ? std::min(th_bound, d.theta_cap) : d.theta_cap;
