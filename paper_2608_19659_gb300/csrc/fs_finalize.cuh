@@ -84,15 +84,6 @@ __device__ __forceinline__ float base_tstar(const Set& set, int p, int sigma) {
   return __uint_as_float(__reduce_max_sync(0xffffffffu, v));
 }
 
-// The caller's copy of the sums of items [beg, end) (nullable), coalesced over the
-// block: the reduction reads them anyway, so no copy follows the call's last kernel.
-__device__ __forceinline__ void copy_sums(const Plan& pl, const uint64_t* sums, uint64_t* out, int beg, int end) {
-  if (!out) return;
-  const size_t b = (size_t)beg * pl.O, e = (size_t)end * pl.O;
-#pragma unroll 4
-  for (size_t x = b + threadIdx.x; x < e; x += blockDim.x) out[x] = __ldg(sums + x);
-}
-
 // Items [beg, end) of problem p, whose first item is pos0 (candidate positions,
 // for the order of equal scores, count from there).
 // LPC: lanes per candidate, 1 (a block takes up to 256 candidates at once) or 4
@@ -101,32 +92,41 @@ __device__ __forceinline__ void copy_sums(const Plan& pl, const uint64_t* sums, 
 template <int LPC = 1>
 __device__ inline Best finalize_problem(const Set& set, const Items& it, const Plan& pl, const uint64_t* sums,
                                  int p, int beg, int end, double* gap, double* score, float* gt_out,
-                                 int pos0) {
+                                 int pos0, uint64_t* sum_out = nullptr) {
   __shared__ Best sb[32];
   const Dims& d = set.d;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nwarp = blockDim.x >> 5;
   // inputs are read-only here (written by earlier kernels): every load goes
-  // through the read-only path and is issued before any store
-  const float gt = __fsub_rn(base_tstar(set, p, 1), base_tstar(set, p, 0));
-  const long long gfix = (long long)fixed40(gt);
+  // through the read-only path, the first candidate's before t* is needed
   const long long n = (long long)pl.O * pl.S;
   const int log2n = (n & (n - 1)) == 0 ? 63 - __clzll(n) : -1;
-  Best b = no_best();
-  // LPC lanes per candidate: each sums every LPC-th outcome, shuffles add them up,
-  // and the lanes share the outputs' conversions
+  // LPC lanes per candidate: each sums every LPC-th outcome (and leaves it in the
+  // caller's copy), shuffles add them up, and the lanes share the conversions
   const int sub = tid % LPC, per = (int)blockDim.x / LPC;
-  for (int q0 = beg; q0 < end; q0 += per) {
-    const int q = q0 + tid / LPC;
-    const bool in = q < end;
+  int cell = 0;
+  auto total = [&](int q) {
     long long tot = 0;
-    int cell = 0;
-    if (in) {
+    if (q < end) {
       cell = __ldg(it.cell + q);
 #pragma unroll 8
-      for (int o = sub; o < pl.O; o += LPC) tot += (long long)__ldg(sums + (size_t)q * pl.O + o);
+      for (int o = sub; o < pl.O; o += LPC) {
+        const size_t x = (size_t)q * pl.O + o;
+        const uint64_t v = __ldg(sums + x);
+        tot += (long long)v;
+        if (sum_out) sum_out[x] = v;
+      }
     }
     for (int o = 1; o < LPC; o <<= 1) tot += __shfl_xor_sync(0xffffffffu, tot, o);
-    if (!in) continue;
+    return tot;
+  };
+  long long tot = total(beg + tid / LPC);
+  const float gt = __fsub_rn(base_tstar(set, p, 1), base_tstar(set, p, 0));
+  const long long gfix = (long long)fixed40(gt);
+  Best b = no_best();
+  for (int q0 = beg; q0 < end; q0 += per) {
+    const int q = q0 + tid / LPC;
+    if (q0 > beg) tot = total(q);
+    if (q >= end) continue;
     const long long sc = gfix * n - tot;
     if (sub == 0 && gap) gap[q] = fixed_mean((unsigned long long)tot, n, log2n);
     if (sub == LPC / 2 && score) score[q] = fixed_mean((unsigned long long)sc, n, log2n);

@@ -855,7 +855,6 @@ __global__ void k_finalize_goodput(Set set, Items it, Plan pl, const uint64_t* s
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nwarp = blockDim.x >> 5;
   const int nb = (int)gridDim.x, per = (it.n + nb - 1) / nb;
   const int beg = min(it.n, (int)blockIdx.x * per), end = min(it.n, beg + per);
-  copy_sums(pl, sums, sum_out, beg, end);
   const long long gm = base[0], gpl = base[1];
   const long long gfix = gpl > gm ? gpl - gm : gm - gpl;
   const long long n = (long long)pl.O * pl.S;
@@ -878,7 +877,12 @@ __global__ void k_finalize_goodput(Set set, Items it, Plan pl, const uint64_t* s
     if (in) {
       cell = __ldg(it.cell + q);
 #pragma unroll 8
-      for (int o = sub; o < pl.O; o += lpc) tot += (long long)__ldg(sums + (size_t)q * pl.O + o);
+      for (int o = sub; o < pl.O; o += lpc) {
+        const size_t x = (size_t)q * pl.O + o;
+        const uint64_t v = __ldg(sums + x);
+        tot += (long long)v;
+        if (sum_out) sum_out[x] = v;  // (the caller's copy)
+      }
     }
     for (int o = 1; o < lpc; o <<= 1) tot += __shfl_xor_sync(0xffffffffu, tot, o);
     if (!in) continue;

@@ -1301,8 +1301,8 @@ __global__ void k_finalize(Set set, Items it, Plan pl, const uint64_t* sums, dou
   const int p = blockIdx.x;
   const int beg = it.off ? it.off[p] : 0;
   const int end = it.off ? it.off[p + 1] : it.n;
-  copy_sums(pl, sums, sum_out, beg, end);
-  const Best b = finalize_problem(set, it, pl, sums, p, beg, end, gap, score, gamma_t ? gamma_t + p : nullptr, beg);
+  const Best b = finalize_problem(set, it, pl, sums, p, beg, end, gap, score, gamma_t ? gamma_t + p : nullptr, beg,
+                                  sum_out);
   if (threadIdx.x == 0 && best) best[p] = b.valid() ? b.cell : -1;
   // every kernel of the call has finished (stream order, and the wait above):
   // its status word can travel with the outputs
@@ -1319,9 +1319,8 @@ __global__ void k_finalize_split(Set set, Items it, Plan pl, const uint64_t* sum
   pdl_wait();
   const int nb = (int)gridDim.x, per = (it.n + nb - 1) / nb;
   const int beg = min(it.n, (int)blockIdx.x * per), end = min(it.n, beg + per);
-  copy_sums(pl, sums, sum_out, beg, end);
   const Best b = finalize_problem<4>(set, it, pl, sums, 0, beg, end, gap, score,
-                                     blockIdx.x == 0 ? gamma_t : nullptr, 0);
+                                     blockIdx.x == 0 ? gamma_t : nullptr, 0, sum_out);
   __shared__ int s_last;
   if (threadIdx.x == 0) {
     part[2 * blockIdx.x] = (uint64_t)b.hi;

@@ -73,16 +73,11 @@ __global__ void __launch_bounds__(kThreshThreads) k_thresh(Set set, int late) {
     const float C = sC[rho], lam = sLam[i], rl = sRl[i], Mf = rep_capf(d, j);
     int n0 = 0, len = 0;
     if (sB[rho] >= 0 && M >= 1) {
-      // (one copy of the code, run twice: this kernel's first pass is latency-bound)
-      int n[2];
-#pragma unroll 1
-      for (int q = 0; q < 2; ++q) {
-        const float lo_f = FL ? fmaxf(sDl[i], __int_as_float(1)) : __int_as_float(1);
-        const int v = min_replicas(q ? 1.0f : lo_f, C, lam, rl, Mf);
-        if (q) n[1] = v; else n[0] = v;
-      }
-      n0 = n[0];
-      if (n0) len = n[1] ? n[1] : M;
+      // (no floor, and every fulfilment positive: the first is that of one replica)
+      const float lo_f = FL ? fmaxf(sDl[i], __int_as_float(1)) : __int_as_float(1);
+      n0 = C > 0.0f && row_in_range(C, lam) && !(FL && sDl[i] > 0.0f) ? 1 : min_replicas(lo_f, C, lam, rl, Mf);
+      const int ns = min_replicas(1.0f, C, lam, rl, Mf);
+      if (n0) len = ns ? ns : M;
     }
     sN0[rho] = n0;
     sOff[rho + 1] = n0 ? len - n0 + 1 : 0;
