@@ -158,7 +158,7 @@ __device__ __forceinline__ float tstar_of(float C, const float* kap, const float
 // they overlap the base solve that precedes this kernel. FL: some class is
 // critical (the model has floors).
 template <bool FL, bool RF>
-__global__ void __launch_bounds__(kPrepThreads) k_prep(Set set, Items it, Plan pl, float* rec,
+__global__ void __launch_bounds__(kPrepThreads, 5) k_prep(Set set, Items it, Plan pl, float* rec,
                                                        uint64_t* sums, int early, int sure) {
   extern __shared__ __align__(16) unsigned char smraw[];
   float* sTh = reinterpret_cast<float*>(smraw);  // [theta_cap], unless a table beyond a thread each is sure
