@@ -222,8 +222,8 @@ int fs_score_candidates_async(fs_model *m, const fs_samples *samples, double *ga
  *   4 Q (only with quantile_dev NULL: the built-in table);
  *   8 T and 8, with T = K (floor(G/1) + floor(G/2) + floor(G/4) + floor(G/8))
  *     (thresholds and their counts);
- *   32 K twice (best capacity and bin per (class, TP) row), 1216 (the two
- *     base allocations), 65536 (their row tables);
+ *   32 K twice (best capacity and bin per (class, TP) row), 1216 (t* of the
+ *     two realisations), 65536 (their row tables);
  *   4 n I with n = max(n_cand, 1), I = 2 (20 + 3 P) + O (4 + 4 ceil(W / 4)),
  *     P the smallest power of two >= max(T + 1, 4), W = Q / O (the
  *     candidates' threshold tables and mapped quantile windows);

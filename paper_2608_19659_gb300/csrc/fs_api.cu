@@ -176,6 +176,7 @@ struct fs_model {
   LaunchCache lc;
   int half = 0;             // the set of what alternates that the last scoring call used
   bool rows_read = false;   // the last scoring call's scenarios read the rows (dump)
+  bool whole = false;       // its records took the whole buffer
   // optional timing events: 5 per timed call (before solve, prep, score,
   // finalize, and after finalize); mode 1 records only the two around score
   int timing = 0;
@@ -372,23 +373,34 @@ Dims call_dims(const fs_model* m, int th_bound) {
   return d;
 }
 
-// Halves of the records and sums (their place depends on the buffers' size alone,
-// so that calls of different sizes never share a byte; a buffer that grows is
-// freed, which waits for the calls in flight).
-float* tables_half(const fs_model* m, int half) {
-  return reinterpret_cast<float*>(static_cast<char*>(m->tables.p) + half * (m->tables.bytes / 2));
-}
-uint64_t* sums_half(const fs_model* m, int half) {
-  return reinterpret_cast<uint64_t*>(static_cast<char*>(m->sums.p) + half * (m->sums.bytes / 2));
+// Buffers of a call's records and sums, sized by the model and the plan alone, so
+// that new bounds never make a later call allocate. The sums have two halves; the
+// records have two where both, with tables for every threshold the model allows,
+// take at most kTwoRecords (a larger call's two halves may still hold its
+// records, whose tables only need the bounds' thresholds). A half's place depends
+// on the buffer's size alone: calls of different sizes never share a byte of
+// different halves, and a buffer that grows is freed, which waits for the calls in
+// flight.
+constexpr size_t kTwoRecords = 64u << 20;
+
+size_t record_bytes(const Dims& d, int n, int O) {
+  const int W = d.Q / O, Wp = 4 + ((W + 3) & ~3);
+  return align_up((size_t)std::max(n, 1) * (2 * (size_t)d.slot_floats + (size_t)O * Wp) * 4, 256);
 }
 
-int ensure_items(fs_model* m, const Dims& d, int n, int O) {
-  int rc;
-  const int W = d.Q / O, Wp = 4 + ((W + 3) & ~3);
-  const size_t item_floats = 2 * (size_t)d.slot_floats + (size_t)O * Wp;
-  if ((rc = m->tables.ensure(2 * align_up((size_t)std::max(n, 1) * item_floats * 4, 256), "candidate records"))) return rc;
+int ensure_items(fs_model* m, int n, int O) {
+  const size_t full = record_bytes(m->d, n, O);
+  int rc = m->tables.ensure(2 * full <= kTwoRecords ? 2 * full : full, "candidate records");
+  if (rc) return rc;
   // sums, then the split reduction's scratch (2 words per block)
   return m->sums.ensure(2 * align_up((size_t)std::max(n, 1) * O * 8 + 16 * (size_t)kFinalizeMaxBlocks, 256), "sums");
+}
+
+float* tables_at(const fs_model* m, int half) {
+  return reinterpret_cast<float*>(static_cast<char*>(m->tables.p) + half * (m->tables.bytes / 512 * 256));
+}
+uint64_t* sums_half(const fs_model* m, int half) {
+  return reinterpret_cast<uint64_t*>(static_cast<char*>(m->sums.p) + half * (m->sums.bytes / 512 * 256));
 }
 
 // The scoring sequence on stream s; cand_dev holds n_cand cell ids.
@@ -401,16 +413,20 @@ int run_score(fs_model* m, Set set, const fs_samples* smp, const int32_t* cand_d
   it.p = nullptr;
   it.cell = cand_dev;
   it.off = nullptr;
-  // this call's set of what alternates: the other one in an asynchronous call,
-  // which may start before the last call has finished, the same in a synchronous
-  // one, which waits for it
+  // What alternates between calls (launch_thresh): the other half in an
+  // asynchronous call, which may start before the last call has finished, the
+  // same in a synchronous one, which waits for it. Records too large for a half
+  // take the whole buffer.
   if (m->th_bound < 0) m->th_bound = threshold_bound(m);
   set.d = call_dims(m, m->th_bound);
+  int rc = ensure_items(m, n, smp->O);
+  if (rc) return rc;
   if (late) m->half ^= 1;
   const int half = m->half;
-  int rc = ensure_items(m, set.d, n, smp->O);
-  if (rc) return rc;
-  float* tables = tables_half(m, half);
+  const bool whole = record_bytes(set.d, n, smp->O) > m->tables.bytes / 512 * 256;
+  const int mode = !late || n == 0 || m->rows_read ? 0 : whole || m->whole ? 1 : 2;
+  m->whole = whole;
+  float* tables = tables_at(m, whole ? 0 : half);
   uint64_t* sums = sums_half(m, half);
   set.tpart += half * 2 * kThreshBlocks;
   set.work += 4 * half;
@@ -429,10 +445,10 @@ int run_score(fs_model* m, Set set, const fs_samples* smp, const int32_t* cand_d
   }
   const bool phases = timed && m->timing == 2;
   if (phases) FS_CUDA(cudaEventRecord(ev[0], s), "record timing event");
-  FS_CUDA(launch_thresh(set, m->lc.floors, m->th_bound, s, late && n > 0 && !m->rows_read), "launch thresholds");
+  FS_CUDA(launch_thresh(set, m->lc.floors, m->th_bound, s, mode), "launch thresholds");
   m->rows_read = dump != nullptr;
   if (phases) FS_CUDA(cudaEventRecord(ev[1], s), "record timing event");
-  FS_CUDA(launch_prep(set, it, pl, tables, sums, late ? 2 : 1, m->sm_count, m->lc, s, m->th_bound), "launch prep");
+  FS_CUDA(launch_prep(set, it, pl, tables, sums, mode == 2 ? 2 : 1, m->sm_count, m->lc, s, m->th_bound), "launch prep");
   if (timed) FS_CUDA(cudaEventRecord(ev[2], s), "record timing event");
   FS_CUDA(launch_score(set, it, pl, tables, sums, dump, fs_dump_stride(m), m->sm_count, m->lc, s), "launch score");
   if (timed) FS_CUDA(cudaEventRecord(ev[3], s), "record timing event");
@@ -851,7 +867,7 @@ int fs_score_goodput(fs_model* m, const fs_samples* smp, double* gap_out, double
   if (m->th_bound < 0) m->th_bound = threshold_bound(m);
   Set set = m->set;
   set.d = call_dims(m, m->th_bound);
-  if ((rc = ensure_items(m, set.d, n, smp->O))) return rc;
+  if ((rc = ensure_items(m, n, smp->O))) return rc;
   cudaStream_t s = m->stream;
   if ((rc = flush_bounds(m, s))) return rc;
   // as in fs_score_candidates, one mapped page-locked block carries the
@@ -882,7 +898,7 @@ int fs_score_goodput(fs_model* m, const fs_samples* smp, double* gap_out, double
   int* span = static_cast<int*>(m->gp.p);
   long long* base = reinterpret_cast<long long*>(span + 2 * kGoodputSpanInts);
   uint64_t* sums = sums_half(m, 0);
-  float* tables = tables_half(m, 0);
+  float* tables = tables_at(m, 0);
   set.gp_span = span;
   FS_CUDA(launch_thresh(set, m->lc.floors, m->th_bound, s), "launch thresholds");
   FS_CUDA(launch_prep(set, it, pl, tables, sums, 1, m->sm_count, m->lc, s, m->th_bound),
@@ -1031,7 +1047,7 @@ int fs_replay(fs_model* m, const fs_replay_spec* sp, int32_t* rounds, int32_t* s
         continue;
       }
       const int n_items = n_active * per;
-      int rc2 = ensure_items(m, m->d, n_items, sp->O);
+      int rc2 = ensure_items(m, n_items, sp->O);
       if (rc2) return rc2;
       Items it{};
       it.n = n_items;
@@ -1041,9 +1057,9 @@ int fs_replay(fs_model* m, const fs_replay_spec* sp, int32_t* rounds, int32_t* s
       fs_samples smp{sp->seed, 0, (uint32_t)r, n_items, sp->O, sp->S, 0, nullptr};
       Plan pl = make_plan(m->d, &smp);
       pl.few = few_path(pl, n_items) ? 1 : 0;
-      FS_CUDA(launch_prep(set, it, pl, tables_half(m, 0), sums_half(m, 0), 0, m->sm_count, m->lc, s),
+      FS_CUDA(launch_prep(set, it, pl, tables_at(m, 0), sums_half(m, 0), 0, m->sm_count, m->lc, s),
               "launch prep");
-      FS_CUDA(launch_score(set, it, pl, tables_half(m, 0), sums_half(m, 0), nullptr, 0, m->sm_count,
+      FS_CUDA(launch_score(set, it, pl, tables_at(m, 0), sums_half(m, 0), nullptr, 0, m->sm_count,
                            m->lc, s),
               "launch score");
       FS_CUDA(launch_replay_reveal(set, rs, it, pl, sums_half(m, 0), n_active, s), "launch reveal");

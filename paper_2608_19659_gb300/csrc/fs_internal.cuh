@@ -509,11 +509,11 @@ cudaError_t launch_solve(const Set& set, int n, const float* cap_x, const float*
 // problem of the set. th_bound > 0: a bound on either realisation's threshold
 // count (theta_cap otherwise). With set.tpart (one problem) the launch's block
 // count is left in set.n_tpart, and the parts hold t*.
-cudaError_t launch_thresh(Set& set, int floors, int th_bound, cudaStream_t s, bool late = false);
+cudaError_t launch_thresh(Set& set, int floors, int th_bound, cudaStream_t s, int late = 0);
 // early: 0 nothing before the wait for the preceding kernel; 1 the candidate ids
 // and bounds were complete before that kernel let this one start, so the
 // bounds-only work runs before the wait; 2 the bounds were, the ids are read again
-// after it (k_thresh's late form).
+// after it (k_thresh's late form 2).
 // Blocks of 256 threads, or of 64 when the launch holds more than two waves
 // of 256-thread blocks (sm_count SMs): each block is mostly a chain of
 // dependent latencies, so more of them in flight per SM finish sooner.

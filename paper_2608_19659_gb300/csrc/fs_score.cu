@@ -155,7 +155,7 @@ __device__ __forceinline__ float tstar_of(float C, const float* kap, const float
 // One CTA per (candidate, realisation sigma). Before the threshold search it
 // maps the quantile strata of the outcomes o = sigma, sigma + 2, ... into the
 // candidate's record: this and Cexcl read only the bounds, so with `early`
-// they overlap the base solve that precedes this kernel. FL: some class is
+// they overlap k_thresh, which precedes this kernel. FL: some class is
 // critical (the model has floors).
 template <bool FL, bool RF>
 __global__ void __launch_bounds__(kPrepThreads, 5) k_prep(Set set, Items it, Plan pl, float* rec,
@@ -487,7 +487,7 @@ __global__ void __launch_bounds__(kPrepThreads, 5) k_prep(Set set, Items it, Pla
     b0 = lo0;
     b1 = lo1;
   }
-  const int Lt = b1 - b0;
+  const int Lt = max(0, b1 - b0);  // (b1 >= b0 for checked inputs; the allocation-free path's are not)
   // Three arrays of Lpad = max(P, 4) entries, P = pow2 >= Lt + 1 (at least 4
   // for 16-byte copies): kappa[u] for u < Lt, +inf beyond, so the scenario
   // search needs no bound checks; thx[pos] = the threshold reached with pos
@@ -615,8 +615,8 @@ __global__ void __launch_bounds__(kPrepThreads, 5) k_prep(Set set, Items it, Pla
     tab[H_RLAM] = rl;
     tab[H_DLT] = dle;
   }
-  // k_score launches only now: its blocks, resident early, slowed the base
-  // solve and this kernel more than their early start saved
+  // k_score launches only now: its blocks, resident early, slowed the kernels
+  // before it more than their early start saved
   pdl_trigger();
 }
 

@@ -116,7 +116,7 @@ extern "C" int fs_score_candidates_noalloc(int32_t K, int32_t B, int32_t G, cons
   const size_t o_theta = take(8 * (size_t)d.theta_cap), o_nth = take(8);
   const size_t o_rowc = take(8 * (size_t)d.K4), o_rowb = take(8 * (size_t)d.K4);
   const size_t o_base = take(2 * sizeof(fs_allocation));
-  const size_t o_rtab = take(4 * (size_t)kRowTabMax);  // row tables of the two base solves
+  const size_t o_rtab = take(4 * (size_t)kRowTabMax);  // row tables of the two realisations
   const int Wq = Q / smp->O, Wp = 4 + ((Wq + 3) & ~3);
   const size_t item_floats = 2 * (size_t)d.slot_floats + (size_t)smp->O * Wp;
   const size_t o_tab = take((size_t)std::max(n, 1) * item_floats * 4);

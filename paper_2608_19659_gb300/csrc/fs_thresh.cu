@@ -46,12 +46,13 @@ __global__ void __launch_bounds__(kThreshThreads) k_thresh(Set set, int late) {
   __shared__ float sLam[FS_MAX_CLASSES], sRl[FS_MAX_CLASSES], sDl[FS_MAX_CLASSES];
   __shared__ int sCover[kWarps][256];  // covers of one threshold (more than 32 rows)
   __shared__ uint32_t s_best;
-  // `late`: what is read here was complete before this kernel could start, and
+  // late 1, 2: what is read here was complete before this kernel could start, and
   // nothing that may still run reads what is written here (launch_thresh), so the
   // wait for the previous kernel comes after the work: the last call's scenarios
-  // overlap this call's thresholds and the part of the preparation before its wait.
-  if (!late) pdl_wait();
-  pdl_trigger();
+  // overlap this call's thresholds and (2) the part of the preparation before its
+  // wait, whose records are not those the scenarios read.
+  if (late == 0) pdl_wait();
+  if (late != 1) pdl_trigger();
   if (set.skip && set.skip[p] >= 0) return;
   const float* bp = set.bounds + (size_t)p * 4 * d.cells;
   const float* cap = bp + (size_t)(sigma ? CAP_HI : CAP_LO) * d.cells;
@@ -183,7 +184,10 @@ __global__ void __launch_bounds__(kThreshThreads) k_thresh(Set set, int late) {
     __syncthreads();
     if (tid == 0) set.tpart[sigma * gridDim.x + blockIdx.x] = __uint_as_float(s_best);
   }
-  if (late) pdl_wait();
+  if (late) {
+    pdl_wait();
+    if (late == 1) pdl_trigger();
+  }
 }
 
 // Measured (one GB300, calls in a row): the eight-class, 256-GPU grid (about 1300
@@ -201,11 +205,12 @@ __global__ void __launch_bounds__(kThreshThreads) k_thresh(Set set, int late) {
 //   - thresholds, rows and tables have no reader left: the preparation of call n -
 //     1 was the last (a dump's scenarios read rows: not late after one; the goodput
 //     stage and the replay are synchronous);
-//   - the parts of t*, the records, the sums and the counters, which call n - 1
-//     still uses, alternate between two sets, call n - 2's being free.
+//   - the parts of t*, the sums, the counters and (late 2: both calls' records fit
+//     a half of their buffer) the records, which call n - 1 still uses, alternate
+//     between two sets, call n - 2's being free.
 // A call without candidates has no preparation and scenarios to hand that on: it
 // waits first.
-cudaError_t launch_thresh(Set& set, int floors, int th_bound, cudaStream_t s, bool late) {
+cudaError_t launch_thresh(Set& set, int floors, int th_bound, cudaStream_t s, int late) {
   const Dims& d = set.d;
   const int bound = th_bound > 0 ? std::min(th_bound, d.theta_cap) : d.theta_cap;
   int gsz = 4;
@@ -216,7 +221,7 @@ cudaError_t launch_thresh(Set& set, int floors, int th_bound, cudaStream_t s, bo
   const int nb = set.P > 1 ? 1 : std::max(1, std::min(kThreshBlocks, (bound + per_block - 1) / per_block));
   set.n_tpart = set.tpart ? nb : 0;
   return launch_pdl(floors ? k_thresh<true> : k_thresh<false>, dim3(nb, 2 * set.P), dim3(kThreshThreads), 0, s, set,
-                    late ? 1 : 0);
+                    late);
 }
 
 }  // namespace fs

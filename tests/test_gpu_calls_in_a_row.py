@@ -75,3 +75,43 @@ def test_calls_in_a_row(fsb, cuda, oracle_lib, K, B, G, side_stream):
         assert float(out[1][0]) == r.gamma_t and int(out[2][0]) == r.best, (k, b)
         assert np.array_equal(out[3].cpu().numpy()[:n], r.sum_eo), (k, b)
         assert np.array_equal(out[0].cpu().numpy()[:n], r.score), (k, b)
+
+
+def test_calls_under_capture(fsb, cuda, oracle_lib):
+    """Three asynchronous calls captured into one CUDA graph after a single
+    warm-up call, the graph replayed between calls made directly."""
+    torch = cuda
+    w = dataclasses.replace(workloads.make_workload(1), S=1000)
+    plans = [(w.candidates, 8, 1000), (w.candidates[::9].copy(), 4, 60), (w.candidates[5:6].copy(), 8, 3000)]
+    st = torch.cuda.Stream()
+    with load_model(fsb, w) as m:
+        ref = [fsb.fs_score_candidates(m, c, O, S, w.seed) for c, O, S in plans]
+    m = fsb.fs_load_model(w.cap_lo, w.cap_hi, w.tail_lo, w.tail_hi, w.slo, w.demand, w.G, w.K, w.B, stream=st)
+    dev = [torch.from_numpy(c).cuda() for c, _, _ in plans]
+    sums = [torch.zeros((len(c), O), dtype=torch.int64, device="cuda") for c, O, _ in plans]
+    torch.cuda.synchronize()
+
+    def call(k):
+        fsb.fs_score_candidates_async(m, dev[k], plans[k][1], plans[k][2], w.seed, sum_eo_dev=sums[k], stream=st)
+
+    with m:
+        call(0)  # the largest: buffers and launch shapes are there
+        call(1)
+        call(2)
+        torch.cuda.synchronize()
+        g = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(g, stream=st):
+            for k in range(3):
+                call(k)
+        for _ in range(4):
+            for s in sums:
+                s.zero_()
+            torch.cuda.synchronize()
+            with torch.cuda.stream(st):
+                call(0)
+                g.replay()
+                call(2)
+                g.replay()
+            torch.cuda.synchronize()
+            for k in range(3):
+                assert np.array_equal(sums[k].cpu().numpy(), ref[k].sum_eo), k
