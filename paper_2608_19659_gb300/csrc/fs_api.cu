@@ -159,7 +159,7 @@ struct fs_model {
   Set set{};
   // per-call scratch
   Buf real, lex, gp;
-  Buf tables, sums;  // records and sums, two halves each: asynchronous calls alternate (launch_thresh)
+  Buf tables, tables2, sums;  // records (two buffers) and sums (two halves): asynchronous calls alternate (launch_thresh)
   Buf replay;     // fs_replay's state of every stream (grown on demand, kept)
   int objective = FS_OBJECTIVE_MAXMIN;  // FS_OBJECTIVE_LEXICOGRAPHIC: fs_solve* and the certificate to tier 4
   // host mirrors
@@ -176,7 +176,8 @@ struct fs_model {
   LaunchCache lc;
   int half = 0;             // the set of what alternates that the last scoring call used
   bool rows_read = false;   // the last scoring call's scenarios read the rows (dump)
-  bool whole = false;       // its records took the whole buffer
+  bool one_buffer = false;  // its records went to the first buffer whatever the half
+  bool async_before = false;
   // optional timing events: 5 per timed call (before solve, prep, score,
   // finalize, and after finalize); mode 1 records only the two around score
   int timing = 0;
@@ -374,14 +375,13 @@ Dims call_dims(const fs_model* m, int th_bound) {
 }
 
 // Buffers of a call's records and sums, sized by the model and the plan alone, so
-// that new bounds never make a later call allocate. The sums have two halves; the
-// records have two where both, with tables for every threshold the model allows,
-// take at most kTwoRecords (a larger call's two halves may still hold its
-// records, whose tables only need the bounds' thresholds). A half's place depends
-// on the buffer's size alone: calls of different sizes never share a byte of
-// different halves, and a buffer that grows is freed, which waits for the calls in
-// flight.
-constexpr size_t kTwoRecords = 64u << 20;
+// that new bounds never make a later call allocate. The sums have two halves. The
+// second buffer of records, of the first's size up to kSecondRecords, comes with
+// the model's second asynchronous call (a first call alone has no use for it, and
+// would pay for its allocation: 55 -> 150 us from 1 MB on), never while the stream
+// is being captured. Calls whose records do not fit it use the first (1024 x 16 x
+// 16384 scenarios without it: 208 us instead of 204).
+constexpr size_t kSecondRecords = 32u << 20;
 
 size_t record_bytes(const Dims& d, int n, int O) {
   const int W = d.Q / O, Wp = 4 + ((W + 3) & ~3);
@@ -390,15 +390,37 @@ size_t record_bytes(const Dims& d, int n, int O) {
 
 int ensure_items(fs_model* m, int n, int O) {
   const size_t full = record_bytes(m->d, n, O);
-  int rc = m->tables.ensure(2 * full <= kTwoRecords ? 2 * full : full, "candidate records");
-  if (rc) return rc;
+  if (full > m->tables.bytes) {
+    int rc = m->tables.ensure(full, "candidate records");
+    if (rc) return rc;
+    // the second buffer grows with the first and at no other time: what a
+    // captured graph holds of either stays while the other does
+    if (m->tables2.p && (rc = m->tables2.ensure(std::min(full, kSecondRecords), "candidate records")))
+      return rc;
+  }
   // sums, then the split reduction's scratch (2 words per block)
   return m->sums.ensure(2 * align_up((size_t)std::max(n, 1) * O * 8 + 16 * (size_t)kFinalizeMaxBlocks, 256), "sums");
 }
 
-float* tables_at(const fs_model* m, int half) {
-  return reinterpret_cast<float*>(static_cast<char*>(m->tables.p) + half * (m->tables.bytes / 512 * 256));
+// The second buffer of records for an asynchronous call that needs `need` bytes
+// of it on stream s: whether it is there.
+bool second_records(fs_model* m, size_t need, cudaStream_t s) {
+  if (m->tables2.p) return m->tables2.bytes >= need;
+  if (!m->async_before || need > kSecondRecords) return false;
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(s, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) {
+    (void)cudaGetLastError();  // (a legacy stream while another captures: not now)
+    return false;
+  }
+  // relaxed: an allocation here must not end a capture that another thread makes
+  cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+  if (cudaThreadExchangeStreamCaptureMode(&mode) != cudaSuccess) return false;
+  const int rc = m->tables2.ensure(std::min(m->tables.bytes, kSecondRecords), "candidate records");
+  (void)cudaThreadExchangeStreamCaptureMode(&mode);
+  if (rc) (void)cudaGetLastError();
+  return rc == FS_OK;
 }
+
 uint64_t* sums_half(const fs_model* m, int half) {
   return reinterpret_cast<uint64_t*>(static_cast<char*>(m->sums.p) + half * (m->sums.bytes / 512 * 256));
 }
@@ -413,20 +435,21 @@ int run_score(fs_model* m, Set set, const fs_samples* smp, const int32_t* cand_d
   it.p = nullptr;
   it.cell = cand_dev;
   it.off = nullptr;
-  // What alternates between calls (launch_thresh): the other half in an
-  // asynchronous call, which may start before the last call has finished, the
-  // same in a synchronous one, which waits for it. Records too large for a half
-  // take the whole buffer.
+  // What alternates between calls (launch_thresh): the other half (the records'
+  // other buffer) in an asynchronous call, which may start before the last call
+  // has finished, the same in a synchronous one, which waits for it. Without a
+  // second buffer the records go to the first.
   if (m->th_bound < 0) m->th_bound = threshold_bound(m);
   set.d = call_dims(m, m->th_bound);
   int rc = ensure_items(m, n, smp->O);
   if (rc) return rc;
   if (late) m->half ^= 1;
   const int half = m->half;
-  const bool whole = record_bytes(set.d, n, smp->O) > m->tables.bytes / 512 * 256;
-  const int mode = !late || n == 0 || m->rows_read ? 0 : whole || m->whole ? 1 : 2;
-  m->whole = whole;
-  float* tables = tables_at(m, whole ? 0 : half);
+  const bool one = !late || !second_records(m, record_bytes(set.d, n, smp->O), s);
+  const int mode = !late || n == 0 || m->rows_read ? 0 : one || m->one_buffer ? 1 : 2;
+  m->one_buffer = one;
+  m->async_before = m->async_before || late;
+  float* tables = static_cast<float*>(half && !one ? m->tables2.p : m->tables.p);
   uint64_t* sums = sums_half(m, half);
   set.tpart += half * 2 * kThreshBlocks;
   set.work += 4 * half;
@@ -898,7 +921,7 @@ int fs_score_goodput(fs_model* m, const fs_samples* smp, double* gap_out, double
   int* span = static_cast<int*>(m->gp.p);
   long long* base = reinterpret_cast<long long*>(span + 2 * kGoodputSpanInts);
   uint64_t* sums = sums_half(m, 0);
-  float* tables = tables_at(m, 0);
+  float* tables = static_cast<float*>(m->tables.p);
   set.gp_span = span;
   FS_CUDA(launch_thresh(set, m->lc.floors, m->th_bound, s), "launch thresholds");
   FS_CUDA(launch_prep(set, it, pl, tables, sums, 1, m->sm_count, m->lc, s, m->th_bound),
@@ -1057,9 +1080,9 @@ int fs_replay(fs_model* m, const fs_replay_spec* sp, int32_t* rounds, int32_t* s
       fs_samples smp{sp->seed, 0, (uint32_t)r, n_items, sp->O, sp->S, 0, nullptr};
       Plan pl = make_plan(m->d, &smp);
       pl.few = few_path(pl, n_items) ? 1 : 0;
-      FS_CUDA(launch_prep(set, it, pl, tables_at(m, 0), sums_half(m, 0), 0, m->sm_count, m->lc, s),
+      FS_CUDA(launch_prep(set, it, pl, static_cast<float*>(m->tables.p), sums_half(m, 0), 0, m->sm_count, m->lc, s),
               "launch prep");
-      FS_CUDA(launch_score(set, it, pl, tables_at(m, 0), sums_half(m, 0), nullptr, 0, m->sm_count,
+      FS_CUDA(launch_score(set, it, pl, static_cast<float*>(m->tables.p), sums_half(m, 0), nullptr, 0, m->sm_count,
                            m->lc, s),
               "launch score");
       FS_CUDA(launch_replay_reveal(set, rs, it, pl, sums_half(m, 0), n_active, s), "launch reveal");
@@ -1179,6 +1202,7 @@ void fs_free_model(fs_model* m) {
   else cudaDeviceSynchronize();
   m->fixed.release();
   m->tables.release();
+  m->tables2.release();
   m->sums.release();
   m->real.release();
   m->lex.release();
