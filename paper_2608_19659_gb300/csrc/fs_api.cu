@@ -395,8 +395,9 @@ int ensure_items(fs_model* m, int n, int O) {
     if (rc) return rc;
     // the second buffer grows with the first and at no other time: what a
     // captured graph holds of either stays while the other does
-    if (m->tables2.p && (rc = m->tables2.ensure(std::min(full, kSecondRecords), "candidate records")))
-      return rc;
+    // (and is optional: without memory for it, calls use the first)
+    if (m->tables2.p && m->tables2.ensure(std::min(full, kSecondRecords), "candidate records"))
+      (void)cudaGetLastError();
   }
   // sums, then the split reduction's scratch (2 words per block)
   return m->sums.ensure(2 * align_up((size_t)std::max(n, 1) * O * 8 + 16 * (size_t)kFinalizeMaxBlocks, 256), "sums");
