@@ -163,7 +163,8 @@ __global__ void __launch_bounds__(kPrepThreads, 5) k_prep(Set set, Items it, Pla
   extern __shared__ __align__(16) unsigned char smraw[];
   float* sTh = reinterpret_cast<float*>(smraw);  // [theta_cap], unless a table beyond a thread each is sure
   __shared__ float s_cx, s_cmax, s_pc, s_po, s_lf, s_hf;
-  __shared__ int s_bx, s_row;
+  __shared__ float4 s_own;  // the candidate cell's cap_lo, cap_hi, tail_lo, tail_hi
+  __shared__ int s_bx, s_row, s_id[2];
   __shared__ float sLam[FS_MAX_CLASSES], sRl[FS_MAX_CLASSES];  // demand and RN(1/demand)
   __shared__ float sDl[FS_MAX_CLASSES];                          // floor delta_i (0: not critical)
   __shared__ int s_res[2][kPrepThreads / 4];
@@ -172,7 +173,19 @@ __global__ void __launch_bounds__(kPrepThreads, 5) k_prep(Set set, Items it, Pla
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nwarp = blockDim.x >> 5;
   if (!early) pdl_wait();
   const int p = it.p ? it.p[item] : 0;
-  int cell = it.cell[item];
+  // early 2: the candidate list may still be being written when it is first read
+  // (by a caller's kernel, or by the last call's reduction through its `best`, that
+  // lets its dependents start before it has finished), and warps that read it for
+  // themselves could get different ids. One thread reads it, before the wait and
+  // after it, and the block takes the id and every decision on it from shared memory.
+  int cell;
+  if (early == 2) {
+    if (tid == 0) s_id[0] = __ldcg(it.cell + item);
+    __syncthreads();
+    cell = s_id[0];
+  } else {
+    cell = it.cell[item];
+  }
   float* base_rec = rec + (size_t)item * pl.item_floats;
   float* tab = base_rec + (size_t)sigma * d.slot_floats;
   if (blockIdx.x == 0 && tid == 0) {
@@ -191,190 +204,181 @@ __global__ void __launch_bounds__(kPrepThreads, 5) k_prep(Set set, Items it, Pla
       tab[H_CELL] = __int_as_float(-1);
     }
   };
-  int rr = 0, ie = 0, jr = 0;
-  float lam = 1.0f, L = 0.0f, rl = 1.0f, dle = 0.0f, lo_c, hi_c, lo_l, hi_l;
-  // The part that reads only the bounds: once, or again when the candidate list
-  // turns out to have changed (read before the wait, it may have belonged to a
-  // kernel of the caller's that lets its dependents start before it has finished).
-  for (bool waited = !early;; waited = true) {
-  if (cell < 0 || cell >= d.cells) {  // device-side candidate ids are checked here
-    if (!waited) pdl_wait();
-    if (!waited && early == 2) {
-      cell = __ldcg(it.cell + item);
-      if (cell >= 0 && cell < d.cells) continue;
+  // The part that reads only the bounds; it leaves its results in shared memory and
+  // in the record.
+  auto bounds_part = [&]() {
+    const int rr = cell / d.B, ie = rr >> 2, be = cell - rr * d.B;
+    const float L = set.slo[ie];
+    if (tid < d.K) {
+      sLam[tid] = set.lam[tid];
+      sRl[tid] = __frcp_rn(set.lam[tid]);
+      if (FL) sDl[tid] = set.slo[d.K + tid];
     }
-    reject(ST_CELL);
-    return;
-  }
-  rr = cell / d.B;
-  ie = rr >> 2;
-  jr = rr & 3;
-  const int be = cell - rr * d.B;
-  lam = set.lam[ie];
-  L = set.slo[ie];
-  rl = __frcp_rn(lam);
-  dle = FL ? set.slo[d.K + ie] : 0.0f;
-  if (tid < d.K) {
-    sLam[tid] = set.lam[tid];
-    sRl[tid] = __frcp_rn(set.lam[tid]);
-    if (FL) sDl[tid] = set.slo[d.K + tid];
-  }
-  const float* bp = set.bounds + (size_t)p * 4 * d.cells;
-  const float* capS = bp + (size_t)(sigma ? CAP_HI : CAP_LO) * d.cells;
-  const float* tailS = bp + (size_t)(sigma ? TAIL_LO : TAIL_HI) * d.cells;
-  lo_c = bp[(size_t)CAP_LO * d.cells + cell];
-  hi_c = bp[(size_t)CAP_HI * d.cells + cell];
-  lo_l = bp[(size_t)TAIL_LO * d.cells + cell];
-  hi_l = bp[(size_t)TAIL_HI * d.cells + cell];
+    const float* bp = set.bounds + (size_t)p * 4 * d.cells;
+    const float* capS = bp + (size_t)(sigma ? CAP_HI : CAP_LO) * d.cells;
+    const float* tailS = bp + (size_t)(sigma ? TAIL_LO : TAIL_HI) * d.cells;
+    const float lo_c = bp[(size_t)CAP_LO * d.cells + cell], hi_c = bp[(size_t)CAP_HI * d.cells + cell];
+    const float lo_l = bp[(size_t)TAIL_LO * d.cells + cell], hi_l = bp[(size_t)TAIL_HI * d.cells + cell];
+    if (tid == 0) s_own = make_float4(lo_c, hi_c, lo_l, hi_l);
 
-  // best SLO-feasible capacity of row r without bin b_e (ties: lower bin)
-  if (RF) {
-    // Under the monotone prior a scenario's draw (c_y, l_y) also refits row
-    // r's other bins (capacity and tail nondecreasing in the load bin). For
-    // realisation sigma the row's capacity is then
-    //   C' = max(g ? max(P_open, c_y) : P_closed, min(max(c_y, F_lo), F_hi)):
-    // A- (sigma 0): a bin below b_e keeps cap_lo and its upper tail falls to
-    //   max(min(tail_hi, l_y), tail_lo), which passes the SLO iff tail_hi <= L,
-    //   or g and tail_lo <= L (P); a bin above b_e passes iff tail_hi <= L and
-    //   its lower capacity rises to min(max(cap_lo, c_y), cap_hi), whose
-    //   maximum over such bins is min(max(c_y, max cap_lo), max cap_hi) (F).
-    // A+ (sigma 1): a bin above b_e keeps cap_hi and its lower tail rises to
-    //   min(max(tail_lo, l_y), tail_hi), which passes iff tail_hi <= L, or g
-    //   and tail_lo <= L (P); a bin below b_e passes iff tail_lo <= L and its
-    //   upper capacity falls to max(min(cap_hi, c_y), cap_lo) (F).
-    // So C' depends on the draw only through (c_y, g), as without the prior.
-    if (warp == 0) {
-      float pc = 0.0f, po = 0.0f, lf = 0.0f, hf = 0.0f;
-      const float* cl = bp + (size_t)CAP_LO * d.cells + (size_t)rr * d.B;
-      const float* ch = bp + (size_t)CAP_HI * d.cells + (size_t)rr * d.B;
-      const float* tl = bp + (size_t)TAIL_LO * d.cells + (size_t)rr * d.B;
-      const float* th = bp + (size_t)TAIL_HI * d.cells + (size_t)rr * d.B;
+    // best SLO-feasible capacity of row r without bin b_e (ties: lower bin)
+    if (RF) {
+      // Under the monotone prior a scenario's draw (c_y, l_y) also refits row
+      // r's other bins (capacity and tail nondecreasing in the load bin). For
+      // realisation sigma the row's capacity is then
+      //   C' = max(g ? max(P_open, c_y) : P_closed, min(max(c_y, F_lo), F_hi)):
+      // A- (sigma 0): a bin below b_e keeps cap_lo and its upper tail falls to
+      //   max(min(tail_hi, l_y), tail_lo), which passes the SLO iff tail_hi <= L,
+      //   or g and tail_lo <= L (P); a bin above b_e passes iff tail_hi <= L and
+      //   its lower capacity rises to min(max(cap_lo, c_y), cap_hi), whose
+      //   maximum over such bins is min(max(c_y, max cap_lo), max cap_hi) (F).
+      // A+ (sigma 1): a bin above b_e keeps cap_hi and its lower tail rises to
+      //   min(max(tail_lo, l_y), tail_hi), which passes iff tail_hi <= L, or g
+      //   and tail_lo <= L (P); a bin below b_e passes iff tail_lo <= L and its
+      //   upper capacity falls to max(min(cap_hi, c_y), cap_lo) (F).
+      // So C' depends on the draw only through (c_y, g), as without the prior.
+      if (warp == 0) {
+        float pc = 0.0f, po = 0.0f, lf = 0.0f, hf = 0.0f;
+        const float* cl = bp + (size_t)CAP_LO * d.cells + (size_t)rr * d.B;
+        const float* ch = bp + (size_t)CAP_HI * d.cells + (size_t)rr * d.B;
+        const float* tl = bp + (size_t)TAIL_LO * d.cells + (size_t)rr * d.B;
+        const float* th = bp + (size_t)TAIL_HI * d.cells + (size_t)rr * d.B;
+        for (int b = lane; b < d.B; b += 32) {
+          if (b == be) continue;
+          const bool p_side = sigma ? b > be : b < be;  // bins refit only in their tail
+          const float cap = sigma ? ch[b] : cl[b];
+          if (p_side) {
+            if (th[b] <= L) pc = fmaxf(pc, cap);
+            if (tl[b] <= L) po = fmaxf(po, cap);
+          } else if ((sigma ? tl[b] : th[b]) <= L) {  // bins refit only in their capacity
+            lf = fmaxf(lf, cl[b]);
+            hf = fmaxf(hf, ch[b]);
+          }
+        }
+        for (int off = 16; off; off >>= 1) {
+          pc = fmaxf(pc, __shfl_xor_sync(0xffffffffu, pc, off));
+          po = fmaxf(po, __shfl_xor_sync(0xffffffffu, po, off));
+          lf = fmaxf(lf, __shfl_xor_sync(0xffffffffu, lf, off));
+          hf = fmaxf(hf, __shfl_xor_sync(0xffffffffu, hf, off));
+        }
+        if (lane == 0) {
+          po = fmaxf(po, pc);
+          // the table covers C' from its least (c_y = cap_lo, gate closed) to
+          // its largest value (c_y = cap_hi, gate open)
+          s_cx = fmaxf(pc, fminf(fmaxf(lo_c, lf), hf));
+          s_cmax = fmaxf(fmaxf(po, hi_c), fminf(fmaxf(hi_c, lf), hf));
+          s_pc = pc;
+          s_po = po;
+          s_lf = lf;
+          s_hf = hf;
+          s_bx = -1;
+          s_row = 0;
+        }
+      }
+    } else if (warp == 0) {
+      float best = 0.0f;
+      int bb = -1;
       for (int b = lane; b < d.B; b += 32) {
         if (b == be) continue;
-        const bool p_side = sigma ? b > be : b < be;  // bins refit only in their tail
-        const float cap = sigma ? ch[b] : cl[b];
-        if (p_side) {
-          if (th[b] <= L) pc = fmaxf(pc, cap);
-          if (tl[b] <= L) po = fmaxf(po, cap);
-        } else if ((sigma ? tl[b] : th[b]) <= L) {  // bins refit only in their capacity
-          lf = fmaxf(lf, cl[b]);
-          hf = fmaxf(hf, ch[b]);
+        const size_t c = (size_t)rr * d.B + b;
+        if (tailS[c] <= L) {
+          const float v = capS[c];
+          if (bb < 0 || v > best) {
+            best = v;
+            bb = b;
+          }
         }
       }
       for (int off = 16; off; off >>= 1) {
-        pc = fmaxf(pc, __shfl_xor_sync(0xffffffffu, pc, off));
-        po = fmaxf(po, __shfl_xor_sync(0xffffffffu, po, off));
-        lf = fmaxf(lf, __shfl_xor_sync(0xffffffffu, lf, off));
-        hf = fmaxf(hf, __shfl_xor_sync(0xffffffffu, hf, off));
+        const float ob = __shfl_xor_sync(0xffffffffu, best, off);
+        const int obb = __shfl_xor_sync(0xffffffffu, bb, off);
+        if (obb >= 0 && (bb < 0 || ob > best || (ob == best && obb < bb))) {
+          best = ob;
+          bb = obb;
+        }
       }
       if (lane == 0) {
-        po = fmaxf(po, pc);
-        // the table covers C' from its least (c_y = cap_lo, gate closed) to
-        // its largest value (c_y = cap_hi, gate open)
-        s_cx = fmaxf(pc, fminf(fmaxf(lo_c, lf), hf));
-        s_cmax = fmaxf(fmaxf(po, hi_c), fminf(fmaxf(hi_c, lf), hf));
-        s_pc = pc;
-        s_po = po;
-        s_lf = lf;
-        s_hf = hf;
-        s_bx = -1;
+        s_cx = bb >= 0 ? best : 0.0f;
+        s_bx = bb;
+        s_cmax = fmaxf(s_cx, hi_c);
+        s_pc = s_po = s_cx;
+        s_lf = s_hf = 0.0f;
         s_row = 0;
       }
     }
-  } else if (warp == 0) {
-    float best = 0.0f;
-    int bb = -1;
-    for (int b = lane; b < d.B; b += 32) {
-      if (b == be) continue;
-      const size_t c = (size_t)rr * d.B + b;
-      if (tailS[c] <= L) {
-        const float v = capS[c];
-        if (bb < 0 || v > best) {
-          best = v;
-          bb = b;
+
+    // Mapped strata (unless the samples are few, whose scorer maps its draws).
+    // Window of outcome o: word 0 = the number of leading
+    // positions whose tail value passes the SLO (the mapped tails are
+    // nondecreasing in the position, so exactly one position ends the run of
+    // passes), words 4.. = the W capacities.
+    if (pl.few) {  // (word 1, 2 of the first window: the cell's capacity bounds, for its draws)
+      if (sigma == 0 && tid == 0) {
+        float* win0 = base_rec + 2 * (size_t)d.slot_floats;
+        win0[1] = lo_c;
+        win0[2] = hi_c;
+      }
+    } else {
+      const int W = pl.W;
+      const float d_c = __fsub_rn(hi_c, lo_c), d_l = __fsub_rn(hi_l, lo_l);
+      const int n_out = (pl.O - sigma + 1) >> 1;  // this block's outcomes
+      const int n_idx = n_out << pl.w;            // (at most Q <= 2^24 positions)
+      float* wins = base_rec + 2 * (size_t)d.slot_floats;
+      // gate positions, an outcome per thread: every position where even the upper
+      // tail passes, none where not even the lower one does, else by bisection
+      for (int x = tid; x < n_out; x += blockDim.x) {
+        const int o = sigma + 2 * x;
+        int pass = hi_l <= L ? W : 0;
+        if (hi_l > L && lo_l <= L) {
+          const float* q = set.qn + (size_t)o * W;
+          for (int step = W; step > 0; step >>= 1)
+            if (pass + step <= W && map_into(lo_l, d_l, hi_l, __ldg(q + pass + step - 1)) <= L) pass += step;
+        }
+        wins[(size_t)o * pl.Wp] = __int_as_float(pass);
+      }
+      if (W >= 4 && (reinterpret_cast<uintptr_t>(set.qn) & 15u) == 0) {
+        // four consecutive positions per thread: one 16-byte load and store
+        // (windows start on 16-byte boundaries)
+        const int n4 = n_idx >> 2;
+  #pragma unroll 4
+        for (int g4 = tid; g4 < n4; g4 += blockDim.x) {
+          const int k = (g4 << 2) & (W - 1), o = sigma + 2 * (g4 >> (pl.w - 2));
+          const float4 v = __ldg(reinterpret_cast<const float4*>(set.qn + (size_t)o * W + k));
+          float4 cm;
+          cm.x = map_into(lo_c, d_c, hi_c, v.x);
+          cm.y = map_into(lo_c, d_c, hi_c, v.y);
+          cm.z = map_into(lo_c, d_c, hi_c, v.z);
+          cm.w = map_into(lo_c, d_c, hi_c, v.w);
+          *reinterpret_cast<float4*>(wins + (size_t)o * pl.Wp + 4 + k) = cm;
+        }
+      } else {
+        // read-only loads, so that the unrolled iterations' loads are issued
+        // together rather than each behind the previous iteration's stores
+  #pragma unroll 4
+        for (int idx = tid; idx < n_idx; idx += blockDim.x) {
+          const int k = idx & (W - 1), o = sigma + 2 * (idx >> pl.w);
+          wins[(size_t)o * pl.Wp + 4 + k] = map_into(lo_c, d_c, hi_c, __ldg(set.qn + (size_t)o * W + k));
         }
       }
     }
-    for (int off = 16; off; off >>= 1) {
-      const float ob = __shfl_xor_sync(0xffffffffu, best, off);
-      const int obb = __shfl_xor_sync(0xffffffffu, bb, off);
-      if (obb >= 0 && (bb < 0 || ob > best || (ob == best && obb < bb))) {
-        best = ob;
-        bb = obb;
-      }
-    }
-    if (lane == 0) {
-      s_cx = bb >= 0 ? best : 0.0f;
-      s_bx = bb;
-      s_cmax = fmaxf(s_cx, hi_c);
-      s_pc = s_po = s_cx;
-      s_lf = s_hf = 0.0f;
-      s_row = 0;
-    }
+  };
+  bool valid;
+  for (bool waited = !early;; waited = true) {  // once, or again when the list turns out to have changed
+    valid = cell >= 0 && cell < d.cells;        // device-side candidate ids are checked here
+    if (valid) bounds_part();
+    if (waited) break;
+    pdl_wait();  // thresholds and rows come from k_thresh
+    if (early != 2) break;
+    if (tid == 0) s_id[1] = __ldcg(it.cell + item);
+    __syncthreads();
+    if (s_id[1] == cell) break;
+    cell = s_id[1];
   }
-
-  // Mapped strata (unless the samples are few, whose scorer maps its draws).
-  // Window of outcome o: word 0 = the number of leading
-  // positions whose tail value passes the SLO (the mapped tails are
-  // nondecreasing in the position, so exactly one position ends the run of
-  // passes), words 4.. = the W capacities.
-  if (pl.few) {  // (word 1, 2 of the first window: the cell's capacity bounds, for its draws)
-    if (sigma == 0 && tid == 0) {
-      float* win0 = base_rec + 2 * (size_t)d.slot_floats;
-      win0[1] = lo_c;
-      win0[2] = hi_c;
-    }
-  } else {
-    const int W = pl.W;
-    const float d_c = __fsub_rn(hi_c, lo_c), d_l = __fsub_rn(hi_l, lo_l);
-    const int n_out = (pl.O - sigma + 1) >> 1;  // this block's outcomes
-    const int n_idx = n_out << pl.w;            // (at most Q <= 2^24 positions)
-    float* wins = base_rec + 2 * (size_t)d.slot_floats;
-    // gate positions, an outcome per thread: every position where even the upper
-    // tail passes, none where not even the lower one does, else by bisection
-    for (int x = tid; x < n_out; x += blockDim.x) {
-      const int o = sigma + 2 * x;
-      int pass = hi_l <= L ? W : 0;
-      if (hi_l > L && lo_l <= L) {
-        const float* q = set.qn + (size_t)o * W;
-        for (int step = W; step > 0; step >>= 1)
-          if (pass + step <= W && map_into(lo_l, d_l, hi_l, __ldg(q + pass + step - 1)) <= L) pass += step;
-      }
-      wins[(size_t)o * pl.Wp] = __int_as_float(pass);
-    }
-    if (W >= 4 && (reinterpret_cast<uintptr_t>(set.qn) & 15u) == 0) {
-      // four consecutive positions per thread: one 16-byte load and store
-      // (windows start on 16-byte boundaries)
-      const int n4 = n_idx >> 2;
-#pragma unroll 4
-      for (int g4 = tid; g4 < n4; g4 += blockDim.x) {
-        const int k = (g4 << 2) & (W - 1), o = sigma + 2 * (g4 >> (pl.w - 2));
-        const float4 v = __ldg(reinterpret_cast<const float4*>(set.qn + (size_t)o * W + k));
-        float4 cm;
-        cm.x = map_into(lo_c, d_c, hi_c, v.x);
-        cm.y = map_into(lo_c, d_c, hi_c, v.y);
-        cm.z = map_into(lo_c, d_c, hi_c, v.z);
-        cm.w = map_into(lo_c, d_c, hi_c, v.w);
-        *reinterpret_cast<float4*>(wins + (size_t)o * pl.Wp + 4 + k) = cm;
-      }
-    } else {
-      // read-only loads, so that the unrolled iterations' loads are issued
-      // together rather than each behind the previous iteration's stores
-#pragma unroll 4
-      for (int idx = tid; idx < n_idx; idx += blockDim.x) {
-        const int k = idx & (W - 1), o = sigma + 2 * (idx >> pl.w);
-        wins[(size_t)o * pl.Wp + 4 + k] = map_into(lo_c, d_c, hi_c, __ldg(set.qn + (size_t)o * W + k));
-      }
-    }
+  if (!valid) {
+    reject(ST_CELL);
+    return;
   }
-  if (waited) break;
-  pdl_wait();  // thresholds and rows come from k_thresh
-  if (early != 2) break;
-  const int again = __ldcg(it.cell + item);
-  if (again == cell) break;
-  cell = again;  // (the same for the whole block)
-  __syncthreads();
-  }
+  const int rr = cell / d.B, ie = rr >> 2, jr = rr & 3;
 
   const size_t ps = (size_t)p * 2 + sigma;
   const float* th_g = set.theta + ps * d.theta_cap;
@@ -418,6 +422,7 @@ __global__ void __launch_bounds__(kPrepThreads, 5) k_prep(Set set, Items it, Pla
   }
   __syncthreads();
   const float cx = s_cx, cmax = s_cmax;
+  const float lam = sLam[ie], rl = sRl[ie], dle = FL ? sDl[ie] : 0.0f;
   const int msent = d.K == 1 ? rep_cap(d, jr) : 0;  // above every threshold only a lone class can go on
 
   // b0: last index feasible at Cexcl; b1: last index feasible at max(Cexcl, cap_hi).
@@ -582,6 +587,7 @@ __global__ void __launch_bounds__(kPrepThreads, 5) k_prep(Set set, Items it, Pla
   if (tid == 0) thx[0] = b0 >= 0 ? th[b0] : 0.0f;
   __syncthreads();
   if (tid == 0) {
+    const float lo_c = s_own.x, hi_c = s_own.y;
     // every row-term quotient x / lambda of a scenario has x = m C' with
     // 1 <= m <= 32767 and C' in {0} or [min(Cexcl, cap_lo), cmax]: in
     // Markstein's range unless a positive C' can fall below 2^-60
@@ -604,9 +610,9 @@ __global__ void __launch_bounds__(kPrepThreads, 5) k_prep(Set set, Items it, Pla
     tab[H_LAM] = lam;
     tab[H_LF] = s_lf;
     tab[H_HF] = s_hf;
-    tab[H_LO_L] = lo_l;
-    tab[H_HI_L] = hi_l;
-    tab[H_SLO] = L;
+    tab[H_LO_L] = s_own.z;
+    tab[H_HI_L] = s_own.w;
+    tab[H_SLO] = set.slo[ie];
     tab[H_CELL] = __int_as_float(cell);
     tab[H_P] = __int_as_float(p);
     tab[H_STEP0] = __int_as_float(Lt ? P >> 1 : 0);

@@ -115,3 +115,39 @@ def test_calls_under_capture(fsb, cuda, oracle_lib):
             torch.cuda.synchronize()
             for k in range(3):
                 assert np.array_equal(sums[k].cpu().numpy(), ref[k].sum_eo), k
+
+
+@pytest.mark.parametrize("at", [0, 7])
+@pytest.mark.parametrize("S", [60, 1500])  # few samples and many
+def test_list_written_by_the_call_before(fsb, cuda, oracle_lib, at, S):
+    """A call whose candidate list holds the best cell of the call queued right
+    before it. That call's reduction lets this one start before it has written
+    the cell, so the entry read first is another one, and no cell at all."""
+    torch = cuda
+    rng = np.random.default_rng(at + S)
+    w = workloads.make_workload(1)
+    n, O, calls = 40, 8, 24
+    lists = [rng.permutation(w.cells)[:n].astype(np.int32) for _ in range(calls)]
+    stale = [-1, int(w.cells), int(lists[0][at])]  # (what the entry holds until then)
+    with load_model(fsb, w) as m:
+        ref = []
+        for k in range(calls):
+            if k:
+                lists[k][at] = ref[-1].best
+            ref.append(fsb.fs_score_candidates(m, lists[k], O, S, k))
+        dev = [torch.from_numpy(c).cuda() for c in lists]
+        best = torch.zeros(1, dtype=torch.int32, device="cuda")
+        sums = [torch.zeros((n, O), dtype=torch.int64, device="cuda") for _ in range(calls)]
+        for _ in range(2):  # (the first calls make the buffers)
+            for k in range(1, calls):
+                dev[k][at] = stale[k % 3]
+            torch.cuda.synchronize()
+            for k in range(calls):
+                nxt = dev[k + 1][at:at + 1] if k + 1 < calls else best
+                fsb.fs_score_candidates_async(m, dev[k], O, S, k, best_dev=nxt, sum_eo_dev=sums[k])
+            fsb.fs_check(m)
+            torch.cuda.synchronize()
+            for k in range(calls):
+                assert np.array_equal(dev[k].cpu().numpy(), lists[k]), k
+                assert np.array_equal(sums[k].cpu().numpy(), ref[k].sum_eo), k
+            assert int(best[0]) == ref[-1].best
