@@ -162,9 +162,9 @@ __global__ void __launch_bounds__(kPrepThreads, 5) k_prep(Set set, Items it, Pla
                                                        uint64_t* sums, int early, int sure) {
   extern __shared__ __align__(16) unsigned char smraw[];
   float* sTh = reinterpret_cast<float*>(smraw);  // [theta_cap], unless a table beyond a thread each is sure
-  __shared__ float s_cx, s_cmax, s_pc, s_po, s_lf, s_hf;
+  __shared__ float s_cx, s_cmax, s_pc, s_po, s_lf, s_hf, s_slo;
   __shared__ float4 s_own;  // the candidate cell's cap_lo, cap_hi, tail_lo, tail_hi
-  __shared__ int s_bx, s_row, s_id[2];
+  __shared__ int s_bx, s_row, s_cell, s_id[2];
   __shared__ float sLam[FS_MAX_CLASSES], sRl[FS_MAX_CLASSES];  // demand and RN(1/demand)
   __shared__ float sDl[FS_MAX_CLASSES];                          // floor delta_i (0: not critical)
   __shared__ int s_res[2][kPrepThreads / 4];
@@ -206,8 +206,10 @@ __global__ void __launch_bounds__(kPrepThreads, 5) k_prep(Set set, Items it, Pla
   };
   // The part that reads only the bounds; it leaves its results in shared memory and
   // in the record.
+  int row = 0;
   auto bounds_part = [&]() {
     const int rr = cell / d.B, ie = rr >> 2, be = cell - rr * d.B;
+    if (!RF) row = rr;
     const float L = set.slo[ie];
     if (tid < d.K) {
       sLam[tid] = set.lam[tid];
@@ -219,7 +221,11 @@ __global__ void __launch_bounds__(kPrepThreads, 5) k_prep(Set set, Items it, Pla
     const float* tailS = bp + (size_t)(sigma ? TAIL_LO : TAIL_HI) * d.cells;
     const float lo_c = bp[(size_t)CAP_LO * d.cells + cell], hi_c = bp[(size_t)CAP_HI * d.cells + cell];
     const float lo_l = bp[(size_t)TAIL_LO * d.cells + cell], hi_l = bp[(size_t)TAIL_HI * d.cells + cell];
-    if (tid == 0) s_own = make_float4(lo_c, hi_c, lo_l, hi_l);
+    if (tid == 0) {  // for the header: kept in shared memory, not in registers
+      s_own = make_float4(lo_c, hi_c, lo_l, hi_l);
+      s_slo = L;
+      s_cell = cell;
+    }
 
     // best SLO-feasible capacity of row r without bin b_e (ties: lower bin)
     if (RF) {
@@ -378,7 +384,8 @@ __global__ void __launch_bounds__(kPrepThreads, 5) k_prep(Set set, Items it, Pla
     reject(ST_CELL);
     return;
   }
-  const int rr = cell / d.B, ie = rr >> 2, jr = rr & 3;
+  const int rr = RF ? cell / d.B : row;  // (the prior's instances have no register for it)
+  const int ie = rr >> 2, jr = rr & 3;
 
   const size_t ps = (size_t)p * 2 + sigma;
   const float* th_g = set.theta + ps * d.theta_cap;
@@ -607,19 +614,19 @@ __global__ void __launch_bounds__(kPrepThreads, 5) k_prep(Set set, Items it, Pla
     tab[H_CX] = s_pc;
     tab[H_BX] = __int_as_float(s_bx);
     tab[H_PO] = s_po;
-    tab[H_LAM] = lam;
+    tab[H_LAM] = sLam[ie];
     tab[H_LF] = s_lf;
     tab[H_HF] = s_hf;
     tab[H_LO_L] = s_own.z;
     tab[H_HI_L] = s_own.w;
-    tab[H_SLO] = set.slo[ie];
-    tab[H_CELL] = __int_as_float(cell);
+    tab[H_SLO] = s_slo;
+    tab[H_CELL] = __int_as_float(s_cell);
     tab[H_P] = __int_as_float(p);
     tab[H_STEP0] = __int_as_float(Lt ? P >> 1 : 0);
     tab[H_ROW] = __int_as_float(s_row);
     tab[H_FAST] = __int_as_float(fast ? 1 : 0);
-    tab[H_RLAM] = rl;
-    tab[H_DLT] = dle;
+    tab[H_RLAM] = sRl[ie];
+    tab[H_DLT] = FL ? sDl[ie] : 0.0f;
   }
   // k_score launches only now: its blocks, resident early, slowed the kernels
   // before it more than their early start saved
