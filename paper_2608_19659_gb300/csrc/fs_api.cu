@@ -149,6 +149,14 @@ struct HostBuf {
 
 using namespace fs;
 
+// What the scoring calls of one sequence alternate (launch_thresh), as the last of
+// them left it.
+struct Sequence {
+  int half = 0;             // the set of parts of t*, sums and counters that it used
+  bool queued = false;      // all its kernels were queued, and its scenarios did not read the rows (no dump)
+  bool one_buffer = false;  // its records went to the first buffer whatever the half
+};
+
 struct fs_model {
   Dims d{};
   int device = 0;
@@ -174,9 +182,9 @@ struct fs_model {
   bool staged = false;  // the staging holds bounds the device copy does not have yet
   int th_bound = -1;    // threshold_bound of the current bounds (-1: not computed yet)
   LaunchCache lc;
-  int half = 0;             // the set of what alternates that the last scoring call used
-  bool rows_read = false;   // the last scoring call's scenarios read the rows (dump)
-  bool one_buffer = false;  // its records went to the first buffer whatever the half
+  Sequence direct;    // calls queued for execution
+  Sequence captured;  // calls recorded by the stream capture capture_id, which run only when its graph does
+  unsigned long long capture_id = 0;
   bool async_before = false;
   // optional timing events: 5 per timed call (before solve, prep, score,
   // finalize, and after finalize); mode 1 records only the two around score
@@ -422,6 +430,25 @@ bool second_records(fs_model* m, size_t need, cudaStream_t s) {
   return rc == FS_OK;
 }
 
+// The sequence an asynchronous call on stream s belongs to. A call under capture
+// does not run now, and its graph may run at any time later, between any two calls:
+// it neither follows the last call queued nor is followed by the next, so the calls
+// of one capture are a sequence of their own (a graph waits for the work before it
+// in its stream, and the work after waits for the graph).
+Sequence& sequence_of(fs_model* m, cudaStream_t s) {
+  cudaStreamCaptureStatus status = cudaStreamCaptureStatusNone;
+  unsigned long long id = 0;
+  if (cudaStreamGetCaptureInfo(s, &status, &id) != cudaSuccess || status == cudaStreamCaptureStatusNone) {
+    (void)cudaGetLastError();  // (a legacy stream while another captures: the launch will say so)
+    return m->direct;
+  }
+  if (id != m->capture_id) {
+    m->capture_id = id;
+    m->captured = Sequence{};
+  }
+  return m->captured;
+}
+
 uint64_t* sums_half(const fs_model* m, int half) {
   return reinterpret_cast<uint64_t*>(static_cast<char*>(m->sums.p) + half * (m->sums.bytes / 512 * 256));
 }
@@ -444,11 +471,13 @@ int run_score(fs_model* m, Set set, const fs_samples* smp, const int32_t* cand_d
   set.d = call_dims(m, m->th_bound);
   int rc = ensure_items(m, n, smp->O);
   if (rc) return rc;
-  if (late) m->half ^= 1;
-  const int half = m->half;
+  Sequence& seq = late ? sequence_of(m, s) : m->direct;
+  if (late) seq.half ^= 1;
+  const int half = seq.half;
   const bool one = !late || !second_records(m, record_bytes(set.d, n, smp->O), s);
-  const int mode = !late || n == 0 || m->rows_read ? 0 : one || m->one_buffer ? 1 : 2;
-  m->one_buffer = one;
+  const int mode = !late || n == 0 || !seq.queued ? 0 : one || seq.one_buffer ? 1 : 2;
+  seq.one_buffer = one;
+  seq.queued = false;
   m->async_before = m->async_before || late;
   float* tables = static_cast<float*>(half && !one ? m->tables2.p : m->tables.p);
   uint64_t* sums = sums_half(m, half);
@@ -470,7 +499,6 @@ int run_score(fs_model* m, Set set, const fs_samples* smp, const int32_t* cand_d
   const bool phases = timed && m->timing == 2;
   if (phases) FS_CUDA(cudaEventRecord(ev[0], s), "record timing event");
   FS_CUDA(launch_thresh(set, m->lc.floors, m->th_bound, s, mode), "launch thresholds");
-  m->rows_read = dump != nullptr;
   if (phases) FS_CUDA(cudaEventRecord(ev[1], s), "record timing event");
   FS_CUDA(launch_prep(set, it, pl, tables, sums, mode == 2 ? 2 : 1, m->sm_count, m->lc, s, m->th_bound), "launch prep");
   if (timed) FS_CUDA(cudaEventRecord(ev[2], s), "record timing event");
@@ -479,6 +507,7 @@ int run_score(fs_model* m, Set set, const fs_samples* smp, const int32_t* cand_d
   FS_CUDA(launch_finalize(set, it, pl, sums, gap, score, gamma_t, best, status_copy,
                           sums + (size_t)std::max(n, 1) * smp->O, sum_out, s),
           "launch finalize");
+  seq.queued = late && !dump;  // (nothing of a synchronous call is left to overlap)
   if (phases) FS_CUDA(cudaEventRecord(ev[4], s), "record timing event");
   return FS_OK;
 }
@@ -737,7 +766,7 @@ int fs_score_candidates(fs_model* m, const fs_samples* smp, double* gap_out, dou
                  dump_dev, sums_mapped ? reinterpret_cast<uint64_t*>(hd + sum_at) : nullptr, s, d_st);
   if (rc) return rc;
   if (sum_bytes && !sums_mapped)
-    FS_CUDA(cudaMemcpyAsync(sum_eo, sums_half(m, m->half), sum_bytes, cudaMemcpyDeviceToHost, s), "read sums");
+    FS_CUDA(cudaMemcpyAsync(sum_eo, sums_half(m, m->direct.half), sum_bytes, cudaMemcpyDeviceToHost, s), "read sums");
   FS_CUDA(cudaStreamSynchronize(s), "synchronize");
   uint32_t st;
   std::memcpy(&st, h + 16 * nn + 32, 4);

@@ -151,3 +151,53 @@ def test_list_written_by_the_call_before(fsb, cuda, oracle_lib, at, S):
                 assert np.array_equal(dev[k].cpu().numpy(), lists[k]), k
                 assert np.array_equal(sums[k].cpu().numpy(), ref[k].sum_eo), k
             assert int(best[0]) == ref[-1].best
+
+
+def _long_plan(w):
+    """Candidates of a call whose scenarios run for milliseconds, its records within the second buffer."""
+    return np.tile(w.candidates, 23)[:1450].astype(np.int32), 8, 1 << 19
+
+
+def test_capture_between_calls(fsb, cuda, oracle_lib):
+    """A call captured between two calls queued without a wait does not run, so
+    the second must keep clear of the first, whose scenarios are still running;
+    the graph gives the captured call's sums later."""
+    torch = cuda
+    w = workloads.make_workload(1)
+    cand, O, S = _long_plan(w)
+    plans = [(cand, S, 1), (w.candidates, 1500, 2), (cand[::-1].copy(), 1500, 3)]  # before, captured, after
+    st = torch.cuda.Stream()
+    with load_model(fsb, w) as m:
+        ref = [fsb.fs_score_candidates(m, c, O, s, seed) for c, s, seed in plans]
+    m = fsb.fs_load_model(w.cap_lo, w.cap_hi, w.tail_lo, w.tail_hi, w.slo, w.demand, w.G, w.K, w.B, stream=st)
+    dev = [torch.from_numpy(c).cuda() for c, _, _ in plans]
+    sums = [torch.zeros((len(c), O), dtype=torch.int64, device="cuda") for c, _, _ in plans]
+
+    def call(k):
+        fsb.fs_score_candidates_async(m, dev[k], O, plans[k][1], plans[k][2], sum_eo_dev=sums[k], stream=st)
+
+    with m:
+        for k in (2, 2, 2):  # buffers of the largest records, both
+            call(k)
+        torch.cuda.synchronize()
+        g = torch.cuda.CUDAGraph()
+        with torch.cuda.stream(st):
+            for _ in range(4):
+                call(0)
+            g.capture_begin()
+            call(1)
+            g.capture_end()
+            running = not st.query()
+            call(2)
+        torch.cuda.synchronize()
+        assert running, "the first call had finished before the capture did: it is too short for this test"
+        assert np.array_equal(sums[0].cpu().numpy(), ref[0].sum_eo)
+        assert np.array_equal(sums[2].cpu().numpy(), ref[2].sum_eo)
+        assert not sums[1].any()
+        with torch.cuda.stream(st):
+            call(2)
+            g.replay()
+            call(0)
+        torch.cuda.synchronize()
+        for k in range(3):
+            assert np.array_equal(sums[k].cpu().numpy(), ref[k].sum_eo), k
