@@ -38,7 +38,8 @@ namespace fs {
 template <bool FL>
 __global__ void __launch_bounds__(kThreshThreads) k_thresh(Set set, int late) {
   const Dims& d = set.d;  // kernel-parameter space: no local copy
-  const int r = blockIdx.y, p = r >> 1, sigma = r & 1;
+  const int r = blockIdx.x, p = r >> 1, sigma = r & 1;
+  const int part = blockIdx.y, n_part = (int)gridDim.y;  // (a replay's realisations may pass 65535: along x)
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   constexpr int kWarps = kThreshThreads / 32;
   __shared__ float sC[256];
@@ -107,7 +108,7 @@ __global__ void __launch_bounds__(kThreshThreads) k_thresh(Set set, int late) {
   const size_t ps = (size_t)p * 2 + sigma;
   float* th = set.theta + ps * d.theta_cap;
   uint16_t* rt = d.K4 * total <= set.rt_cap ? set.rtab + ps * set.rt_cap : nullptr;
-  if (blockIdx.x == 0) {
+  if (part == 0) {
     for (int rho = tid; rho < d.K4; rho += kThreshThreads) {
       set.rowC[ps * d.K4 + rho] = sC[rho];
       set.rowB[ps * d.K4 + rho] = sB[rho];
@@ -122,9 +123,9 @@ __global__ void __launch_bounds__(kThreshThreads) k_thresh(Set set, int late) {
   int lgs = 2;
   while ((1 << lgs) < d.K4 && lgs < 5) ++lgs;
   const int gsz = 1 << lgs, gl = lane & (gsz - 1), per = 32 >> lgs;  // thresholds of a warp at a time
-  const int stride = (int)gridDim.x * kWarps * per;
+  const int stride = n_part * kWarps * per;
   uint32_t best = 0u;  // the largest feasible threshold's bits
-  for (int x0 = ((int)blockIdx.x * kWarps + warp) * per; x0 < total; x0 += stride) {
+  for (int x0 = (part * kWarps + warp) * per; x0 < total; x0 += stride) {
     const int x = min(x0 + (lane >> lgs), total - 1);  // (a spare group repeats the last one)
     int row = 0, hi = d.K4 - 1;
     while (row < hi) {
@@ -182,7 +183,7 @@ __global__ void __launch_bounds__(kThreshThreads) k_thresh(Set set, int late) {
     best = __reduce_max_sync(0xffffffffu, best);
     if (lane == 0) atomicMax(&s_best, best);
     __syncthreads();
-    if (tid == 0) set.tpart[sigma * gridDim.x + blockIdx.x] = __uint_as_float(s_best);
+    if (tid == 0) set.tpart[sigma * n_part + part] = __uint_as_float(s_best);
   }
   if (late) {
     pdl_wait();
@@ -220,7 +221,7 @@ cudaError_t launch_thresh(Set& set, int floors, int th_bound, cudaStream_t s, in
   const int per_block = 2 * (kThreshThreads / gsz);
   const int nb = set.P > 1 ? 1 : std::max(1, std::min(kThreshBlocks, (bound + per_block - 1) / per_block));
   set.n_tpart = set.tpart ? nb : 0;
-  return launch_pdl(floors ? k_thresh<true> : k_thresh<false>, dim3(nb, 2 * set.P), dim3(kThreshThreads), 0, s, set,
+  return launch_pdl(floors ? k_thresh<true> : k_thresh<false>, dim3(2 * set.P, nb), dim3(kThreshThreads), 0, s, set,
                     late);
 }
 

@@ -127,3 +127,21 @@ def test_policy_comparison_runs(fsb, cuda):
     s = compare.summarise(runs["fleetsieve"], runs["uniform_random"], n_boot=200)
     lo, hi = s["ci95"]
     assert lo <= s["advantage"] <= hi and len(s["per_class"]) == w.K
+
+
+def test_replay_more_streams_than_a_grid_dimension(fsb, cuda, oracle_lib):
+    """Streams whose realisations (two each) outnumber the 65535 blocks that a
+    grid holds along y or z."""
+    rng = np.random.default_rng(3)
+    n, w = 32800, workloads.random_small(rng, 1, 2, 4)
+    u = rng.random((2, n, w.cells)).astype(np.float32)
+    cap, tail = (lo.reshape(-1) + (hi - lo).reshape(-1) * x
+                 for lo, hi, x in ((w.cap_lo, w.cap_hi, u[0]), (w.tail_lo, w.tail_hi, u[1])))
+    perm = rng.permuted(np.tile(np.arange(w.cells, dtype=np.int32), (n, 1)), axis=1)
+    rp = workloads.Replay(w, cap, tail, perm, 1, 0.01, 3)
+    q = oracle_lib.triangular_table(8)
+    with load_model(fsb, w, quantile=q) as m:
+        res = fsb.fs_replay(m, cap, tail, perm, rp.r0, rp.eps, 2, 4, 11, rp.max_rounds)
+    assert len(set(res.rounds)) > 1  # (some go on, some stop)
+    for k in list(range(0, n, 1093)) + [32767, 32768, n - 1]:
+        _compare(fsb, res, rp, k, oracle_lib.replay_stream(rp, k, q, seed=11, S=4, O=2), w.K)
