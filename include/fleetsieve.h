@@ -30,7 +30,9 @@
  *     *_async / *_batch take device pointers and a cudaStream_t (as void*),
  *     enqueue their work and return; fs_check() synchronises such a stream and
  *     reports device-side errors;
- *   - one fs_model is not thread-safe; separate models are independent.
+ *   - one fs_model is not thread-safe; separate models are independent. A
+ *     model's calls share its device state: a caller that queues them on
+ *     several streams orders each after the one before (an event, or a wait).
  */
 #ifndef FLEETSIEVE_H
 #define FLEETSIEVE_H
@@ -104,7 +106,8 @@ int fs_load_model(const fs_bounds *bounds, const float *slo, const float *demand
  * capacity and tail intervals"). Revealed flags are kept. The arrays are
  * copied (into page-locked staging) before the call returns, which queues no
  * device work: the next call that needs the bounds on the device queues their
- * copy on the model's stream (work it queues on another stream waits for it),
+ * copy on the model's stream, after the work already queued on its own stream
+ * (which reads the old bounds; what it queues there then waits for the copy),
  * and fs_score_candidates reads freshly staged bounds where they are. Every
  * later call on the model sees the new bounds.
  */

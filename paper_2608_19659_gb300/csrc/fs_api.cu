@@ -177,7 +177,7 @@ struct fs_model {
   // page-locked staging: the last bounds upload (its copy may still be in
   // flight until up_done), and a synchronous call's outputs and status word
   HostBuf h_up, h_out;
-  cudaEvent_t up_done = nullptr, round_done = nullptr;  // (created on first use)
+  cudaEvent_t up_done = nullptr, read_done = nullptr, round_done = nullptr;  // (created on first use)
   bool up_pending = false;
   bool staged = false;  // the staging holds bounds the device copy does not have yet
   int th_bound = -1;    // threshold_bound of the current bounds (-1: not computed yet)
@@ -301,10 +301,30 @@ int threshold_bound(const fs_model* m) {
   return (int)std::min<long long>(most, d.theta_cap);
 }
 
+// The model's stream goes on once the work queued on s has finished: earlier calls
+// there may still read what is about to be written on the model's stream. (The
+// calls before them on other streams had to finish first: a model's calls share its
+// device state. Not while s is being captured: a capture waits for no such copy.)
+int wait_for_readers(fs_model* m, cudaStream_t s) {
+  if (s == m->stream) return FS_OK;
+  cudaStreamCaptureStatus status = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(s, &status) != cudaSuccess || status != cudaStreamCaptureStatusNone) {
+    (void)cudaGetLastError();
+    return FS_OK;
+  }
+  if (!m->read_done) FS_CUDA(cudaEventCreateWithFlags(&m->read_done, cudaEventDisableTiming), "create read event");
+  FS_CUDA(cudaEventRecord(m->read_done, s), "record read event");
+  FS_CUDA(cudaStreamWaitEvent(m->stream, m->read_done, 0), "order after the readers");
+  return FS_OK;
+}
+
 // Queue the device copy of staged bounds (if any) on the model's stream without
-// waiting, and order work on stream s after the last such copy.
+// waiting, after the work queued on s, and order work on stream s after the last
+// such copy.
 int flush_bounds(fs_model* m, cudaStream_t s) {
   if (m->staged) {
+    int rc = wait_for_readers(m, s);
+    if (rc) return rc;
     const size_t span = (size_t)(reinterpret_cast<char*>(m->set.revealed) - reinterpret_cast<char*>(m->set.bounds)) +
                         m->h_revealed.size();
     FS_CUDA(cudaMemcpyAsync(m->set.bounds, m->h_up.p, span, cudaMemcpyHostToDevice, m->stream), "upload bounds");
@@ -1240,6 +1260,7 @@ void fs_free_model(fs_model* m) {
   m->replay.release();
   for (cudaEvent_t e : m->ev) cudaEventDestroy(e);
   if (m->up_done) cudaEventDestroy(m->up_done);
+  if (m->read_done) cudaEventDestroy(m->read_done);
   if (m->round_done) cudaEventDestroy(m->round_done);
   m->h_up.release();
   m->h_out.release();
