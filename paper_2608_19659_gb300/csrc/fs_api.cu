@@ -179,6 +179,7 @@ struct fs_model {
   HostBuf h_up, h_out;
   cudaEvent_t up_done = nullptr, read_done = nullptr, round_done = nullptr;  // (created on first use)
   bool up_pending = false;
+  bool other_stream = false;  // calls were queued on another stream than the model's since the floors were set
   bool staged = false;  // the staging holds bounds the device copy does not have yet
   int th_bound = -1;    // threshold_bound of the current bounds (-1: not computed yet)
   LaunchCache lc;
@@ -320,8 +321,9 @@ int wait_for_readers(fs_model* m, cudaStream_t s) {
 
 // Queue the device copy of staged bounds (if any) on the model's stream without
 // waiting, after the work queued on s, and order work on stream s after the last
-// such copy.
+// such copy. Every call on a stream of the caller's starts with it.
 int flush_bounds(fs_model* m, cudaStream_t s) {
+  m->other_stream = m->other_stream || s != m->stream;
   if (m->staged) {
     int rc = wait_for_readers(m, s);
     if (rc) return rc;
@@ -744,7 +746,10 @@ int fs_set_floors(fs_model* m, const float* floor) {
     }
   m->h_dlt = v;
   // a small copy, finished before the call returns: every later call on any
-  // stream sees the new floors (they follow the SLOs on the device)
+  // stream sees the new floors (they follow the SLOs on the device), and every
+  // earlier one has read the old
+  if (m->other_stream) FS_CUDA(cudaDeviceSynchronize(), "wait for the queued calls");
+  m->other_stream = false;
   FS_CUDA(cudaMemcpyAsync((void*)(m->set.slo + K), m->h_dlt.data(), 4 * (size_t)K, cudaMemcpyHostToDevice,
                           m->stream),
           "upload floors");

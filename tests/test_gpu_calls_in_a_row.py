@@ -203,28 +203,35 @@ def test_capture_between_calls(fsb, cuda, oracle_lib):
             assert np.array_equal(sums[k].cpu().numpy(), ref[k].sum_eo), k
 
 
-def test_bounds_replaced_while_calls_run_on_another_stream(fsb, cuda, oracle_lib):
-    """The model's stream is not the one its calls are queued on: new bounds
-    reach the device only once the calls queued with the old ones have read them."""
+@pytest.mark.parametrize("what", ["bounds", "floors"])
+def test_inputs_replaced_while_calls_run_on_another_stream(fsb, cuda, oracle_lib, what):
+    """The model's stream is not the one its calls are queued on: new bounds and
+    floors reach the device only once the calls queued with the old have read them."""
     torch = cuda
-    w = workloads.make_workload(1)
-    w2 = dataclasses.replace(w, cap_lo=w.cap_lo * np.float32(0.5), cap_hi=w.cap_hi * np.float32(0.75))
+    w = dataclasses.replace(workloads.make_workload(1), floor=np.array([0.125, 0.0], np.float32))
+    if what == "bounds":
+        w2 = dataclasses.replace(w, cap_lo=w.cap_lo * np.float32(0.5), cap_hi=w.cap_hi * np.float32(0.75))
+    else:
+        w2 = dataclasses.replace(w, floor=np.array([0.0, 1.0], np.float32))
     cand, O, S = _long_plan(w)
     st = torch.cuda.Stream()
     with load_model(fsb, w2) as m:
         ref2 = fsb.fs_score_candidates(m, w.candidates, O, 1500, 5)
     with load_model(fsb, w) as m:  # (on the default stream)
         ref = fsb.fs_score_candidates(m, cand, O, S, 5)
+        assert not np.array_equal(fsb.fs_score_candidates(m, w.candidates, O, 1500, 5).sum_eo, ref2.sum_eo)
         dev = [torch.from_numpy(c).cuda() for c in (cand, w.candidates)]
         sums = [torch.zeros((len(cand), O), dtype=torch.int64, device="cuda") for _ in range(4)]
         sums2 = torch.zeros((len(w.candidates), O), dtype=torch.int64, device="cuda")
         torch.cuda.synchronize()
         for x in sums:
             fsb.fs_score_candidates_async(m, dev[0], O, S, 5, sum_eo_dev=x, stream=st)
-        fsb.fs_update_bounds(m, w2.cap_lo, w2.cap_hi, w2.tail_lo, w2.tail_hi)
+        if what == "bounds":
+            fsb.fs_update_bounds(m, w2.cap_lo, w2.cap_hi, w2.tail_lo, w2.tail_hi)
+        else:
+            fsb.fs_set_floors(m, w2.floor)
         fsb.fs_score_candidates_async(m, dev[1], O, 1500, 5, sum_eo_dev=sums2, stream=st)
         fsb.fs_check(m, st)
     for x in sums:
         assert np.array_equal(x.cpu().numpy(), ref.sum_eo)
-    assert np.array_equal(sums2.cpu().numpy(), ref2.sum_eo) and ref2.sum_eo.any()
-    assert not np.array_equal(ref2.sum_eo, ref.sum_eo[:len(w.candidates)])
+    assert np.array_equal(sums2.cpu().numpy(), ref2.sum_eo)
