@@ -17,6 +17,7 @@
 #include <nvtx3/nvToolsExt.h>
 
 #include "fs_internal.cuh"
+#include "fs_optional_buf.h"
 
 namespace fs {
 
@@ -112,6 +113,17 @@ struct Buf {
   }
 };
 
+// Device memory for what calls can do without: a refusal is no error.
+struct QuietDevice {
+  static void* alloc(size_t bytes) {
+    void* p = nullptr;
+    if (cudaMalloc(&p, bytes) == cudaSuccess) return p;
+    (void)cudaGetLastError();
+    return nullptr;
+  }
+  static void free(void* p) { cudaFree(p); }
+};
+
 // Page-locked host memory that grows on demand, mapped into the device's
 // address space: copies to and from it are asynchronous, so a call can queue
 // them and wait once, and kernels can read and write it directly (dev).
@@ -167,7 +179,8 @@ struct fs_model {
   Set set{};
   // per-call scratch
   Buf real, lex, gp;
-  Buf tables, tables2, sums;  // records (two buffers) and sums (two halves): asynchronous calls alternate (launch_thresh)
+  Buf tables, sums;  // records (in two buffers) and sums (two halves): asynchronous calls alternate (launch_thresh)
+  OptionalBuf<QuietDevice> tables2;
   Buf replay;     // fs_replay's state of every stream (grown on demand, kept)
   int objective = FS_OBJECTIVE_MAXMIN;  // FS_OBJECTIVE_LEXICOGRAPHIC: fs_solve* and the certificate to tier 4
   // host mirrors
@@ -409,8 +422,8 @@ Dims call_dims(const fs_model* m, int th_bound) {
 // second buffer of records, of the first's size up to kSecondRecords, comes with
 // the model's second asynchronous call (a first call alone has no use for it, and
 // would pay for its allocation: 55 -> 150 us from 1 MB on), never while the stream
-// is being captured. Calls whose records do not fit it use the first (1024 x 16 x
-// 16384 scenarios without it: 208 us instead of 204).
+// is being captured. Calls whose records do not fit it, or find no memory for it,
+// use the first (1024 x 16 x 16384 scenarios without it: 208 us instead of 204).
 constexpr size_t kSecondRecords = 32u << 20;
 
 size_t record_bytes(const Dims& d, int n, int O) {
@@ -425,9 +438,8 @@ int ensure_items(fs_model* m, int n, int O) {
     if (rc) return rc;
     // the second buffer grows with the first and at no other time: what a
     // captured graph holds of either stays while the other does
-    // (and is optional: without memory for it, calls use the first)
-    if (m->tables2.p && m->tables2.ensure(std::min(full, kSecondRecords), "candidate records"))
-      (void)cudaGetLastError();
+    m->tables2.retry();
+    if (m->tables2.p) m->tables2.ensure(std::min(full, kSecondRecords));
   }
   // sums, then the split reduction's scratch (2 words per block)
   return m->sums.ensure(2 * align_up((size_t)std::max(n, 1) * O * 8 + 16 * (size_t)kFinalizeMaxBlocks, 256), "sums");
@@ -437,7 +449,7 @@ int ensure_items(fs_model* m, int n, int O) {
 // of it on stream s: whether it is there.
 bool second_records(fs_model* m, size_t need, cudaStream_t s) {
   if (m->tables2.p) return m->tables2.bytes >= need;
-  if (!m->async_before || need > kSecondRecords) return false;
+  if (!m->async_before || need > kSecondRecords || m->tables2.declined) return false;
   cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
   if (cudaStreamIsCapturing(s, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) {
     (void)cudaGetLastError();  // (a legacy stream while another captures: not now)
@@ -446,10 +458,9 @@ bool second_records(fs_model* m, size_t need, cudaStream_t s) {
   // relaxed: an allocation here must not end a capture that another thread makes
   cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
   if (cudaThreadExchangeStreamCaptureMode(&mode) != cudaSuccess) return false;
-  const int rc = m->tables2.ensure(std::min(m->tables.bytes, kSecondRecords), "candidate records");
+  const bool there = m->tables2.ensure(std::min(m->tables.bytes, kSecondRecords));
   (void)cudaThreadExchangeStreamCaptureMode(&mode);
-  if (rc) (void)cudaGetLastError();
-  return rc == FS_OK;
+  return there;
 }
 
 // The sequence an asynchronous call on stream s belongs to. A call under capture
