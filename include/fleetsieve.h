@@ -192,7 +192,18 @@ int fs_score_candidates(fs_model *m, const fs_samples *samples, double *gap_out,
                         double *score_out, float *gamma_t, int32_t *best, int64_t *sum_eo,
                         void *dump_dev);
 
-/* Same with samples->cand and every output on the device, enqueued on cuda_stream. */
+/*
+ * Same with samples->cand and every output on the device, enqueued on cuda_stream.
+ * Device memory: a call with more candidates or outcomes than any before it on the
+ * model allocates room for its candidates' records (4 n I bytes, as given at
+ * fs_score_candidates_noalloc) and sums (16 n O bytes). The second call of this kind
+ * on a model that is not being captured also allocates a second buffer for records,
+ * as large as the first but at most 32 MiB: a call whose records fit it starts
+ * before the one before has finished. (A loop that must not allocate is preceded by
+ * two calls of its largest plan. Without memory for the second buffer every call
+ * uses the first.) A call can be captured into a CUDA graph once no allocation and
+ * no upload of new bounds is left to do.
+ */
 int fs_score_candidates_async(fs_model *m, const fs_samples *samples, double *gap_dev,
                               double *score_dev, float *gamma_t_dev, int32_t *best_dev,
                               int64_t *sum_eo_dev, void *dump_dev, void *cuda_stream);
