@@ -294,7 +294,7 @@ static __device__ __noinline__ int min_replicas_ieee(float t, float c, float lam
 // (row_in_range(c, lam) and M >= 1)
 __device__ __forceinline__ int min_replicas_fast(float t, float c, float lam, float rlam, float M) {
   const float y = ceilf(__fdividef(__fmul_rn(t, lam), c));  // estimate only (c == 0: infinite)
-  float n = fminf(fmaxf(y, 1.0f), M);
+  float n = fmaxf(fminf(y, M), 1.0f);  // (0 / 0, no capacity and t lambda underflowed: M, which fails)
   while (n > 1.0f && fulfil_fast(n - 1.0f, c, lam, rlam) >= t) n -= 1.0f;
   while (n <= M && fulfil_fast(n, c, lam, rlam) < t) n += 1.0f;
   return n <= M ? (int)n : 0;

@@ -6,6 +6,7 @@ capacities outside the fast quotient's range, thresholds far below 1. Every
 comparison is bit for bit."""
 
 import dataclasses
+import time
 
 import numpy as np
 import pytest
@@ -69,3 +70,24 @@ def test_scoring_thresholds(fsb, cuda, oracle_lib, K, B, G, demand, ties, floors
     assert r.gamma_t == ref.gamma_t and np.array_equal(r.sum_eo, ref.sum_eo)
     assert np.array_equal(r.score, ref.score) and r.best == ref.best
     assert np.array_equal(many.sum_eo, np.tile(ref.sum_eo, (400, 1)))
+
+
+def test_no_capacity_and_a_small_demand(fsb, cuda, oracle_lib):
+    """Rows without capacity whose smallest threshold times the demand underflows
+    (demand 0.25; not at 1.0) are dismissed at once, not after a walk over all
+    replica counts, in the solver and in a scoring call's thresholds."""
+    w = workloads.random_small(np.random.default_rng(1), 1, 2, 8700, p_infeasible=0.0)
+    zero = np.zeros_like(w.cap_lo)
+    us = {}
+    for lam in (1.0, 0.25):
+        x = dataclasses.replace(w, cap_lo=zero, cap_hi=zero, demand=np.array([lam], np.float32), O=4, S=6)
+        with load_model(fsb, x) as m:
+            t = []
+            for _ in range(30):
+                a = time.perf_counter()
+                am, _, gt = fsb.fs_solve_bounds(m)
+                r = fsb.fs_score_candidates(m, x.candidates[:4], x.O, x.S, 1)
+                t.append(time.perf_counter() - a)
+        assert am["t_star"] == 0.0 and gt == 0.0 and not r.sum_eo.any()
+        us[lam] = 1e6 * sorted(t)[len(t) // 2]
+    assert us[0.25] < 1.5 * us[1.0], us  # (51 us both; with the walk 622)
