@@ -376,7 +376,12 @@ int fs_set_objective(fs_model *m, int32_t objective);
  * Needs sum_i lambda_i <= 2^20 req/s, G <= 1024, (K + 1)(G + 1) <= 4 Mi and
  * Q / O <= 4096 (2048 under the monotone prior: a segment's table of
  * positions lives in shared memory) (FS_EINVAL otherwise). Synchronous.
- * Independent of fs_set_objective.
+ * Independent of fs_set_objective. Device memory: records and sums as for
+ * fs_score_candidates_async, and 16 (G + 5) (T + 2) K bytes of tables of the other
+ * classes' goodput (T as given at fs_score_candidates_noalloc: 41 kB at K = 2,
+ * G = 16, 128 MB at K = 8, G = 256), but at most 512 MiB of them, or one class's
+ * share where that is more (the classes are then taken in several passes). The model
+ * keeps them; new bounds never make a call allocate.
  */
 int fs_score_goodput(fs_model *m, const fs_samples *samples, double *gap_out, double *score_out,
                      double *gamma_gp, int32_t *best, int64_t *sum_eo);

@@ -980,8 +980,9 @@ int fs_score_goodput(fs_model* m, const fs_samples* smp, double* gap_out, double
   const Plan pl = make_plan(set.d, smp);
   if (pl.W > (m->set.prior == 1 ? 2048 : 4096))  // a segment's table of positions lives in shared memory
     return fail(FS_EINVAL, "the goodput stage needs Q / O <= 2048 under the monotone prior, 4096 otherwise");
-  // the rows wanted and the base goodputs, then the pool of rows
-  const size_t rows = goodput_pool_rows(m->d, m->th_bound, kGoodputPoolMax);
+  // the rows wanted and the base goodputs, then the pool of rows (for any bounds of
+  // the model, so that new ones never make a later call allocate)
+  const size_t rows = goodput_pool_rows(m->d, kGoodputPoolMax);
   const size_t head = align_up(8 * (size_t)kGoodputSpanInts + 16 * (nn + 1), 256);
   if ((rc = m->gp.ensure(head + rows * goodput_row_bytes(m->d), "goodput tables"))) return rc;
   int* span = static_cast<int*>(m->gp.p);

@@ -558,7 +558,7 @@ cudaError_t launch_solve_lex(const Set& set, int n, const float* cap_x, const fl
 // want, or as many whole classes' as most_bytes holds, at least one's: the
 // scorer then takes the classes in several passes).
 constexpr size_t kGoodputPoolMax = 512u << 20;
-size_t goodput_pool_rows(const Dims& d, int th_bound, size_t most_bytes);
+size_t goodput_pool_rows(const Dims& d, size_t most_bytes);
 size_t goodput_row_bytes(const Dims& d);
 constexpr int kGoodputSpanInts = 4 * FS_MAX_CLASSES;  // wanted rows per (realisation, class): least, most
 cudaError_t launch_score_goodput(const Set& set, const Items& it, const Plan& pl, const float* tables,

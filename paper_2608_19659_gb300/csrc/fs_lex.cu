@@ -969,8 +969,8 @@ static long long goodput_rows_per_class(const Dims& d, int th_bound) {
   return 2LL * (bound + 2);
 }
 
-size_t goodput_pool_rows(const Dims& d, int th_bound, size_t most_bytes) {
-  const long long per = goodput_rows_per_class(d, th_bound);
+size_t goodput_pool_rows(const Dims& d, size_t most_bytes) {
+  const long long per = goodput_rows_per_class(d, d.theta_cap);
   const long long row = 8LL * (d.G + 1 + kT);
   long long classes = (long long)most_bytes / (per * row);
   classes = classes < 1 ? 1 : classes > d.K ? d.K : classes;

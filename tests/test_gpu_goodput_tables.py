@@ -50,3 +50,19 @@ def test_goodput_pool_in_passes(fsb, cuda, oracle_lib):
     lam = rng.uniform(600.0, 900.0, 8).astype(np.float32)
     w = dataclasses.replace(w, demand=lam, O=4, S=3, candidates=np.array([0, 13, 37, 63], np.int32))
     _check(fsb, oracle_lib, w)
+
+
+def test_new_bounds_allocate_nothing(fsb, cuda, oracle_lib):
+    """A goodput call after one of the same plan takes no device memory, however
+    many more thresholds its bounds have (some 90 a realisation, then 1200)."""
+    torch = cuda
+    w = workloads.random_small(np.random.default_rng(2), 8, 2, 256, p_infeasible=0.0)
+    w = dataclasses.replace(w, candidates=w.candidates[:5].copy(), O=4, S=3, demand=np.full(8, 60.0, np.float32))
+    many = dataclasses.replace(w, cap_lo=w.cap_lo * np.float32(200), cap_hi=w.cap_hi * np.float32(200))
+    with load_model(fsb, many) as m:
+        fsb.fs_score_goodput(m, w.candidates, w.O, w.S, w.seed)
+        before = torch.cuda.mem_get_info()[0]
+        fsb.fs_update_bounds(m, w.cap_lo, w.cap_hi, w.tail_lo, w.tail_hi)
+        r = fsb.fs_score_goodput(m, w.candidates, w.O, w.S, w.seed)
+        assert torch.cuda.mem_get_info()[0] == before
+    assert np.array_equal(r.sum_eo, oracle_lib.score_goodput(w, oracle_lib.triangular_table(4096)).sum_eo)
