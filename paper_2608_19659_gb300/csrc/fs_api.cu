@@ -495,7 +495,6 @@ int run_score(fs_model* m, Set set, const fs_samples* smp, const int32_t* cand_d
   it.n = n;
   it.p = nullptr;
   it.cell = cand_dev;
-  it.off = nullptr;
   // What alternates between calls (launch_thresh): the other half (the records'
   // other buffer) in an asynchronous call, which may start before the last call
   // has finished, the same in a synchronous one, which waits for it. Without a
@@ -1143,7 +1142,6 @@ int fs_replay(fs_model* m, const fs_replay_spec* sp, int32_t* rounds, int32_t* s
       it.n = n_items;
       it.p = rs.item_p;
       it.cell = rs.item_cell;
-      it.off = nullptr;
       fs_samples smp{sp->seed, 0, (uint32_t)r, n_items, sp->O, sp->S, 0, nullptr};
       Plan pl = make_plan(m->d, &smp);
       pl.few = few_path(pl, n_items) ? 1 : 0;

@@ -209,7 +209,6 @@ struct Items {
   int n;
   const int* p;         // [n] problem of the item, nullptr = all problem 0
   const int* cell;      // [n] candidate cell
-  const int* off;       // [P + 1] item range of each problem (grouped by problem)
 };
 
 // ---------------------------------------------------------------- arithmetic

@@ -1311,18 +1311,14 @@ __global__ void k_finalize(Set set, Items it, Plan pl, const uint64_t* sums, dou
                            float* gamma_t, int32_t* best, uint32_t* status_copy, uint64_t* sum_out) {
   pdl_trigger();
   pdl_wait();
-  const int p = blockIdx.x;
-  const int beg = it.off ? it.off[p] : 0;
-  const int end = it.off ? it.off[p + 1] : it.n;
-  const Best b = finalize_problem(set, it, pl, sums, p, beg, end, gap, score, gamma_t ? gamma_t + p : nullptr, beg,
-                                  sum_out);
-  if (threadIdx.x == 0 && best) best[p] = b.valid() ? b.cell : -1;
+  const Best b = finalize_problem(set, it, pl, sums, 0, 0, it.n, gap, score, gamma_t, 0, sum_out);
+  if (threadIdx.x == 0 && best) *best = b.valid() ? b.cell : -1;
   // every kernel of the call has finished (stream order, and the wait above):
   // its status word can travel with the outputs
-  if (threadIdx.x == 0 && p == 0 && status_copy) *status_copy = *set.status;
+  if (threadIdx.x == 0 && status_copy) *status_copy = *set.status;
 }
 
-// One problem with many candidates, split over the CTAs: each writes its
+// Many candidates, split over the CTAs: each writes its
 // candidates' expectations and scores and its best entry into part[2 b ..],
 // and the last to finish (a ticket in work[1], zeroed by k_prep) reduces them.
 __global__ void k_finalize_split(Set set, Items it, Plan pl, const uint64_t* sums, double* gap, double* score,
@@ -1508,7 +1504,7 @@ cudaError_t launch_score(const Set& set, const Items& it, const Plan& pl, const 
 }
 
 int finalize_blocks(const Items& it) {
-  if (it.off || it.n <= 256) return 0;
+  if (it.n <= 256) return 0;
   return std::min(kFinalizeMaxBlocks, (it.n + 63) / 64);  // four lanes per candidate: one pass of a block
 }
 
@@ -1519,7 +1515,7 @@ cudaError_t launch_finalize(const Set& set, const Items& it, const Plan& pl, con
   if (nb > 0 && part)
     return launch_pdl(k_finalize_split, dim3(nb), dim3(256), 0, s, set, it, pl, sums, gap, score, gamma_t, best,
                       status_copy, part, sum_out);
-  return launch_pdl(k_finalize, dim3(it.off ? set.P : 1), dim3(256), 0, s, set, it, pl, sums, gap, score, gamma_t,
+  return launch_pdl(k_finalize, dim3(1), dim3(256), 0, s, set, it, pl, sums, gap, score, gamma_t,
                     best, status_copy, sum_out);
 }
 

@@ -174,7 +174,6 @@ extern "C" int fs_score_candidates_noalloc(int32_t K, int32_t B, int32_t G, cons
   it.n = n;
   it.p = nullptr;
   it.cell = smp->cand;
-  it.off = nullptr;
   Plan pl{};
   pl.key0 = (uint32_t)smp->seed;
   pl.key1 = (uint32_t)(smp->seed >> 32);
