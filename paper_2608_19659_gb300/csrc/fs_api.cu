@@ -573,9 +573,9 @@ int solve_lex_pass(fs_model* m, const Set& set, int n, const float* cap_x, const
 // memory that the last kernel writes, so no copy follows it, and the inputs are
 // read from mapped memory where they were staged (measured against device copies
 // of them: fs_solve_bounds after an update 21.8 against 23.3 us at 64 cells, 30.6
-// against 34.6 at 1024, 219 against 475 at 262,144; with the pageable result
-// copies that stood here before, about 35 us at 64). cap_x, tail_x as
-// for launch_solve; `at`: bytes of h_out the caller uses before the results.
+// against 34.6 at 1024, 219 against 475 at 262,144; with pageable result copies
+// about 35 us at 64). cap_x, tail_x as for launch_solve; `at`: bytes of h_out the
+// caller uses before the results.
 int solve_to_host(fs_model* m, const Set& set, int n, const float* cap_x, const float* tail_x, fs_allocation* out,
                   size_t at, fs_allocation* result) {
   HostOut host;

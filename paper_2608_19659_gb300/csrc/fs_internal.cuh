@@ -288,8 +288,8 @@ static __device__ __noinline__ int min_replicas_ieee(float t, float c, float lam
 }
 
 // In range, the answer is reached from the estimate by steps of one: two
-// fulfilments when the estimate is right (the bracket of seven tested at once
-// that stood here before took 2.5 times the instructions).
+// fulfilments when the estimate is right (a bracket of seven tested at once takes
+// 2.5 times the instructions).
 // (row_in_range(c, lam) and M >= 1)
 __device__ __forceinline__ int min_replicas_fast(float t, float c, float lam, float rlam, float M) {
   const float y = ceilf(__fdividef(__fmul_rn(t, lam), c));  // estimate only (c == 0: infinite)

@@ -169,11 +169,10 @@ constexpr size_t kLexCellsWide = 128 * 1024;
 // sum m_i can be spent freely, and S_i is needed (and reachable) for h = 0..slack
 // GPUs above the cheapest options of classes i..K-1. An option of cost c takes e
 // = c - m_i of them. Where t* is tight the slack is a few GPUs and a class's
-// options with e <= slack are few; the table over all of [0, G] that stood here
-// before, with a division per option and cell, took 66 us on 1000 realisations of
-// the four-class, 64-GPU grid and 180 us on two of the eight-class, 256-GPU one
-// (its last step, the walk forward, one thread's); measured now: see
-// launch_solve_lex.
+// options with e <= slack are few. A table over all of [0, G] with a division per
+// option and cell, and one thread's walk forward, takes 66 us on 1000 realisations
+// of the four-class, 64-GPU grid and 180 us on two of the eight-class, 256-GPU one
+// (this one: see launch_solve_lex).
 template <bool PACK, int NW>
 __global__ void __launch_bounds__(NW == 1 ? 128 : 32 * NW) k_solve_lex(Set set, int n_real, const float* cap_x,
                                                                        const float* tail_x, fs_allocation* out_x,
@@ -1007,9 +1006,9 @@ cudaError_t launch_score_goodput(const Set& set, const Items& it, const Plan& pl
   // evens them out
   const long long n_seg = (long long)it.n * pl.O;
   // beyond a few waves of blocks the closed-gate goodputs are evaluated once per
-  // candidate rather than by each of its segments (294 us in all on the largest
-  // call with them and the block-wide k_other, 352 us before both; 1.2 us more of
-  // a launch on the paper-scale one, whose 512 segments are one wave)
+  // candidate rather than by each of its segments (with the block-wide k_other 294 us
+  // in all on the largest call, 352 us without both; 1.2 us more of a launch on the
+  // paper-scale one, whose 512 segments are one wave)
   gt.closed = !rf && n_seg > 8LL * sm_count ? base + 2 : nullptr;
   const unsigned grid = (unsigned)(n_seg < 0x7fffffffLL ? n_seg : 0x7fffffffLL);
   // many segments: 128 threads (a segment's set-up is paid by fewer; the largest call

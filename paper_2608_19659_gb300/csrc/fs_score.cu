@@ -1318,9 +1318,9 @@ __global__ void k_finalize(Set set, Items it, Plan pl, const uint64_t* sums, dou
   if (threadIdx.x == 0 && status_copy) *status_copy = *set.status;
 }
 
-// Many candidates, split over the CTAs: each writes its
-// candidates' expectations and scores and its best entry into part[2 b ..],
-// and the last to finish (a ticket in work[1], zeroed by k_prep) reduces them.
+// Many candidates, split over the CTAs: each writes its candidates' expectations and
+// scores and its best entry into part[2 b ..], and the last to finish (a ticket in
+// work[1], zeroed by k_prep) reduces them.
 __global__ void k_finalize_split(Set set, Items it, Plan pl, const uint64_t* sums, double* gap, double* score,
                                  float* gamma_t, int32_t* best, uint32_t* status_copy, uint64_t* part,
                                  uint64_t* sum_out) {

@@ -24,9 +24,8 @@
 // are met when those fit in G together; with t* = 0 and the floors met, that
 // cover is the class's allocation.
 // What bounds it: the dependent chain of about a dozen probes (latency for a
-// few realisations, issue slots for a batch). Before, a 256-thread block per
-// realisation listed and sorted the thresholds first; measured: see
-// launch_solve.
+// few realisations, issue slots for a batch). Measured, against a 256-thread block
+// per realisation that lists and sorts the thresholds: see launch_solve.
 #include <cuda_runtime.h>
 
 #include <cstddef>

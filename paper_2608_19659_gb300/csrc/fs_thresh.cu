@@ -20,11 +20,9 @@
 //
 // What bounds it: dependent latencies (the cells' loads, a row's two covers,
 // one cover per row and threshold); every block finds the rows for itself (a
-// few kB from L2) rather than wait for another to hand them over. Before, one
-// block per realisation sorted the values and probed them (20 us on the
-// eight-class, 256-GPU grid, whose tables above 8192 words it left out, so that
-// the preparation searched for each candidate: 60 us); measured now: see
-// launch_thresh.
+// few kB from L2) rather than wait for another to hand them over. One block per
+// realisation that sorts the values and probes them takes 19 us on the
+// eight-class, 256-GPU grid against 7 (launch_thresh).
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -192,8 +190,9 @@ __global__ void __launch_bounds__(kThreshThreads) k_thresh(Set set, int late) {
 }
 
 // Measured (one GB300, calls in a row): the eight-class, 256-GPU grid (about 1300
-// thresholds a realisation, 55 blocks each) 19.2 -> 7.3 us, and with its tables
-// the preparation of 1024 candidates 60.6 -> 14 us: 1024 x 16 x 16384 scenarios
+// thresholds a realisation, 55 blocks each) 19.2 -> 7.3 us; with its tables, which
+// one block left out above 8192 words, so that the preparation searched for each
+// candidate, the preparation of 1024 candidates 60.6 -> 14 us: 1024 x 16 x 16384 scenarios
 // 270 -> 206 us, 1024 x 8 x 60 116 -> 51 us; four classes, 64 GPUs 51 -> 45 us.
 //
 // late: for a scoring call n on the model's own device bounds, of at least one
@@ -202,15 +201,19 @@ __global__ void __launch_bounds__(kThreshThreads) k_thresh(Set set, int late) {
 // was itself let start by the scenarios, after call n - 1's preparation and so
 // (each waits for its predecessor) its thresholds had finished, which had waited
 // for call n - 2's reduction. So
-//   - the bounds are only written by copies (a full barrier in the stream);
+//   - the bounds are only written by copies, which are ordered after the calls
+//     queued before them (a full barrier in the stream, flush_bounds on another);
 //   - thresholds, rows and tables have no reader left: the preparation of call n -
 //     1 was the last (a dump's scenarios read rows: not late after one; the goodput
 //     stage and the replay are synchronous);
-//   - the parts of t*, the sums, the counters and (late 2: both calls' records fit
-//     a half of their buffer) the records, which call n - 1 still uses, alternate
-//     between two sets, call n - 2's being free.
+//   - the parts of t*, the sums and the counters, which call n - 1 still uses,
+//     alternate between two sets, call n - 2's being free;
+//   - late 2: so do the records, between two buffers (both calls' fit the second).
+//     Late 1: one of them keeps its records in the first buffer whatever its turn,
+//     so the preparation starts only after the wait.
 // A call without candidates has no preparation and scenarios to hand that on: it
-// waits first.
+// waits first. Calls are counted as they are queued; those that a stream capture
+// records are counted by themselves (sequence_of).
 cudaError_t launch_thresh(Set& set, int floors, int th_bound, cudaStream_t s, int late) {
   const Dims& d = set.d;
   const int bound = th_bound > 0 ? std::min(th_bound, d.theta_cap) : d.theta_cap;
