@@ -476,11 +476,9 @@ cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t s
   return cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
 }
 
-// Per-model launch state: whether floors are set, and the launch shapes
-// (filled on first use) per kernel instance: [floors] for the solve and the
-// preparation, [path][floors] for the scorer (plain, dump, table over one
-// problem, table over several).
-// The preparation's and the scorer's instances are indexed by mode = floors +
+// Per-model launch state: whether floors are set, and the launch shapes (filled on
+// first use) per kernel instance: [mode] for the preparation, [path][mode] for the
+// scorer (plain, dump, table over one problem, table over several), mode = floors +
 // 2 prior (0..3).
 constexpr int kScoreVariants = 4;
 struct LaunchCache {

@@ -235,3 +235,39 @@ def test_inputs_replaced_while_calls_run_on_another_stream(fsb, cuda, oracle_lib
     for x in sums:
         assert np.array_equal(x.cpu().numpy(), ref.sum_eo)
     assert np.array_equal(sums2.cpu().numpy(), ref2.sum_eo)
+
+
+def test_records_past_the_second_buffer(fsb, cuda, oracle_lib):
+    """Calls whose records do not fit the second buffer (32 MiB: more than 1842
+    candidates here) among calls whose records do, in a mixed order without a wait,
+    with plans of many and few samples and bounds replaced in between."""
+    torch = cuda
+    w = workloads.make_workload(1)
+    ws = [w, dataclasses.replace(w, cap_lo=w.cap_lo * np.float32(0.5), cap_hi=w.cap_hi * np.float32(0.75))]
+    rng = np.random.default_rng(12)
+    O = 8
+    plans = [(rng.permutation(np.tile(w.candidates, 32))[:n].astype(np.int32), S)
+             for n, S in ((2000, 1500), (1800, 1500), (64, 4096), (2000, 60), (16, 60))]
+    ref = {}
+    for b, x in enumerate(ws):
+        with load_model(fsb, x) as m:
+            for k, (cand, S) in enumerate(plans):
+                ref[k, b] = fsb.fs_score_candidates(m, cand, O, S, k)
+    order = [int(k) for k in rng.integers(len(plans), size=48)]
+    order[:8] = [0, 0, 2, 1, 0, 1, 1, 2]  # (large first, then each change of buffer)
+    at = [int(b) for b in np.cumsum(rng.random(48) < 0.2) % 2]
+    dev = [torch.from_numpy(c).cuda() for c, _ in plans]
+    sums = [torch.zeros((len(plans[k][0]), O), dtype=torch.int64, device="cuda") for k in order]
+    best = torch.zeros(len(order), dtype=torch.int32, device="cuda")
+    torch.cuda.synchronize()
+    with load_model(fsb, ws[at[0]]) as m:
+        for i, k in enumerate(order):
+            if i and at[i] != at[i - 1]:
+                x = ws[at[i]]
+                fsb.fs_update_bounds(m, x.cap_lo, x.cap_hi, x.tail_lo, x.tail_hi)
+            fsb.fs_score_candidates_async(m, dev[k], O, plans[k][1], k, best_dev=best[i:i + 1], sum_eo_dev=sums[i])
+        fsb.fs_check(m)
+        torch.cuda.synchronize()
+    for i, k in enumerate(order):
+        assert np.array_equal(sums[i].cpu().numpy(), ref[k, at[i]].sum_eo), (i, k)
+        assert int(best[i]) == ref[k, at[i]].best, (i, k)

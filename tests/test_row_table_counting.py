@@ -1,15 +1,15 @@
-"""The counting rule behind the base solve's row table, on the CPU.
+"""The counting rule behind the thresholds' ranks, on the CPU.
 
 A row (capacity c, demand lambda, at most M replicas) covers a threshold t with
 its smallest n such that f(n) = min(1, RN(RN(n c) / lambda)) >= t (Section 3,
-Eqs. 2 and 4; a critical class covers max(t, delta)). The GPU solve does not
-evaluate f for every (row, threshold): it counts how many of the row's own
-values f(n0) <= ... <= f(len) lie below t, where n0 is the first n with
-f(n) >= max(delta, the smallest positive float) and len the first n with
-f(n) = 1 (else M), and takes n0 plus that count (no cover when every value is
-below t). This checks that rule against brute force with the oracle's
-fulfilment arithmetic, at thresholds taken from the row's own values, their
-float neighbours and elsewhere in (0, 1].
+Eqs. 2 and 4; a critical class covers max(t, delta)). Of the row's own values
+f(n0) <= ... <= f(len), where n0 is the first n with f(n) >= max(delta, the
+smallest positive float) and len the first n with f(n) = 1 (else M), as many lie
+below t as that cover is above n0, and all of them when there is no cover. The
+GPU's thresholds kernel takes those counts from the covers: their sum over the
+rows is t's rank in the sorted set, so that it needs no sort. This checks the
+rule against brute force with the oracle's fulfilment arithmetic, at thresholds
+taken from the row's own values, their float neighbours and elsewhere in (0, 1].
 """
 
 import numpy as np
