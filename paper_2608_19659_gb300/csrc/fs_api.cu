@@ -165,7 +165,7 @@ using namespace fs;
 // them left it.
 struct Sequence {
   int half = 0;             // the set of parts of t*, sums and counters that it used
-  bool queued = false;      // all its kernels were queued, and its scenarios did not read the rows (no dump)
+  bool queued = false;      // all its kernels were queued (it had candidates), and none reads the rows late (no dump)
   bool one_buffer = false;  // its records went to the first buffer whatever the half
 };
 
@@ -539,7 +539,7 @@ int run_score(fs_model* m, Set set, const fs_samples* smp, const int32_t* cand_d
   FS_CUDA(launch_finalize(set, it, pl, sums, gap, score, gamma_t, best, status_copy,
                           sums + (size_t)std::max(n, 1) * smp->O, sum_out, s),
           "launch finalize");
-  seq.queued = late && !dump;  // (nothing of a synchronous call is left to overlap)
+  seq.queued = late && !dump && n > 0;  // (nothing of a synchronous call is left to overlap)
   if (phases) FS_CUDA(cudaEventRecord(ev[4], s), "record timing event");
   return FS_OK;
 }

@@ -196,7 +196,7 @@ __global__ void __launch_bounds__(kThreshThreads) k_thresh(Set set, int late) {
 // 270 -> 206 us, 1024 x 8 x 60 116 -> 51 us; four classes, 64 GPUs 51 -> 45 us.
 //
 // late: for a scoring call n on the model's own device bounds, of at least one
-// candidate, after another on its stream. What may still run when it starts is
+// candidate, after another such call. What may still run when it starts is
 // call n - 1's scenarios and reduction: that reduction let this kernel start, and
 // was itself let start by the scenarios, after call n - 1's preparation and so
 // (each waits for its predecessor) its thresholds had finished, which had waited
@@ -212,7 +212,7 @@ __global__ void __launch_bounds__(kThreshThreads) k_thresh(Set set, int late) {
 //     Late 1: one of them keeps its records in the first buffer whatever its turn,
 //     so the preparation starts only after the wait.
 // A call without candidates has no preparation and scenarios to hand that on: it
-// waits first. Calls are counted as they are queued; those that a stream capture
+// and the call after it wait first. Calls are counted as they are queued; those that a stream capture
 // records are counted by themselves (sequence_of).
 cudaError_t launch_thresh(Set& set, int floors, int th_bound, cudaStream_t s, int late) {
   const Dims& d = set.d;
